@@ -46,6 +46,8 @@ struct KrylovDev {
   double w2[2];           // selective reorthogonalisation: ||w||^2 before the projection
   int reorth[2];          // ... this Arnoldi step needs the second Gram-Schmidt pass
   int reorth_count[2];    // Arnoldi steps of this time step that took the second pass
+  double hsq[2];          // ||w||^2 after both Gram-Schmidt passes (CGS2)
+  int corr32;             // the second pass's update may be formed in FP32 (k_orth_close)
 };
 
 // Preconditioned MINRES scalars of one run, per species (the Lanczos process on P^-1 A in the
@@ -295,8 +297,10 @@ __global__ void k_scale4(Seg sg, const double4_32a* src, double4_32a* dst, const
 // ---------------------------------------------------------------- Gram-Schmidt passes
 // Classical Gram-Schmidt twice (CGS2, gs_reorth = 0):
 // MODE 0: h1[s][k] = <V_k, W>_s                       k = 0..nv-1
-// MODE 1: W -= sum_k h1[s][k] V_k;  h2[s][k] = <V_k, W>_s
-// MODE 2: W -= sum_k h2[s][k] V_k;  ||W||_s^2, then the Hessenberg / Givens update (last block)
+// MODE 1: W -= sum_k h1[s][k] V_k;  h2[s][k] = <V_k, W>_s and ||W||_s^2, hence the norm after the
+//         second projection, ||W - V h2||^2 = ||W||^2 - ||h2||^2 (V orthonormal)
+// then k_orth_close: V_{j+1} = (W - sum_k h2[s][k] V_k) / h_{j+1,j} and, beside it, the column's Givens
+// update.
 // Selective reorthogonalisation (gs_reorth = 1; Daniel, Gragg, Kaufman and Stewart 1976): MODE 0
 // with with_norm also records ||W||_s^2, then
 // MODE 3: W -= sum_k h1[s][k] V_k;  ||W||_s^2; a species whose norm kept at least half its square
@@ -306,6 +310,7 @@ __global__ void k_scale4(Seg sg, const double4_32a* src, double4_32a* dst, const
 // MODE 5: W -= sum_k h2[s][k] V_k;  ||W||_s^2, the column of the flagged species
 // Blocks of a run with no flagged species leave MODE 4 and 5 at entry.
 // <a, b>_s sums components (x, z) for species 0 and (y, w) for species 1 over the run's nodes.
+constexpr double ORTH_CORR32 = 0x1p-30;  // largest |h2_k| / ||W|| whose correction may be formed in FP32
 constexpr int KC = 16;                // basis vectors per chunk: 2 KC = 32 values, one per lane
 constexpr int ORTH_BLOCKS = 152 * 2;  // target grid of the segmented kernels (2 blocks per SM)
 // threads per block of the Gram-Schmidt passes; measured (ms per step, 512 x 512 FP64 / mixed /
@@ -367,10 +372,10 @@ __device__ __forceinline__ double block_sum_n(int nvals, double (&a)[32], double
   return block_sum_v<NT, 32>(a, sm);
 }
 
-// W[v] -= sum_{k < nv} c[s][k] V_k[v] for one node (two partial sums, even / odd k, halve the
+// w -= sum_{k < nv} c[s][k] V_k[v] for one node (two partial sums, even / odd k, halve the
 // FP64 dependency chains)
-__device__ __forceinline__ void orth_update_node(const double4_32a* __restrict__ V, double4_32a* __restrict__ W,
-                                                 size_t N, int nv, const double (*coef)[MAXM + 1], int v) {
+__device__ __forceinline__ void orth_update_value(const double4_32a* __restrict__ V, double4_32a& w, size_t N,
+                                                  int nv, const double (*coef)[MAXM + 1], int v) {
   double ax = 0, ay = 0, az = 0, aw = 0, bx = 0, by = 0, bz = 0, bw = 0;
   int k = 0;
   for (; k + 1 < nv; k += 2) {
@@ -385,24 +390,35 @@ __device__ __forceinline__ void orth_update_node(const double4_32a* __restrict__
     ax = fma(coef[0][k], q0.x, ax); az = fma(coef[0][k], q0.z, az);
     ay = fma(coef[1][k], q0.y, ay); aw = fma(coef[1][k], q0.w, aw);
   }
-  double4_32a w = W[v];
   w.x -= ax + bx;
   w.y -= ay + by;
   w.z -= az + bz;
   w.w -= aw + bw;
+}
+
+// W[v] -= sum_{k < nv} c[s][k] V_k[v] for one node
+__device__ __forceinline__ void orth_update_node(const double4_32a* __restrict__ V, double4_32a* __restrict__ W,
+                                                 size_t N, int nv, const double (*coef)[MAXM + 1], int v) {
+  double4_32a w = W[v];
+  orth_update_value(V, w, N, nv, coef, v);
   W[v] = w;
 }
 
 // Dots of W with the KW basis vectors k0 .. k0+KW-1 over this thread's nodes, into acc[2t] (species
 // 0) and acc[2t+1] (species 1).  KW is exact, so no FP64 slot is spent on absent vectors.  With
-// UPD the node is first updated with all nv vectors (the same vectors are then re-read from L1).
+// UPD the node is first updated with all nv vectors (the same vectors are then re-read from L1) and
+// the updated vector's squared norm is taken, into nrm[0], nrm[1].
 template <int KW, bool UPD>
 __device__ __forceinline__ void orth_dots_chunk(const double4_32a* __restrict__ V, double4_32a* __restrict__ W,
                                                 size_t N, int k0, int nv, const double (*coef)[MAXM + 1],
-                                                int v0, int v1, double (&acc)[32]) {
+                                                int v0, int v1, double (&acc)[32], double (&nrm)[2]) {
   for (int v = v0; v < v1; v += blockDim.x) {
     if (UPD) orth_update_node(V, W, N, nv, coef, v);
     const double4_32a w = W[v];
+    if (UPD) {
+      nrm[0] = fma(w.x, w.x, fma(w.z, w.z, nrm[0]));
+      nrm[1] = fma(w.y, w.y, fma(w.w, w.w, nrm[1]));
+    }
 #pragma unroll
     for (int t = 0; t < KW; ++t) {
       const double4_32a q = V[(size_t)(k0 + t) * N + v];
@@ -416,13 +432,13 @@ template <bool UPD>
 __device__ __forceinline__ void orth_dots_dispatch(int kw, const double4_32a* __restrict__ V,
                                                    double4_32a* __restrict__ W, size_t N, int k0, int nv,
                                                    const double (*coef)[MAXM + 1], int v0, int v1,
-                                                   double (&acc)[32]) {
+                                                   double (&acc)[32], double (&nrm)[2]) {
 #define CH_ORTH_CASE(n) \
-  case n: orth_dots_chunk<n, UPD>(V, W, N, k0, nv, coef, v0, v1, acc); break;
+  case n: orth_dots_chunk<n, UPD>(V, W, N, k0, nv, coef, v0, v1, acc, nrm); break;
   switch (kw) {
     CH_ORTH_CASE(1) CH_ORTH_CASE(2) CH_ORTH_CASE(3) CH_ORTH_CASE(4) CH_ORTH_CASE(5) CH_ORTH_CASE(6)
     CH_ORTH_CASE(7) CH_ORTH_CASE(8) CH_ORTH_CASE(9) CH_ORTH_CASE(10) CH_ORTH_CASE(11) CH_ORTH_CASE(12)
-    CH_ORTH_CASE(13) CH_ORTH_CASE(14) CH_ORTH_CASE(15) default: orth_dots_chunk<16, UPD>(V, W, N, k0, nv, coef, v0, v1, acc);
+    CH_ORTH_CASE(13) CH_ORTH_CASE(14) CH_ORTH_CASE(15) default: orth_dots_chunk<16, UPD>(V, W, N, k0, nv, coef, v0, v1, acc, nrm);
   }
 #undef CH_ORTH_CASE
 }
@@ -460,8 +476,10 @@ __device__ __forceinline__ void stage_columns(const KrylovDev* kd, int j, bool o
 
 // Column j of the Arnoldi process for species sp once w is orthogonal to V_0..V_j with squared norm
 // hsq, from the staged h and rotations: h_{j+1} = ||w||, the previous Givens rotations, a new one, the
-// residual estimate |g_{j+1}| and the cycle's stopping tests.
-__device__ __forceinline__ void arnoldi_column(KrylovDev* kd, int sp, int j, double hsq, ColumnStage* cst) {
+// residual estimate |g_{j+1}| and the cycle's stopping tests.  set_hinv = false: 1 / h_{j+1} is already
+// in place (and being read).
+__device__ __forceinline__ void arnoldi_column(KrylovDev* kd, int sp, int j, double hsq, ColumnStage* cst,
+                                               bool set_hinv) {
   double* h = cst->h[sp];
   const double hn = sqrt(hsq);
   double cur = h[0];  // entry k after the rotations 0..k-1
@@ -487,7 +505,7 @@ __device__ __forceinline__ void arnoldi_column(KrylovDev* kd, int sp, int j, dou
   kd->its[sp] = cst->its[sp] + 1;
   if (!isfinite(hn) || !isfinite(den)) kd->nonfinite = 1;
   const bool breakdown = !(hn > 1e-300);
-  kd->hinv[sp] = breakdown ? 0.0 : 1.0 / hn;
+  if (set_hinv) kd->hinv[sp] = breakdown ? 0.0 : 1.0 / hn;
   if (fabs(gj1) <= cst->tol[sp] || breakdown || den == 0.0) kd->cycle_active[sp] = 0;
 }
 
@@ -502,7 +520,7 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
   KrylovDev* kd = kds + run;
   if (MODE >= 4 && !(kd->reorth[0] | kd->reorth[1])) return;  // the run needs no second pass
   const int v0 = sg.lo[blockIdx.x] + threadIdx.x, v1 = sg.hi[blockIdx.x];
-  if (MODE == 1 || MODE == 2 || MODE == 3 || MODE == 5) {
+  if (MODE == 1 || MODE == 3 || MODE == 5) {
     const bool first = MODE == 1 || MODE == 3;
     for (int k = threadIdx.x; k < nv; k += blockDim.x) {
       coef[0][k] = first ? kd->h1[0][k] : kd->h2[0][k];
@@ -510,11 +528,13 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
     }
     __syncthreads();
   }
-  if (MODE == 2 || MODE == 3 || MODE == 5) {
+  if (MODE == 3 || MODE == 5) {
     for (int v = v0; v < v1; v += blockDim.x) orth_update_node(V, W, (size_t)N, nv, coef, v);
   }
   const int b0 = sg.first[run], b1 = sg.first[run + 1];
   if (DOTS) {
+    const bool norm = MODE == 1 || (MODE == 0 && with_norm);
+    double nrm[2] = {0.0, 0.0};
     for (int k0 = 0; k0 < nv; k0 += KC) {
       double acc[32];
 #pragma unroll
@@ -522,22 +542,23 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
       const int kw = nv - k0 < KC ? nv - k0 : KC;
       // MODE 1: the update of each node is fused into the first chunk's dots
       if (MODE == 1 && k0 == 0)
-        orth_dots_dispatch<true>(kw, V, W, (size_t)N, k0, nv, coef, v0, v1, acc);
+        orth_dots_dispatch<true>(kw, V, W, (size_t)N, k0, nv, coef, v0, v1, acc, nrm);
       else
-        orth_dots_dispatch<false>(kw, V, W, (size_t)N, k0, nv, coef, v0, v1, acc);
+        orth_dots_dispatch<false>(kw, V, W, (size_t)N, k0, nv, coef, v0, v1, acc, nrm);
       const double tot = block_sum_n<ORTH_TPB>(2 * kw, acc, sm);
       if (threadIdx.x < 2 * kw) partials[(size_t)blockIdx.x * MAXV + 2 * k0 + threadIdx.x] = tot;
     }
-    const bool norm = MODE == 0 && with_norm;
-    if (norm) {  // ||W||_s^2 before the projection, into the slots after the dots
-      double acc[32];
-#pragma unroll
-      for (int t = 0; t < 32; ++t) acc[t] = 0.0;
+    if (MODE == 0 && with_norm) {  // ||W||_s^2 before the projection
       for (int v = v0; v < v1; v += blockDim.x) {
         const double4_32a w = W[v];
-        acc[0] = fma(w.x, w.x, fma(w.z, w.z, acc[0]));
-        acc[1] = fma(w.y, w.y, fma(w.w, w.w, acc[1]));
+        nrm[0] = fma(w.x, w.x, fma(w.z, w.z, nrm[0]));
+        nrm[1] = fma(w.y, w.y, fma(w.w, w.w, nrm[1]));
       }
+    }
+    if (norm) {  // the norms go into the slots after the dots
+      double acc[32];
+      acc[0] = nrm[0];
+      acc[1] = nrm[1];
       const double bt = block_sum_v<ORTH_TPB, 2>(acc, sm);
       if (threadIdx.x < 2) partials[(size_t)blockIdx.x * MAXV + 2 * nv + threadIdx.x] = bt;
     }
@@ -549,12 +570,38 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
       dst0[k] = MODE == 4 && !kd->reorth[0] ? 0.0 : tot[2 * k];
       dst1[k] = MODE == 4 && !kd->reorth[1] ? 0.0 : tot[2 * k + 1];
     }
-    if (norm && threadIdx.x < 2) kd->w2[threadIdx.x] = tot[2 * nv + threadIdx.x];
+    if (MODE == 0 && norm && threadIdx.x < 2) kd->w2[threadIdx.x] = tot[2 * nv + threadIdx.x];
+    if (MODE == 1 && threadIdx.x < 64) {  // warp s: ||W - V h2||_s^2 and 1 / h_{j+1,j} of species s
+      const int sp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+      double q = 0.0, mx = 0.0;
+      for (int k = lane; k < nv; k += 32) {
+        const double h = tot[2 * k + sp];
+        q = fma(h, h, q);
+        mx = fmax(mx, fabs(h));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        q += __shfl_xor_sync(0xffffffffu, q, o);
+        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      }
+      if (lane == 0) {
+        const double w2 = tot[2 * nv + sp];
+        double hsq = w2 - q;
+        if (hsq < 0.0) hsq = 0.0;  // (a NaN stays a NaN)
+        const double hn = sqrt(hsq);
+        kd->hsq[sp] = hsq;
+        kd->hinv[sp] = (kd->cycle_active[sp] && hn > 1e-300) ? 1.0 / hn : 0.0;
+        sm[sp] = (isfinite(w2) && isfinite(q) && mx <= ORTH_CORR32 * sqrt(w2)) ? 1.0 : 0.0;
+      }
+    }
+    if (MODE == 1) {
+      __syncthreads();
+      if (threadIdx.x == 0) kd->corr32 = sm[0] != 0.0 && sm[1] != 0.0;
+    }
     if (threadIdx.x == 0) kd->ticket = 0;
   } else {
     double acc[32];
-#pragma unroll
-    for (int t = 0; t < 32; ++t) acc[t] = 0.0;
+    acc[0] = acc[1] = 0.0;
     for (int v = v0; v < v1; v += blockDim.x) {
       const double4_32a w = W[v];
       acc[0] = fma(w.x, w.x, fma(w.z, w.z, acc[0]));
@@ -568,19 +615,12 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
     stage_columns(kd, nv - 1, MODE == 3, &cst);
     if (threadIdx.x < 2) {
       const int sp = threadIdx.x;
-      if (MODE == 2) {
-        if (cst.active[sp]) {
-          arnoldi_column(kd, sp, nv - 1, tot[sp], &cst);
-          kd->reorth_count[sp] = cst.rcount[sp] + 1;
-        } else {
-          kd->hinv[sp] = 0.0;
-        }
-      } else if (MODE == 3) {
+      if (MODE == 3) {
         kd->reorth[sp] = 0;
         if (kd->cycle_active[sp]) {
           if (tot[sp] >= 0.5 * kd->w2[sp]) {
             for (int k = 0; k < nv; ++k) kd->h2[sp][k] = 0.0;
-            arnoldi_column(kd, sp, nv - 1, tot[sp], &cst);
+            arnoldi_column(kd, sp, nv - 1, tot[sp], &cst, true);
           } else {
             kd->reorth[sp] = 1;
           }
@@ -588,7 +628,7 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
           kd->hinv[sp] = 0.0;
         }
       } else if (kd->reorth[sp]) {  // MODE 5
-        arnoldi_column(kd, sp, nv - 1, tot[sp], &cst);
+        arnoldi_column(kd, sp, nv - 1, tot[sp], &cst, true);
         kd->reorth_count[sp] += 1;
       }
     }
@@ -597,6 +637,79 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
       if (threadIdx.x < 2) kd->reorth[threadIdx.x] = 0;
     }
     if (threadIdx.x == 0) kd->ticket = 0;
+  }
+}
+
+// v rounded towards zero to FP32 by integer operations (the conversion instruction runs at the FP64
+// pipe's rate).  For |v| < 2^128; values below FP32's normal range come out as zero or denormal.
+__device__ __forceinline__ float trunc_f32(double v) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const int e = max((hi & 0x7fffffff) - 0x38000000, 0);  // exponent bias 1023 -> 127
+  return __int_as_float((int)__funnelshift_l((unsigned)lo, (unsigned)e, 3) | (hi & 0x80000000));
+}
+
+// The end of CGS2: V_{j+1} = (W - sum_k h2[s][k] V_k) / h_{j+1,j} (0 for a species that sits out).  W
+// itself is not written: the next Arnoldi step overwrites it.  The blocks past the segments, one per
+// run, apply the column's Givens rotations meanwhile.
+//
+// h2 is the rounding error that the first projection left (1e-16 to 1e-14 of ||W||), so where every
+// |h2_k| <= 2^-30 ||W|| (kd->corr32) the correction V h2 is formed in FP32: its error, nv 2^-23 2^-30
+// ||W|| |V_k[v]|, is below the FP64 rounding of W, and the FP64 pipe (2 FMA per clock and SM, what
+// bounds these passes) is left with three instructions per component instead of nv + 2.  A larger h2
+// (a vector that lies almost in the span of the basis) or a non-finite value takes the FP64 sum.
+// Measured (512 x 512, 10 basis vectors on average): this pass and the normalisation it now includes
+// 43.6 us before (FP64 update with its own norm reduction, then a scaling kernel).
+__global__ void __launch_bounds__(ORTH_TPB, 2) k_orth_close(Seg sg, int N, int nv, const double4_32a* __restrict__ V,
+                                                            const double4_32a* __restrict__ W,
+                                                            double4_32a* __restrict__ vnext, KrylovDev* kds) {
+  if ((int)blockIdx.x >= sg.nblocks) {
+    KrylovDev* kd = kds + ((int)blockIdx.x - sg.nblocks);
+    __shared__ ColumnStage cst;
+    stage_columns(kd, nv - 1, false, &cst);
+    if (threadIdx.x < 2) {
+      const int sp = threadIdx.x;
+      if (cst.active[sp]) {
+        arnoldi_column(kd, sp, nv - 1, kd->hsq[sp], &cst, false);
+        kd->reorth_count[sp] = cst.rcount[sp] + 1;
+      }
+    }
+    return;
+  }
+  __shared__ double coef[2][MAXM + 1];
+  __shared__ float coef32[2][MAXM + 1];
+  const KrylovDev* kd = kds + sg.run[blockIdx.x];
+  for (int k = threadIdx.x; k < nv; k += blockDim.x) {
+    const double h0 = kd->h2[0][k], h1 = kd->h2[1][k];
+    coef[0][k] = h0;
+    coef[1][k] = h1;
+    coef32[0][k] = (float)h0;
+    coef32[1][k] = (float)h1;
+  }
+  const double s0 = kd->hinv[0], s1 = kd->hinv[1];
+  const bool c32 = kd->corr32 != 0;
+  __syncthreads();
+  const int v1 = sg.hi[blockIdx.x];
+  for (int v = sg.lo[blockIdx.x] + threadIdx.x; v < v1; v += blockDim.x) {
+    double4_32a w = W[v];
+    if (c32) {
+      float ax = 0.f, ay = 0.f, az = 0.f, aw = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < nv; ++k) {
+        const double4_32a q = V[(size_t)k * N + v];
+        const float c0 = coef32[0][k], c1 = coef32[1][k];
+        ax = fmaf(c0, trunc_f32(q.x), ax);
+        ay = fmaf(c1, trunc_f32(q.y), ay);
+        az = fmaf(c0, trunc_f32(q.z), az);
+        aw = fmaf(c1, trunc_f32(q.w), aw);
+      }
+      w.x -= (double)ax;
+      w.y -= (double)ay;
+      w.z -= (double)az;
+      w.w -= (double)aw;
+    } else {
+      orth_update_value(V, w, (size_t)N, nv, coef, v);
+    }
+    vnext[v] = make_double4_32a(w.x * s0, w.y * s1, w.z * s0, w.w * s1);
   }
 }
 
@@ -1151,8 +1264,8 @@ static ch_status read_flags(ch_state_s* S, cudaStream_t st) {
 
 static double res4_bytes(const ch_system_s* s) { return 20.0 * s->nnz + 4.0 * (s->N + 1) + 96.0 * s->N; }
 
-// One Arnoldi step j for all systems: Z_j = Prec(V_j) (Algorithm 1), W = A Z_j, CGS2 against
-// V_0..V_j with the Givens update and V_{j+1} = W / h_{j+1,j}.  Everything is enqueued on `st`
+// One Arnoldi step j for all systems: Z_j = Prec(V_j) (Algorithm 1), W = A Z_j, Gram-Schmidt against
+// V_0..V_j, the Givens update and V_{j+1} = W / h_{j+1,j}.  Everything is enqueued on `st`
 // with no host synchronisation, so it can be captured.
 static ch_status arnoldi_step(ch_state_s* S, int j, cudaStream_t st) {
   const ch_system_s* s = S->sys;
@@ -1183,23 +1296,23 @@ static ch_status arnoldi_step(ch_state_s* S, int j, cudaStream_t st) {
       ProfScope ps(st, K_ORTH_RE, 0, (nv + 2) * n32, 4.0 * nv * N + 4.0 * N);
       k_orth<5><<<nb, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, S->partials, S->kd);
     }
+    {
+      ProfScope ps(st, K_SCALE4, 0, 64.0 * N, 0.0);
+      k_scale4<<<nb, TPB, 0, st>>>(S->seg, W4, V4 + (size_t)(j + 1) * N, S->kd);
+    }
   } else {
     {
       ProfScope ps(st, K_ORTH0, 0, (nv + 1) * n32, 4.0 * nv * N);
       k_orth<0><<<nb, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, S->partials, S->kd);
     }
     {
-      ProfScope ps(st, K_ORTH1, 0, (nv + 2) * n32, 8.0 * nv * N);
+      ProfScope ps(st, K_ORTH1, 0, (nv + 2) * n32, 8.0 * nv * N + 4.0 * N);
       k_orth<1><<<nb, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, S->partials, S->kd);
     }
     {
-      ProfScope ps(st, K_ORTH2, 0, (nv + 2) * n32, 4.0 * nv * N + 4.0 * N);
-      k_orth<2><<<nb, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, S->partials, S->kd);
+      ProfScope ps(st, K_ORTH2, 0, (nv + 2) * n32, 12.0 * N);
+      k_orth_close<<<nb + S->R, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, V4 + (size_t)(j + 1) * N, S->kd);
     }
-  }
-  {
-    ProfScope ps(st, K_SCALE4, 0, 64.0 * N, 0.0);
-    k_scale4<<<nb, TPB, 0, st>>>(S->seg, W4, V4 + (size_t)(j + 1) * N, S->kd);
   }
   CH_LAUNCHED();
   return CH_OK;
