@@ -29,36 +29,32 @@ template <typename T> struct V2T;
 template <> struct V2T<double> { using t = double2; };
 template <> struct V2T<float> { using t = float2; };
 
-// Fine-level operator of a uniform mesh as diagonals: row i's neighbours sit at i + lat_off(d),
-// the lattice directions a + b W + c WH (W, WH: the row's run's strides), ascending in d for any
-// W, H >= 2, i.e. in CSR column order; val[d * n + i] is zero where row i has no such neighbour
-// (the clamped column index is then read but multiplied by zero).
+// Fine-level operator of a uniform mesh in lattice form: node i's neighbours sit at i + lat_off(d)
+// and its row is the table row of its class id (Lattice): nd values in ascending direction, i.e. in
+// CSR column order (zero where the class has no such neighbour: the clamped index is then read but
+// multiplied by zero), padded to `ts` with the class's factor in slot nd (LatTab).  The assembled
+// rows of a class agree to the rounding of the node coordinates (checked at set-up, below 2^-36 of
+// the diagonal), and the table holds those of the class's representative node.
 template <typename T>
-struct Dia {
+struct LatOp {
   int nd = 0;                      // 7 (2D) or 15 (3D); 0: not structured, use the CSR form
-  int W = 0, WH = 0;               // strides of a single-run mesh
-  const int* node_run = nullptr;   // several runs: run of each row ...
-  const int2* run_wh = nullptr;    // ... and (W, WH) of each run
-  T* val = nullptr;
+  int ts = 0;                      // values per table row: 8 or 16
+  Lattice L;
+  const T* tab = nullptr;          // nids x ts: the operator's rows (slot nd: 1 / diagonal)
+  // FP64: the Chebyshev steps' tables (deg x nids x ts each, see lat_step_tables); FP32 steps use tab
+  T* steps = nullptr;              // of the V-cycle's smoother
+  T* semi = nullptr;               // of the semi-iteration (precond_M = 1)
+  T* scratch = nullptr;            // of ch_smooth's own degree, rebuilt by each call
 };
-
-// direction d of the 2D (7: uniform triangles) or 3D (15: Kuhn tetrahedra) lattice stencil
-__host__ __device__ __forceinline__ int lat_off(int nd, int d, int W, int WH) {
-  constexpr int a2[7] = {-1, 0, -1, 0, 1, 0, 1}, b2[7] = {-1, -1, 0, 0, 0, 1, 1};
-  constexpr int a3[15] = {-1, 0, -1, 0, -1, 0, -1, 0, 1, 0, 1, 0, 1, 0, 1};
-  constexpr int b3[15] = {-1, -1, 0, 0, -1, -1, 0, 0, 0, 1, 1, 0, 0, 1, 1};
-  constexpr int c3[15] = {-1, -1, -1, -1, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1};
-  return nd == 7 ? a2[d] + b2[d] * W : a3[d] + b3[d] * W + c3[d] * WH;
-}
 
 template <typename T>
 struct LevelT {
   Csr<T> A, P, R;
-  Dia<T> dia;                          // level 0 of a structured mesh
+  LatOp<T> lat;                        // level 0 of a structured mesh
   int tprA = 1, tprP = 1, tprR = 1;  // lanes per row of the SpMV-type kernels (autotuned)
   bool pdl = false;                  // launch the V-cycle kernels as programmatic dependents
   T* dinv = nullptr;
-  typename V2T<T>::t *x = nullptr, *x2 = nullptr, *d = nullptr, *r = nullptr, *b = nullptr;
+  typename V2T<T>::t *x = nullptr, *x2 = nullptr, *r = nullptr, *b = nullptr;
 };
 
 struct Hierarchy {
@@ -78,6 +74,7 @@ struct Hierarchy {
   double cheb_lower = 0.3;
   int autotune = 1;
   bool pdl = true;
+  double* lat_tab = nullptr;          // FP64 table of the finest level's lattice form (null: CSR form)
   Alloc mem;
 };
 
@@ -567,7 +564,7 @@ static ch_status level_setup(Hierarchy* h, int l, const ch_params& p, cudaStream
 
 template <typename T, typename V2>
 static void launch_residual(int tpr, const Csr<T>& A, const V2* b, const V2* x, V2* r, cudaStream_t st,
-                            const Dia<T>* dia = nullptr, bool pdl = false);
+                            const LatOp<T>* lat = nullptr, bool pdl = false);
 template <typename T, typename V2, bool ACC>
 static void launch_spmv2(int tpr, const Csr<T>& A, const V2* x, V2* y, cudaStream_t st, bool pdl = false);
 
@@ -646,12 +643,12 @@ static ch_status autotune_levels(Hierarchy* h, std::vector<LevelT<T>>& L, int mo
   using V2 = typename V2T<T>::t;
   for (int l = 0; l < h->nlev; ++l) {
     const int n = L[l].A.nrows;
-    V2* vecs[5] = {L[l].x, L[l].x2, L[l].d, L[l].r, L[l].b};
-    for (int k = 0; k < 5; ++k) CH_CUDA(cudaMemsetAsync(vecs[k], 0, sizeof(V2) * n, st));
+    V2* vecs[4] = {L[l].x, L[l].x2, L[l].r, L[l].b};
+    for (int k = 0; k < 4; ++k) CH_CUDA(cudaMemsetAsync(vecs[k], 0, sizeof(V2) * n, st));
   }
   for (int l = 0; l < h->nlev; ++l) {
     LevelT<T>& W = L[l];
-    W.tprA = W.dia.nd ? 1
+    W.tprA = W.lat.nd ? 1
                       : tune_tpr(0, W.A.nrows, W.A.ncols, W.A.nnz, sizeof(T), mode,
                                  [&](int t) { launch_residual<T, V2>(t, W.A, W.b, W.x, W.r, st); }, st);
     if (l + 1 < h->nlev) {
@@ -667,73 +664,120 @@ static ch_status autotune_levels(Hierarchy* h, std::vector<LevelT<T>>& L, int mo
   return CH_OK;
 }
 
-__global__ void k_csr_to_dia(Csr<double> A, Dia<double> D) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= A.nrows) return;
-  int W = D.W, WH = D.WH;
-  if (D.node_run) {
-    const int2 w = D.run_wh[D.node_run[i]];
-    W = w.x;
-    WH = w.y;
-  }
-  for (int q = A.rowptr[i]; q < A.rowptr[i + 1]; ++q) {
-    const int o = A.col[q] - i;
-    for (int d = 0; d < D.nd; ++d)
-      if (lat_off(D.nd, d, W, WH) == o) D.val[(size_t)d * A.nrows + i] = A.val[q];
-  }
+// Table rows of the lattice form from the representative nodes' CSR rows (slot nd: 1 / diagonal).
+__global__ void k_lat_table(Csr<double> A, Lattice L, int nd, int ts, double* tab) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  if (id >= L.nids) return;
+  const int i = L.rep[id];
+  const int2 w = L.wh[id];
+  double* row = tab + (size_t)id * ts;
+  for (int d = 0; d < ts; ++d) row[d] = 0.0;
+  for (int q = A.rowptr[i]; q < A.rowptr[i + 1]; ++q)
+    for (int d = 0; d < nd; ++d)
+      if (lat_off(nd, d, w.x, w.y) == A.col[q] - i) row[d] = A.val[q];
+  row[nd] = 1.0 / row[nd / 2];
 }
 
-// The diagonal form of A when every stored entry of every row lies on the lattice stencil of its
-// run (checked on the host from the pattern at set-up); else nd = 0 and the level stays CSR.
-static ch_status dia_build(const Csr<double>& A, const FineLattice* lat, Alloc& mem, Dia<double>* out,
-                           cudaStream_t st) {
-  out->nd = 0;
-  if (!lat || (lat->dim != 2 && lat->dim != 3)) return CH_OK;
-  const int n = A.nrows, R = (int)lat->W.size();
-  if (R < 1 || (int)lat->run_off.size() != R + 1 || lat->run_off[R] != n) return CH_OK;
-  const int nd = lat->dim == 2 ? 7 : 15;
-  std::vector<int> rp(n + 1), col((size_t)A.nnz);
-  CH_CUDA(cudaMemcpyAsync(rp.data(), A.rowptr, sizeof(int) * (n + 1), cudaMemcpyDeviceToHost, st));
-  CH_CUDA(cudaMemcpyAsync(col.data(), A.col, sizeof(int) * (size_t)A.nnz, cudaMemcpyDeviceToHost, st));
-  CH_CUDA(cudaStreamSynchronize(st));
-  for (int r = 0; r < R; ++r) {
-    const int W = lat->W[r], WH = lat->WH[r];
-    if (W < 2 || WH < 2 * W) return CH_OK;
-    int offs[15];
-    for (int d = 0; d < nd; ++d) offs[d] = lat_off(nd, d, W, WH);
-    for (int i = lat->run_off[r]; i < lat->run_off[r + 1]; ++i)
-      for (int q = rp[i]; q < rp[i + 1]; ++q) {
-        const int o = col[q] - i;
-        bool on = false;
-        for (int d = 0; d < nd && !on; ++d) on = offs[d] == o;
-        if (!on) return CH_OK;
-      }
+// bad = 1 if a stored entry lies off its run's lattice stencil or away from its class's table value
+__global__ void k_lat_check(Csr<double> A, Lattice L, int nd, int ts, const double* tab, int* bad) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= A.nrows) return;
+  const int id = lat_id(L, i);
+  const int2 w = L.wh[id];
+  const double* row = tab + (size_t)id * ts;
+  const double tol = 0x1p-36 * fabs(row[nd / 2]);
+  bool ok = true;
+  double seen = 0.0, sum = 0.0;
+  for (int q = A.rowptr[i]; q < A.rowptr[i + 1]; ++q) {
+    int at = -1;
+    for (int d = 0; d < nd; ++d)
+      if (lat_off(nd, d, w.x, w.y) == A.col[q] - i) at = d;
+    if (at < 0 || !(fabs(A.val[q] - row[at]) <= tol)) ok = false;
+    if (at >= 0) seen += fabs(row[at]);
   }
-  Dia<double> D;
-  D.nd = nd;
-  if (R == 1) {
-    D.W = lat->W[0];
-    D.WH = lat->WH[0];
-  } else {
-    std::vector<int2> wh(R);
-    for (int r = 0; r < R; ++r) wh[r] = make_int2(lat->W[r], lat->WH[r]);
-    int2* d_wh = nullptr;
-    CH_TRY(mem.get(&d_wh, (size_t)R));
-    CH_CUDA(cudaMemcpyAsync(d_wh, wh.data(), sizeof(int2) * R, cudaMemcpyHostToDevice, st));
-    CH_CUDA(cudaStreamSynchronize(st));  // wh is a host temporary
-    D.node_run = lat->node_run;
-    D.run_wh = d_wh;
-  }
-  CH_TRY(mem.get(&D.val, (size_t)nd * n));
-  CH_CUDA(cudaMemsetAsync(D.val, 0, sizeof(double) * (size_t)nd * n, st));
-  k_csr_to_dia<<<blocks_for(n), TPB, 0, st>>>(A, D);
-  CH_LAUNCHED();
-  *out = D;
-  return CH_OK;
+  for (int d = 0; d < nd; ++d) sum += fabs(row[d]);
+  if (!(fabs(sum - seen) <= tol)) ok = false;  // the class has an entry that the row lacks
+  if (!ok) *bad = 1;
 }
 
 template <typename T>
-static ch_status make_working(Hierarchy* h, const FineLattice* lat, std::vector<LevelT<T>>& L, cudaStream_t st) {
+__global__ void k_lat_cast(const double* a, T* b, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) b[i] = (T)a[i];
+}
+
+// The Chebyshev step x' = x + alpha (x - xp) + beta D^-1 (b - A x) with everything that depends on the
+// class folded into one table row: x' = g (A' x - b) - alpha xp with g = -beta / a_ii (slot nd) and
+// A' = A but for the diagonal, a_ii' = a_ii + (1 + alpha) / g = a_ii (1 - (1 + alpha) / beta).  Nine
+// FP64 instructions per right-hand side in 2D (seven for the row, two for g and xp) instead of ten
+// and a scaling per row: FP64 V-cycles are bound by that pipe.  FP32 steps are bound by their vectors
+// and keep the operator's own rounded values (k_cheb_step_lat).
+struct StepCoefs {
+  int n;
+  double alpha[16], beta[16];
+};
+__global__ void k_lat_steps(const double* tab, int nids, int nd, int ts, StepCoefs c, double* out) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
+  if (id >= nids) return;
+  const double* row = tab + (size_t)id * ts;
+  double* o = out + ((size_t)s * nids + id) * ts;
+  const double diag = row[nd / 2];
+  for (int d = 0; d < ts; ++d) {
+    double v = d < nd ? row[d] : 0.0;
+    if (d == nd / 2) v = diag * (1.0 - (1.0 + c.alpha[s]) / c.beta[s]);
+    if (d == nd) v = -c.beta[s] / diag;
+    o[d] = v;
+  }
+}
+
+// The lattice form's FP64 table of A where every row fits it (tab stays null where not: the level
+// then keeps the CSR form).
+static ch_status lat_build(const Csr<double>& A, const Lattice* L, Alloc& mem, double** tab, cudaStream_t st) {
+  *tab = nullptr;
+  if (!L || (L->dim != 2 && L->dim != 3)) return CH_OK;
+  const int nd = L->dim == 2 ? 7 : 15, ts = nd + 1;
+  Alloc tmp;
+  int* bad = nullptr;
+  double* t = nullptr;
+  CH_TRY(tmp.get(&bad, 1));
+  CH_TRY(mem.get(&t, (size_t)L->nids * ts));
+  CH_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), st));
+  k_lat_table<<<blocks_for(L->nids), TPB, 0, st>>>(A, *L, nd, ts, t);
+  k_lat_check<<<blocks_for(A.nrows), TPB, 0, st>>>(A, *L, nd, ts, t, bad);
+  CH_LAUNCHED();
+  int hb = 0;
+  CH_CUDA(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CH_CUDA(cudaStreamSynchronize(st));
+  if (!hb) *tab = t;
+  return CH_OK;
+}
+
+struct ChebCoef {
+  double invtheta;
+  double alpha[16], beta[16];
+};
+static ChebCoef cheb_coef(double rho, int deg, double lower);
+static ChebCoef cheb_coef_interval(double lo, double hi, int deg);
+
+// the tables of `deg` steps with coefficients c
+static void lat_step_tables(const double* tab64, const LatOp<double>& op, const ChebCoef& c, int deg, double* out,
+                            cudaStream_t st) {
+  StepCoefs sc;
+  sc.n = deg;
+  for (int s = 0; s < 16; ++s) {
+    sc.alpha[s] = c.alpha[s];
+    sc.beta[s] = c.beta[s];
+  }
+  k_lat_steps<<<dim3(blocks_for(op.L.nids, 64), deg), 64, 0, st>>>(tab64, op.L.nids, op.nd, op.ts, sc, out);
+}
+
+static int semi_steps(const ch_params& p) { return p.cheb_M_steps > 0 ? p.cheb_M_steps : 5; }
+// Wathen's bounds of the eigenvalues of D^-1 M: [1/2, 2] (triangles), [1/2, 5/2] (tetrahedra)
+static ChebCoef semi_coef(int dim, int steps) { return cheb_coef_interval(0.5, dim == 2 ? 2.0 : 2.5, steps); }
+
+template <typename T>
+static ch_status make_working(Hierarchy* h, const Lattice* lat, const ch_params& p, std::vector<LevelT<T>>& L,
+                              cudaStream_t st) {
   using V2 = typename V2T<T>::t;
   L.resize(h->nlev);
   for (int l = 0; l < h->nlev; ++l) {
@@ -768,35 +812,40 @@ static ch_status make_working(Hierarchy* h, const FineLattice* lat, std::vector<
     }
     CH_TRY(h->mem.get(&w.x, (size_t)n));
     CH_TRY(h->mem.get(&w.x2, (size_t)n));
-    CH_TRY(h->mem.get(&w.d, (size_t)n));
     CH_TRY(h->mem.get(&w.r, (size_t)n));
     CH_TRY(h->mem.get(&w.b, (size_t)n));
     w.pdl = h->pdl;
   }
 
-  // the fine level of a uniform mesh in diagonal form
-  Dia<double> d64;
-  CH_TRY(dia_build(h->A[0], lat, h->mem, &d64, st));
-  if (d64.nd) {
-    Dia<T>& d = L[0].dia;
-    d.nd = d64.nd;
-    d.W = d64.W;
-    d.WH = d64.WH;
-    d.node_run = d64.node_run;
-    d.run_wh = d64.run_wh;
-    const size_t cnt = (size_t)d64.nd * h->A[0].nrows;
-    if (std::is_same<T, double>::value) {
-      d.val = reinterpret_cast<T*>(d64.val);
-    } else {
-      CH_TRY(h->mem.get(&d.val, cnt));
-      k_copy_cast<T><<<blocks_for((int64_t)cnt), TPB, 0, st>>>(d64.val, d.val, (int64_t)cnt);
-      CH_LAUNCHED();
+  // the fine level of a uniform mesh in lattice form
+  CH_TRY(lat_build(h->A[0], lat, h->mem, &h->lat_tab, st));
+  if (h->lat_tab) {
+    LatOp<T>& op = L[0].lat;
+    op.nd = lat->dim == 2 ? 7 : 15;
+    op.ts = op.nd + 1;
+    op.L = *lat;
+    const int cnt = lat->nids * op.ts;
+    T* tab = nullptr;
+    CH_TRY(h->mem.get(&tab, (size_t)cnt));
+    k_lat_cast<T><<<blocks_for(cnt), TPB, 0, st>>>(h->lat_tab, tab, cnt);
+    op.tab = tab;
+    if constexpr (std::is_same<T, double>::value) {
+      CH_TRY(h->mem.get(&op.steps, (size_t)h->cheb_degree * cnt));
+      CH_TRY(h->mem.get(&op.scratch, (size_t)16 * cnt));
+      lat_step_tables(h->lat_tab, op, cheb_coef(h->rho[0], h->cheb_degree, h->cheb_lower), h->cheb_degree, op.steps,
+                      st);
+      if (p.precond_M == 1) {
+        const int ns = semi_steps(p);
+        CH_TRY(h->mem.get(&op.semi, (size_t)ns * cnt));
+        lat_step_tables(h->lat_tab, op, semi_coef(lat->dim, ns), ns, op.semi, st);
+      }
     }
+    CH_LAUNCHED();
   }
   return autotune_levels<T>(h, L, h->autotune, st);
 }
 
-ch_status hierarchy_build(const Csr<double>& A0, const FineLattice* lat, const ch_params& p, int precision, cudaStream_t st,
+ch_status hierarchy_build(const Csr<double>& A0, const Lattice* lat, const ch_params& p, int precision, cudaStream_t st,
                           Hierarchy** out) {
   *out = nullptr;
   Hierarchy* h = new Hierarchy();
@@ -868,9 +917,9 @@ ch_status hierarchy_build(const Csr<double>& A0, const FineLattice* lat, const c
   }
   if (s == CH_OK) {
     if (precision == 0) {
-      s = make_working<double>(h, lat, h->Ld, st);
+      s = make_working<double>(h, lat, p, h->Ld, st);
     } else {
-      s = make_working<float>(h, lat, h->Lf, st);
+      s = make_working<float>(h, lat, p, h->Lf, st);
       if (s == CH_OK) s = h->mem.get(&h->cinvf, (size_t)h->nc * h->nc);
       if (s == CH_OK) {
         k_d2f<<<blocks_for((int64_t)h->nc * h->nc), TPB, 0, st>>>(h->cinv, h->cinvf,
@@ -960,9 +1009,9 @@ __device__ __forceinline__ V2 mk2(T a, T b) {
   return v;
 }
 
-// x = D^-1 b / theta (first Chebyshev step from a zero guess); d = x
+// x = D^-1 b / theta (first Chebyshev step from a zero guess)
 template <typename T, typename V2>
-__global__ void k_cheb_first(int n, const T* dinv, const V2* b, T invtheta, V2* x, V2* d) {
+__global__ void k_cheb_first(int n, const T* dinv, const V2* b, T invtheta, V2* x) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const T di = i < n ? dinv[i] : T(0);  // set-up data: read before the dependency wait
   pdl_wait();
@@ -970,9 +1019,7 @@ __global__ void k_cheb_first(int n, const T* dinv, const V2* b, T invtheta, V2* 
   if (i >= n) return;
   const T s = invtheta * di;
   const V2 bi = b[i];
-  const V2 v = mk2<T, V2>(s * bi.x, s * bi.y);
-  x[i] = v;
-  d[i] = v;
+  x[i] = mk2<T, V2>(s * bi.x, s * bi.y);
 }
 
 // Row sums of A x for both right-hand sides with TPR lanes per row: lane `sub` takes entries
@@ -1044,14 +1091,16 @@ __device__ __forceinline__ void row_acc(const Csr<T>& A, const CsrRow<T, TPR>& r
   }
 }
 
-// r = b - A x;  d = alpha d + beta D^-1 r;  xo = x + d.  The row sum starts from -b, so it is
-// -r, and nbeta = -beta turns it back: d = alpha d + (nbeta D^-1) (A x - b), three FP64
-// instructions per right-hand side after the sum (multiply, fused multiply-add, add).
+// One Chebyshev step of the two-term form, x' = x + alpha (x - xp) + beta D^-1 (b - A x), with the
+// iterate before x in the output's own place: xo holds xp on entry and x' on exit, so a step moves
+// four vectors (x, xp, b, x') and keeps no direction.
+enum XPrev { XP_NONE = 0, XP_READ = 1, XP_ZERO = 2 };  // alpha = 0; xp in xo; xp = 0 (x is the first iterate)
+
+// The row sum starts from -b, so it is -r, and nbeta = -beta turns it back.
 template <typename T, typename V2, int TPR>
 __global__ void __launch_bounds__(TPB) k_cheb_step(Csr<T> A, const T* __restrict__ dinv,
                                                    const V2* __restrict__ b, const V2* __restrict__ x,
-                                                   V2* __restrict__ d, V2* __restrict__ xo, T alpha,
-                                                   T nbeta) {
+                                                   V2* __restrict__ xo, T alpha, T nbeta, int mode) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = t / TPR, sub = t % TPR;
   CsrRow<T, TPR> row;
@@ -1067,16 +1116,18 @@ __global__ void __launch_bounds__(TPB) k_cheb_step(Csr<T> A, const T* __restrict
   }
   row_acc<T, V2, TPR>(A, row, x, s0, s1);
   if (i >= A.nrows || sub != 0) return;
-  const V2 xi = x[i];
-  V2 dd;
-  if (alpha != T(0)) {
-    const V2 dold = d[i];
-    dd = mk2<T, V2>(fma(alpha, dold.x, di * s0), fma(alpha, dold.y, di * s1));
-  } else {
-    dd = mk2<T, V2>(di * s0, di * s1);
+  V2 y = x[i];
+  if (mode != XP_NONE) {
+    V2 d = y;
+    if (mode == XP_READ) {
+      const V2 xp = xo[i];
+      d.x -= xp.x;
+      d.y -= xp.y;
+    }
+    y.x = fma(alpha, d.x, y.x);
+    y.y = fma(alpha, d.y, y.y);
   }
-  d[i] = dd;
-  xo[i] = mk2<T, V2>(xi.x + dd.x, xi.y + dd.y);
+  xo[i] = mk2<T, V2>(fma(di, s0, y.x), fma(di, s1, y.y));
 }
 
 template <typename T, typename V2, int TPR>
@@ -1115,32 +1166,37 @@ __global__ void __launch_bounds__(TPB) k_spmv2(Csr<T> A, const V2* __restrict__ 
   }
 }
 
-// ---------------------------------------------------------------- structured (diagonal) fine level
-// One row of the lattice form: its ND operator values and its run's strides (set-up data, so the
-// kernels read them before their dependency wait).
+// ---------------------------------------------------------------- structured (lattice) fine level
+// One row of the lattice form: the class's ND values and factor and its run's strides (set-up data, so
+// the kernels read them before their dependency wait).  Rows of a warp are almost always of one class:
+// the table reads are broadcasts from L1.
 template <typename T, int ND>
-struct DiaRow {
-  T a[ND];
+struct LatRow {
+  T a[ND + 1];
   int W, WH;
 };
 template <typename T, int ND>
-__device__ __forceinline__ DiaRow<T, ND> dia_row(const Dia<T>& D, int n, int i) {
-  DiaRow<T, ND> r;
-  r.W = D.W;
-  r.WH = D.WH;
-  if (D.node_run) {
-    const int2 w = D.run_wh[D.node_run[i]];
+__device__ __forceinline__ LatRow<T, ND> lat_row(const LatOp<T>& D, const T* __restrict__ tab, int i) {
+  LatRow<T, ND> r;
+  const int id = lat_id(D.L, i);
+  r.W = D.L.W;
+  r.WH = D.L.WH;
+  if (D.L.nids > D.L.ncls) {
+    const int2 w = D.L.wh[id];
     r.W = w.x;
     r.WH = w.y;
   }
+  constexpr int NQ = (ND + 1) * (int)sizeof(T) / 16;  // 16-byte loads (rows are 32 to 128 bytes, aligned)
+  const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)id * (ND + 1));
+  uint4* dst = reinterpret_cast<uint4*>(r.a);
 #pragma unroll
-  for (int d = 0; d < ND; ++d) r.a[d] = D.val[(size_t)d * n + i];
+  for (int q = 0; q < NQ; ++q) dst[q] = src[q];
   return r;
 }
 
 // Row sum of the lattice form onto the caller's (s0, s1) (zero, or -b for a residual's negative).
 template <typename T, typename V2, int ND>
-__device__ __forceinline__ void dia_row_acc(const DiaRow<T, ND>& r, int n, int i, const V2* __restrict__ x,
+__device__ __forceinline__ void lat_row_acc(const LatRow<T, ND>& r, int n, int i, const V2* __restrict__ x,
                                             T& s0, T& s1) {
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
@@ -1152,76 +1208,91 @@ __device__ __forceinline__ void dia_row_acc(const DiaRow<T, ND>& r, int n, int i
   }
 }
 
-// k_cheb_step on the lattice form (same arithmetic: the sum starts from -b, nbeta = -beta)
+// One Chebyshev step on the lattice form.  FP32 is bound by its vectors (34 bytes per row: x, xp, b, x'
+// and the class id; one value per stored entry and a kept direction made it 72 in 2D, 104 in 3D), FP64
+// by its pipe.  Measured, us per step in a run of launches: FP32 4.01 -> 3.26 (512 x 512), 9.88 -> 8.21
+// (3D 128 x 128 x 32), 16.8 -> 10.2 (64 runs, 1.46 M rows); 512 x 512 FP64 steps 20.8 -> 18.9 ms.
+// xp is read from and x' written to xo.  FP64: the step's table
+// (lat_step_tables), x' = g (A' x - b) - alpha xp.  FP32: the operator's table, x' = x + alpha (x - xp)
+// + (nbeta D^-1) (A x - b).
 template <typename T, typename V2, int ND>
-__global__ void __launch_bounds__(TPB) k_cheb_step_dia(Dia<T> D, int n, const T* __restrict__ dinv,
+__global__ void __launch_bounds__(TPB) k_cheb_step_lat(LatOp<T> D, int n, const T* __restrict__ tab,
                                                        const V2* __restrict__ b, const V2* __restrict__ x,
-                                                       V2* __restrict__ d, V2* __restrict__ xo, T alpha, T nbeta) {
+                                                       V2* __restrict__ xo, T alpha, T nbeta, int mode) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  DiaRow<T, ND> row;
-  T di = 0;
-  if (i < n) {
-    row = dia_row<T, ND>(D, n, i);
-    di = dinv[i] * nbeta;
-  }
+  LatRow<T, ND> row;
+  if (i < n) row = lat_row<T, ND>(D, tab, i);
   pdl_wait();
   pdl_trigger_t<T>();
   if (i >= n) return;
   const V2 bi = b[i];
   T s0 = -bi.x, s1 = -bi.y;
-  dia_row_acc<T, V2, ND>(row, n, i, x, s0, s1);
-  const V2 xi = x[i];
-  V2 dd;
-  if (alpha != T(0)) {
-    const V2 dold = d[i];
-    dd = mk2<T, V2>(fma(alpha, dold.x, di * s0), fma(alpha, dold.y, di * s1));
+  lat_row_acc<T, V2, ND>(row, n, i, x, s0, s1);
+  const T g = row.a[ND];
+  if (sizeof(T) == 8) {
+    if (mode == XP_READ) {
+      const V2 xp = xo[i];
+      xo[i] = mk2<T, V2>(fma(g, s0, -alpha * xp.x), fma(g, s1, -alpha * xp.y));
+    } else {
+      xo[i] = mk2<T, V2>(g * s0, g * s1);
+    }
   } else {
-    dd = mk2<T, V2>(di * s0, di * s1);
+    V2 y = x[i];
+    if (mode != XP_NONE) {
+      V2 d = y;
+      if (mode == XP_READ) {
+        const V2 xp = xo[i];
+        d.x -= xp.x;
+        d.y -= xp.y;
+      }
+      y.x = fma(alpha, d.x, y.x);
+      y.y = fma(alpha, d.y, y.y);
+    }
+    const T di = g * nbeta;
+    xo[i] = mk2<T, V2>(fma(di, s0, y.x), fma(di, s1, y.y));
   }
-  d[i] = dd;
-  xo[i] = mk2<T, V2>(xi.x + dd.x, xi.y + dd.y);
 }
 
 template <typename T, typename V2, int ND>
-__global__ void __launch_bounds__(TPB) k_residual_dia(Dia<T> D, int n, const V2* __restrict__ b,
+__global__ void __launch_bounds__(TPB) k_residual_lat(LatOp<T> D, int n, const V2* __restrict__ b,
                                                       const V2* __restrict__ x, V2* __restrict__ r) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  DiaRow<T, ND> row;
-  if (i < n) row = dia_row<T, ND>(D, n, i);
+  LatRow<T, ND> row;
+  if (i < n) row = lat_row<T, ND>(D, D.tab, i);
   pdl_wait();
   pdl_trigger_t<T>();
   if (i >= n) return;
   T s0 = 0, s1 = 0;
-  dia_row_acc<T, V2, ND>(row, n, i, x, s0, s1);
+  lat_row_acc<T, V2, ND>(row, n, i, x, s0, s1);
   const V2 bi = b[i];
   r[i] = mk2<T, V2>(bi.x - s0, bi.y - s1);
 }
 
 template <typename T, typename V2, int ND>
-__global__ void __launch_bounds__(TPB) k_spmv2_dia(Dia<T> D, int n, const V2* __restrict__ x, V2* __restrict__ y) {
+__global__ void __launch_bounds__(TPB) k_spmv2_lat(LatOp<T> D, int n, const V2* __restrict__ x, V2* __restrict__ y) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  DiaRow<T, ND> row;
-  if (i < n) row = dia_row<T, ND>(D, n, i);
+  LatRow<T, ND> row;
+  if (i < n) row = lat_row<T, ND>(D, D.tab, i);
   pdl_wait();
   pdl_trigger_t<T>();
   if (i >= n) return;
   T s0 = 0, s1 = 0;
-  dia_row_acc<T, V2, ND>(row, n, i, x, s0, s1);
+  lat_row_acc<T, V2, ND>(row, n, i, x, s0, s1);
   y[i] = mk2<T, V2>(s0, s1);
 }
 
-#define CH_DIA_DISPATCH(nd, KCALL)                    \
+#define CH_LAT_DISPATCH(nd, KCALL)                    \
   switch (nd) {                                       \
     case 7: { constexpr int NDC = 7; KCALL; } break;  \
     default: { constexpr int NDC = 15; KCALL; } break; \
   }
 
 // b_c = R r, fused with the coarse level's first Chebyshev step from a zero guess (pointwise:
-// x_c = d_c = invtheta D_c^-1 b_c, the arithmetic of k_cheb_first): one launch instead of two.
+// x_c = invtheta D_c^-1 b_c, the arithmetic of k_cheb_first): one launch instead of two.
 template <typename T, typename V2, int TPR>
 __global__ void __launch_bounds__(TPB) k_restrict_first(Csr<T> R, const V2* __restrict__ r, V2* __restrict__ bc,
                                                         const T* __restrict__ dinv_c, T invtheta,
-                                                        V2* __restrict__ xc, V2* __restrict__ dc) {
+                                                        V2* __restrict__ xc) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = t / TPR, sub = t % TPR;
   CsrRow<T, TPR> row;
@@ -1233,9 +1304,7 @@ __global__ void __launch_bounds__(TPB) k_restrict_first(Csr<T> R, const V2* __re
   row_acc<T, V2, TPR>(R, row, r, s0, s1);
   if (i >= R.nrows || sub != 0) return;
   bc[i] = mk2<T, V2>(s0, s1);
-  const V2 v = mk2<T, V2>(s * s0, s * s1);
-  xc[i] = v;
-  dc[i] = v;
+  xc[i] = mk2<T, V2>(s * s0, s * s1);
 }
 
 #define CH_TPR_DISPATCH(tpr, KCALL)                      \
@@ -1248,39 +1317,32 @@ __global__ void __launch_bounds__(TPB) k_restrict_first(Csr<T> R, const V2* __re
     default: { constexpr int TPRC = 32; KCALL; } break;  \
   }
 
-// one Chebyshev step d = alpha d + beta D^-1 (b - A x), xo = x + d (the kernels take -beta)
+// one Chebyshev step on a CSR level (the kernel takes -beta)
 template <typename T, typename V2>
-static void launch_cheb_step(int tpr, const Csr<T>& A, const T* dinv, const V2* b, const V2* x, V2* d,
-                             V2* xo, T alpha, T beta, cudaStream_t st, const Dia<T>* dia = nullptr,
-                             bool pdl = false) {
+static void launch_cheb_step(int tpr, const Csr<T>& A, const T* dinv, const V2* b, const V2* x, V2* xo, T alpha,
+                             T beta, int mode, cudaStream_t st, bool pdl) {
   const T nbeta = -beta;
-  if (dia && dia->nd) {
-    const int g = blocks_for(A.nrows);
-    CH_DIA_DISPATCH(dia->nd, (launch_k(pdl, k_cheb_step_dia<T, V2, NDC>, g, TPB, 0, st, *dia, A.nrows, dinv, b,
-                                       x, d, xo, alpha, nbeta)));
-    return;
-  }
   const int g = blocks_for((int64_t)A.nrows * tpr);
-  CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_cheb_step<T, V2, TPRC>, g, TPB, 0, st, A, dinv, b, x, d, xo, alpha,
-                                 nbeta)));
+  CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_cheb_step<T, V2, TPRC>, g, TPB, 0, st, A, dinv, b, x, xo, alpha, nbeta,
+                                 mode)));
 }
 template <typename T, typename V2>
 static void launch_residual(int tpr, const Csr<T>& A, const V2* b, const V2* x, V2* r, cudaStream_t st,
-                            const Dia<T>* dia, bool pdl) {
-  if (dia && dia->nd) {
+                            const LatOp<T>* lat, bool pdl) {
+  if (lat && lat->nd) {
     const int g = blocks_for(A.nrows);
-    CH_DIA_DISPATCH(dia->nd, (launch_k(pdl, k_residual_dia<T, V2, NDC>, g, TPB, 0, st, *dia, A.nrows, b, x, r)));
+    CH_LAT_DISPATCH(lat->nd, (launch_k(pdl, k_residual_lat<T, V2, NDC>, g, TPB, 0, st, *lat, A.nrows, b, x, r)));
     return;
   }
   const int g = blocks_for((int64_t)A.nrows * tpr);
   CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_residual<T, V2, TPRC>, g, TPB, 0, st, A, b, x, r)));
 }
-// y = A x with the level's operator (the diagonal form where there is one)
+// y = A x with the level's operator (the lattice form where there is one)
 template <typename T, typename V2>
 static void launch_apply_level(const LevelT<T>& L, const V2* x, V2* y, cudaStream_t st) {
-  if (L.dia.nd) {
+  if (L.lat.nd) {
     const int g = blocks_for(L.A.nrows);
-    CH_DIA_DISPATCH(L.dia.nd, (launch_k(L.pdl, k_spmv2_dia<T, V2, NDC>, g, TPB, 0, st, L.dia, L.A.nrows, x, y)));
+    CH_LAT_DISPATCH(L.lat.nd, (launch_k(L.pdl, k_spmv2_lat<T, V2, NDC>, g, TPB, 0, st, L.lat, L.A.nrows, x, y)));
     return;
   }
   launch_spmv2<T, V2, false>(L.tprA, L.A, x, y, st, L.pdl);
@@ -1381,10 +1443,10 @@ __global__ void k_load2(int n, const double* src, int ld, V2* dst) {
   dst[i] = mk2<T, V2>((T)v.x, (T)v.y);
 }
 // k_load2 fused with the finest level's first Chebyshev step from a zero guess (the arithmetic of
-// k_cheb_first on the converted values): b = (T) src, x = d = invtheta D^-1 b.  One launch instead
+// k_cheb_first on the converted values): b = (T) src, x = invtheta D^-1 b.  One launch instead
 // of two at the start of the first V-cycle of a solve.
 template <typename T, typename V2>
-__global__ void k_load2_first(int n, const double* src, int ld, const T* dinv, T invtheta, V2* b, V2* x, V2* d) {
+__global__ void k_load2_first(int n, const double* src, int ld, const T* dinv, T invtheta, V2* b, V2* x) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const T di = i < n ? dinv[i] : T(0);  // set-up data: read before the dependency wait
   pdl_wait();
@@ -1394,9 +1456,7 @@ __global__ void k_load2_first(int n, const double* src, int ld, const T* dinv, T
   const V2 bi = mk2<T, V2>((T)v.x, (T)v.y);
   b[i] = bi;
   const T s = invtheta * di;
-  const V2 w = mk2<T, V2>(s * bi.x, s * bi.y);
-  x[i] = w;
-  d[i] = w;
+  x[i] = mk2<T, V2>(s * bi.x, s * bi.y);
 }
 template <typename T, typename V2>
 __global__ void k_store2(int n, const V2* src, double* dst, int ld) {
@@ -1409,11 +1469,6 @@ __global__ void k_store2(int n, const V2* src, double* dst, int ld) {
 }
 
 // ---------------------------------------------------------------- V-cycle driver
-struct ChebCoef {
-  double invtheta;
-  double alpha[16], beta[16];
-};
-
 // Coefficients of `deg` Chebyshev semi-iteration steps for eigenvalues in [lo, hi]: the first
 // step from zero is x = D^-1 b / theta, then d = alpha_s d + beta_s D^-1 (b - A x), x += d.
 static ChebCoef cheb_coef_interval(double lo, double hi, int deg) {
@@ -1438,12 +1493,16 @@ static ChebCoef cheb_coef(double rho, int deg, double lower) {
   return cheb_coef_interval(lower * hi, hi, deg);
 }
 
-// `deg` Chebyshev steps with coefficients c on level L (accounted as kernels kfirst / kstep).
-// zero_guess: 0 continue from *xcur; 1 start from zero (the first step is pointwise); 2 start from
-// zero with that first step already taken by the caller (fused into the restriction)
+// bytes per row of the fine level's lattice form beyond its vectors: the class id
+static double lat_bytes(const Lattice& L, double n) { return (L.id32 ? 4.0 : 2.0) * n; }
+
+// `deg` Chebyshev steps with coefficients c on level L (accounted as kernels kfirst / kstep); tabs: the
+// steps' tables where the level has the lattice form in FP64.  zero_guess: 0 continue from *xcur; 1 start from
+// zero (the first step is pointwise); 2 start from zero with that first step already taken by the
+// caller (fused into the restriction or the input conversion)
 template <typename T_>
-static ch_status smooth_coef(LevelT<T_>& L, const ChebCoef& c, int deg, int zero_guess, int kfirst, int kstep,
-                             typename V2T<T_>::t** xcur, cudaStream_t st) {
+static ch_status smooth_coef(LevelT<T_>& L, const ChebCoef& c, const T_* tabs, int deg, int zero_guess, int kfirst,
+                             int kstep, typename V2T<T_>::t** xcur, cudaStream_t st) {
   using V2 = typename V2T<T_>::t;
   const int n = L.A.nrows;
   V2* x = *xcur;
@@ -1451,18 +1510,24 @@ static ch_status smooth_coef(LevelT<T_>& L, const ChebCoef& c, int deg, int zero
   int s0 = 0;
   const double T = sizeof(T_), nnz = (double)L.A.nnz;
   if (zero_guess == 1) {
-    ProfScope ps(st, kfirst, sizeof(T_) == 4, 7.0 * T * n, 2.0 * n);
-    launch_k(L.pdl, k_cheb_first<T_, V2>, blocks_for(n), TPB, 0, st, n, L.dinv, L.b, (T_)c.invtheta, x, L.d);
+    ProfScope ps(st, kfirst, sizeof(T_) == 4, 5.0 * T * n, 2.0 * n);
+    launch_k(L.pdl, k_cheb_first<T_, V2>, blocks_for(n), TPB, 0, st, n, L.dinv, L.b, (T_)c.invtheta, x);
     s0 = 1;
   } else if (zero_guess == 2) {
     s0 = 1;
   }
-  // operator bytes: CSR values + column indices + row pointers, or the diagonals' values
-  const double opb = L.dia.nd ? T * L.dia.nd * (double)n : nnz * (4 + T) + 4.0 * (n + 1);
+  // operator bytes: CSR values + column indices + row pointers and D^-1, or the class ids
+  const double opb = L.lat.nd ? lat_bytes(L.lat.L, n) : nnz * (4 + T) + 4.0 * (n + 1) + T * n;
   for (int s = s0; s < deg; ++s) {
-    ProfScope ps(st, kstep, sizeof(T_) == 4, opb + T * n * (c.alpha[s] != 0.0 ? 11 : 9), 2.0 * nnz + 4.0 * n);
-    launch_cheb_step<T_, V2>(L.tprA, L.A, L.dinv, L.b, x, L.d, other, (T_)c.alpha[s], (T_)c.beta[s], st,
-                             &L.dia, L.pdl);
+    const int mode = s == 0 ? XP_NONE : (s == 1 && s0 == 1 ? XP_ZERO : XP_READ);
+    ProfScope ps(st, kstep, sizeof(T_) == 4, opb + T * n * (mode == XP_READ ? 8 : 6), 2.0 * nnz + 4.0 * n);
+    if (L.lat.nd) {
+      const T_* tab = sizeof(T_) == 8 ? tabs + (size_t)s * L.lat.L.nids * L.lat.ts : L.lat.tab;
+      CH_LAT_DISPATCH(L.lat.nd, (launch_k(L.pdl, k_cheb_step_lat<T_, V2, NDC>, blocks_for(n), TPB, 0, st, L.lat, n,
+                                          tab, L.b, x, other, (T_)c.alpha[s], (T_)-c.beta[s], mode)));
+    } else {
+      launch_cheb_step<T_, V2>(L.tprA, L.A, L.dinv, L.b, x, other, (T_)c.alpha[s], (T_)c.beta[s], mode, st, L.pdl);
+    }
     std::swap(x, other);
   }
   CH_LAUNCHED();
@@ -1476,24 +1541,23 @@ static ch_status smooth(Hierarchy* h, LevelT<T_>& L, int l, int zero_guess,
                         typename V2T<T_>::t** xcur, cudaStream_t st) {
   const int deg = l == 0 ? h->cheb_degree : h->cheb_degree_coarse;
   const ChebCoef c = cheb_coef(h->rho[l], deg, h->cheb_lower);
-  return smooth_coef<T_>(L, c, deg, zero_guess, l == 0 ? K_CHEB_FIRST : K_CHEB_FIRST_C,
+  return smooth_coef<T_>(L, c, L.lat.steps, deg, zero_guess, l == 0 ? K_CHEB_FIRST : K_CHEB_FIRST_C,
                          l == 0 ? K_CHEB_STEP : K_CHEB_STEP_C, xcur, st);
 }
 
 // M~^-1 by the Chebyshev semi-iteration (Section 3's alternative to AMG for the mass matrix):
 // `steps` steps on D^-1 M from a zero guess over Wathen's bounds of its eigenvalues for P1
-// simplices, [1/2, 2] (triangles) and [1/2, 5/2] (tetrahedra), on the finest level of M's
-// hierarchy (its working-precision copy of M and D^-1).  b in L.b; result in *xres.
+// simplices (semi_coef), on the finest level of M's hierarchy (its working-precision copy of M and
+// D^-1).  b in L.b; result in *xres.
 template <typename T_>
 static ch_status semi_iteration(LevelT<T_>& L, int dim, int steps, typename V2T<T_>::t** xres, cudaStream_t st) {
-  const ChebCoef c = cheb_coef_interval(0.5, dim == 2 ? 2.0 : 2.5, steps);
   *xres = L.x;
-  return smooth_coef<T_>(L, c, steps, 1, K_CHEB_SEMI, K_CHEB_SEMI, xres, st);
+  return smooth_coef<T_>(L, semi_coef(dim, steps), L.lat.semi, steps, 1, K_CHEB_SEMI, K_CHEB_SEMI, xres, st);
 }
 
-// one V-cycle at level l on L[l].b; result in *xres (L[l].x or L[l].x2)
+// one V-cycle at level l on L[l].b; result in *xres (L[l].x or L[l].x2).  zero_guess: as smooth_coef
 template <typename T>
-static ch_status vcycle(Hierarchy* h, std::vector<LevelT<T>>& Ls, const T* cinv, int l,
+static ch_status vcycle(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l,
                         int zero_guess, typename V2T<T>::t** xres, cudaStream_t st) {
   using V2 = typename V2T<T>::t;
   LevelT<T>& L = Ls[l];
@@ -1511,21 +1575,21 @@ static ch_status vcycle(Hierarchy* h, std::vector<LevelT<T>>& Ls, const T* cinv,
   LevelT<T>& C = Ls[l + 1];
   const int nc = C.A.nrows;
   {
-    const double opb = L.dia.nd ? Tb * L.dia.nd * (double)n : L.A.nnz * (4 + Tb) + 4.0 * (n + 1);
+    const double opb = L.lat.nd ? lat_bytes(L.lat.L, n) : L.A.nnz * (4 + Tb) + 4.0 * (n + 1);
     ProfScope ps(st, l == 0 ? K_VRESIDUAL : K_VRESIDUAL_C, sizeof(T) == 4, opb + 6.0 * Tb * n, 2.0 * L.A.nnz);
-    launch_residual<T, V2>(L.tprA, L.A, L.b, x, L.r, st, &L.dia, L.pdl);
+    launch_residual<T, V2>(L.tprA, L.A, L.b, x, L.r, st, &L.lat, L.pdl);
   }
   const bool fuse = l + 1 < h->nlev - 1;  // the coarse level smooths: fuse its first step
   {
     ProfScope ps(st, l == 0 ? K_RESTRICT : K_RESTRICT_C, sizeof(T) == 4,
-                 L.R.nnz * (4 + Tb) + 4.0 * (nc + 1) + 2.0 * Tb * (n + nc) + (fuse ? 5.0 * Tb * nc : 0.0),
+                 L.R.nnz * (4 + Tb) + 4.0 * (nc + 1) + 2.0 * Tb * (n + nc) + (fuse ? 3.0 * Tb * nc : 0.0),
                  2.0 * L.R.nnz + (fuse ? 2.0 * nc : 0.0));
     if (fuse) {
       const int degc = h->cheb_degree_coarse;
       const ChebCoef cc = cheb_coef(h->rho[l + 1], degc, h->cheb_lower);
       const int g = blocks_for((int64_t)L.R.nrows * L.tprR);
       CH_TPR_DISPATCH(L.tprR, (launch_k(L.pdl, k_restrict_first<T, V2, TPRC>, g, TPB, 0, st, L.R, L.r, C.b,
-                                        C.dinv, (T)cc.invtheta, C.x, C.d)));
+                                        C.dinv, (T)cc.invtheta, C.x)));
     } else {
       launch_spmv2<T, V2, false>(L.tprR, L.R, L.r, C.b, st, L.pdl);
     }
@@ -1545,7 +1609,7 @@ static ch_status vcycle(Hierarchy* h, std::vector<LevelT<T>>& Ls, const T* cinv,
 }
 
 template <typename T>
-static ch_status solve_t(Hierarchy* h, std::vector<LevelT<T>>& Ls, const T* cinv, const double* b,
+static ch_status solve_t(Hierarchy* h, LevelT<T>* Ls, const T* cinv, const double* b,
                          int ldb, double* x, int ldx, int ncyc, cudaStream_t st) {
   using V2 = typename V2T<T>::t;
   LevelT<T>& L = Ls[0];
@@ -1568,6 +1632,16 @@ static ch_status smooth_t(Hierarchy* h, std::vector<LevelT<T>>& Ls, const double
   LevelT<T>& L = Ls[0];
   const int n = L.A.nrows;
   const double io = n * (16.0 + 2.0 * sizeof(T));
+  const ChebCoef c = cheb_coef(h->rho[0], degree, h->cheb_lower);
+  const T* tabs = L.lat.steps;
+  if constexpr (std::is_same<T, double>::value) {
+    if (L.lat.nd && degree != h->cheb_degree) {
+      // this degree's tables; the two loads below lie between them and the steps, which read the
+      // tables before their dependency wait
+      lat_step_tables(h->lat_tab, L.lat, c, degree, L.lat.scratch, st);
+      tabs = L.lat.scratch;
+    }
+  }
   {
     ProfScope ps(st, K_VLOAD, sizeof(T) == 4, 2.0 * io, 0.0);
     launch_k(L.pdl, k_load2<T, V2>, blocks_for(n), TPB, 0, st, n, b, 2, L.b);
@@ -1577,9 +1651,9 @@ static ch_status smooth_t(Hierarchy* h, std::vector<LevelT<T>>& Ls, const double
     launch_k(L.pdl, k_load2<T, V2>, blocks_for(n), TPB, 0, st, n, x, 2, L.x);
   }
   CH_LAUNCHED();
-  const ChebCoef c = cheb_coef(h->rho[0], degree, h->cheb_lower);
   V2* xr = L.x;
-  for (int k = 0; k < passes; ++k) CH_TRY(smooth_coef<T>(L, c, degree, 0, K_CHEB_FIRST, K_CHEB_STEP, &xr, st));
+  for (int k = 0; k < passes; ++k)
+    CH_TRY(smooth_coef<T>(L, c, tabs, degree, 0, K_CHEB_FIRST, K_CHEB_STEP, &xr, st));
   {
     ProfScope ps(st, K_VSTORE, sizeof(T) == 4, io, 0.0);
     launch_k(L.pdl, k_store2<T, V2>, blocks_for(n), TPB, 0, st, n, xr, x, 2);
@@ -1595,15 +1669,13 @@ ch_status hierarchy_smooth(Hierarchy* h, const double* b, double* x, int degree,
 
 ch_status hierarchy_solve(Hierarchy* h, const double* b, int ldb, double* x, int ldx, int ncyc,
                           cudaStream_t st) {
-  if (h->precision == 0) return solve_t<double>(h, h->Ld, h->cinv, b, ldb, x, ldx, ncyc, st);
-  return solve_t<float>(h, h->Lf, h->cinvf, b, ldb, x, ldx, ncyc, st);
+  if (h->precision == 0) return solve_t<double>(h, h->Ld.data(), h->cinv, b, ldb, x, ldx, ncyc, st);
+  return solve_t<float>(h, h->Lf.data(), h->cinvf, b, ldb, x, ldx, ncyc, st);
 }
 
 // ---------------------------------------------------------------- Algorithm 1
 // w_1 = AMG(M) v_1;  w_2 = AMG(H) v_2;  w_2 = M w_2;  w_2 = AMG(H) w_2.
 // v, w are N x 4 (phi_p, phi_n, mu_p, mu_n per node): block 1 at offset 0, block 2 at offset 2.
-static int semi_steps(const ch_params& p) { return p.cheb_M_steps > 0 ? p.cheb_M_steps : 5; }
-
 // The fine-level input of a solve: b = (T) v (strided FP64 pairs).  With AMG V-cycles on a
 // hierarchy of more than one level the first V-cycle's first smoothing step (from zero) is done in
 // the same launch (k_load2_first), and the V-cycle then starts at its second step (zero_guess 2).
@@ -1614,9 +1686,8 @@ static int load_input(Hierarchy* h, LevelT<T>& L, bool amg, const double* v, int
   const int n = L.A.nrows;
   if (amg && h->nlev > 1) {
     const ChebCoef c = cheb_coef(h->rho[0], h->cheb_degree, h->cheb_lower);
-    ProfScope ps(st, K_VLOAD, sizeof(T) == 4, n * (16.0 + 7.0 * sizeof(T)), 2.0 * n);
-    launch_k(L.pdl, k_load2_first<T, V2>, blocks_for(n), TPB, 0, st, n, v, ld, L.dinv, (T)c.invtheta, L.b, L.x,
-             L.d);
+    ProfScope ps(st, K_VLOAD, sizeof(T) == 4, n * (16.0 + 5.0 * sizeof(T)), 2.0 * n);
+    launch_k(L.pdl, k_load2_first<T, V2>, blocks_for(n), TPB, 0, st, n, v, ld, L.dinv, (T)c.invtheta, L.b, L.x);
     return 2;
   }
   ProfScope ps(st, K_VLOAD, sizeof(T) == 4, n * (16.0 + 2.0 * sizeof(T)), 0.0);
@@ -1650,7 +1721,7 @@ static ch_status precond_t(ch_precond_s* pc, std::vector<LevelT<T>>& LM, std::ve
     if (p.precond_M == 1) {
       CH_TRY(semi_iteration<T>(L, pc->sys->mesh->dim, semi_steps(p), &xr, sm));
     } else {
-      for (int c = 0; c < p.vcycles_M; ++c) CH_TRY(vcycle<T>(pc->hM, LM, cinvM, 0, c == 0 ? zg : 0, &xr, sm));
+      for (int c = 0; c < p.vcycles_M; ++c) CH_TRY(vcycle<T>(pc->hM, LM.data(), cinvM, 0, c == 0 ? zg : 0, &xr, sm));
     }
     {
       ProfScope ps(sm, K_VSTORE, sizeof(T) == 4, n * (16.0 + 2.0 * sizeof(T)), 0.0);
@@ -1664,17 +1735,17 @@ static ch_status precond_t(ch_precond_s* pc, std::vector<LevelT<T>>& LM, std::ve
     LevelT<T>& L = LH[0];
     const int zg = load_input<T>(pc->hH, L, true, v + 2, 4, st);
     V2* xr = L.x;
-    for (int c = 0; c < p.vcycles_H; ++c) CH_TRY(vcycle<T>(pc->hH, LH, cinvH, 0, c == 0 ? zg : 0, &xr, st));
+    for (int c = 0; c < p.vcycles_H; ++c) CH_TRY(vcycle<T>(pc->hH, LH.data(), cinvH, 0, c == 0 ? zg : 0, &xr, st));
     // b <- M x (M's fine level in working precision); the V-cycle reads only L.b afterwards
     {
       const double Tb = sizeof(T), nnz = (double)LM[0].A.nnz;
-      const double opb = LM[0].dia.nd ? Tb * LM[0].dia.nd * (double)n : nnz * (4 + Tb) + 4.0 * (n + 1);
+      const double opb = LM[0].lat.nd ? lat_bytes(LM[0].lat.L, n) : nnz * (4 + Tb) + 4.0 * (n + 1);
       ProfScope ps(st, K_SPMV_M, sizeof(T) == 4, opb + 4.0 * Tb * n, 2.0 * nnz);
       launch_apply_level<T, V2>(LM[0], xr, L.b, st);
     }
     CH_LAUNCHED();
     xr = L.x;  // the first solve's result now lives in L.b as M x; start afresh
-    for (int c = 0; c < p.vcycles_H; ++c) CH_TRY(vcycle<T>(pc->hH, LH, cinvH, 0, c == 0, &xr, st));
+    for (int c = 0; c < p.vcycles_H; ++c) CH_TRY(vcycle<T>(pc->hH, LH.data(), cinvH, 0, c == 0, &xr, st));
     {
       ProfScope ps(st, K_VSTORE, sizeof(T) == 4, n * (16.0 + 2.0 * sizeof(T)), 0.0);
       launch_k(L.pdl, k_store2<T, V2>, blocks_for(n), TPB, 0, st, n, xr, w + 2, 4);
@@ -1705,7 +1776,7 @@ static ch_status mass_solve_t(ch_precond_s* pc, std::vector<LevelT<T>>& LM, cons
   if (p.precond_M == 1) {
     CH_TRY(semi_iteration<T>(L, pc->sys->mesh->dim, semi_steps(p), &xr, st));
   } else {
-    for (int c = 0; c < p.vcycles_M; ++c) CH_TRY(vcycle<T>(pc->hM, LM, cinvM, 0, c == 0, &xr, st));
+    for (int c = 0; c < p.vcycles_M; ++c) CH_TRY(vcycle<T>(pc->hM, LM.data(), cinvM, 0, c == 0, &xr, st));
   }
   k_store2<T, V2><<<blocks_for(n), TPB, 0, st>>>(n, xr, x, 2);
   CH_LAUNCHED();
@@ -1721,7 +1792,7 @@ ch_status mass_solve(ch_precond_s* pc, const double* b, double* x, cudaStream_t 
 
 // ---------------------------------------------------------------- allocation-free V-cycles
 // ch_vcycle_noalloc runs the same V-cycles as ch_vcycle, but the per-level work vectors
-// (x, x2, d, r, b for every level, two right-hand sides each) are carved out of one
+// (x, x2, r, b for every level, two right-hand sides each) are carved out of one
 // file-scope device array instead of the preconditioner's own buffers, so a call needs no
 // device memory beyond the caller's b and x and the already-built hierarchy.  The array is
 // reserved in every GPU that loads the library for the life of the process.
@@ -1760,48 +1831,6 @@ ch_status noalloc_scratch(void** out) {
 }  // namespace
 
 template <typename T>
-static ch_status vcycle_static(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l, bool zero_guess,
-                               typename V2T<T>::t** xres, cudaStream_t st) {
-  using V2 = typename V2T<T>::t;
-  LevelT<T>& L = Ls[l];
-  const int n = L.A.nrows;
-  if (l == h->nlev - 1) {
-    launch_dense_solve<T, V2>(L.pdl, n, cinv, L.b, L.x, st);
-    CH_LAUNCHED();
-    *xres = L.x;
-    return CH_OK;
-  }
-  const int deg = l == 0 ? h->cheb_degree : h->cheb_degree_coarse;
-  const ChebCoef c = cheb_coef(h->rho[l], deg, h->cheb_lower);
-  V2* x = *xres;
-  auto smooth_static = [&](bool zg) {
-    V2* other = (x == L.x) ? L.x2 : L.x;
-    int s0 = 0;
-    if (zg) {
-      k_cheb_first<T, V2><<<blocks_for(n), TPB, 0, st>>>(n, L.dinv, L.b, (T)c.invtheta, x, L.d);
-      s0 = 1;
-    }
-    for (int s = s0; s < deg; ++s) {
-      launch_cheb_step<T, V2>(L.tprA, L.A, L.dinv, L.b, x, L.d, other, (T)c.alpha[s], (T)c.beta[s], st,
-                              &L.dia);
-      std::swap(x, other);
-    }
-  };
-  smooth_static(zero_guess);
-  LevelT<T>& C = Ls[l + 1];
-  launch_residual<T, V2>(L.tprA, L.A, L.b, x, L.r, st, &L.dia);
-  launch_spmv2<T, V2, false>(L.tprR, L.R, L.r, C.b, st);
-  CH_LAUNCHED();
-  V2* xc = C.x;
-  CH_TRY(vcycle_static<T>(h, Ls, cinv, l + 1, true, &xc, st));
-  launch_spmv2<T, V2, true>(L.tprP, L.P, xc, x, st);
-  smooth_static(false);
-  CH_LAUNCHED();
-  *xres = x;
-  return CH_OK;
-}
-
-template <typename T>
 static ch_status solve_static(Hierarchy* h, const std::vector<LevelT<T>>& src, const T* cinv,
                               const double* b, double* x, int ncyc, cudaStream_t st) {
   using V2 = typename V2T<T>::t;
@@ -1810,7 +1839,7 @@ static ch_status solve_static(Hierarchy* h, const std::vector<LevelT<T>>& src, c
     set_error("ch_vcycle_noalloc: hierarchy has %d levels (max %d)", h->nlev, MAXLEV);
     return CH_ERR_ARG;
   }
-  // 5 vectors of n_l pairs per level, each rounded up to 256 bytes
+  // The documented limit: 5 vectors of n_l pairs per level, each rounded up to 256 bytes (4 are used)
   size_t need = 0;
   for (int l = 0; l < h->nlev; ++l) need += 5 * ((src[l].A.nrows * sizeof(V2) + 255) / 256 * 256);
   if (need > NOALLOC_SCRATCH_BYTES) {
@@ -1832,7 +1861,6 @@ static ch_status solve_static(Hierarchy* h, const std::vector<LevelT<T>>& src, c
     const int n = src[l].A.nrows;
     Ls[l].x = carve(n);
     Ls[l].x2 = carve(n);
-    Ls[l].d = carve(n);
     Ls[l].r = carve(n);
     Ls[l].b = carve(n);
   }
@@ -1842,7 +1870,7 @@ static ch_status solve_static(Hierarchy* h, const std::vector<LevelT<T>>& src, c
   k_load2<T, V2><<<blocks_for(n0), TPB, 0, st>>>(n0, b, 2, Ls[0].b);
   CH_LAUNCHED();
   V2* xr = Ls[0].x;
-  for (int c = 0; c < ncyc; ++c) CH_TRY(vcycle_static<T>(h, Ls, cinv, 0, c == 0, &xr, st));
+  for (int c = 0; c < ncyc; ++c) CH_TRY(vcycle<T>(h, Ls, cinv, 0, c == 0, &xr, st));
   k_store2<T, V2><<<blocks_for(n0), TPB, 0, st>>>(n0, xr, x, 2);
   CH_LAUNCHED();
   return CH_OK;

@@ -154,6 +154,20 @@ __global__ void k_facet_vol(const double* X, const int* f, int F, double* vol) {
   }
 }
 
+// class id of every node of one run (Lattice)
+__global__ void k_lat_ids(ch_params p, int N, int node_off, int base, int id32, void* out) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= N) return;
+  const int i = n % (p.nx + 1), j = (n / (p.nx + 1)) % (p.ny + 1);
+  int c = (i == 0 ? 0 : (i == p.nx ? 2 : 1)) + 3 * (j == 0 ? 0 : (j == p.ny ? 2 : 1));
+  if (p.dim == 3) {
+    const int k = n / ((p.nx + 1) * (p.ny + 1));
+    c += 9 * (k == 0 ? 0 : (k == p.nz ? 2 : 1));
+  }
+  if (id32) static_cast<int*>(out)[node_off + n] = base + c;
+  else static_cast<uint16_t*>(out)[node_off + n] = (uint16_t)(base + c);
+}
+
 // counts of one box mesh
 static void box_counts(const ch_params& p, int* N, int* E, int* F) {
   if (p.dim == 2) {
@@ -200,6 +214,36 @@ ch_status mesh_build(ch_mesh_s* m, cudaStream_t st) {
   CH_TRY(m->mem.get(&m->tvol, (size_t)m->Ft));
   CH_TRY(m->mem.get(&m->node_run, (size_t)m->N));
   CH_TRY(m->mem.get(&m->run_off_d, (size_t)R + 1));
+  Lattice& L = m->lat;
+  L.dim = d;
+  L.ncls = d == 2 ? 9 : 27;
+  if ((int64_t)R * L.ncls > 2000000000LL) {
+    set_error("batched mesh too large for int32 indexing");
+    return CH_ERR_ARG;
+  }
+  L.nids = R * L.ncls;
+  L.id32 = L.nids > 65536;
+  L.W = m->runs[0].nx + 1;
+  L.WH = L.W * (m->runs[0].ny + 1);
+  uint8_t* ids = nullptr;
+  CH_TRY(m->mem.get(&ids, (size_t)m->N * (L.id32 ? 4 : 2)));
+  L.id = ids;
+  CH_TRY(m->mem.get(&L.wh, (size_t)L.nids));
+  CH_TRY(m->mem.get(&L.rep, (size_t)L.nids));
+  std::vector<int2> wh(L.nids);
+  std::vector<int> rep(L.nids);
+  for (int r = 0; r < R; ++r) {
+    const ch_params& p = m->runs[r];
+    const int W = p.nx + 1, WH = W * (p.ny + 1), nz = d == 3 ? p.nz : 0;
+    for (int c = 0; c < L.ncls; ++c) {
+      const auto pick = [](int cls, int cells) { return cls == 0 ? 0 : (cls == 1 ? cells / 2 : cells); };
+      const int x = pick(c % 3, p.nx), y = pick(c / 3 % 3, p.ny), z = d == 3 ? pick(c / 9, nz) : 0;
+      wh[(size_t)r * L.ncls + c] = make_int2(W, WH);
+      rep[(size_t)r * L.ncls + c] = m->run_off[r] + x + W * y + WH * z;
+    }
+  }
+  CH_CUDA(cudaMemcpyAsync(L.wh, wh.data(), sizeof(int2) * L.nids, cudaMemcpyHostToDevice, st));
+  CH_CUDA(cudaMemcpyAsync(L.rep, rep.data(), sizeof(int) * L.nids, cudaMemcpyHostToDevice, st));
   for (int r = 0; r < R; ++r) {
     const ch_params& p = m->runs[r];
     const int n = m->run_off[r + 1] - m->run_off[r], e = eoff[r + 1] - eoff[r], f = foff[r + 1] - foff[r];
@@ -208,6 +252,7 @@ ch_status mesh_build(ch_mesh_s* m, cudaStream_t st) {
     k_mesh_facets<<<blocks_for(f), TPB, 0, st>>>(p, f, m->run_off[r], m->bot + (size_t)foff[r] * d,
                                                   m->top + (size_t)foff[r] * d);
     k_fill_int<<<blocks_for(n), TPB, 0, st>>>(m->node_run + m->run_off[r], n, r);
+    k_lat_ids<<<blocks_for(n), TPB, 0, st>>>(p, n, m->run_off[r], r * L.ncls, L.id32, L.id);
   }
   CH_LAUNCHED();
   CH_CUDA(cudaMemcpyAsync(m->run_off_d, m->run_off.data(), sizeof(int) * (R + 1), cudaMemcpyHostToDevice, st));

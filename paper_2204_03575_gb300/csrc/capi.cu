@@ -283,14 +283,6 @@ ch_status ch_precond_setup(const ch_system_t* s, void* stream, ch_precond_t** ou
   M.col = H.col = s->col;
   M.val = s->valM;
   H.val = s->valH;
-  ch::FineLattice lat;
-  lat.dim = s->mesh->dim;
-  lat.run_off = s->mesh->run_off;
-  for (const ch_params& rp : s->mesh->runs) {
-    lat.W.push_back(rp.nx + 1);
-    lat.WH.push_back((rp.nx + 1) * (rp.ny + 1));
-  }
-  lat.node_run = s->mesh->node_run;
   // The finest level's Chebyshev degree, cheb_degree 0: 5 in both precisions.  (FP64 512 x 512:
   // 79.8 / 76.0 steps/s at degree 5 / 6.  FP32 V-cycles: degree 6 gained 3 % on 512 x 512 steps
   // 4..63 but lost 3.6 % on the 3D box and 2-5 % on the 256 x 256 warm-start runs.)
@@ -300,8 +292,8 @@ ch_status ch_precond_setup(const ch_system_t* s, void* stream, ch_precond_t** ou
   if (ph.cheb_degree == 0) ph.cheb_degree = 5;
   ch_params pm = ph;
   pm.cheb_degree = ph.cheb_degree_M > 0 ? ph.cheb_degree_M : std::min(3, ph.cheb_degree);
-  ch_status r = ch::hierarchy_build(M, &lat, pm, pc->precision, S(stream), &pc->hM);
-  if (r == CH_OK) r = ch::hierarchy_build(H, &lat, ph, pc->precision, S(stream), &pc->hH);
+  ch_status r = ch::hierarchy_build(M, &s->mesh->lat, pm, pc->precision, S(stream), &pc->hM);
+  if (r == CH_OK) r = ch::hierarchy_build(H, &s->mesh->lat, ph, pc->precision, S(stream), &pc->hH);
   if (r == CH_OK && (cudaStreamCreateWithFlags(&pc->side, cudaStreamNonBlocking) != cudaSuccess ||
                      cudaEventCreateWithFlags(&pc->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
                      cudaEventCreateWithFlags(&pc->ev_join, cudaEventDisableTiming) != cudaSuccess)) {

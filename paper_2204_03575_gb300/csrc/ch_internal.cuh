@@ -189,6 +189,35 @@ void prof_add_slot(int kid, int f32, int64_t launches, double bytes, double fmas
 
 }  // namespace ch
 
+// ---------------------------------------------------------------- lattice classes of a uniform mesh
+namespace ch {
+// On a uniform box mesh an assembled row depends only on the run's cell size and on whether the node
+// is the first, an inner or the last one along each axis: 9 classes in 2D, 27 in 3D.  Every node
+// carries its class id, run * classes + class, and a fine-level operator is one table row per id
+// instead of one value per stored entry.
+struct Lattice {
+  int dim = 0, ncls = 0;        // 9 (2D) or 27 (3D) classes per run
+  int nids = 0;                 // runs x ncls
+  int W = 0, WH = 0;            // strides nx + 1 and (nx + 1)(ny + 1) of a single run
+  int id32 = 0;                 // ids are 32-bit (more than 65536 of them), else 16-bit
+  void* id = nullptr;           // N class ids
+  int2* wh = nullptr;           // nids: strides of the id's run
+  int* rep = nullptr;           // nids: a node of the class (the middle one along its inner axes)
+};
+// strides of the lattice directions: 7 in 2D (the triangles' edges), 15 in 3D (the Kuhn tetrahedra's),
+// ascending for any W, H >= 2, i.e. in CSR column order; direction ND / 2 is the node itself
+__host__ __device__ __forceinline__ int lat_off(int nd, int d, int W, int WH) {
+  constexpr int a2[7] = {-1, 0, -1, 0, 1, 0, 1}, b2[7] = {-1, -1, 0, 0, 0, 1, 1};
+  constexpr int a3[15] = {-1, 0, -1, 0, -1, 0, -1, 0, 1, 0, 1, 0, 1, 0, 1};
+  constexpr int b3[15] = {-1, -1, 0, 0, -1, -1, 0, 0, 0, 1, 1, 0, 0, 1, 1};
+  constexpr int c3[15] = {-1, -1, -1, -1, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1};
+  return nd == 7 ? a2[d] + b2[d] * W : a3[d] + b3[d] * W + c3[d] * WH;
+}
+__device__ __forceinline__ int lat_id(const Lattice& L, int i) {
+  return L.id32 ? static_cast<const int*>(L.id)[i] : static_cast<const uint16_t*>(L.id)[i];
+}
+}  // namespace ch
+
 // ---------------------------------------------------------------- opaque handles
 struct ch_mesh_s {
   ch_params p{};                 // parameters of run 0 (the only run of a plain mesh)
@@ -208,6 +237,7 @@ struct ch_mesh_s {
   int *n2e_ptr = nullptr, *n2e = nullptr;  // node -> incident elements (sorted)
   int *n2b_ptr = nullptr, *n2b = nullptr;  // node -> incident bottom facets
   int *n2t_ptr = nullptr, *n2t = nullptr;  // node -> incident top facets
+  ch::Lattice lat;
   ch::Alloc mem;
 };
 
@@ -230,15 +260,7 @@ struct ch_system_s {
 
 namespace ch {
 struct Hierarchy;  // amg.cu
-// The fine level's mesh structure, for the structured (diagonal) form of level 0: node i of run r
-// has its neighbours at i + a + b W_r + c WH_r over the uniform mesh's lattice directions.
-struct FineLattice {
-  int dim = 0;                    // 2 or 3
-  std::vector<int> run_off;       // host, runs + 1
-  std::vector<int> W, WH;         // host, per run: nx + 1 and (nx + 1)(ny + 1)
-  const int* node_run = nullptr;  // device, N (used when there are several runs)
-};
-ch_status hierarchy_build(const Csr<double>& A0, const FineLattice* lat, const ch_params& p, int precision,
+ch_status hierarchy_build(const Csr<double>& A0, const Lattice* lat, const ch_params& p, int precision,
                           cudaStream_t st, Hierarchy** out);
 void hierarchy_free(Hierarchy* h);
 int hierarchy_levels(const Hierarchy* h);
@@ -254,7 +276,6 @@ ch_status hierarchy_solve(Hierarchy* h, const double* b, int ldb, double* x, int
 ch_status hierarchy_smooth(Hierarchy* h, const double* b, double* x, int degree, int passes, cudaStream_t st);
 // as hierarchy_solve (strides 2), work vectors in a static device array: no device allocation
 ch_status hierarchy_solve_noalloc(Hierarchy* h, const double* b, double* x, int ncyc, cudaStream_t st);
-// y (N x 2, fp64, stride ldy) = A0 x (N x 2, fp64, stride ldx) in the hierarchy's working precision
 
 // assemble.cu
 ch_status loads(const ch_system_s* s, const double* pp, const double* pn, double* Fp, double* Fn,
