@@ -22,14 +22,15 @@
 // (k_conv3x3: 16 pixels per warp, 8 channels per tile; each lane gathers its A-fragment elements
 // straight from the shifted input, zero outside the image, the B fragments from the weights
 // staged in shared memory).
-// Weight gradients are reduced over pixels by FP32 FMAs in fixed-size pixel chunks and summed in
-// chunk order (deterministic).
+// Weight gradients are GEMMs over the pixels on mma.sync, per strip of image rows, the strips' partial
+// sums added in order (deterministic).
 #include <cuda_bf16.h>
 
 #include <cmath>
 #include <vector>
 
 #include <algorithm>
+#include <initializer_list>
 
 #include "ch_internal.cuh"
 
@@ -38,7 +39,6 @@ namespace ch {
 constexpr int WS_C = 32;       // hidden channels
 constexpr int WS_CIN = 16;     // input channels padded for the k16 MMA (12 used)
 constexpr int WS_COUT = 8;     // output channels padded for the n8 MMA (4 used)
-constexpr int WS_CHUNK = 1024; // pixels per weight-gradient partial
 
 struct WsParams {  // FP32 master parameters, contiguous
   float* w1;  // [9][WS_CIN][WS_C]
@@ -383,22 +383,47 @@ __global__ void __launch_bounds__(TC_M) k_conv3x3_tc(const __nv_bfloat16* __rest
 // part[smp][b][8]; k_ws_rms_fin adds a sample's block partials in block order.
 constexpr int WS_RMS_BLOCKS = 256;  // most blocks per sample of the first pass
 
+// The four channels of pixel i (N x 4 node-major arrays): one vector load where the caller's array is
+// aligned for it (al: 32 bytes for fp64, 16 for fp32), four scalar loads otherwise.
+template <typename T> struct Quad { T x, y, z, w; };
+__device__ __forceinline__ Quad<double> ld4(const double* p, size_t i, bool al) {
+  if (al) {
+    const double4_32a v = reinterpret_cast<const double4_32a*>(p)[i];
+    return {v.x, v.y, v.z, v.w};
+  }
+  return {p[4 * i], p[4 * i + 1], p[4 * i + 2], p[4 * i + 3]};
+}
+__device__ __forceinline__ Quad<float> ld4(const float* p, size_t i, bool al) {
+  if (al) {
+    const float4 v = reinterpret_cast<const float4*>(p)[i];
+    return {v.x, v.y, v.z, v.w};
+  }
+  return {p[4 * i], p[4 * i + 1], p[4 * i + 2], p[4 * i + 3]};
+}
+static bool aligned4(size_t elem, std::initializer_list<const void*> ps) {
+  uintptr_t u = 0;
+  for (const void* p : ps) u |= reinterpret_cast<uintptr_t>(p);
+  return (u & (4 * elem - 1)) == 0;
+}
+
 template <typename T>
 __global__ void k_ws_rms_part(const T* __restrict__ s, const T* __restrict__ q, const T* __restrict__ q2, int P,
-                              int chunk, double* __restrict__ part) {
+                              int chunk, bool al, double* __restrict__ part) {
   __shared__ double red[8][256];
   const int smp = blockIdx.y, b = blockIdx.x;
   const int i0 = b * chunk, i1 = min(P, i0 + chunk);
   double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    const size_t o = ((size_t)smp * P + i) * 4;
+    const size_t o = (size_t)smp * P + i;
+    const Quad<T> sv = ld4(s, o, al), qv = ld4(q, o, al), q2v = q2 ? ld4(q2, o, al) : Quad<T>{};
+    const T sc[4] = {sv.x, sv.y, sv.z, sv.w}, qc[4] = {qv.x, qv.y, qv.z, qv.w}, q2c[4] = {q2v.x, q2v.y, q2v.z, q2v.w};
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const double a = s[o + c], bq = q[o + c];
+      const double a = sc[c], bq = qc[c];
       const double d = a - bq;
       acc[c] = fma(d, d, acc[c]);
       if (q2) {
-        const double D = a - 2.0 * bq + (double)q2[o + c];
+        const double D = a - 2.0 * bq + (double)q2c[c];
         acc[4 + c] = fma(D, D, acc[4 + c]);
       }
     }
@@ -416,45 +441,49 @@ __global__ void k_ws_rms_part(const T* __restrict__ s, const T* __restrict__ q, 
   if (threadIdx.x < 8) part[((size_t)smp * gridDim.x + b) * 8 + threadIdx.x] = red[threadIdx.x][0];
 }
 
-__global__ void k_ws_rms_fin(const double* __restrict__ part, int nblk, int P, int has_q2, float* __restrict__ dscale) {
+__global__ void k_ws_rms_fin(const double* __restrict__ part, int nblk, int P, int has_q2, float* __restrict__ dscale,
+                             double* __restrict__ dinv) {
   const int smp = blockIdx.x, c = threadIdx.x;
   if (c >= 8) return;
   double sum = 0.0;
   for (int b = 0; b < nblk; ++b) sum += part[((size_t)smp * nblk + b) * 8 + c];
-  dscale[smp * 8 + c] = (c >= 4 && !has_q2) ? 1.f : (float)fmax(sqrt(sum / (double)P), 1e-30);
+  const float d = (c >= 4 && !has_q2) ? 1.f : (float)fmax(sqrt(sum / (double)P), 1e-30);
+  dscale[smp * 8 + c] = d;
+  dinv[smp * 8 + c] = 1.0 / (double)d;
 }
 
+// dinv = 1 / dscale in FP64: the per-pixel kernels multiply by it (an FP64 division per channel and
+// pixel bound them: packing 8 x 257 x 257 pixels took 100 us).
 // Input image of the network from the states s, q, q2 (N x 4 each, fp64 node major or fp32
 // sample-major): channels 0-3 = (s - mean[0:4]) * inv_std[0:4] (the fields at step k), channels
 // 4-7 = ((s - q) / r1 - mean[4:8]) * inv_std[4:8] (the last change in units of its RMS), channels
 // 8-11 = (s - 2 q + q2) / r2 (the second difference in units of its RMS), channels 12-15 zero.
 template <typename T>
-__global__ void k_ws_pack(const T* __restrict__ s, const T* __restrict__ q, const T* __restrict__ q2, int P,
+__global__ void k_ws_pack(const T* __restrict__ s, const T* __restrict__ q, const T* __restrict__ q2, int P, bool al,
                           const float* __restrict__ mean, const float* __restrict__ inv_std,
-                          const float* __restrict__ dscale, __nv_bfloat16* __restrict__ x) {
+                          const double* __restrict__ dinv, __nv_bfloat16* __restrict__ x) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // pixel; blockIdx.y = sample
   const int smp = blockIdx.y;
   if (i >= (size_t)P) return;
-  const size_t o = ((size_t)smp * P + i) * 4;
-  const T* a = s + o;
-  const T* b = q + o;
-  const T* b2 = q2 + o;
-  const float* sc = dscale + smp * 8;
-  __nv_bfloat16* dst = x + ((size_t)smp * P + i) * WS_CIN;
+  const size_t o = (size_t)smp * P + i;
+  const Quad<T> sv = ld4(s, o, al), qv = ld4(q, o, al), q2v = ld4(q2, o, al);
+  const T a[4] = {sv.x, sv.y, sv.z, sv.w}, b[4] = {qv.x, qv.y, qv.z, qv.w}, b2[4] = {q2v.x, q2v.y, q2v.z, q2v.w};
+  const double* sc = dinv + smp * 8;
+  float v[12];
 #pragma unroll
-  for (int c = 0; c < WS_CIN; ++c) {
-    float v = 0.f;
-    if (c < 4) {
-      v = ((float)a[c] - mean[c]) * inv_std[c];
-    } else if (c < 8) {
-      const double d = ((double)a[c - 4] - (double)b[c - 4]) / (double)sc[c - 4];
-      v = ((float)d - mean[c]) * inv_std[c];
-    } else if (c < 12) {
-      const double D = (double)a[c - 8] - 2.0 * (double)b[c - 8] + (double)b2[c - 8];
-      v = (float)(D / (double)sc[c - 4]);
-    }
-    dst[c] = __float2bfloat16_rn(v);
+  for (int c = 0; c < 4; ++c) {
+    v[c] = ((float)a[c] - mean[c]) * inv_std[c];
+    const double d = ((double)a[c] - (double)b[c]) * sc[c];
+    v[4 + c] = ((float)d - mean[4 + c]) * inv_std[4 + c];
+    const double D = (double)a[c] - 2.0 * (double)b[c] + (double)b2[c];
+    v[8 + c] = (float)(D * sc[4 + c]);
   }
+  uint32_t w[8] = {};
+#pragma unroll
+  for (int c = 0; c < 6; ++c) w[c] = pack_bf16(__float2bfloat16_rn(v[2 * c]), __float2bfloat16_rn(v[2 * c + 1]));
+  uint4* dst = reinterpret_cast<uint4*>(x + o * WS_CIN);
+  dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+  dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
 // State-space error of the prediction in units of the change's RMS, E = (theta D - e) / r1 with
@@ -462,7 +491,7 @@ __global__ void k_ws_pack(const T* __restrict__ s, const T* __restrict__ q, cons
 // the factor dE/dy = out_scale D / r1 (fp32 inputs, sample-major B x N x 4).
 __global__ void k_ws_err_theta(const float* __restrict__ y, const float* __restrict__ s, const float* __restrict__ q,
                                const float* __restrict__ q2, const float* __restrict__ n, int P,
-                               const float* __restrict__ out_scale, const float* __restrict__ dscale,
+                               const float* __restrict__ out_scale, const double* __restrict__ dinv,
                                float* __restrict__ e, float* __restrict__ fac) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int smp = blockIdx.y;
@@ -473,26 +502,34 @@ __global__ void k_ws_err_theta(const float* __restrict__ y, const float* __restr
     const double a = s[o + c], b = q[o + c];
     const double D = a - 2.0 * b + (double)q2[o + c];
     const double err = (double)n[o + c] - 2.0 * a + b;
-    const double r1 = dscale[smp * 8 + c], os = out_scale[c];
+    const double r1i = dinv[smp * 8 + c], os = out_scale[c];
     const double th = (double)y[((size_t)smp * P + i) * WS_COUT + c] * os;
-    e[o + c] = (float)((th * D - err) / r1);
-    fac[o + c] = (float)(os * D / r1);
+    e[o + c] = (float)((th * D - err) * r1i);
+    fac[o + c] = (float)(os * D * r1i);
   }
 }
 
 // pred = s + (s - q) + y * out_scale * (s - 2 q + q2) (fp64, N x 4): the learned second-order
 // extrapolation
 __global__ void k_ws_unpack(const double* __restrict__ s, const double* __restrict__ q, const double* __restrict__ q2,
-                            const float* __restrict__ y, int P, const float* __restrict__ out_scale,
+                            const float* __restrict__ y, int P, bool al, const float* __restrict__ out_scale,
                             double* __restrict__ pred) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= P) return;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const size_t o = (size_t)i * 4 + c;
-    const double a = s[o], b = q[o];
-    const double D = a - 2.0 * b + q2[o];
-    pred[o] = a + (a - b) + (double)y[(size_t)i * WS_COUT + c] * (double)out_scale[c] * D;
+  const Quad<double> a = ld4(s, i, al), b = ld4(q, i, al), b2 = ld4(q2, i, al);
+  const float4 yv = *reinterpret_cast<const float4*>(y + (size_t)i * WS_COUT);
+  const double p0 = a.x + (a.x - b.x) + (double)yv.x * (double)out_scale[0] * (a.x - 2.0 * b.x + b2.x);
+  const double p1 = a.y + (a.y - b.y) + (double)yv.y * (double)out_scale[1] * (a.y - 2.0 * b.y + b2.y);
+  const double p2 = a.z + (a.z - b.z) + (double)yv.z * (double)out_scale[2] * (a.z - 2.0 * b.z + b2.z);
+  const double p3 = a.w + (a.w - b.w) + (double)yv.w * (double)out_scale[3] * (a.w - 2.0 * b.w + b2.w);
+  if (al) {
+    reinterpret_cast<double4_32a*>(pred)[i] = make_double4_32a(p0, p1, p2, p3);
+  } else {
+    double* o = pred + (size_t)i * 4;
+    o[0] = p0;
+    o[1] = p1;
+    o[2] = p2;
+    o[3] = p3;
   }
 }
 
@@ -564,63 +601,182 @@ __global__ void k_ws_dy(const float* __restrict__ e, const float* __restrict__ g
 }
 
 // ---------------------------------------------------------------- weight gradients
-// dW[tap][ci][co] = sum_p X[p + off(tap)][ci] dY[p][co], db[co] = sum_p dY[p][co], over a chunk
-// of WS_CHUNK pixels of one sample per block (partials[(sample * nchunk + chunk)][...]).
-// One thread per (tap, ci) pair keeps COUT accumulators; dY of 64 pixels is staged in shared memory.
+// dW[tap][ci][co] = sum_p X[p + off(tap)][ci] dY[p][co], db[co] = sum_p dY[p][co]: per tap a GEMM with
+// M = input channels, N = output channels and K = pixels, both operands stored pixel-major (K x M and
+// K x N), which is what ldmatrix.trans turns into mma.sync fragments.  A block takes a strip of image
+// rows of one column segment of one sample; per row it needs the input rows r - 1, r, r + 1 (a ring of
+// four bands in shared memory, one new band and one dY row copied by cp.async while the row before
+// is multiplied) and warp t < 9 multiplies tap t, whose A operand is the band (tap / 3) shifted by
+// tap % 3 pixels.  Warp 9 adds the bias gradient.  A row's MMAs (FP32 accumulate) start from zero and
+// are added to the strip's FP32 sums, so no accumulation chain is longer than a row or a strip.
+// Each strip writes its own partial gradient; k_ws_reduce adds them in order (deterministic).
+//
+// Pixel rows are padded by 16 bytes (80 or 48 bytes: 8 consecutive pixels hit distinct banks).  The
+// FP32-FMA form before it (one thread per (tap, ci), X read through L1 for every pixel) was bound by
+// its loads: batch of 8 at 257 x 257, us per layer 664 / 873 / 469.
+constexpr int WG_SEG = 160;     // most pixels of a segment
+constexpr int WG_BLOCKS = 304;  // strips aimed at: two blocks on each of the 152 SMs
+constexpr int WG_WARPS = 10;
+struct WgTiles {
+  int nseg, seg, rows, nstrip;  // column segments, pixels of one, image rows per strip, strips per segment
+};
+inline WgTiles wg_tiles(int H, int W, int B) {
+  WgTiles t;
+  t.nseg = (W + WG_SEG - 1) / WG_SEG;
+  t.seg = (W + t.nseg - 1) / t.nseg;
+  const int64_t rows = ((int64_t)H * t.nseg * B + WG_BLOCKS - 1) / WG_BLOCKS;
+  t.rows = (int)(rows < 2 ? 2 : rows);
+  t.nstrip = (H + t.rows - 1) / t.rows;
+  return t;
+}
+template <int CIN, int COUTG>
+constexpr int wg_smem(int kp) {
+  return 4 * (kp + 2) * (2 * CIN + 16) + 2 * kp * (2 * COUTG + 16);
+}
+
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+
 template <int CIN, int COUTG, int COUTW>  // COUTG: channels stored in dY; COUTW: channels of dW
-__global__ void __launch_bounds__(256) k_ws_wgrad(const __nv_bfloat16* __restrict__ X,
-                                                  const __nv_bfloat16* __restrict__ dY, int H, int W,
-                                                  int nchunk, float* __restrict__ partials) {
-  constexpr int NP = 9 * CIN;  // (tap, ci) pairs
-  constexpr int TILE = 64;
-  __shared__ float dys[TILE][COUTW];
-  const int P = H * W;
-  const int smp = blockIdx.y, chunk = blockIdx.x;
+__global__ void __launch_bounds__(32 * WG_WARPS) k_ws_wgrad(const __nv_bfloat16* __restrict__ X,
+                                                            const __nv_bfloat16* __restrict__ dY, int H, int W,
+                                                            int nseg, int seg, int rows, int kp,
+                                                            float* __restrict__ partials) {
+  constexpr int XS = 2 * CIN + 16, DS = 2 * COUTG + 16;  // bytes per pixel in shared memory
+  constexpr int MT = CIN / 16, NT = COUTW / 8;
+  extern __shared__ __align__(16) unsigned char wg_smem_raw[];
+  const int P = H * W, smp = blockIdx.z, c0 = blockIdx.y * seg, len = min(seg, W - c0);
+  const int r0 = blockIdx.x * rows, r1 = min(H, r0 + rows);
   const __nv_bfloat16* Xs = X + (size_t)smp * P * CIN;
   const __nv_bfloat16* Ds = dY + (size_t)smp * P * COUTG;
-  float* out = partials + ((size_t)smp * nchunk + chunk) * (NP * COUTW + COUTW);
-  for (int pair0 = 0; pair0 < NP; pair0 += blockDim.x) {
-    const int pair = pair0 + threadIdx.x;
-    const int tap = pair / CIN, ci = pair % CIN;
-    const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-    float acc[COUTW];
-#pragma unroll
-    for (int c = 0; c < COUTW; ++c) acc[c] = 0.f;
-    float bacc = 0.f;  // bias gradient (thread 0 of the first pass only)
-    const int pbeg = chunk * WS_CHUNK, pend = min(P, pbeg + WS_CHUNK);
-    for (int pt = pbeg; pt < pend; pt += TILE) {
-      __syncthreads();
-      for (int i = threadIdx.x; i < TILE * COUTW; i += blockDim.x) {
-        const int pp = pt + i / COUTW, c = i % COUTW;
-        dys[i / COUTW][c] = pp < pend ? __bfloat162float(Ds[(size_t)pp * COUTG + c]) : 0.f;
-      }
-      __syncthreads();
-      if (pair < NP) {
-        for (int k = 0; k < TILE && pt + k < pend; ++k) {
-          const int p = pt + k, r = p / W + dy, q = p % W + dx;
-          const float xv = (r >= 0 && r < H && q >= 0 && q < W)
-                               ? __bfloat162float(Xs[((size_t)r * W + q) * CIN + ci]) : 0.f;
-#pragma unroll
-          for (int c = 0; c < COUTW; ++c) acc[c] = fmaf(xv, dys[k][c], acc[c]);
-        }
-      }
-      if (pair0 == 0 && threadIdx.x < COUTW)
-        for (int k = 0; k < TILE && pt + k < pend; ++k) bacc += dys[k][threadIdx.x];
+  const uint32_t sx = smem_u32(wg_smem_raw), sd = sx + 4 * (kp + 2) * XS;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // band of image row r: slot (r + 1) & 3, pixel j = column c0 - 1 + j, zero outside the image
+  const auto load_band = [&](int r) {
+    constexpr int CH = CIN / 8;  // 16-byte chunks per pixel
+    const bool in_r = r >= 0 && r < H;
+    for (int f = tid; f < (kp + 2) * CH; f += 32 * WG_WARPS) {
+      const int j = f / CH, ch = f % CH, q = c0 - 1 + j;
+      const bool in = in_r && q >= 0 && q < W && j < len + 2;
+      cp_async16(sx + ((r + 1) & 3) * (kp + 2) * XS + j * XS + ch * 16,
+                 in ? Xs + ((size_t)r * W + q) * CIN + ch * 8 : Xs, in);
     }
-    if (pair < NP)
+  };
+  const auto load_dy = [&](int r) {
+    constexpr int CH = COUTG / 8;
+    for (int f = tid; f < kp * CH; f += 32 * WG_WARPS) {
+      const int j = f / CH, ch = f % CH;
+      const bool in = j < len && r < r1;
+      cp_async16(sd + (r & 1) * kp * DS + j * DS + ch * 16,
+                 in ? Ds + ((size_t)r * W + c0 + j) * COUTG + ch * 8 : Ds, in);
+    }
+  };
+  const auto commit = [] { asm volatile("cp.async.commit_group;\n" ::: "memory"); };
+  load_band(r0 - 1);
+  load_band(r0);
+  load_band(r0 + 1);
+  load_dy(r0);
+  commit();
+  float sum[MT][NT][4] = {};
+  float bsum[2] = {0.f, 0.f};
+  constexpr int NPAIR = COUTW / 2, PAR = 32 / NPAIR;  // bias warp: lane = channel pair + NPAIR x pixel class
+  for (int r = r0; r < r1; ++r) {
+    load_band(r + 2);  // the next row's new band and dY, in flight while this row is multiplied
+    load_dy(r + 1);
+    commit();
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();
+    const uint32_t dy = sd + (r & 1) * kp * DS;
+    if (warp < 9) {
+      const int band = r + warp / 3 - 1, dx = warp % 3;
+      const uint32_t xb = sx + ((band + 1) & 3) * (kp + 2) * XS + dx * XS;
+      float acc[MT][NT][4] = {};
+      const int q = lane >> 3, l8 = lane & 7;
+      for (int k0 = 0; k0 < kp; k0 += 16) {
+        uint32_t a[MT][4], b[(NT + 1) / 2][4];
 #pragma unroll
-      for (int c = 0; c < COUTW; ++c) out[pair * COUTW + c] = acc[c];
-    if (pair0 == 0 && threadIdx.x < COUTW) out[NP * COUTW + threadIdx.x] = bacc;
+        for (int m = 0; m < MT; ++m)  // matrices (k half, m half): q >> 1, q & 1
+          ldsm4_t(a[m], xb + (k0 + (q >> 1) * 8 + l8) * XS + (m * 16 + (q & 1) * 8) * 2);
+#pragma unroll
+        for (int n = 0; n < (NT + 1) / 2; ++n) {  // matrices (k half, n half): q & 1, q >> 1 (one n tile: q >> 1 = 0)
+          const int nh = NT > 1 ? q >> 1 : 0;
+          ldsm4_t(b[n], dy + (k0 + (q & 1) * 8 + l8) * DS + (n * 16 + nh * 8) * 2);
+        }
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+          for (int n = 0; n < NT; ++n) {
+            const uint32_t bb[2] = {b[n / 2][2 * (n & 1)], b[n / 2][2 * (n & 1) + 1]};
+            mma_bf16(acc[m][n], a[m], bb);
+          }
+      }
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) sum[m][n][e] += acc[m][n][e];
+    } else {
+      const unsigned char* row = wg_smem_raw + (dy - sx) + (lane % NPAIR) * 4;
+      float t0 = 0.f, t1 = 0.f;
+      for (int j = lane / NPAIR; j < len; j += PAR) {
+        const uint32_t v = *reinterpret_cast<const uint32_t*>(row + j * DS);
+        t0 += __uint_as_float(v << 16);
+        t1 += __uint_as_float(v & 0xFFFF0000u);
+      }
+      bsum[0] += t0;
+      bsum[1] += t1;
+    }
+    __syncthreads();  // every read of band r - 1 and of this dY row precedes the next copies into them
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");  // the last prefetch
+  float* out = partials + (((size_t)smp * nseg + blockIdx.y) * gridDim.x + blockIdx.x) * (9 * CIN * COUTW + COUTW);
+  if (warp < 9) {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          out[(warp * CIN + m * 16 + g + (e >> 1) * 8) * COUTW + n * 8 + 2 * t + (e & 1)] = sum[m][n][e];
+  } else {
+#pragma unroll
+    for (int o = NPAIR; o < 32; o <<= 1) {
+      bsum[0] += __shfl_xor_sync(0xffffffffu, bsum[0], o);
+      bsum[1] += __shfl_xor_sync(0xffffffffu, bsum[1], o);
+    }
+    if (lane < NPAIR) {
+      out[9 * CIN * COUTW + 2 * lane] = bsum[0];
+      out[9 * CIN * COUTW + 2 * lane + 1] = bsum[1];
+    }
   }
 }
 
-// sum of nparts partial gradient vectors of length len, in part order
-__global__ void k_ws_reduce(const float* __restrict__ partials, int nparts, int len, float* __restrict__ g) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= len) return;
+// sum of nparts partial gradient vectors of length len: eight threads per value take a contiguous
+// eighth of the parts each, in part order, and their sums are added in order
+__global__ void __launch_bounds__(256) k_ws_reduce(const float* __restrict__ partials, int nparts, int len,
+                                                   float* __restrict__ g) {
+  __shared__ float sm[8][32];
+  const int i = blockIdx.x * 32 + threadIdx.x, y = threadIdx.y;
+  const int per = (nparts + 7) / 8, k0 = y * per, k1 = min(nparts, k0 + per);
   float s = 0.f;
-  for (int k = 0; k < nparts; ++k) s += partials[(size_t)k * len + i];
-  g[i] = s;
+  if (i < len) {
+#pragma unroll 8
+    for (int k = k0; k < k1; ++k) s += partials[(size_t)k * len + i];
+  }
+  sm[y][threadIdx.x] = s;
+  __syncthreads();
+  if (y == 0 && i < len) {
+    float t = sm[0][threadIdx.x];
+#pragma unroll
+    for (int q = 1; q < 8; ++q) t += sm[q][threadIdx.x];
+    g[i] = t;
+  }
 }
 
 // Adam (Kingma & Ba 2015) on the FP32 master parameters
@@ -682,6 +838,7 @@ struct ch_ws_s {
   __nv_bfloat16 *c1 = nullptr, *c2 = nullptr, *c3 = nullptr;       // the same as tcgen05 B operands
   __nv_bfloat16 *c2f = nullptr, *c3f = nullptr;
   float* norm = nullptr;  // mean[8], inv_std[8], out_scale[4]
+  double* dinv = nullptr;   // 1 / dscale
   float* dscale = nullptr;  // Bmax x 8: RMS of the last change and of the second difference per sample and channel
   float* t = nullptr;       // Bmax x P x 4: dE/dy of the state-space loss
   float* e = nullptr;       // Bmax x P x 4 output errors y - t
@@ -690,6 +847,8 @@ struct ch_ws_s {
   double* rres = nullptr;   // Bmax x P x 4 residuals of the prediction
   double *tmp1 = nullptr, *tmp2 = nullptr;  // P x 4
   double* nrm = nullptr;    // Bmax x 8 squared residual norms per channel
+  double* rn_part = nullptr;          // the residual norms' block partials
+  unsigned int* rn_ticket = nullptr;  // ... and their last-block counter
   double *zex = nullptr, *zr = nullptr;  // preconditioned residuals: P x 4, Bmax x P x 4
   __nv_bfloat16 *x0 = nullptr, *a1 = nullptr, *a2 = nullptr;      // Bmax x P x {16, 32, 32}
   __nv_bfloat16 *dy = nullptr, *dz2 = nullptr, *dz1 = nullptr;    // Bmax x P x {16, 32, 32}
@@ -748,6 +907,13 @@ static ch_status ws_tc_setup() {
                                tc_smem_bytes<16, WS_C>()));
   CH_CUDA(cudaFuncSetAttribute(k_conv3x3_tc<WS_C, WS_C, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                tc_smem_bytes<WS_C, WS_C>()));
+  const int kp = (WG_SEG + 15) / 16 * 16;
+  CH_CUDA(cudaFuncSetAttribute(k_ws_wgrad<WS_C, 16, WS_COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               wg_smem<WS_C, 16>(kp)));
+  CH_CUDA(cudaFuncSetAttribute(k_ws_wgrad<WS_C, WS_C, WS_C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               wg_smem<WS_C, WS_C>(kp)));
+  CH_CUDA(cudaFuncSetAttribute(k_ws_wgrad<WS_CIN, WS_C, WS_C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               wg_smem<WS_CIN, WS_C>(kp)));
   return CH_OK;
 }
 
@@ -757,8 +923,8 @@ static void ws_rms(ch_ws_s* w, const T* s, const T* q, const T* q2, int B, cudaS
   const int P = w->P;
   const int chunk = std::max(1024, (P + WS_RMS_BLOCKS - 1) / WS_RMS_BLOCKS);
   const int nblk = (P + chunk - 1) / chunk;
-  k_ws_rms_part<T><<<dim3(nblk, B), 256, 0, st>>>(s, q, q2, P, chunk, w->rms_part);
-  k_ws_rms_fin<<<B, 32, 0, st>>>(w->rms_part, nblk, P, q2 != nullptr, w->dscale);
+  k_ws_rms_part<T><<<dim3(nblk, B), 256, 0, st>>>(s, q, q2, P, chunk, aligned4(sizeof(T), {s, q, q2}), w->rms_part);
+  k_ws_rms_fin<<<B, 32, 0, st>>>(w->rms_part, nblk, P, q2 != nullptr, w->dscale, w->dinv);
 }
 
 // One convolution of B samples on the handle's engine.
@@ -826,7 +992,8 @@ ch_status ws_create(int H, int W, int Bmax, ch_ws_s** out) {
   w->P = H * W;
   w->Bmax = Bmax;
   const size_t P = (size_t)w->P * Bmax;
-  const int nchunk = (w->P + WS_CHUNK - 1) / WS_CHUNK;
+  // weight-gradient partials: at most WG_BLOCKS strips and one more per segment and sample
+  const size_t nparts = WG_BLOCKS + (size_t)Bmax * ((W + WG_SEG - 1) / WG_SEG);
   ch_status r = CH_OK;
   if (r == CH_OK) r = w->mem.get(&w->params, WS_NPARAM);
   if (r == CH_OK) r = w->mem.get(&w->grads, WS_NPARAM);
@@ -844,6 +1011,7 @@ ch_status ws_create(int H, int W, int Bmax, ch_ws_s** out) {
   if (r == CH_OK) r = w->mem.get(&w->c3f, 9 * 16 * WS_C);
   if (r == CH_OK) r = w->mem.get(&w->norm, 20);
   if (r == CH_OK) r = w->mem.get(&w->dscale, (size_t)Bmax * 8);
+  if (r == CH_OK) r = w->mem.get(&w->dinv, (size_t)Bmax * 8);
   if (r == CH_OK) r = w->mem.get(&w->t, P * 4);
   if (r == CH_OK) r = w->mem.get(&w->e, P * 4);
   if (r == CH_OK) r = w->mem.get(&w->ge, P * 4);
@@ -854,7 +1022,7 @@ ch_status ws_create(int H, int W, int Bmax, ch_ws_s** out) {
   if (r == CH_OK) r = w->mem.get(&w->dz2, P * WS_C);
   if (r == CH_OK) r = w->mem.get(&w->dz1, P * WS_C);
   if (r == CH_OK) r = w->mem.get(&w->y, P * WS_COUT);
-  if (r == CH_OK) r = w->mem.get(&w->part, (size_t)Bmax * nchunk * (9 * WS_C * WS_C + WS_C));
+  if (r == CH_OK) r = w->mem.get(&w->part, nparts * (9 * WS_C * WS_C + WS_C));
   if (r == CH_OK) r = w->mem.get(&w->loss_part, 1024);
   if (r == CH_OK) r = w->mem.get(&w->rms_part, (size_t)Bmax * WS_RMS_BLOCKS * 8);
   if (r == CH_OK) {
@@ -913,23 +1081,27 @@ ch_status ws_set_norm(ch_ws_s* w, const float* host20, cudaStream_t st) {
   return CH_OK;
 }
 
+// The weight and bias gradients of one convolution of B samples into g (weights, then biases).
+template <int CIN, int COUTG, int COUTW>
+static void ws_wgrad(ch_ws_s* w, const __nv_bfloat16* X, const __nv_bfloat16* dY, int B, float* g, cudaStream_t st) {
+  const WgTiles t = wg_tiles(w->H, w->W, B);
+  const int kp = (t.seg + 15) / 16 * 16, len = 9 * CIN * COUTW + COUTW;
+  k_ws_wgrad<CIN, COUTG, COUTW><<<dim3(t.nstrip, t.nseg, B), 32 * WG_WARPS, wg_smem<CIN, COUTG>(kp), st>>>(
+      X, dY, w->H, w->W, t.nseg, t.seg, t.rows, kp, w->part);
+  k_ws_reduce<<<(len + 31) / 32, dim3(32, 8), 0, st>>>(w->part, t.nstrip * t.nseg * B, len, g);
+}
+
 // Backward pass from dy (already in w->dy) and, if lr > 0, an Adam step.
 static ch_status ws_backward_update(ch_ws_s* w, int B, float lr, cudaStream_t st) {
-  const int P = w->P;
   // backward through the data: dz2 = (W3 flipped * dy) . [a2 > 0];  dz1 = (W2 flipped * dz2) . [a1 > 0]
   ws_conv<16, WS_C, 2>(w, w->dy, w->w3f, w->c3f, nullptr, w->dz2, nullptr, w->a2, B, st);
   ws_conv<WS_C, WS_C, 2>(w, w->dz2, w->w2f, w->c2f, nullptr, w->dz1, nullptr, w->a1, B, st);
   CH_LAUNCHED();
-  // weight gradients, per sample and pixel chunk, then summed in order
-  const int nchunk = (P + WS_CHUNK - 1) / WS_CHUNK;
+  // weight gradients, per strip of image rows, then summed in order
   WsParams g = ws_views(w->grads);
-  const dim3 wg(nchunk, B);
-  k_ws_wgrad<WS_C, 16, WS_COUT><<<wg, 256, 0, st>>>(w->a2, w->dy, w->H, w->W, nchunk, w->part);
-  k_ws_reduce<<<blocks_for(WS_N3 + WS_COUT), TPB, 0, st>>>(w->part, B * nchunk, WS_N3 + WS_COUT, g.w3);
-  k_ws_wgrad<WS_C, WS_C, WS_C><<<wg, 256, 0, st>>>(w->a1, w->dz2, w->H, w->W, nchunk, w->part);
-  k_ws_reduce<<<blocks_for(WS_N2 + WS_C), TPB, 0, st>>>(w->part, B * nchunk, WS_N2 + WS_C, g.w2);
-  k_ws_wgrad<WS_CIN, WS_C, WS_C><<<wg, 256, 0, st>>>(w->x0, w->dz1, w->H, w->W, nchunk, w->part);
-  k_ws_reduce<<<blocks_for(WS_N1 + WS_C), TPB, 0, st>>>(w->part, B * nchunk, WS_N1 + WS_C, g.w1);
+  ws_wgrad<WS_C, 16, WS_COUT>(w, w->a2, w->dy, B, g.w3, st);
+  ws_wgrad<WS_C, WS_C, WS_C>(w, w->a1, w->dz2, B, g.w2, st);
+  ws_wgrad<WS_CIN, WS_C, WS_C>(w, w->x0, w->dz1, B, g.w1, st);
   CH_LAUNCHED();
   if (lr > 0.f) {
     w->adam_t += 1;
@@ -950,14 +1122,16 @@ ch_status ws_predict(ch_ws_s* w, const double* state, const double* prev, const 
   {
     ProfScope ps(st, K_WS_IO, 0, w->P * (32.0 * 3 + 32.0), 0.0);
     ws_rms<double>(w, state, prev, prev2, 1, st);
-    k_ws_pack<double><<<dim3(blocks_for(w->P), 1), TPB, 0, st>>>(state, prev, prev2, w->P, w->norm, w->norm + 8,
-                                                                  w->dscale, w->x0);
+    k_ws_pack<double><<<dim3(blocks_for(w->P), 1), TPB, 0, st>>>(state, prev, prev2, w->P,
+                                                                  aligned4(8, {state, prev, prev2}), w->norm,
+                                                                  w->norm + 8, w->dinv, w->x0);
   }
   CH_LAUNCHED();
   CH_TRY(ws_forward_packed(w, 1, st));
   {
     ProfScope ps(st, K_WS_IO, 0, w->P * (32.0 * 3 + 32.0 + 32.0), 0.0);
-    k_ws_unpack<<<blocks_for(w->P), TPB, 0, st>>>(state, prev, prev2, w->y, w->P, w->norm + 16, pred);
+    k_ws_unpack<<<blocks_for(w->P), TPB, 0, st>>>(state, prev, prev2, w->y, w->P,
+                                                      aligned4(8, {state, prev, prev2, pred}), w->norm + 16, pred);
   }
   CH_LAUNCHED();
   return CH_OK;
@@ -978,11 +1152,12 @@ ch_status ws_train_step(ch_ws_s* w, const float* x, const float* q, const float*
   }
   const int P = w->P;
   ws_rms<float>(w, x, q, q2, B, st);
-  k_ws_pack<float><<<dim3(blocks_for(P), B), TPB, 0, st>>>(x, q, q2, P, w->norm, w->norm + 8, w->dscale, w->x0);
+  k_ws_pack<float><<<dim3(blocks_for(P), B), TPB, 0, st>>>(x, q, q2, P, aligned4(4, {x, q, q2}), w->norm,
+                                                            w->norm + 8, w->dinv, w->x0);
   CH_LAUNCHED();
   CH_TRY(ws_forward_packed(w, B, st));
   const int lb = 304;
-  k_ws_err_theta<<<dim3(blocks_for(P), B), TPB, 0, st>>>(w->y, x, q, q2, n, P, w->norm + 16, w->dscale, w->e, w->t);
+  k_ws_err_theta<<<dim3(blocks_for(P), B), TPB, 0, st>>>(w->y, x, q, q2, n, P, w->norm + 16, w->dinv, w->e, w->t);
   k_ws_lap_loss<<<lb, 256, 0, st>>>(w->e, w->H, w->W, B, lap, w->ge, w->loss_part);
   k_ws_dy<<<lb, 256, 0, st>>>(w->e, w->ge, w->t, w->H, w->W, B, lap, w->dy);
   CH_TRY(ws_backward_update(w, B, lr, st));
@@ -1001,77 +1176,112 @@ ch_status ws_train_step(ch_ws_s* w, const float* x, const float* q, const float*
 // ---------------------------------------------------------------- residual-loss training
 // The correction c = y * out_scale * D (fp64, N x 4, D = s - 2 q + q2) of one sample, or the
 // linear extrapolation 2 s - q (mode 0).
-__global__ void k_ws_guess_part(int P, int mode, const double* __restrict__ s, const double* __restrict__ q,
+__global__ void k_ws_guess_part(int P, int mode, bool al, const double* __restrict__ s, const double* __restrict__ q,
                                 const double* __restrict__ q2, const float* __restrict__ y,
-                                const float* __restrict__ out_scale, double* __restrict__ out) {
+                                const float* __restrict__ out_scale, double4_32a* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= P) return;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const size_t o = (size_t)i * 4 + c;
-    out[o] = mode == 0 ? 2.0 * s[o] - q[o]
-                       : (double)y[(size_t)i * WS_COUT + c] * (double)out_scale[c] * (s[o] - 2.0 * q[o] + q2[o]);
+  const Quad<double> a = ld4(s, i, al), b = ld4(q, i, al);
+  if (mode == 0) {
+    out[i] = make_double4_32a(2.0 * a.x - b.x, 2.0 * a.y - b.y, 2.0 * a.z - b.z, 2.0 * a.w - b.w);
+  } else {
+    const Quad<double> c = ld4(q2, i, al);
+    const float4 yv = *reinterpret_cast<const float4*>(y + (size_t)i * WS_COUT);
+    out[i] = make_double4_32a((double)yv.x * (double)out_scale[0] * (a.x - 2.0 * b.x + c.x),
+                              (double)yv.y * (double)out_scale[1] * (a.y - 2.0 * b.y + c.y),
+                              (double)yv.z * (double)out_scale[2] * (a.z - 2.0 * b.z + c.z),
+                              (double)yv.w * (double)out_scale[3] * (a.w - 2.0 * b.w + c.w));
   }
 }
 
 // out = a - b (N x 4)
-__global__ void k_ws_sub(int n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out) {
+__global__ void k_ws_sub(int P, const double4_32a* __restrict__ a, const double4_32a* b, double4_32a* out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = a[i] - b[i];
+  if (i >= P) return;
+  const double4_32a u = a[i], v = b[i];
+  out[i] = make_double4_32a(u.x - v.x, u.y - v.y, u.z - v.z, u.w - v.w);
 }
 
 // nrm[0..3] = per channel sum of rex * zex, nrm[4..7] = per channel sum of r * z, where z = P^-1 r
-// (or z = r for the plain norm); one block, fixed order
-__global__ void k_ws_resnorm(int P, const double* __restrict__ rex, const double* __restrict__ zex,
-                             const double* __restrict__ r, const double* __restrict__ z, double* __restrict__ nrm) {
-  __shared__ double red[8][256];
+// (or z = r for the plain norm), in a fixed order: block b adds its chunk of pixels into part[b][8]
+// and the last block to finish adds the blocks' sums in block order.  (One block over the whole
+// image took 222 us at 257 x 257, latency alone.)
+constexpr int RN_BLOCKS = 152;
+__global__ void __launch_bounds__(256) k_ws_resnorm(int P, const double4_32a* __restrict__ rex,
+                                                    const double4_32a* __restrict__ zex,
+                                                    const double4_32a* __restrict__ r,
+                                                    const double4_32a* __restrict__ z, double* __restrict__ part,
+                                                    unsigned int* __restrict__ ticket, double* __restrict__ nrm) {
+  __shared__ double red[8][8];
+  __shared__ bool last;
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int i = threadIdx.x; i < P; i += blockDim.x) {
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const size_t o = (size_t)i * 4 + c;
-      acc[c] = fma(rex[o], zex[o], acc[c]);
-      acc[4 + c] = fma(r[o], z[o], acc[4 + c]);
-    }
+  const int chunk = (P + gridDim.x - 1) / gridDim.x, i1 = min(P, ((int)blockIdx.x + 1) * chunk);
+  for (int i = blockIdx.x * chunk + threadIdx.x; i < i1; i += blockDim.x) {
+    const double4_32a a = rex[i], b = zex[i], c = r[i], d = z[i];
+    acc[0] = fma(a.x, b.x, acc[0]);
+    acc[1] = fma(a.y, b.y, acc[1]);
+    acc[2] = fma(a.z, b.z, acc[2]);
+    acc[3] = fma(a.w, b.w, acc[3]);
+    acc[4] = fma(c.x, d.x, acc[4]);
+    acc[5] = fma(c.y, d.y, acc[5]);
+    acc[6] = fma(c.z, d.z, acc[6]);
+    acc[7] = fma(c.w, d.w, acc[7]);
   }
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-  for (int c = 0; c < 8; ++c) red[c][threadIdx.x] = acc[c];
+  for (int c = 0; c < 8; ++c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+    if (lane == 0) red[w][c] = acc[c];
+  }
   __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-#pragma unroll
-      for (int c = 0; c < 8; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + h];
-    }
-    __syncthreads();
+  if (threadIdx.x < 8) {
+    double t = 0.0;
+    for (int q = 0; q < 8; ++q) t += red[q][threadIdx.x];
+    part[blockIdx.x * 8 + threadIdx.x] = t;
   }
-  if (threadIdx.x < 8) nrm[threadIdx.x] = red[threadIdx.x][0];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // warp w: value w, lanes over blocks (lane, lane + 32, ...), then the lanes' sums
+  double t = 0.0;
+  for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(part + b * 8 + w);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) nrm[w] = t;
+  if (threadIdx.x == 0) *ticket = 0;
 }
 
 // dy of one sample from g = A z: L = sum_species ln(<r, z>_sp / <rex, zex>_sp) / (2B) with
 // z = P^-1 r (P^-1 symmetric, or the identity), r = rex - A c, so dL/dc = -2 A z / <r, z>_sp / (2B)
 // and dL/dy_c = dL/dc_c * out_scale_c * D_c (c = y out_scale D).
 // Channel c belongs to species c % 2 (channels phi_p, phi_n, mu_p, mu_n).
-__global__ void k_ws_res_dy(int P, int B, const double* __restrict__ g, const double* __restrict__ nrm,
+__global__ void k_ws_res_dy(int P, int B, const double4_32a* __restrict__ g, const double* __restrict__ nrm,
                             const float* __restrict__ out_scale, const double* __restrict__ s,
-                            const double* __restrict__ q, const double* __restrict__ q2,
+                            const double* __restrict__ q, const double* __restrict__ q2, bool al,
                             __nv_bfloat16* __restrict__ dy) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= P) return;
-  double wsp[2];
-#pragma unroll
-  for (int sp = 0; sp < 2; ++sp) {
+  __shared__ double wsp[2];
+  if (threadIdx.x < 2) {  // once per block: an FP64 division per pixel would cost more than the rest
+    const int sp = threadIdx.x;
     const double den = nrm[sp] + nrm[sp + 2], num = nrm[4 + sp] + nrm[6 + sp];
     wsp[sp] = (den > 0.0 && num > 0.0) ? 1.0 / (num * (double)B) : 0.0;
   }
-#pragma unroll
-  for (int c = 0; c < 16; ++c) {
-    float v = 0.f;
-    if (c < 4) {
-      const size_t o = (size_t)i * 4 + c;
-      v = (float)(-g[o] * wsp[c % 2] * ((double)out_scale[c] * (s[o] - 2.0 * q[o] + q2[o])));
-    }
-    dy[(size_t)i * 16 + c] = __float2bfloat16_rn(v);
-  }
+  __syncthreads();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= P) return;
+  const double4_32a gv = g[i];
+  const Quad<double> sv = ld4(s, i, al), qv = ld4(q, i, al), q2v = ld4(q2, i, al);
+  const float v0 = (float)(-gv.x * wsp[0] * ((double)out_scale[0] * (sv.x - 2.0 * qv.x + q2v.x)));
+  const float v1 = (float)(-gv.y * wsp[1] * ((double)out_scale[1] * (sv.y - 2.0 * qv.y + q2v.y)));
+  const float v2 = (float)(-gv.z * wsp[0] * ((double)out_scale[2] * (sv.z - 2.0 * qv.z + q2v.z)));
+  const float v3 = (float)(-gv.w * wsp[1] * ((double)out_scale[3] * (sv.w - 2.0 * qv.w + q2v.w)));
+  uint4* o = reinterpret_cast<uint4*>(dy + (size_t)i * 16);
+  o[0] = make_uint4(pack_bf16(__float2bfloat16_rn(v0), __float2bfloat16_rn(v1)),
+                    pack_bf16(__float2bfloat16_rn(v2), __float2bfloat16_rn(v3)), 0u, 0u);
+  o[1] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 ch_status ws_train_residual(ch_ws_s* w, const ch_system_s* sys, ch_precond_s* pc, const double* x,
@@ -1100,12 +1310,18 @@ ch_status ws_train_residual(ch_ws_s* w, const ch_system_s* sys, ch_precond_s* pc
     CH_TRY(w->mem.get(&w->tmp1, (size_t)P * 4));
     CH_TRY(w->mem.get(&w->tmp2, (size_t)P * 4));
     CH_TRY(w->mem.get(&w->nrm, (size_t)w->Bmax * 8));
+    CH_TRY(w->mem.get(&w->rn_part, (size_t)RN_BLOCKS * 8));
+    CH_TRY(w->mem.get(&w->rn_ticket, 1));
+    CH_CUDA(cudaMemsetAsync(w->rn_ticket, 0, sizeof(unsigned int), st));
   }
   ws_rms<double>(w, x, q, q2, B, st);
-  k_ws_pack<double><<<dim3(blocks_for(P), B), TPB, 0, st>>>(x, q, q2, P, w->norm, w->norm + 8, w->dscale, w->x0);
+  const bool al = aligned4(8, {x, q, q2});  // (a sample is a multiple of 32 bytes)
+  k_ws_pack<double><<<dim3(blocks_for(P), B), TPB, 0, st>>>(x, q, q2, P, al, w->norm, w->norm + 8, w->dinv, w->x0);
   CH_LAUNCHED();
   CH_TRY(ws_forward_packed(w, B, st));
-  const int nb = blocks_for(P), nb4 = blocks_for(4 * P);
+  const int nb = blocks_for(P), rnb = std::min(RN_BLOCKS, nb);
+  const auto v4 = [](const double* p) { return reinterpret_cast<const double4_32a*>(p); };
+  const auto m4 = [](double* p) { return reinterpret_cast<double4_32a*>(p); };
   for (int b = 0; b < B; ++b) {
     const double* xs = x + (size_t)b * P * 4;
     const double* qs = q + (size_t)b * P * 4;
@@ -1114,15 +1330,16 @@ ch_status ws_train_residual(ch_ws_s* w, const ch_system_s* sys, ch_precond_s* pc
     double* r = w->rres + (size_t)b * P * 4;
     // rex = b(s) - A (2 s - q)
     CH_TRY(rhs_strided(sys, xs, xs + 1, 4, w->tmp1, st));
-    k_ws_guess_part<<<nb, TPB, 0, st>>>(P, 0, xs, qs, q2s, nullptr, nullptr, w->tmp2);
+    k_ws_guess_part<<<nb, TPB, 0, st>>>(P, 0, al, xs, qs, q2s, nullptr, nullptr, m4(w->tmp2));
     CH_LAUNCHED();
     CH_TRY(apply_A(sys, w->tmp2, rex, st));
-    k_ws_sub<<<nb4, TPB, 0, st>>>(4 * P, w->tmp1, rex, rex);
+    k_ws_sub<<<nb, TPB, 0, st>>>(P, v4(w->tmp1), v4(rex), m4(rex));
     // r = rex - A c
-    k_ws_guess_part<<<nb, TPB, 0, st>>>(P, 1, xs, qs, q2s, w->y + (size_t)b * P * WS_COUT, w->norm + 16, w->tmp2);
+    k_ws_guess_part<<<nb, TPB, 0, st>>>(P, 1, al, xs, qs, q2s, w->y + (size_t)b * P * WS_COUT, w->norm + 16,
+                                        m4(w->tmp2));
     CH_LAUNCHED();
     CH_TRY(apply_A(sys, w->tmp2, w->tmp1, st));
-    k_ws_sub<<<nb4, TPB, 0, st>>>(4 * P, rex, w->tmp1, r);
+    k_ws_sub<<<nb, TPB, 0, st>>>(P, v4(rex), v4(w->tmp1), m4(r));
     // z = P^-1 r, zex = P^-1 rex (Algorithm 1), or the residuals themselves
     const double* zex = rex;
     const double* z = r;
@@ -1132,10 +1349,10 @@ ch_status ws_train_residual(ch_ws_s* w, const ch_system_s* sys, ch_precond_s* pc
       zex = w->zex;
       z = w->zr + (size_t)b * P * 4;
     }
-    k_ws_resnorm<<<1, 256, 0, st>>>(P, rex, zex, r, z, w->nrm + 8 * b);
+    k_ws_resnorm<<<rnb, 256, 0, st>>>(P, v4(rex), v4(zex), v4(r), v4(z), w->rn_part, w->rn_ticket, w->nrm + 8 * b);
     // g = A z (A is symmetric) -> dy of this sample
     CH_TRY(apply_A(sys, z, w->tmp1, st));
-    k_ws_res_dy<<<nb, TPB, 0, st>>>(P, B, w->tmp1, w->nrm + 8 * b, w->norm + 16, xs, qs, q2s,
+    k_ws_res_dy<<<nb, TPB, 0, st>>>(P, B, v4(w->tmp1), w->nrm + 8 * b, w->norm + 16, xs, qs, q2s, al,
                                     w->dy + (size_t)b * P * 16);
     CH_LAUNCHED();
   }
