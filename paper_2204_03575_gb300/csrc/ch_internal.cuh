@@ -134,8 +134,7 @@ inline void launch_k(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, size_
 }
 
 // ---------------------------------------------------------------- primitives (sparse.cu)
-// exclusive scan of n int64 values in place; returns the total in *total (host)
-ch_status scan_i64(int64_t* data, int64_t n, int64_t* total, cudaStream_t st, Alloc& tmp);
+// rowptr (n + 1) = exclusive scan of the counts; returns the total in *total (host)
 ch_status scan_i32_to_rowptr(const int* counts, int* rowptr, int n, int64_t* total,
                              cudaStream_t st, Alloc& tmp);
 // incidence lists: for each of nitems items with k entries (ids in [0,nkeys)), build the
