@@ -134,12 +134,7 @@ inline void launch_k(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, size_
 }
 
 // ---------------------------------------------------------------- primitives (sparse.cu)
-<<<<<<< paper_2204_03575_gb300/csrc/ch_internal.cuh
 // rowptr (n + 1) = exclusive scan of the counts; returns the total in *total (host)
-=======
-// exclusive scan of n int64 values in place; returns the total in *total (host)
-ch_status scan_i64(int64_t* data, int64_t n, int64_t* total, cudaStream_t st, Alloc& tmp);
->>>>>>> _work/ldt/paper_2204_03575_gb300/csrc/ch_internal.cuh
 ch_status scan_i32_to_rowptr(const int* counts, int* rowptr, int n, int64_t* total,
                              cudaStream_t st, Alloc& tmp);
 // incidence lists: for each of nitems items with k entries (ids in [0,nkeys)), build the
@@ -208,13 +203,6 @@ struct Lattice {
   int2* wh = nullptr;           // nids: strides of the id's run
   int* rep = nullptr;           // nids: a node of the class (the middle one along its inner axes)
 };
-<<<<<<< paper_2204_03575_gb300/csrc/ch_internal.cuh
-=======
-// The grid of one run: first node, first cell, cells per axis.
-struct CellGrid {
-  int node0, cell0, nx, ny, nz;
-};
->>>>>>> _work/ldt/paper_2204_03575_gb300/csrc/ch_internal.cuh
 // strides of the lattice directions: 7 in 2D (the triangles' edges), 15 in 3D (the Kuhn tetrahedra's),
 // ascending for any W, H >= 2, i.e. in CSR column order; direction ND / 2 is the node itself
 __host__ __device__ __forceinline__ int lat_off(int nd, int d, int W, int WH) {
@@ -249,10 +237,6 @@ struct ch_mesh_s {
   int *n2b_ptr = nullptr, *n2b = nullptr;  // node -> incident bottom facets
   int *n2t_ptr = nullptr, *n2t = nullptr;  // node -> incident top facets
   ch::Lattice lat;
-<<<<<<< paper_2204_03575_gb300/csrc/ch_internal.cuh
-=======
-  ch::CellGrid* cell_grid = nullptr;  // device, per run
->>>>>>> _work/ldt/paper_2204_03575_gb300/csrc/ch_internal.cuh
   ch::Alloc mem;
 };
 
@@ -267,12 +251,7 @@ struct ch_system_s {
   double* valK = nullptr;
   double* valH = nullptr;
   int* diag = nullptr;  // position of the diagonal entry of each row
-<<<<<<< paper_2204_03575_gb300/csrc/ch_internal.cuh
   double* eload = nullptr;  // E x (dim+1) x 2: per element and vertex, the f-load contributions
-=======
-  double2* eload = nullptr;  // per grid cell and corner, the f-load contributions (polymer, NFA)
-  void* log_tables = nullptr;  // potential = 3: the load's logarithm tables
->>>>>>> _work/ldt/paper_2204_03575_gb300/csrc/ch_internal.cuh
   double* bw = nullptr;     // pattern = 1: Fb x 2 species x (dim + dim^2) substrate weights, else null
   double a = 0, c = 0;  // A = [[M, aK], [aK, -cM]]
   ch::Alloc mem;
