@@ -1,8 +1,9 @@
 // Mesh generation, P1 assembly, explicit loads and the block operator of Eq. (14).
 //
-// Everything is node-centric ("gather"): the thread of node i visits the simplices or
+// Everything is node-centric ("gather"): the thread of node i visits the simplices, cells or
 // boundary facets incident to i in increasing index order and adds their contributions,
 // so every sum has a fixed order and results are bitwise reproducible (no atomics).
+#include <algorithm>
 #include <cmath>
 
 #include "ch_internal.cuh"
@@ -243,6 +244,13 @@ ch_status mesh_build(ch_mesh_s* m, cudaStream_t st) {
     }
   }
   CH_CUDA(cudaMemcpyAsync(L.wh, wh.data(), sizeof(int2) * L.nids, cudaMemcpyHostToDevice, st));
+  std::vector<CellGrid> grid(R);
+  for (int r = 0; r < R; ++r) {
+    const ch_params& p = m->runs[r];
+    grid[r] = {m->run_off[r], eoff[r] / (d == 2 ? 2 : 6), p.nx, p.ny, d == 3 ? p.nz : 0};
+  }
+  CH_TRY(m->mem.get(&m->cell_grid, (size_t)R));
+  CH_CUDA(cudaMemcpyAsync(m->cell_grid, grid.data(), sizeof(CellGrid) * R, cudaMemcpyHostToDevice, st));
   CH_CUDA(cudaMemcpyAsync(L.rep, rep.data(), sizeof(int) * L.nids, cudaMemcpyHostToDevice, st));
   for (int r = 0; r < R; ++r) {
     const ch_params& p = m->runs[r];
@@ -484,6 +492,8 @@ __global__ void k_facet_pattern(const double* coords, const int* bot, int nf, do
   for (int q = 0; q < 2 * NW; ++q) bw[(size_t)f * 2 * NW + q] = W[q / NW][q % NW];
 }
 
+static ch_status log_tables(ch_system_s* s, cudaStream_t st);
+
 // Weights of every run's bottom facets (each run's box is [0, Lx_r] in x).
 static ch_status substrate_weights(const ch_mesh_s* m, ch_system_s* s, cudaStream_t st) {
   const int d = m->dim, R = (int)m->runs.size();
@@ -525,7 +535,7 @@ ch_status assemble_system(const ch_mesh_s* m, ch_system_s* s, cudaStream_t st) {
   CH_TRY(s->mem.get(&s->valM, (size_t)nnz));
   CH_TRY(s->mem.get(&s->valK, (size_t)nnz));
   CH_TRY(s->mem.get(&s->valH, (size_t)nnz));
-  CH_TRY(s->mem.get(&s->eload, (size_t)m->E * (d + 1) * 2));
+  CH_TRY(s->mem.get(&s->eload, (size_t)(m->E / (d == 2 ? 2 : 6)) * (d == 2 ? 4 : 8)));
   CH_TRY(s->mem.get(&s->diag, (size_t)N));
   k_pattern<<<blocks_for(N), TPB, 0, st>>>(m->elems, d + 1, m->n2e_ptr, m->n2e, N, s->rowptr,
                                             nullptr, s->col, overflow);
@@ -540,6 +550,7 @@ ch_status assemble_system(const ch_mesh_s* m, ch_system_s* s, cudaStream_t st) {
   // H = a K + sqrt(c) M  (Section 3, matching Schur approximation)
   k_axpby_vals<<<blocks_for(nnz), TPB, 0, st>>>(s->valK, s->valM, s->a, sqrt(s->c), s->valH, nnz);
   CH_LAUNCHED();
+  if (s->p.potential == 3) CH_TRY(log_tables(s, st));
   if (s->p.pattern && s->p.bc_mode) CH_TRY(substrate_weights(m, s, st));
   int ovf = 0;
   CH_CUDA(cudaMemcpyAsync(&ovf, overflow, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -564,36 +575,70 @@ ch_status assemble_system(const ch_mesh_s* m, ch_system_s* s, cudaStream_t st) {
 // where <x> is the sum of x over the simplex's vertices.
 
 struct MeshPod {
-  int dim, N, E;
-  const double* coords;
+  int dim, N, C;                // nodes, cells (the 2 triangles or 6 tetrahedra of a grid cell)
   const int* elems;
   const int* bot;
   const int* top;
   const double* vol;
   const double* bvol;
   const double* tvol;
-  const int *n2e_ptr, *n2e, *n2b_ptr, *n2b, *n2t_ptr, *n2t;
+  const int *n2b_ptr, *n2b, *n2t_ptr, *n2t;
+  const int* node_run;
+  const CellGrid* grid;         // per run
 };
 
 static MeshPod mesh_pod(const ch_mesh_s* s) {
   MeshPod v;
   v.dim = s->dim;
   v.N = s->N;
-  v.E = s->E;
-  v.coords = s->coords;
+  v.C = s->E / (s->dim == 2 ? 2 : 6);
   v.elems = s->elems;
   v.bot = s->bot;
   v.top = s->top;
   v.vol = s->vol;
   v.bvol = s->bvol;
   v.tvol = s->tvol;
-  v.n2e_ptr = s->n2e_ptr;
-  v.n2e = s->n2e;
   v.n2b_ptr = s->n2b_ptr;
   v.n2b = s->n2b;
   v.n2t_ptr = s->n2t_ptr;
   v.n2t = s->n2t;
+  v.node_run = s->node_run;
+  v.grid = s->cell_grid;
   return v;
+}
+
+// Corners of a cell: bit 0 is +x, bit 1 +y, bit 2 +z.  Simplex t of the cell runs from corner 0 over
+// path[t][0] (and path[t][1]) to the opposite corner (k_mesh_elems' order of triangles and tetrahedra).
+template <int D> struct CellSimplices;
+template <> struct CellSimplices<2> {
+  static constexpr int NT = 2, NC = 4;
+  __host__ __device__ static constexpr int corner(int t, int a) {  // t = 0: (0, 1, 3), 1: (0, 3, 2)
+    constexpr int c[2][3] = {{0, 1, 3}, {0, 3, 2}};
+    return c[t][a];
+  }
+};
+template <> struct CellSimplices<3> {
+  static constexpr int NT = 6, NC = 8;
+  __host__ __device__ static constexpr int corner(int t, int a) {
+    constexpr int c[6][4] = {{0, 1, 3, 7}, {0, 1, 5, 7}, {0, 2, 3, 7}, {0, 2, 6, 7}, {0, 4, 5, 7}, {0, 4, 6, 7}};
+    return c[t][a];
+  }
+};
+// the nodes of a cell's corners, read from its simplices
+template <int D>
+__device__ __forceinline__ void cell_nodes(const int* elems, int cell, int (&v)[CellSimplices<D>::NC]) {
+  using S = CellSimplices<D>;
+  const int* e = elems + (size_t)cell * S::NT * (D + 1);
+#pragma unroll
+  for (int t = 0; t < S::NT; ++t)
+#pragma unroll
+    for (int a = 0; a <= D; ++a) {
+      bool first = true;  // each corner once
+#pragma unroll
+      for (int q = 0; q < t * (D + 1) + a; ++q)
+        if (S::corner(q / (D + 1), q % (D + 1)) == S::corner(t, a)) first = false;
+      if (first) v[S::corner(t, a)] = e[t * (D + 1) + a];
+    }
 }
 
 struct LoadCoef {
@@ -604,54 +649,69 @@ struct LoadCoef {
   const double* bw;  // patterned substrate weights (Fb x 2 x (D + D^2)), or null for p = 1
 };
 
-// Per element e and vertex a, eload[(e (D+1) + a) 2 + {0, 1}] = |T| (7 int p q^2 l_a - 0.2 int phi_s l_a)
-// / |T| and the same with p and q exchanged (Eq. (15)'s f' for polymer and NFA against the hat
-// function of vertex a).  The vertex sums are formed once per element; int_pqq_li's terms that do
-// not involve the vertex (A, B, C below) are element constants (the closed form above).
+// The loads are formed per grid cell, one entry per corner, and each node then adds its 4 (8) cells'
+// entries: eload[(cell NC + corner) 2 + {0, 1}] = int over the cell of f_p' and f_n' against the corner's
+// hat function.  Per simplex T with vertex sums <.> the closed form above is, with c = |T| 7 d!/(d+4)!
+// and b = |T| 0.2 / ((d+1)(d+2)),
+//   c (<p><q>^2 + 2<pq><q> + <q^2><p> + 2<pq^2>) - b (<phi_s> + 1)            element constants
+//   + p_i (c (<q>^2 + <q^2>) + b + q_i (4 c <q> + 6 c q_i)) + q_i (2 c (<p><q> + <pq>) + b + 2 c <p> q_i)
+// five FMAs per vertex and species.  FP64-pipe bound (about 95 instructions per tetrahedron): 518 us on
+// 128 x 128 x 32 cells and 83 us on 512 x 512, where one thread per simplex with a store per vertex
+// took 875 and 122 us.  A
+// thread takes a cell, so the products of the nodal values are formed once for its simplices and
+// there is one entry per corner instead of one per simplex and vertex (a third of the stores in 3D).
 template <int D>
-__global__ void k_elem_loads(const MeshPod m, LoadCoef L, const double* pp, const double* pn, int ld,
-                             double* __restrict__ eload) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= m.E) return;
+__global__ void __launch_bounds__(128) k_cell_loads(const MeshPod m, LoadCoef L, const double* pp, const double* pn,
+                                                    int ld, double2* __restrict__ eload) {
+  using S = CellSimplices<D>;
+  const int cell = blockIdx.x * blockDim.x + threadIdx.x;
+  if (cell >= m.C) return;
   constexpr double c4 = (D == 2) ? 1.0 / 360.0 : 1.0 / 840.0;  // d!/(d+4)!
   constexpr double c2 = 1.0 / ((D + 1) * (D + 2));             // int lambda_a lambda_i / |T|, a != i
-  const int* ev = m.elems + (D + 1) * e;
-  double P[D + 1], Q[D + 1];
+  int v[S::NC];
+  cell_nodes<D>(m.elems, cell, v);
+  double P[S::NC], Q[S::NC], PQ[S::NC], Fp[S::NC], Fn[S::NC];
 #pragma unroll
-  for (int a = 0; a <= D; ++a) {
-    P[a] = pp[(size_t)ld * ev[a]];
-    Q[a] = pn[(size_t)ld * ev[a]];
+  for (int a = 0; a < S::NC; ++a) {
+    P[a] = pp[(size_t)ld * v[a]];
+    Q[a] = pn[(size_t)ld * v[a]];
+    PQ[a] = P[a] * Q[a];
+    Fp[a] = Fn[a] = 0.0;
   }
-  double Sp = 0, Sq = 0, Spq = 0, Spp = 0, Sqq = 0, Spqq = 0, Sppq = 0;
+  const double vol = m.vol[(size_t)cell * S::NT];  // the cell's simplices are congruent
+  const double c = vol * L.cubic * c4, b = vol * L.cs * c2;
+  const double c_2 = 2.0 * c, c_4 = 4.0 * c, c_6 = 6.0 * c;
 #pragma unroll
-  for (int a = 0; a <= D; ++a) {
-    Sp += P[a];
-    Sq += Q[a];
-    const double pq = P[a] * Q[a];
-    Spq += pq;
-    Spp += P[a] * P[a];
-    Sqq += Q[a] * Q[a];
-    Spqq += pq * Q[a];
-    Sppq += pq * P[a];
-  }
-  // int p q^2 l_i / (c4 |T|) = A + p_i B + q_i (C + 2 q_i Sp) + p_i q_i (4 Sq + 6 q_i), and the
-  // same with p and q exchanged (C is symmetric)
-  const double Ap = Sp * Sq * Sq + 2.0 * Spq * Sq + Sqq * Sp + 2.0 * Spqq, Bp = Sq * Sq + Sqq;
-  const double An = Sq * Sp * Sp + 2.0 * Spq * Sp + Spp * Sq + 2.0 * Sppq, Bn = Sp * Sp + Spp;
-  const double C = 2.0 * (Sp * Sq + Spq);
-  const double vol = m.vol[e];
-  const double ss = (D + 1) - Sp - Sq;  // sum of phi_s over the vertices
+  for (int t = 0; t < S::NT; ++t) {
+    double Sp = 0, Sq = 0, Spq = 0, Spp = 0, Sqq = 0, Spqq = 0, Sppq = 0;
 #pragma unroll
-  for (int a = 0; a <= D; ++a) {
-    const double pi = P[a], qi = Q[a];
-    const double Ip = c4 * (Ap + pi * Bp + qi * (C + 2.0 * qi * Sp) + pi * qi * (4.0 * Sq + 6.0 * qi));
-    const double In = c4 * (An + qi * Bn + pi * (C + 2.0 * pi * Sq) + qi * pi * (4.0 * Sp + 6.0 * pi));
-    const double Is = c2 * (ss + (1.0 - pi - qi));  // int phi_s lambda_i / |T|
-    double2 out;
-    out.x = vol * (L.cubic * Ip - L.cs * Is);
-    out.y = vol * (L.cubic * In - L.cs * Is);
-    reinterpret_cast<double2*>(eload)[(size_t)e * (D + 1) + a] = out;
+    for (int a = 0; a <= D; ++a) {
+      const int k = S::corner(t, a);
+      Sp += P[k];
+      Sq += Q[k];
+      Spq += PQ[k];
+      Spp = fma(P[k], P[k], Spp);
+      Sqq = fma(Q[k], Q[k], Sqq);
+      Spqq = fma(PQ[k], Q[k], Spqq);
+      Sppq = fma(PQ[k], P[k], Sppq);
+    }
+    const double bs = b * ((D + 2) - Sp - Sq);  // b (<phi_s> + 1)
+    const double cSp = c * Sp, cSq = c * Sq, cpq = c_2 * Spq;
+    const double Ap = fma(c_2, Spqq, fma(cSp, fma(Sq, Sq, Sqq), cpq * Sq)) - bs;
+    const double An = fma(c_2, Sppq, fma(cSq, fma(Sp, Sp, Spp), cpq * Sp)) - bs;
+    const double Bp = fma(c, fma(Sq, Sq, Sqq), b), Bn = fma(c, fma(Sp, Sp, Spp), b);
+    const double C = fma(2.0 * cSp, Sq, cpq) + b;
+    const double Sp2 = 2.0 * cSp, Sq2 = 2.0 * cSq, Sp4 = c_4 * Sp, Sq4 = c_4 * Sq;
+#pragma unroll
+    for (int a = 0; a <= D; ++a) {
+      const int k = S::corner(t, a);
+      const double p = P[k], q = Q[k];
+      Fp[k] += fma(p, fma(q, fma(c_6, q, Sq4), Bp), fma(q, fma(Sp2, q, C), Ap));
+      Fn[k] += fma(q, fma(p, fma(c_6, p, Sp4), Bn), fma(p, fma(Sq2, p, C), An));
+    }
   }
+#pragma unroll
+  for (int a = 0; a < S::NC; ++a) eload[(size_t)cell * S::NC + a] = make_double2(Fp[a], Fn[a]);
 }
 
 // ---- The Flory-Huggins load (potential = 3).  Section 2's bulk energy
@@ -663,12 +723,6 @@ __global__ void k_elem_loads(const MeshPod m, LoadCoef L, const double* pp, cons
 // with each logarithm taken at max(phi, delta) (a NaN stays a NaN).  The integrand is not a
 // polynomial, so a fixed rule defines the load: on every simplex the product of 3-point
 // Gauss-Legendre rules collapsed onto it (Duffy), 9 points on a triangle, 27 on a tetrahedron.
-struct FhRule {
-  int nq;
-  double lam[27][4];  // barycentric coordinates of the points
-  double w[27];       // weights, summing to 1: int_T g ~ |T| sum_q w_q g(x_q)
-};
-
 struct FhCoef {
   double chi_pn, chi_ps, chi_ns, inv_np, inv_nn, inv_ns, delta;
 };
@@ -677,90 +731,210 @@ struct FhCoef {
 // Square (u, v) -> triangle (u, v (1 - u)), Jacobian 1 - u; cube (u, v, t) -> tetrahedron
 // (u, v (1 - u), t (1 - u)(1 - v)), Jacobian (1 - u)^2 (1 - v); normalised by the reference
 // simplex's measure (1/2, 1/6).
-static FhRule fh_rule(int dim) {
-  const double g[3] = {0.5 - std::sqrt(15.0) / 10.0, 0.5, 0.5 + std::sqrt(15.0) / 10.0};
-  const double w[3] = {5.0 / 18.0, 4.0 / 9.0, 5.0 / 18.0};
-  FhRule R{};
-  int q = 0;
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j)
-      for (int k = 0; k < (dim == 3 ? 3 : 1); ++k) {
-        const double u = g[i], v = g[j];
-        double xi[3] = {u, v * (1.0 - u), 0.0};
-        double wt;
-        if (dim == 2) {
-          wt = 2.0 * w[i] * w[j] * (1.0 - u);
-        } else {
-          xi[2] = g[k] * (1.0 - u) * (1.0 - v);
-          wt = 6.0 * w[i] * w[j] * w[k] * (1.0 - u) * (1.0 - u) * (1.0 - v);
-        }
-        R.lam[q][0] = 1.0 - xi[0] - xi[1] - xi[2];
-        for (int a = 1; a <= dim; ++a) R.lam[q][a] = xi[a - 1];
-        R.w[q] = wt;
-        ++q;
+__device__ __forceinline__ constexpr double gl_x(int i) {
+  return i == 0 ? 0.11270166537925831148 : (i == 1 ? 0.5 : 0.88729833462074168852);
+}
+__device__ __forceinline__ constexpr double gl_w(int i) { return i == 1 ? 4.0 / 9.0 : 5.0 / 18.0; }
+
+// Natural logarithm of a positive value by tables over the mantissa and the exponent (Tang 1990,
+// "Table-driven implementation of the logarithm function in IEEE floating-point arithmetic"): x = 2^k m,
+// with f the reciprocal of the middle of m's interval (1024 of them) rounded to FP32, r = m f - 1 (one
+// FMA; |r| <= 2^-11 and a little), log x = k log 2 - log f + log1p(r) and log1p by its Taylor series
+// through r^4 (the next term is below 2^-57).  Seven FP64 instructions where the general function
+// takes several times as many, and the kernel is bound by that pipe; the absolute error stays within
+// 2^-53 (1 + |log x|) and a rounding, which is what the sums it enters can resolve.  Other values (zero,
+// negative, denormal, infinite, NaN) take CUDA's log.
+struct LogTables {
+  double2 m[1024];  // f, -log f
+  double k[2048];   // (biased exponent - 1023) log 2
+};
+__global__ void k_log_tables(LogTables* t) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < 1024) {
+    const double f = (double)(float)(1.0 / (1.0 + (i + 0.5) / 1024.0));
+    t->m[i] = make_double2(f, -log(f));
+  }
+  if (i < 2048) t->k[i] = (i - 1023) * 0.69314718055994530942;
+}
+// log of max(x, delta), delta > 0; a NaN stays a NaN.  Positive doubles compare like their bits (an FP64
+// comparison would take the pipe).
+__device__ __forceinline__ double guarded_log(double x, double delta, const LogTables* tab) {
+  long long bits = __double_as_longlong(x);
+  const long long lo = __double_as_longlong(delta);
+  if ((unsigned)(bits >> 32) - 0x00100000u >= 0x7fe00000u) {
+    x = x < delta ? delta : x;
+    bits = __double_as_longlong(x);
+    if ((unsigned)(bits >> 32) - 0x00100000u >= 0x7fe00000u) return log(x);
+  }
+  bits = bits < lo ? lo : bits;
+  const unsigned hi = (unsigned)(bits >> 32);
+  if (hi < 0x00100000u) return log(__longlong_as_double(bits));  // a denormal delta
+  const double m = __longlong_as_double((bits & 0x000fffffffffffffLL) | 0x3ff0000000000000LL);
+  const double2 e = tab->m[(hi >> 10) & 1023u];
+  const double r = fma(m, e.x, -1.0), r2 = r * r;
+  const double p = fma(r, fma(r, -0.25, 1.0 / 3.0), -0.5);
+  return (tab->k[hi >> 20] + e.y) + fma(r2, p, r);
+}
+
+// eload as k_cell_loads, f' of the Flory-Huggins energy by the product rule.  The terms of f' that are
+// linear in the concentrations are integrated exactly (the rule is exact for them); the rule takes the
+// logarithms' part
+//   g_p = ln phi_p / N_p - ln phi_s / N_s,  g_n = ln phi_n / N_n - ln phi_s / N_s,
+// along the innermost direction the concentrations are a + t b and the hat functions 1 and t, so a
+// point costs three FMAs for the concentrations, three logarithms, three for g and four to
+// accumulate (about 38 FP64 instructions against 144 with the hat functions tabulated per point and
+// CUDA's log: 19.5 ms on 128 x 128 x 32 cells, 7.1 ms now).  A thread takes a simplex, a block 32 cells at a time;
+// the simplices' corner values are added in shared memory in simplex order.  Three blocks per SM
+// with the tables in shared memory.
+template <int D>
+constexpr int fh_smem() {
+  return (int)(sizeof(LogTables) + sizeof(double2) * CellSimplices<D>::NT * (D + 1) * 32);
+}
+template <int D>
+__global__ void __launch_bounds__(32 * CellSimplices<D>::NT) k_cell_loads_fh(const MeshPod m, const FhCoef F,
+                                                                             const LogTables* __restrict__ tables,
+                                                                             const double* pp, const double* pn,
+                                                                             int ld, double2* __restrict__ eload) {
+  using S = CellSimplices<D>;
+  extern __shared__ __align__(16) unsigned char fh_raw[];
+  LogTables* tab = reinterpret_cast<LogTables*>(fh_raw);
+  double2(*part)[D + 1][32] = reinterpret_cast<double2(*)[D + 1][32]>(fh_raw + sizeof(LogTables));
+  for (int e = threadIdx.x; e < (int)(sizeof(LogTables) / 16); e += blockDim.x)
+    reinterpret_cast<uint4*>(tab)[e] = reinterpret_cast<const uint4*>(tables)[e];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, t = threadIdx.x >> 5;  // one simplex per warp: uniform corners
+  for (int c0 = blockIdx.x * 32; c0 < m.C; c0 += gridDim.x * 32) {
+    const int cell = c0 + lane;
+    if (cell < m.C) {
+      const int* ev = m.elems + ((size_t)cell * S::NT + t) * (D + 1);
+      double P[D + 1], Q[D + 1];
+#pragma unroll
+      for (int a = 0; a <= D; ++a) {
+        P[a] = pp[(size_t)ld * ev[a]];
+        Q[a] = pn[(size_t)ld * ev[a]];
       }
-  R.nq = q;
-  return R;
+      double Gp[D + 1], Gn[D + 1];  // [0]: against 1, [a]: against lambda_a
+#pragma unroll
+      for (int a = 0; a <= D; ++a) Gp[a] = Gn[a] = 0.0;
+      const auto line = [&](double p0, double dp, double n0, double dn, double (&s)[4]) {
+        // s = sums over the innermost points of w g_p, w x g_p, w g_n, w x g_n
+        const double s0 = 1.0 - p0 - n0, ds = -(dp + dn);
+        s[0] = s[1] = s[2] = s[3] = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const double x = gl_x(k), w = gl_w(k);
+          const double p = fma(x, dp, p0), n = fma(x, dn, n0), ps = fma(x, ds, s0);
+          const double ls = guarded_log(ps, F.delta, tab) * F.inv_ns;
+          const double gp = fma(guarded_log(p, F.delta, tab), F.inv_np, -ls);
+          const double gn = fma(guarded_log(n, F.delta, tab), F.inv_nn, -ls);
+          s[0] = fma(w, gp, s[0]);
+          s[1] = fma(w * x, gp, s[1]);
+          s[2] = fma(w, gn, s[2]);
+          s[3] = fma(w * x, gn, s[3]);
+        }
+      };
+      if (D == 2) {
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) {
+          const double u = gl_x(i), w1 = 1.0 - u, c = 2.0 * gl_w(i) * w1;
+          double s[4];
+          line(fma(u, P[1] - P[0], P[0]), w1 * (P[2] - P[0]), fma(u, Q[1] - Q[0], Q[0]), w1 * (Q[2] - Q[0]), s);
+          Gp[0] = fma(c, s[0], Gp[0]);
+          Gp[1] = fma(c * u, s[0], Gp[1]);
+          Gp[2] = fma(c * w1, s[1], Gp[2]);
+          Gn[0] = fma(c, s[2], Gn[0]);
+          Gn[1] = fma(c * u, s[2], Gn[1]);
+          Gn[2] = fma(c * w1, s[3], Gn[2]);
+        }
+      } else {
+#pragma unroll 1
+        for (int ij = 0; ij < 9; ++ij) {
+          const double u = gl_x(ij / 3), v = gl_x(ij % 3), w1 = 1.0 - u, w2 = w1 * (1.0 - v), vv = v * w1;
+          const double c = 6.0 * gl_w(ij / 3) * gl_w(ij % 3) * w1 * w2;
+          double s[4];
+          line(fma(u, P[1] - P[0], fma(vv, P[2] - P[0], P[0])), w2 * (P[D] - P[0]),
+               fma(u, Q[1] - Q[0], fma(vv, Q[2] - Q[0], Q[0])), w2 * (Q[D] - Q[0]), s);
+          Gp[0] = fma(c, s[0], Gp[0]);
+          Gp[1] = fma(c * u, s[0], Gp[1]);
+          Gp[2] = fma(c * vv, s[0], Gp[2]);
+          Gp[D] = fma(c * w2, s[1], Gp[D]);
+          Gn[0] = fma(c, s[2], Gn[0]);
+          Gn[1] = fma(c * u, s[2], Gn[1]);
+          Gn[2] = fma(c * vv, s[2], Gn[2]);
+          Gn[D] = fma(c * w2, s[3], Gn[D]);
+        }
+      }
+#pragma unroll
+      for (int a = 1; a <= D; ++a) {  // lambda_0 = 1 - the others
+        Gp[0] -= Gp[a];
+        Gn[0] -= Gn[a];
+      }
+      // the linear part, f_p' = kp + lp phi_p + mp phi_n and f_n' alike: int lambda_i = 1 / (d+1),
+      // int phi lambda_i = (<phi> + phi_i) / ((d+1)(d+2)), in units of |T|
+      const double kp = F.inv_np - F.inv_ns + F.chi_ps, lp = -2.0 * F.chi_ps, mp = F.chi_pn - F.chi_ps - F.chi_ns;
+      const double kn = F.inv_nn - F.inv_ns + F.chi_ns, ln = F.chi_pn - F.chi_ps - F.chi_ns, mn = -2.0 * F.chi_ns;
+      constexpr double q1 = 1.0 / (D + 1), q2 = 1.0 / ((D + 1) * (D + 2));
+      double Sp = 0.0, Sq = 0.0;
+#pragma unroll
+      for (int a = 0; a <= D; ++a) {
+        Sp += P[a];
+        Sq += Q[a];
+      }
+      const double vol = m.vol[(size_t)cell * S::NT + t];
+#pragma unroll
+      for (int a = 0; a <= D; ++a) {
+        const double sp = q2 * (Sp + P[a]), sq = q2 * (Sq + Q[a]);
+        part[t][a][lane] = make_double2(vol * (Gp[a] + fma(lp, sp, fma(mp, sq, kp * q1))),
+                                        vol * (Gn[a] + fma(ln, sp, fma(mn, sq, kn * q1))));
+      }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 32 * S::NC; e += blockDim.x) {
+      const int cl = e / S::NC, corner = e % S::NC;
+      if (c0 + cl >= m.C) continue;
+      double fp = 0.0, fn = 0.0;
+#pragma unroll
+      for (int q = 0; q < S::NT; ++q)
+#pragma unroll
+        for (int a = 0; a <= D; ++a)
+          if (S::corner(q, a) == corner) {
+            const double2 v = part[q][a][cl];
+            fp += v.x;
+            fn += v.y;
+          }
+      eload[((size_t)c0 + cl) * S::NC + corner] = make_double2(fp, fn);
+    }
+    __syncthreads();  // before the next cells' values
+  }
 }
 
-__device__ __forceinline__ double guarded_log(double x, double delta) { return log(x < delta ? delta : x); }
-
-// eload[(e (D+1) + a) 2 + {0, 1}] = |T| sum_q w_q f_{p,n}'(phi_h(x_q)) lambda_a(x_q)
-template <int D>
-__global__ void k_elem_loads_fh(const MeshPod m, const FhRule R, const FhCoef F, const double* pp,
-                                const double* pn, int ld, double* __restrict__ eload) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= m.E) return;
-  const int* ev = m.elems + (D + 1) * e;
-  double P[D + 1], Q[D + 1], Fp[D + 1], Fn[D + 1];
-#pragma unroll
-  for (int a = 0; a <= D; ++a) {
-    P[a] = pp[(size_t)ld * ev[a]];
-    Q[a] = pn[(size_t)ld * ev[a]];
-    Fp[a] = 0.0;
-    Fn[a] = 0.0;
-  }
-  for (int q = 0; q < R.nq; ++q) {
-    double p = 0.0, n = 0.0;
-#pragma unroll
-    for (int a = 0; a <= D; ++a) {
-      p += R.lam[q][a] * P[a];
-      n += R.lam[q][a] * Q[a];
-    }
-    const double s = 1.0 - p - n;
-    const double ls = (guarded_log(s, F.delta) + 1.0) * F.inv_ns;
-    const double fp = (guarded_log(p, F.delta) + 1.0) * F.inv_np - ls + F.chi_pn * n + F.chi_ps * (s - p) -
-                      F.chi_ns * n;
-    const double fn = (guarded_log(n, F.delta) + 1.0) * F.inv_nn - ls + (F.chi_pn - F.chi_ps) * p +
-                      F.chi_ns * (s - n);
-    const double wq = R.w[q];
-#pragma unroll
-    for (int a = 0; a <= D; ++a) {
-      Fp[a] += wq * fp * R.lam[q][a];
-      Fn[a] += wq * fn * R.lam[q][a];
-    }
-  }
-  const double vol = m.vol[e];
-#pragma unroll
-  for (int a = 0; a <= D; ++a)
-    reinterpret_cast<double2*>(eload)[(size_t)e * (D + 1) + a] = make_double2(vol * Fp[a], vol * Fn[a]);
+// the Flory-Huggins load's logarithm tables, once per system, and its shared-memory limits
+static ch_status log_tables(ch_system_s* s, cudaStream_t st) {
+  LogTables* t = nullptr;
+  CH_TRY(s->mem.get(&t, 1));
+  s->log_tables = t;
+  k_log_tables<<<blocks_for(2048), TPB, 0, st>>>(t);
+  CH_LAUNCHED();
+  CH_CUDA(cudaFuncSetAttribute(k_cell_loads_fh<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, fh_smem<2>()));
+  CH_CUDA(cudaFuncSetAttribute(k_cell_loads_fh<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, fh_smem<3>()));
+  return CH_OK;
 }
 
 template <int D>
-__device__ void node_loads(const MeshPod& m, const LoadCoef& L, const double* __restrict__ eload,
+__device__ void node_loads(const MeshPod& m, const LoadCoef& L, const double2* __restrict__ eload,
                            const double* pp, const double* pn, int ld, int v, double* Fp, double* Fn,
                            double* Gp, double* Gn) {
   double fp = 0.0, fn = 0.0;
-  for (int q = m.n2e_ptr[v]; q < m.n2e_ptr[v + 1]; ++q) {  // incident elements in a fixed order
-    const int e = m.n2e[q];
-    const int* ev = m.elems + (D + 1) * e;
-    int li = 0;
+  const CellGrid G = m.grid[m.node_run[v]];
+  const int l = v - G.node0, x = l % (G.nx + 1), yz = l / (G.nx + 1), y = yz % (G.ny + 1), z = yz / (G.ny + 1);
+  constexpr int NC = CellSimplices<D>::NC;
 #pragma unroll
-    for (int a = 0; a <= D; ++a)
-      if (ev[a] == v) li = a;
-    const double2 c = reinterpret_cast<const double2*>(eload)[(size_t)e * (D + 1) + li];
-    fp += c.x;
-    fn += c.y;
+  for (int c = NC - 1; c >= 0; --c) {  // cells in increasing order: the node is their corner c
+    const int cx = x - (c & 1), cy = y - ((c >> 1) & 1), cz = z - (c >> 2);
+    if (cx < 0 || cx >= G.nx || cy < 0 || cy >= G.ny || (D == 3 && (cz < 0 || cz >= G.nz))) continue;
+    const double2 e = eload[((size_t)G.cell0 + cx + (size_t)G.nx * (cy + (size_t)G.ny * (D == 3 ? cz : 0))) * NC + c];
+    fp += e.x;
+    fn += e.y;
   }
   *Fp = fp;
   *Fn = fn;
@@ -847,7 +1021,7 @@ static LoadCoef load_coef(const ch_params& p) {
 }
 
 template <int D>
-__global__ void k_loads(const MeshPod m, LoadCoef L, const double* eload, const double* pp,
+__global__ void k_loads(const MeshPod m, LoadCoef L, const double2* eload, const double* pp,
                         const double* pn, int ld, double* Fp, double* Fn, double* Gp, double* Gn) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= m.N) return;
@@ -861,7 +1035,7 @@ __global__ void k_loads(const MeshPod m, LoadCoef L, const double* eload, const 
 
 // b (N x 4) = (M phi_p + tau g_p, M phi_n + tau g_n, -c F_p, -c F_n)   (Eq. (13) -> Eq. (14))
 template <int D>
-__global__ void k_rhs(const MeshPod m, LoadCoef L, const double* eload, const int* rowptr,
+__global__ void k_rhs(const MeshPod m, LoadCoef L, const double2* eload, const int* rowptr,
                       const int* col, const double* valM, const double* pp, const double* pn, int ld,
                       double tau, double c, double* b) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
@@ -882,28 +1056,30 @@ __global__ void k_rhs(const MeshPod m, LoadCoef L, const double* eload, const in
   reinterpret_cast<double4_32a*>(b)[v] = out;
 }
 
-// Per-element load contributions into s->eload (the system's scratch: calls on one system must
-// not overlap on the GPU).  Algorithmic bytes: the vertex values gathered, element indices and
-// measures, the contributions written.
-static void elem_loads(const ch_system_s* s, const MeshPod& m, const LoadCoef& L, const double* pp,
+// Per-cell load contributions into s->eload (the system's scratch: calls on one system must not overlap
+// on the GPU).  Algorithmic bytes: the vertex values gathered, element indices and measures, the
+// contributions written.
+static void cell_loads(const ch_system_s* s, const MeshPod& m, const LoadCoef& L, const double* pp,
                        const double* pn, int ld, cudaStream_t st) {
-  const double E = m.E, d1 = m.dim + 1;
+  const double C = m.C, nc = m.dim == 2 ? 4 : 8, nt = m.dim == 2 ? 2 : 6, d1 = m.dim + 1;
+  const double bytes = C * (nc * (4.0 + 16.0 + 16.0) + 8.0);
   if (s->p.potential == 3) {
-    const FhRule R = fh_rule(m.dim);
     const ch_params& p = s->p;
     const FhCoef F{p.chi_pn, p.chi_ps, p.chi_ns, 1.0 / p.N_p, 1.0 / p.N_nfa, 1.0 / p.N_s, p.fh_delta};
-    ProfScope ps(st, K_ELEM_LOADS, 0, E * (d1 * (4.0 + 16.0) + 8.0 + 16.0 * d1), E * R.nq * (4.0 * d1 + 10.0));
+    ProfScope ps(st, K_ELEM_LOADS, 0, bytes, C * nt * (m.dim == 2 ? 9 : 27) * 40.0);
     if (m.dim == 2)
-      k_elem_loads_fh<2><<<blocks_for(m.E), TPB, 0, st>>>(m, R, F, pp, pn, ld, s->eload);
+      k_cell_loads_fh<2><<<std::min(blocks_for(m.C, 32), 5 * 152), 64, fh_smem<2>(), st>>>(
+          m, F, static_cast<const LogTables*>(s->log_tables), pp, pn, ld, s->eload);
     else
-      k_elem_loads_fh<3><<<blocks_for(m.E), TPB, 0, st>>>(m, R, F, pp, pn, ld, s->eload);
+      k_cell_loads_fh<3><<<std::min(blocks_for(m.C, 32), 3 * 152), 192, fh_smem<3>(), st>>>(
+          m, F, static_cast<const LogTables*>(s->log_tables), pp, pn, ld, s->eload);
     return;
   }
-  ProfScope ps(st, K_ELEM_LOADS, 0, E * (d1 * (4.0 + 16.0) + 8.0 + 16.0 * d1), E * (22.0 + 12.0 * d1));
+  ProfScope ps(st, K_ELEM_LOADS, 0, bytes, C * nt * (40.0 + 10.0 * d1));
   if (m.dim == 2)
-    k_elem_loads<2><<<blocks_for(m.E), TPB, 0, st>>>(m, L, pp, pn, ld, s->eload);
+    k_cell_loads<2><<<blocks_for(m.C, 128), 128, 0, st>>>(m, L, pp, pn, ld, s->eload);
   else
-    k_elem_loads<3><<<blocks_for(m.E), TPB, 0, st>>>(m, L, pp, pn, ld, s->eload);
+    k_cell_loads<3><<<blocks_for(m.C, 128), 128, 0, st>>>(m, L, pp, pn, ld, s->eload);
 }
 
 ch_status loads(const ch_system_s* s, const double* pp, const double* pn, double* Fp, double* Fn,
@@ -911,7 +1087,7 @@ ch_status loads(const ch_system_s* s, const double* pp, const double* pn, double
   const MeshPod m = mesh_pod(s->mesh);
   LoadCoef L = load_coef(s->p);
   L.bw = s->bw;
-  elem_loads(s, m, L, pp, pn, 1, st);
+  cell_loads(s, m, L, pp, pn, 1, st);
   ProfScope ps(st, K_LOADS, 0, 16.0 * m.N + 32.0 * m.N, 0.0);
   if (m.dim == 2)
     k_loads<2><<<blocks_for(m.N), TPB, 0, st>>>(m, L, s->eload, pp, pn, 1, Fp, Fn, gp, gn);
@@ -926,11 +1102,9 @@ ch_status rhs_strided(const ch_system_s* s, const double* pp, const double* pn, 
   const MeshPod m = mesh_pod(s->mesh);
   LoadCoef L = load_coef(s->p);
   L.bw = s->bw;
-  elem_loads(s, m, L, pp, pn, ld, st);
-  const double E = s->mesh->E, d1 = m.dim + 1;
-  // phi read + b written + M (values, columns, row pointers) + incidence and the element
-  // contributions gathered
-  ProfScope ps(st, K_RHS, 0, 48.0 * m.N + 12.0 * s->nnz + 4.0 * m.N + E * d1 * (4.0 + 4.0 + 16.0),
+  cell_loads(s, m, L, pp, pn, ld, st);
+  // phi read + b written + M (values, columns, row pointers) + the cells' contributions gathered
+  ProfScope ps(st, K_RHS, 0, 48.0 * m.N + 12.0 * s->nnz + 4.0 * m.N + m.C * (m.dim == 2 ? 64.0 : 128.0),
                2.0 * s->nnz);
   if (m.dim == 2)
     k_rhs<2><<<blocks_for(m.N), TPB, 0, st>>>(m, L, s->eload, s->rowptr, s->col, s->valM, pp, pn, ld,

@@ -203,6 +203,10 @@ struct Lattice {
   int2* wh = nullptr;           // nids: strides of the id's run
   int* rep = nullptr;           // nids: a node of the class (the middle one along its inner axes)
 };
+// The grid of one run: first node, first cell, cells per axis.
+struct CellGrid {
+  int node0, cell0, nx, ny, nz;
+};
 // strides of the lattice directions: 7 in 2D (the triangles' edges), 15 in 3D (the Kuhn tetrahedra's),
 // ascending for any W, H >= 2, i.e. in CSR column order; direction ND / 2 is the node itself
 __host__ __device__ __forceinline__ int lat_off(int nd, int d, int W, int WH) {
@@ -237,6 +241,7 @@ struct ch_mesh_s {
   int *n2b_ptr = nullptr, *n2b = nullptr;  // node -> incident bottom facets
   int *n2t_ptr = nullptr, *n2t = nullptr;  // node -> incident top facets
   ch::Lattice lat;
+  ch::CellGrid* cell_grid = nullptr;  // device, per run
   ch::Alloc mem;
 };
 
@@ -251,7 +256,8 @@ struct ch_system_s {
   double* valK = nullptr;
   double* valH = nullptr;
   int* diag = nullptr;  // position of the diagonal entry of each row
-  double* eload = nullptr;  // E x (dim+1) x 2: per element and vertex, the f-load contributions
+  double2* eload = nullptr;  // per grid cell and corner, the f-load contributions (polymer, NFA)
+  void* log_tables = nullptr;  // potential = 3: the load's logarithm tables
   double* bw = nullptr;     // pattern = 1: Fb x 2 species x (dim + dim^2) substrate weights, else null
   double a = 0, c = 0;  // A = [[M, aK], [aK, -cM]]
   ch::Alloc mem;
