@@ -516,14 +516,90 @@ static ch_status substrate_weights(const ch_mesh_s* m, ch_system_s* s, cudaStrea
   return CH_OK;
 }
 
+// ---------------------------------------------------------------- the operator's lattice table
+template <int ND>
+__global__ void k_lat_operator(int nids, const int* rep, const int2* wh, const int* rowptr, const int* col,
+                               const double* valM, const double* valK, double a, double c, double* tab) {
+  using X = LatAxes<ND>;
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  if (id >= nids) return;
+  const int i = rep[id];
+  const int2 w = wh[id];
+  double* t = tab + (size_t)id * X::TS;
+  for (int k = 0; k < X::TS; ++k) t[k] = 0.0;
+  for (int q = rowptr[i]; q < rowptr[i + 1]; ++q)
+    for (int d = 0; d < ND; ++d)
+      if (lat_off(ND, d, w.x, w.y) == col[q] - i) {
+        t[d] = valM[q];
+        t[ND + d] = -c * valM[q];
+        if (X::index(d) >= 0) t[2 * ND + X::index(d)] = a * valK[q];
+      }
+}
+
+// bad = 1 where a row's entries differ from its class's table by more than 2^-36 of its diagonal, or K
+// has an entry off the axes
+template <int ND>
+__global__ void k_lat_operator_check(Lattice L, int N, const int* rowptr, const int* col, const double* valM,
+                                     const double* valK, double a, const double* tab, int* bad) {
+  using X = LatAxes<ND>;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const int id = lat_id(L, i);
+  const int2 w = L.wh[id];
+  const double* t = tab + (size_t)id * X::TS;
+  const double tm = 0x1p-36 * fabs(t[ND / 2]), tk = 0x1p-36 * fabs(t[2 * ND + X::index(ND / 2)]);
+  bool ok = true;
+  double seen = 0.0, sum = 0.0;
+  for (int q = rowptr[i]; q < rowptr[i + 1]; ++q) {
+    int at = -1;
+    for (int d = 0; d < ND; ++d)
+      if (lat_off(ND, d, w.x, w.y) == col[q] - i) at = d;
+    if (at < 0) {
+      ok = false;
+      continue;
+    }
+    int e = -1;
+    for (int d = 0; d < ND; ++d)
+      if (d == at) e = X::index(d);
+    const double k = e >= 0 ? t[2 * ND + e] : 0.0;
+    if (!(fabs(valM[q] - t[at]) <= tm) || !(fabs(a * valK[q] - k) <= tk)) ok = false;
+    seen += fabs(t[at]);
+  }
+  for (int d = 0; d < ND; ++d) sum += fabs(t[d]);
+  if (!(fabs(sum - seen) <= tm)) ok = false;  // the class has an entry that the row lacks
+  if (!ok) *bad = 1;
+}
+
+static ch_status lattice_operator(const ch_mesh_s* m, ch_system_s* s, int* bad, cudaStream_t st) {
+  const Lattice& L = m->lat;
+  const int ts = m->dim == 2 ? LatAxes<7>::TS : LatAxes<15>::TS;
+  double* tab = nullptr;
+  CH_TRY(s->mem.get(&tab, (size_t)L.nids * ts));
+  s->lat.L = L;
+  s->lat.tab = tab;
+  if (m->dim == 2) {
+    k_lat_operator<7><<<blocks_for(L.nids, 64), 64, 0, st>>>(L.nids, L.rep, L.wh, s->rowptr, s->col, s->valM, s->valK,
+                                                             s->a, s->c, tab);
+    k_lat_operator_check<7><<<blocks_for(s->N), TPB, 0, st>>>(L, s->N, s->rowptr, s->col, s->valM, s->valK, s->a, tab,
+                                                              bad);
+  } else {
+    k_lat_operator<15><<<blocks_for(L.nids, 64), 64, 0, st>>>(L.nids, L.rep, L.wh, s->rowptr, s->col, s->valM,
+                                                              s->valK, s->a, s->c, tab);
+    k_lat_operator_check<15><<<blocks_for(s->N), TPB, 0, st>>>(L, s->N, s->rowptr, s->col, s->valM, s->valK, s->a,
+                                                               tab, bad);
+  }
+  CH_LAUNCHED();
+  return CH_OK;
+}
+
 ch_status assemble_system(const ch_mesh_s* m, ch_system_s* s, cudaStream_t st) {
   const int N = m->N, d = m->dim;
   s->N = N;
   Alloc tmp;
   int *cnt = nullptr, *overflow = nullptr;
   CH_TRY(tmp.get(&cnt, (size_t)N));
-  CH_TRY(tmp.get(&overflow, 1));
-  CH_CUDA(cudaMemsetAsync(overflow, 0, sizeof(int), st));
+  CH_TRY(tmp.get(&overflow, 2));  // ... and the lattice operator's misfit flag
+  CH_CUDA(cudaMemsetAsync(overflow, 0, 2 * sizeof(int), st));
   k_pattern<<<blocks_for(N), TPB, 0, st>>>(m->elems, d + 1, m->n2e_ptr, m->n2e, N, nullptr, cnt,
                                             nullptr, overflow);
   CH_LAUNCHED();
@@ -552,10 +628,12 @@ ch_status assemble_system(const ch_mesh_s* m, ch_system_s* s, cudaStream_t st) {
   CH_LAUNCHED();
   if (s->p.potential == 3) CH_TRY(log_tables(s, st));
   if (s->p.pattern && s->p.bc_mode) CH_TRY(substrate_weights(m, s, st));
-  int ovf = 0;
-  CH_CUDA(cudaMemcpyAsync(&ovf, overflow, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CH_TRY(lattice_operator(m, s, overflow + 1, st));
+  int ovf[2] = {0, 0};
+  CH_CUDA(cudaMemcpyAsync(ovf, overflow, sizeof(ovf), cudaMemcpyDeviceToHost, st));
   CH_CUDA(cudaStreamSynchronize(st));
-  if (ovf) {
+  if (ovf[1]) s->lat.tab = nullptr;  // (a very long, thin grid's coordinates round too unevenly)
+  if (ovf[0]) {
     set_error("a node has more than %d incident simplex vertices", MAXADJ);
     return CH_ERR_INTERNAL;
   }
@@ -1035,7 +1113,7 @@ __global__ void k_loads(const MeshPod m, LoadCoef L, const double2* eload, const
 
 // b (N x 4) = (M phi_p + tau g_p, M phi_n + tau g_n, -c F_p, -c F_n)   (Eq. (13) -> Eq. (14))
 template <int D>
-__global__ void k_rhs(const MeshPod m, LoadCoef L, const double2* eload, const int* rowptr,
+__global__ void k_rhs(const MeshPod m, LoadCoef L, const double2* eload, const LatOperator A, const int* rowptr,
                       const int* col, const double* valM, const double* pp, const double* pn, int ld,
                       double tau, double c, double* b) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1043,10 +1121,23 @@ __global__ void k_rhs(const MeshPod m, LoadCoef L, const double2* eload, const i
   double Fp, Fn, Gp, Gn;
   node_loads<D>(m, L, eload, pp, pn, ld, v, &Fp, &Fn, &Gp, &Gn);
   double mp = 0.0, mn = 0.0;
-  for (int q = rowptr[v]; q < rowptr[v + 1]; ++q) {
-    const int j = col[q];
-    mp = fma(valM[q], pp[(size_t)ld * j], mp);
-    mn = fma(valM[q], pn[(size_t)ld * j], mn);
+  if (A.tab) {
+    constexpr int ND = D == 2 ? 7 : 15;
+    const int id = lat_id(A.L, v);
+    const int2 w = A.L.wh[id];
+    const double* t = A.tab + (size_t)id * LatAxes<ND>::TS;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      const int j = __double2hiint(t[d]) != 0 ? v + lat_off(ND, d, w.x, w.y) : v;  // (as lat_apply_A)
+      mp = fma(t[d], pp[(size_t)ld * j], mp);
+      mn = fma(t[d], pn[(size_t)ld * j], mn);
+    }
+  } else {
+    for (int q = rowptr[v]; q < rowptr[v + 1]; ++q) {
+      const int j = col[q];
+      mp = fma(valM[q], pp[(size_t)ld * j], mp);
+      mn = fma(valM[q], pn[(size_t)ld * j], mn);
+    }
   }
   double4_32a out;
   out.x = mp + tau * Gp;
@@ -1107,10 +1198,10 @@ ch_status rhs_strided(const ch_system_s* s, const double* pp, const double* pn, 
   ProfScope ps(st, K_RHS, 0, 48.0 * m.N + 12.0 * s->nnz + 4.0 * m.N + m.C * (m.dim == 2 ? 64.0 : 128.0),
                2.0 * s->nnz);
   if (m.dim == 2)
-    k_rhs<2><<<blocks_for(m.N), TPB, 0, st>>>(m, L, s->eload, s->rowptr, s->col, s->valM, pp, pn, ld,
+    k_rhs<2><<<blocks_for(m.N), TPB, 0, st>>>(m, L, s->eload, s->lat, s->rowptr, s->col, s->valM, pp, pn, ld,
                                                s->p.tau, s->c, b);
   else
-    k_rhs<3><<<blocks_for(m.N), TPB, 0, st>>>(m, L, s->eload, s->rowptr, s->col, s->valM, pp, pn, ld,
+    k_rhs<3><<<blocks_for(m.N), TPB, 0, st>>>(m, L, s->eload, s->lat, s->rowptr, s->col, s->valM, pp, pn, ld,
                                                s->p.tau, s->c, b);
   CH_LAUNCHED();
   return CH_OK;
@@ -1146,12 +1237,28 @@ __global__ void k_apply_A(int N, const int* rowptr, const int* col, const double
   y[v] = out;
 }
 
+// The lattice form: no indices or values but the class id, so the FP64 pipe alone bounds it (54
+// instructions per node at most).  512 x 512: 23.9 us, 33.6 in CSR form; 3D 128 x 128 x 32: 83, 127 in
+// CSR form.
+template <int ND>
+__global__ void __launch_bounds__(128) k_apply_A_lat(LatOperator A, int N, const double4_32a* __restrict__ x,
+                                                     double4_32a* __restrict__ y) {
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v < N) y[v] = lat_apply_A<ND>(A, v, x);
+}
+
 ch_status apply_A(const ch_system_s* s, const double* x, double* y, cudaStream_t st) {
-  ProfScope ps(st, K_APPLY_A, 0, 20.0 * s->nnz + 4.0 * (s->N + 1) + 64.0 * s->N,
-               8.0 * s->nnz + 4.0 * s->N);
-  k_apply_A<<<blocks_for(s->N), TPB, 0, st>>>(s->N, s->rowptr, s->col, s->valM, s->valK, s->a,
-                                               s->c, reinterpret_cast<const double4_32a*>(x),
-                                               reinterpret_cast<double4_32a*>(y));
+  const double4_32a* x4 = reinterpret_cast<const double4_32a*>(x);
+  double4_32a* y4 = reinterpret_cast<double4_32a*>(y);
+  if (s->lat.tab) {
+    const double f = s->mesh->dim == 2 ? 48.0 : 88.0;
+    ProfScope ps(st, K_APPLY_A, 0, 66.0 * s->N, f * s->N);
+    if (s->mesh->dim == 2) k_apply_A_lat<7><<<blocks_for(s->N, 128), 128, 0, st>>>(s->lat, s->N, x4, y4);
+    else k_apply_A_lat<15><<<blocks_for(s->N, 128), 128, 0, st>>>(s->lat, s->N, x4, y4);
+  } else {
+    ProfScope ps(st, K_APPLY_A, 0, 20.0 * s->nnz + 4.0 * (s->N + 1) + 64.0 * s->N, 8.0 * s->nnz + 4.0 * s->N);
+    k_apply_A<<<blocks_for(s->N), TPB, 0, st>>>(s->N, s->rowptr, s->col, s->valM, s->valK, s->a, s->c, x4, y4);
+  }
   CH_LAUNCHED();
   return CH_OK;
 }

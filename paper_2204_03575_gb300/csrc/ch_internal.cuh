@@ -219,6 +219,68 @@ __host__ __device__ __forceinline__ int lat_off(int nd, int d, int W, int WH) {
 __device__ __forceinline__ int lat_id(const Lattice& L, int i) {
   return L.id32 ? static_cast<const int*>(L.id)[i] : static_cast<const uint16_t*>(L.id)[i];
 }
+
+// The block operator of Eq. (14) on the lattice: per class id a table row of the mass entries m_d, of
+// -c m_d and of a k_e over the axis directions e -- the only ones where the stiffness matrix of a box
+// mesh is not zero (5 of 7 in 2D, 7 of 15 in 3D).  tab is null where the mesh does not fit its
+// classes (set-up check): the CSR form then.
+struct LatOperator {
+  Lattice L;
+  const double* tab = nullptr;
+};
+template <int ND> struct LatAxes;
+template <> struct LatAxes<7> {
+  static constexpr int NK = 5, TS = 20;  // axis directions; doubles per table row (2 ND + NK, even)
+  __host__ __device__ static constexpr int index(int d) { return d >= 1 && d <= 5 ? d - 1 : -1; }
+};
+template <> struct LatAxes<15> {
+  static constexpr int NK = 7, TS = 38;
+  __host__ __device__ static constexpr int index(int d) {
+    constexpr int k[15] = {-1, -1, -1, 0, -1, 1, 2, 3, 4, 5, -1, 6, -1, -1, -1};
+    return k[d];
+  }
+};
+
+// (A x)_i for both species: y1 = M x1 + a K x2, y2 = a K x1 - c M x2.  4 FMAs per direction and 4 more
+// per axis direction (48 in 2D, 88 in 3D, against 8 per stored entry, 56 and 120, in CSR form).
+template <int ND>
+__device__ __forceinline__ double4_32a lat_apply_A(const LatOperator& A, int i, const double4_32a* __restrict__ x) {
+  using X = LatAxes<ND>;
+  const int id = lat_id(A.L, i);
+  int W = A.L.W, WH = A.L.WH;
+  if (A.L.nids > A.L.ncls) {
+    const int2 w = A.L.wh[id];
+    W = w.x;
+    WH = w.y;
+  }
+  const double2* row = reinterpret_cast<const double2*>(A.tab + (size_t)id * X::TS);
+  double t[X::TS];
+#pragma unroll
+  for (int q = 0; q < X::TS / 2; ++q) {
+    const double2 v = row[q];
+    t[2 * q] = v.x;
+    t[2 * q + 1] = v.y;
+  }
+  double4_32a y = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+#pragma unroll
+  for (int d = 0; d < ND; ++d) {
+    // a neighbour the class lacks (mass entry zero) reads the node itself, not another row's or run's value
+    const int j = __double2hiint(t[d]) != 0 ? i + lat_off(ND, d, W, WH) : i;
+    const double4_32a z = x[j];
+    y.x = fma(t[d], z.x, y.x);
+    y.y = fma(t[d], z.y, y.y);
+    y.z = fma(t[ND + d], z.z, y.z);
+    y.w = fma(t[ND + d], z.w, y.w);
+    if (X::index(d) >= 0) {
+      const double k = t[2 * ND + (X::index(d) >= 0 ? X::index(d) : 0)];
+      y.x = fma(k, z.z, y.x);
+      y.y = fma(k, z.w, y.y);
+      y.z = fma(k, z.x, y.z);
+      y.w = fma(k, z.y, y.w);
+    }
+  }
+  return y;
+}
 }  // namespace ch
 
 // ---------------------------------------------------------------- opaque handles
@@ -260,6 +322,7 @@ struct ch_system_s {
   void* log_tables = nullptr;  // potential = 3: the load's logarithm tables
   double* bw = nullptr;     // pattern = 1: Fb x 2 species x (dim + dim^2) substrate weights, else null
   double a = 0, c = 0;  // A = [[M, aK], [aK, -cM]]
+  ch::LatOperator lat;  // ... on the lattice
   ch::Alloc mem;
 };
 

@@ -189,12 +189,46 @@ __device__ bool reduce_run(const Seg& sg, double* partials, unsigned int* run_ti
 // ---------------------------------------------------------------- residual / norms
 // W = b - A x (all systems), then per run the last block computes ||b_s||, ||r_s||, relres and
 // sets active / cycle flags, beta and g for a (re)start.  If init, also tol_s = rtol ||b_s||.
+// The end of k_residual4: the run's norms from the blocks' sums, then (last block) the flags.
+__device__ void residual_close(const Seg& sg, double (&acc)[4], double* partials, KrylovDev* kds, int init,
+                               double rtol) {
+  __shared__ double sm[(TPB / 32) * 4];
+  const int run = sg.run[blockIdx.x];
+  block_sum<4>(acc, sm);
+  if (threadIdx.x < 4) partials[(size_t)blockIdx.x * MAXV + threadIdx.x] = sm[threadIdx.x];
+  KrylovDev* kd = kds + run;
+  const int b0 = sg.first[run], b1 = sg.first[run + 1];
+  __shared__ double tot[4];
+  if (!reduce_run(sg, partials, &kd->ticket, b0, b1, 4, tot)) return;
+  if (threadIdx.x < 2) {
+    const int s = threadIdx.x;
+    const double bn = sqrt(tot[s]), rn = sqrt(tot[2 + s]);
+    if (init) {
+      kd->bnorm[s] = bn;
+      kd->tol[s] = rtol * bn;
+      kd->its[s] = 0;
+      kd->reorth_count[s] = 0;
+      kd->active[s] = 1;
+      if (s == 0) kd->nonfinite = 0;
+    }
+    __syncwarp(0x3u);
+    if (!isfinite(bn) || !isfinite(rn)) kd->nonfinite = 1;
+    kd->relres[s] = bn > 0.0 ? rn / bn : 0.0;
+    const int act = kd->active[s] && rn > kd->tol[s] && bn > 0.0;
+    kd->active[s] = act;
+    kd->cycle_active[s] = act;
+    kd->k[s] = 0;
+    kd->beta[s] = rn;
+    kd->g[s][0] = rn;
+    kd->hinv[s] = (act && rn > 0.0) ? 1.0 / rn : 0.0;
+  }
+  if (threadIdx.x == 0) kd->ticket = 0;
+}
+
 __global__ void k_residual4(Seg sg, const int* rowptr, const int* col, const double* valM,
                             const double* valK, double a, double c, const double4_32a* x,
                             const double4_32a* b, double4_32a* W, double* partials, KrylovDev* kds,
                             int init, double rtol) {
-  __shared__ double sm[(TPB / 32) * 4];
-  const int run = sg.run[blockIdx.x];
   double acc[4] = {0, 0, 0, 0};  // ||b_p||^2, ||b_n||^2, ||r_p||^2, ||r_n||^2
   // Two nodes per iteration (v and v + blockDim.x, the order of the plain loop) with their rows
   // walked in one loop, so that both rows' gathers are in flight together: the segmented grid has
@@ -253,35 +287,28 @@ __global__ void k_residual4(Seg sg, const int* rowptr, const int* col, const dou
       acc[3] += r.y * r.y + r.w * r.w;
     }
   }
-  block_sum<4>(acc, sm);
-  if (threadIdx.x < 4) partials[(size_t)blockIdx.x * MAXV + threadIdx.x] = sm[threadIdx.x];
-  KrylovDev* kd = kds + run;
-  const int b0 = sg.first[run], b1 = sg.first[run + 1];
-  __shared__ double tot[4];
-  if (!reduce_run(sg, partials, &kd->ticket, b0, b1, 4, tot)) return;
-  if (threadIdx.x < 2) {
-    const int s = threadIdx.x;
-    const double bn = sqrt(tot[s]), rn = sqrt(tot[2 + s]);
-    if (init) {
-      kd->bnorm[s] = bn;
-      kd->tol[s] = rtol * bn;
-      kd->its[s] = 0;
-      kd->reorth_count[s] = 0;
-      kd->active[s] = 1;
-      if (s == 0) kd->nonfinite = 0;
-    }
-    __syncwarp(0x3u);
-    if (!isfinite(bn) || !isfinite(rn)) kd->nonfinite = 1;
-    kd->relres[s] = bn > 0.0 ? rn / bn : 0.0;
-    const int act = kd->active[s] && rn > kd->tol[s] && bn > 0.0;
-    kd->active[s] = act;
-    kd->cycle_active[s] = act;
-    kd->k[s] = 0;
-    kd->beta[s] = rn;
-    kd->g[s][0] = rn;
-    kd->hinv[s] = (act && rn > 0.0) ? 1.0 / rn : 0.0;
+  residual_close(sg, acc, partials, kds, init, rtol);
+}
+
+// k_residual4 with the operator in lattice form (lat_apply_A), two nodes per iteration so that both rows'
+// gathers are in flight.  512 x 512: 43 us, 53 in CSR form; 3D 128 x 128 x 32: 112, 161 in CSR form.
+template <int ND>
+__global__ void __launch_bounds__(TPB, 2) k_residual4_lat(Seg sg, LatOperator A, const double4_32a* __restrict__ x,
+                                                          const double4_32a* __restrict__ b, double4_32a* __restrict__ W,
+                                                          double* partials, KrylovDev* kds, int init, double rtol) {
+  double acc[4] = {0, 0, 0, 0};  // ||b_p||^2, ||b_n||^2, ||r_p||^2, ||r_n||^2
+  const int hi = sg.hi[blockIdx.x];
+#pragma unroll 2
+  for (int v = sg.lo[blockIdx.x] + threadIdx.x; v < hi; v += blockDim.x) {
+    const double4_32a bb = b[v], y = lat_apply_A<ND>(A, v, x);
+    const double4_32a r = make_double4_32a(bb.x - y.x, bb.y - y.y, bb.z - y.z, bb.w - y.w);
+    W[v] = r;
+    acc[0] += bb.x * bb.x + bb.z * bb.z;
+    acc[1] += bb.y * bb.y + bb.w * bb.w;
+    acc[2] += r.x * r.x + r.z * r.z;
+    acc[3] += r.y * r.y + r.w * r.w;
   }
-  if (threadIdx.x == 0) kd->ticket = 0;
+  residual_close(sg, acc, partials, kds, init, rtol);
 }
 
 // dst = src * hinv[s] per system of the block's run (components x,z: polymer; y,w: NFA)
@@ -657,8 +684,8 @@ __device__ __forceinline__ float trunc_f32(double v) {
 // ||W|| |V_k[v]|, is below the FP64 rounding of W, and the FP64 pipe (2 FMA per clock and SM, what
 // bounds these passes) is left with three instructions per component instead of nv + 2.  A larger h2
 // (a vector that lies almost in the span of the basis) or a non-finite value takes the FP64 sum.
-// Measured (512 x 512, 10 basis vectors on average): this pass and the normalisation it now includes
-// 43.6 us before (FP64 update with its own norm reduction, then a scaling kernel).
+// Measured (512 x 512, 10 basis vectors on average): 20.6 us, where the FP64 update with its own norm
+// reduction and the scaling kernel after it took 43.6.
 __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth_close(Seg sg, int N, int nv, const double4_32a* __restrict__ V,
                                                             const double4_32a* __restrict__ W,
                                                             double4_32a* __restrict__ vnext, KrylovDev* kds) {
@@ -1327,12 +1354,23 @@ static ch_status arnoldi_launch(ch_state_s* S, int j, cudaStream_t st) {
 
 static ch_status residual_launch(ch_state_s* S, int init, cudaStream_t st, const double* x = nullptr) {
   const ch_system_s* s = S->sys;
-  ProfScope ps(st, K_RESIDUAL4, 0, res4_bytes(s), 8.0 * s->nnz + 12.0 * S->N);
-  k_residual4<<<S->nblocks, TPB, 0, st>>>(S->seg, s->rowptr, s->col, s->valM, s->valK, s->a, s->c,
-                                           reinterpret_cast<const double4_32a*>(x ? x : S->x),
-                                           reinterpret_cast<const double4_32a*>(S->b),
-                                           reinterpret_cast<double4_32a*>(S->W), S->partials, S->kd,
-                                           init, s->p.rtol);
+  const double4_32a* x4 = reinterpret_cast<const double4_32a*>(x ? x : S->x);
+  const double4_32a* b4 = reinterpret_cast<const double4_32a*>(S->b);
+  double4_32a* W4 = reinterpret_cast<double4_32a*>(S->W);
+  if (s->lat.tab) {
+    const double f = s->mesh->dim == 2 ? 48.0 : 88.0;
+    ProfScope ps(st, K_RESIDUAL4, 0, 98.0 * S->N, (f + 12.0) * S->N);
+    if (s->mesh->dim == 2)
+      k_residual4_lat<7><<<S->nblocks, TPB, 0, st>>>(S->seg, s->lat, x4, b4, W4, S->partials, S->kd, init,
+                                                     s->p.rtol);
+    else
+      k_residual4_lat<15><<<S->nblocks, TPB, 0, st>>>(S->seg, s->lat, x4, b4, W4, S->partials, S->kd, init,
+                                                      s->p.rtol);
+  } else {
+    ProfScope ps(st, K_RESIDUAL4, 0, res4_bytes(s), 8.0 * s->nnz + 12.0 * S->N);
+    k_residual4<<<S->nblocks, TPB, 0, st>>>(S->seg, s->rowptr, s->col, s->valM, s->valK, s->a, s->c, x4, b4, W4,
+                                             S->partials, S->kd, init, s->p.rtol);
+  }
   CH_LAUNCHED();
   return CH_OK;
 }
