@@ -47,10 +47,30 @@ struct LatOp {
   T* scratch = nullptr;            // of ch_smooth's own degree, rebuilt by each call
 };
 
+// One tile of the 2D lattice form for k_smooth_tile: the run's first node, strides and ids, and the
+// tile's first output column and row.
+struct LatTile {
+  int off, W, H, x0, y0, id0;
+};
+template <typename T> struct TileShape;  // columns of a region, nodes per thread, most groups
+template <> struct TileShape<float> { static constexpr int RW = 64, ROWS = 4, GMAX = 16; };
+template <> struct TileShape<double> { static constexpr int RW = 16, ROWS = 1, GMAX = 16; };
+// FP64 passes are bound by the FP64 pipe, where recomputed halo nodes cost as much as any: tiles only
+// while the mesh is too small to fill the chip and a step is a launch's latency
+constexpr int TILE_MAX_F64 = 152;
+struct TilePlan {
+  int ntiles = 0;  // 0: the pass runs as one launch per step
+  int groups = 0;  // thread rows of a block
+  int halo = 0;    // operator applications of the pass
+  const LatTile* tiles = nullptr;
+};
+
 template <typename T>
 struct LevelT {
   Csr<T> A, P, R;
   LatOp<T> lat;                        // level 0 of a structured mesh
+  TilePlan plan, plan_r;               // ... its smoothing passes as single launches, and those from a
+                                       // given iterate that also form the residual
   int tprA = 1, tprP = 1, tprR = 1;  // lanes per row of the SpMV-type kernels (autotuned)
   bool pdl = false;                  // launch the V-cycle kernels as programmatic dependents
   T* dinv = nullptr;
@@ -599,6 +619,8 @@ static ch_status level_setup(Hierarchy* h, int l, const ch_params& p, cudaStream
   return CH_OK;
 }
 
+template <typename T>
+static ch_status tile_setup();
 template <typename T, typename V2>
 static void launch_residual(int tpr, const Csr<T>& A, const V2* b, const V2* x, V2* r, cudaStream_t st,
                             const LatOp<T>* lat = nullptr, bool pdl = false);
@@ -808,12 +830,60 @@ static void lat_step_tables(const double* tab64, const LatOp<double>& op, const 
   k_lat_steps<<<dim3(blocks_for(op.L.nids, 64), deg), 64, 0, st>>>(tab64, op.L.nids, op.nd, op.ts, sc, out);
 }
 
+// Tiles of a pass of `halo` operator applications over every run of a 2D mesh: the block height whose
+// tiles leave the busiest SM the fewest region nodes (tall blocks recompute less halo, short ones
+// spread a small mesh over more SMs).
+template <typename T>
+static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* out, cudaStream_t st) {
+  using S = TileShape<T>;
+  *out = TilePlan();
+  const int tw = S::RW - 2 * halo;
+  if (tw < S::RW / 4) return CH_OK;
+  const auto count = [&](int th) {
+    int64_t n = 0;
+    for (const ch_params& p : m->runs) n += (int64_t)((p.nx + tw) / tw) * ((p.ny + th) / th);
+    return n;
+  };
+  int64_t best = 0;
+  int G = 0;
+  for (int g = 2; g <= S::GMAX; ++g) {
+    const int rh = S::ROWS * g, th = rh - 2 * halo;
+    if (th < 1 || S::RW * g % 32 != 0) continue;
+    // region rows on the busiest SM, in tenths; two blocks of up to 8 groups share an SM and overlap,
+    // taller ones run alone and wait out their loads once there is more than one per SM
+    const int64_t n = count(th), cost = (n + 151) / 152 * rh * (g > 8 && n > 152 ? 11 : 10);
+    if (G == 0 || cost < best) {
+      best = cost;
+      G = g;
+    }
+  }
+  if (G == 0) return CH_OK;
+  const int th = S::ROWS * G - 2 * halo;
+  if (sizeof(T) == 8 && count(th) > TILE_MAX_F64) return CH_OK;
+  std::vector<LatTile> tiles;
+  for (size_t r = 0; r < m->runs.size(); ++r) {
+    const ch_params& p = m->runs[r];
+    for (int y = 0; y <= p.ny; y += th)
+      for (int x = 0; x <= p.nx; x += tw)
+        tiles.push_back({m->run_off[r], p.nx + 1, p.ny + 1, x, y, (int)r * m->lat.ncls});
+  }
+  LatTile* d = nullptr;
+  CH_TRY(mem.get(&d, tiles.size()));
+  CH_CUDA(cudaMemcpyAsync(d, tiles.data(), sizeof(LatTile) * tiles.size(), cudaMemcpyHostToDevice, st));
+  CH_CUDA(cudaStreamSynchronize(st));  // tiles is a host temporary
+  out->ntiles = (int)tiles.size();
+  out->groups = G;
+  out->halo = halo;
+  out->tiles = d;
+  return CH_OK;
+}
+
 static int semi_steps(const ch_params& p) { return p.cheb_M_steps > 0 ? p.cheb_M_steps : 5; }
 // Wathen's bounds of the eigenvalues of D^-1 M: [1/2, 2] (triangles), [1/2, 5/2] (tetrahedra)
 static ChebCoef semi_coef(int dim, int steps) { return cheb_coef_interval(0.5, dim == 2 ? 2.0 : 2.5, steps); }
 
 template <typename T>
-static ch_status make_working(Hierarchy* h, const Lattice* lat, const ch_params& p, std::vector<LevelT<T>>& L,
+static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, const ch_params& p, std::vector<LevelT<T>>& L,
                               cudaStream_t st) {
   using V2 = typename V2T<T>::t;
   L.resize(h->nlev);
@@ -855,6 +925,7 @@ static ch_status make_working(Hierarchy* h, const Lattice* lat, const ch_params&
   }
 
   // the fine level of a uniform mesh in lattice form
+  const Lattice* lat = &mesh->lat;
   CH_TRY(lat_build(h->A[0], lat, h->mem, &h->lat_tab, st));
   if (h->lat_tab) {
     LatOp<T>& op = L[0].lat;
@@ -878,11 +949,16 @@ static ch_status make_working(Hierarchy* h, const Lattice* lat, const ch_params&
       }
     }
     CH_LAUNCHED();
+    if (lat->dim == 2 && h->nlev > 1) {
+      CH_TRY(tile_setup<T>());
+      CH_TRY(tile_plan<T>(mesh, h->cheb_degree, h->mem, &L[0].plan, st));
+      CH_TRY(tile_plan<T>(mesh, h->cheb_degree + 1, h->mem, &L[0].plan_r, st));
+    }
   }
   return autotune_levels<T>(h, L, h->autotune, st);
 }
 
-ch_status hierarchy_build(const Csr<double>& A0, const Lattice* lat, const ch_params& p, int precision, cudaStream_t st,
+ch_status hierarchy_build(const Csr<double>& A0, const ch_mesh_s* mesh, const ch_params& p, int precision, cudaStream_t st,
                           Hierarchy** out) {
   *out = nullptr;
   Hierarchy* h = new Hierarchy();
@@ -948,9 +1024,9 @@ ch_status hierarchy_build(const Csr<double>& A0, const Lattice* lat, const ch_pa
   }
   if (s == CH_OK) {
     if (precision == 0) {
-      s = make_working<double>(h, lat, p, h->Ld, st);
+      s = make_working<double>(h, mesh, p, h->Ld, st);
     } else {
-      s = make_working<float>(h, lat, p, h->Lf, st);
+      s = make_working<float>(h, mesh, p, h->Lf, st);
       if (s == CH_OK) s = h->mem.get(&h->cinvf, (size_t)h->nc * h->nc);
       if (s == CH_OK) {
         k_d2f<<<blocks_for((int64_t)h->nc * h->nc), TPB, 0, st>>>(h->cinv, h->cinvf,
@@ -1312,6 +1388,188 @@ __global__ void __launch_bounds__(TPB) k_spmv2_lat(LatOp<T> D, int n, const V2* 
   y[i] = mk2<T, V2>(s0, s1);
 }
 
+// A whole smoothing pass of the 2D lattice form in one launch.  A block holds a region of RW columns x
+// (ROWS x groups) rows: a tile of outputs and a halo as deep as the pass applies the operator
+// (deg times), in shared memory (two buffers of the iterate); a thread owns ROWS nodes of one column
+// with their iterate, the one before it and b in registers.  Every application spoils one ring of the
+// region, so the tile's own nodes end exact: the same operations in the same order as k_cheb_step_lat
+// and k_residual_lat, bitwise.  Operators being one table row per class, nothing but b (and x, unless
+// the pass starts from zero) is read, once per pass instead of four vectors per step.
+//   ZERO: the pass starts from a zero guess (its first step is pointwise);  RES: r = b - A x' as well.
+// Nodes outside the mesh stay zero (their coefficients are zero).
+// Bound by instruction issue and the waves' load latency, not memory.  Algorithm 1 per application, us, one
+// launch per step -> per pass: FP32 64 x 64 77.8 -> 51.6, 256 x 256 143 -> 124, 512 x 512 247 -> 202, 1024 x
+// 1024 655 -> 523, 64 runs 1071 -> 960; FP64 32 x 32 131 -> 117 (larger FP64 meshes keep the steps: 96 x 96
+// 202 either way).
+template <typename T, typename V2>
+struct TileArgs {
+  const LatTile* tiles;
+  const T *tab, *steps;  // the operator's table; FP64: the steps' tables
+  const V2 *b, *x;
+  V2 *xo, *r;
+  int nids, deg, halo;
+  T invtheta, alpha[16], nbeta[16];
+};
+template <typename T>
+constexpr int tile_smem(int groups) {
+  return 2 * (TileShape<T>::ROWS * groups + 3) * (TileShape<T>::RW + 2) * 2 * (int)sizeof(T);
+}
+
+// a x + y and the like on both right-hand sides: packed FP32 (one instruction for two fused
+// multiply-adds, each rounded as fmaf), plain FP64
+__device__ __forceinline__ unsigned long long pk2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 up2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float c, float2 x, float2 a) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pk2(c, c)), "l"(pk2(x.x, x.y)), "l"(pk2(a.x, a.y)));
+  return up2(r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(-1.f, b, a); }  // exact product
+__device__ __forceinline__ double2 fma2(double c, double2 x, double2 a) {
+  return make_double2(fma(c, x.x, a.x), fma(c, x.y, a.y));
+}
+__device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+
+// One block's tile.  EDGE: the region reaches the mesh's boundary (or past it), so nodes carry their own
+// class row and those outside the mesh stay zero; the other tiles (all but the rim) keep one row in
+// registers and test nothing.
+template <typename T, typename V2, bool ZERO, bool RES, bool EDGE>
+__device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatTile& tl, V2* buf) {
+  constexpr int RW = TileShape<T>::RW, ROWS = TileShape<T>::ROWS, ST = RW + 2;
+  const int tid = threadIdx.x, c = tid % RW, g = tid / RW, RH = ROWS * (blockDim.x / RW);
+  const int plane = (RH + 3) * ST;  // node (r, c) of a buffer at (r + 1, c + 1)
+  const int h = a.halo, x = tl.x0 - h + c, y0 = tl.y0 - h + g * ROWS;
+  const bool col_in = !EDGE || (x >= 0 && x < tl.W);
+  const int cx = !EDGE ? 1 : (x <= 0 ? 0 : (x >= tl.W - 1 ? 2 : 1));
+  const auto in = [&](int t) { return !EDGE || (col_in && y0 + t >= 0 && y0 + t < tl.H); };
+  const auto load_row = [&](const T* tab, int cy, T (&o)[8]) {
+    constexpr int NQ = 8 * (int)sizeof(T) / 16;
+    const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)(tl.id0 + cx + 3 * cy) * 8);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) reinterpret_cast<uint4*>(o)[q] = src[q];
+  };
+  const auto edge = [&](int t) { return y0 + t == 0 ? 0 : (y0 + t == tl.H - 1 ? 2 : 1); };
+  T row[8];
+  load_row(a.tab, 1, row);
+  pdl_wait();
+  pdl_trigger_t<T>();
+  const size_t node0 = (size_t)tl.off + (size_t)((long long)y0 * tl.W) + x;  // (used only inside the mesh)
+  V2 b[ROWS], cur[ROWS], prev[ROWS];
+#pragma unroll
+  for (int t = 0; t < ROWS; ++t) {
+    b[t] = cur[t] = prev[t] = mk2<T, V2>(T(0), T(0));
+    if (in(t)) {
+      b[t] = a.b[node0 + (size_t)t * tl.W];
+      if (!ZERO) cur[t] = a.x[node0 + (size_t)t * tl.W];
+    }
+  }
+  if (ZERO) {
+#pragma unroll
+    for (int t = 0; t < ROWS; ++t) {
+      T di = row[7];
+      if (EDGE && edge(t) != 1) {
+        T e[8];
+        load_row(a.tab, edge(t), e);
+        di = e[7];
+      }
+      const T s = a.invtheta * di;
+      cur[t] = mk2<T, V2>(s * b[t].x, s * b[t].y);
+    }
+  }
+  V2* mine = buf + (g * ROWS + 1) * ST + c + 1;  // this thread's first node in buffer 0
+#pragma unroll
+  for (int t = 0; t < ROWS; ++t) mine[t * ST] = cur[t];
+  __syncthreads();
+  int p = 0, margin = 0;  // rings of the region that are spoiled
+  // one application of the rows `tab` (the interior one in `row`) to the iterate, seeded with -b or 0:
+  // f(t, row, sum) for the thread's nodes that a later application or the output needs
+  const auto apply = [&](const T* tab, bool seed_b, auto f) {
+    const V2* q = mine + p * plane;
+    V2 south = q[-ST], wprev = q[-ST - 1], wcur = q[-1], ecur = q[1], enext = q[ST + 1];
+#pragma unroll
+    for (int t = 0; t < ROWS; ++t) {
+      const V2 north = t + 1 < ROWS ? cur[t + 1 < ROWS ? t + 1 : t] : q[ROWS * ST];
+      const V2 center = cur[t];
+      const int r = g * ROWS + t;
+      if (r > margin && r < RH - 1 - margin && in(t)) {
+        V2 s = seed_b ? mk2<T, V2>(-b[t].x, -b[t].y) : mk2<T, V2>(T(0), T(0));
+        const V2 nb[7] = {wprev, south, wcur, center, ecur, north, enext};
+        if (EDGE && edge(t) != 1) {
+          T e[8];
+          load_row(tab, edge(t), e);
+#pragma unroll
+          for (int d = 0; d < 7; ++d) s = fma2(e[d], nb[d], s);
+          f(t, e[7], s);
+        } else {
+#pragma unroll
+          for (int d = 0; d < 7; ++d) s = fma2(row[d], nb[d], s);
+          f(t, row[7], s);
+        }
+      }
+      south = center;
+      wprev = wcur;
+      wcur = q[(t + 1) * ST - 1];
+      ecur = enext;
+      enext = q[(t + 2) * ST + 1];
+    }
+    ++margin;
+  };
+  for (int s = ZERO ? 1 : 0; s < a.deg; ++s) {
+    const int mode = s == 0 ? XP_NONE : (ZERO && s == 1 ? XP_ZERO : XP_READ);
+    const T alpha = a.alpha[s], nbeta = a.nbeta[s];
+    const T* tab = sizeof(T) == 8 ? a.steps + (size_t)s * a.nids * 8 : a.tab;
+    if (sizeof(T) == 8) load_row(tab, 1, row);
+    apply(tab, true, [&](int t, T g7, V2 sum) {
+      V2 v;
+      if (sizeof(T) == 8) {
+        v = mode == XP_READ ? fma2(g7, sum, mk2<T, V2>(-alpha * prev[t].x, -alpha * prev[t].y))
+                            : mk2<T, V2>(g7 * sum.x, g7 * sum.y);
+      } else {
+        v = cur[t];
+        if (mode == XP_READ) v = fma2(alpha, sub2(v, prev[t]), v);
+        else if (mode == XP_ZERO) v = fma2(alpha, v, v);
+        v = fma2(g7 * nbeta, sum, v);
+      }
+      prev[t] = cur[t];
+      cur[t] = v;
+    });
+    p ^= 1;
+#pragma unroll
+    for (int t = 0; t < ROWS; ++t) mine[p * plane + t * ST] = cur[t];
+    __syncthreads();
+  }
+  const bool col_out = col_in && c >= h && c < RW - h;
+  const auto out = [&](int t) { return col_out && in(t) && g * ROWS + t >= h && g * ROWS + t < RH - h; };
+#pragma unroll
+  for (int t = 0; t < ROWS; ++t)
+    if (out(t)) a.xo[node0 + (size_t)t * tl.W] = cur[t];
+  if (RES) {
+    if (sizeof(T) == 8) load_row(a.tab, 1, row);
+    apply(a.tab, false, [&](int t, T, V2 sum) {
+      if (out(t)) a.r[node0 + (size_t)t * tl.W] = sub2(b[t], sum);
+    });
+  }
+}
+
+template <typename T, typename V2, bool ZERO, bool RES>
+__global__ void __launch_bounds__(TileShape<T>::RW* TileShape<T>::GMAX) k_smooth_tile(TileArgs<T, V2> a) {
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  V2* buf = reinterpret_cast<V2*>(tile_raw);
+  const LatTile tl = a.tiles[blockIdx.x];
+  constexpr int RW = TileShape<T>::RW, ROWS = TileShape<T>::ROWS;
+  const int RH = ROWS * (blockDim.x / RW), xl = tl.x0 - a.halo, yl = tl.y0 - a.halo;
+  if (xl > 0 && yl > 0 && xl + RW < tl.W && yl + RH < tl.H) smooth_tile<T, V2, ZERO, RES, false>(a, tl, buf);
+  else smooth_tile<T, V2, ZERO, RES, true>(a, tl, buf);
+}
+
 #define CH_LAT_DISPATCH(nd, KCALL)                    \
   switch (nd) {                                       \
     case 7: { constexpr int NDC = 7; KCALL; } break;  \
@@ -1524,6 +1782,49 @@ static ChebCoef cheb_coef(double rho, int deg, double lower) {
   return cheb_coef_interval(lower * hi, hi, deg);
 }
 
+// the tile kernels' shared-memory limits (above the 48 KB default)
+template <typename T>
+static ch_status tile_setup() {
+  using V2 = typename V2T<T>::t;
+  const auto set = [](auto kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem<T>(TileShape<T>::GMAX));
+  };
+  CH_CUDA(set(k_smooth_tile<T, V2, true, true>));
+  CH_CUDA(set(k_smooth_tile<T, V2, false, true>));
+  CH_CUDA(set(k_smooth_tile<T, V2, false, false>));
+  return CH_OK;
+}
+
+// the V-cycle smoother's pass on the finest level in one launch (see k_smooth_tile)
+template <typename T, bool ZERO, bool RES>
+static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename V2T<T>::t* x,
+                               typename V2T<T>::t* xo, cudaStream_t st) {
+  using V2 = typename V2T<T>::t;
+  const TilePlan& pl = RES && !ZERO ? L.plan_r : L.plan;
+  const ChebCoef c = cheb_coef(h->rho[0], h->cheb_degree, h->cheb_lower);
+  TileArgs<T, V2> a;
+  a.tiles = pl.tiles;
+  a.tab = L.lat.tab;
+  a.steps = L.lat.steps;
+  a.b = L.b;
+  a.x = x;
+  a.xo = xo;
+  a.r = L.r;
+  a.nids = L.lat.L.nids;
+  a.deg = h->cheb_degree;
+  a.halo = pl.halo;
+  a.invtheta = (T)c.invtheta;
+  for (int s = 0; s < 16; ++s) {
+    a.alpha[s] = (T)c.alpha[s];
+    a.nbeta[s] = (T)-c.beta[s];
+  }
+  const double n = L.A.nrows, apps = pl.halo;
+  ProfScope ps(st, K_CHEB_STEP, sizeof(T) == 4, n * 2.0 * sizeof(T) * ((ZERO ? 1 : 2) + (RES ? 2 : 1)),
+               apps * (2.0 * L.A.nnz + 4.0 * n));
+  launch_k(L.pdl, k_smooth_tile<T, V2, ZERO, RES>, pl.ntiles, TileShape<T>::RW * pl.groups, tile_smem<T>(pl.groups),
+           st, a);
+}
+
 // bytes per row of the fine level's lattice form beyond its vectors: the class id
 static double lat_bytes(const Lattice& L, double n) { return (L.id32 ? 4.0 : 2.0) * n; }
 
@@ -1602,10 +1903,17 @@ static ch_status vcycle(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l,
     return CH_OK;
   }
   V2* x = *xres;
-  CH_TRY(smooth<T>(h, L, l, zero_guess, &x, st));
   LevelT<T>& C = Ls[l + 1];
   const int nc = C.A.nrows;
-  {
+  const bool tiles = l == 0 && L.plan.ntiles > 0 && L.plan_r.ntiles > 0;
+  if (tiles) {
+    V2* to = x == L.x ? L.x2 : L.x;
+    if (zero_guess) launch_smooth_tile<T, true, true>(h, L, nullptr, to, st);
+    else launch_smooth_tile<T, false, true>(h, L, x, to, st);
+    CH_LAUNCHED();
+    x = to;
+  } else {
+    CH_TRY(smooth<T>(h, L, l, zero_guess, &x, st));
     const double opb = L.lat.nd ? lat_bytes(L.lat.L, n) : L.A.nnz * (4 + Tb) + 4.0 * (n + 1);
     ProfScope ps(st, l == 0 ? K_VRESIDUAL : K_VRESIDUAL_C, sizeof(T) == 4, opb + 6.0 * Tb * n, 2.0 * L.A.nnz);
     launch_residual<T, V2>(L.tprA, L.A, L.b, x, L.r, st, &L.lat, L.pdl);
@@ -1634,7 +1942,14 @@ static ch_status vcycle(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l,
     launch_spmv2<T, V2, true>(L.tprP, L.P, xc, x, st, L.pdl);
   }
   CH_LAUNCHED();
-  CH_TRY(smooth<T>(h, L, l, 0, &x, st));
+  if (tiles) {
+    V2* to = x == L.x ? L.x2 : L.x;
+    launch_smooth_tile<T, false, false>(h, L, x, to, st);
+    CH_LAUNCHED();
+    x = to;
+  } else {
+    CH_TRY(smooth<T>(h, L, l, 0, &x, st));
+  }
   *xres = x;
   return CH_OK;
 }
@@ -1715,7 +2030,7 @@ template <typename T>
 static int load_input(Hierarchy* h, LevelT<T>& L, bool amg, const double* v, int ld, cudaStream_t st) {
   using V2 = typename V2T<T>::t;
   const int n = L.A.nrows;
-  if (amg && h->nlev > 1) {
+  if (amg && h->nlev > 1 && !(L.plan.ntiles > 0 && L.plan_r.ntiles > 0)) {
     const ChebCoef c = cheb_coef(h->rho[0], h->cheb_degree, h->cheb_lower);
     ProfScope ps(st, K_VLOAD, sizeof(T) == 4, n * (16.0 + 5.0 * sizeof(T)), 2.0 * n);
     launch_k(L.pdl, k_load2_first<T, V2>, blocks_for(n), TPB, 0, st, n, v, ld, L.dinv, (T)c.invtheta, L.b, L.x);

@@ -292,8 +292,8 @@ ch_status ch_precond_setup(const ch_system_t* s, void* stream, ch_precond_t** ou
   if (ph.cheb_degree == 0) ph.cheb_degree = 5;
   ch_params pm = ph;
   pm.cheb_degree = ph.cheb_degree_M > 0 ? ph.cheb_degree_M : std::min(3, ph.cheb_degree);
-  ch_status r = ch::hierarchy_build(M, &s->mesh->lat, pm, pc->precision, S(stream), &pc->hM);
-  if (r == CH_OK) r = ch::hierarchy_build(H, &s->mesh->lat, ph, pc->precision, S(stream), &pc->hH);
+  ch_status r = ch::hierarchy_build(M, s->mesh, pm, pc->precision, S(stream), &pc->hM);
+  if (r == CH_OK) r = ch::hierarchy_build(H, s->mesh, ph, pc->precision, S(stream), &pc->hH);
   if (r == CH_OK && (cudaStreamCreateWithFlags(&pc->side, cudaStreamNonBlocking) != cudaSuccess ||
                      cudaEventCreateWithFlags(&pc->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
                      cudaEventCreateWithFlags(&pc->ev_join, cudaEventDisableTiming) != cudaSuccess)) {

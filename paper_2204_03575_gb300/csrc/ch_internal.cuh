@@ -328,7 +328,7 @@ struct ch_system_s {
 
 namespace ch {
 struct Hierarchy;  // amg.cu
-ch_status hierarchy_build(const Csr<double>& A0, const Lattice* lat, const ch_params& p, int precision,
+ch_status hierarchy_build(const Csr<double>& A0, const ch_mesh_s* mesh, const ch_params& p, int precision,
                           cudaStream_t st, Hierarchy** out);
 void hierarchy_free(Hierarchy* h);
 int hierarchy_levels(const Hierarchy* h);
