@@ -224,7 +224,8 @@ ch_status ch_precond_level(const ch_precond_t* pc, int32_t which, int32_t level,
                            int32_t* A_rowptr, int32_t* A_col, double* A_val, int32_t* P_rowptr,
                            int32_t* P_col, double* P_val, void* stream);
 /* Lanes per row chosen for the level's A (smoothing, residual), R (restriction) and P
- * (prolongation) SpMVs (host outputs; R and P are 0 on the coarsest level). */
+ * (prolongation) SpMVs (host outputs; R and P are 0 on the coarsest level); 256 for R is a block per
+ * row. */
 ch_status ch_precond_tiles(const ch_precond_t* pc, int32_t which, int32_t level, int32_t* tpr_A,
                            int32_t* tpr_R, int32_t* tpr_P);
 /* Algorithm 1 on both species: w_1 ~ M^-1 v_1 and w_2 ~ H^-1 M H^-1 v_2 (AMG V-cycles); the

@@ -626,10 +626,12 @@ static void launch_residual(int tpr, const Csr<T>& A, const V2* b, const V2* x, 
                             const LatOp<T>* lat = nullptr, bool pdl = false);
 template <typename T, typename V2, bool ACC>
 static void launch_spmv2(int tpr, const Csr<T>& A, const V2* x, V2* y, cudaStream_t st, bool pdl = false);
+template <typename T, typename V2>
+static void launch_restrict(int tpr, const Csr<T>& R, const V2* x, V2* y, cudaStream_t st, bool pdl);
 
 // ---------------------------------------------------------------- SpMV tile autotuner
-// Lanes per row (1..32) for each matrix the V-cycle multiplies by: A (smoother steps and
-// residuals), R (restriction), P (prolongation).  autotune = 0 takes the rule below; 1 times
+// Lanes per row (1..32, or a whole block for restrictions of long rows) for each matrix the V-cycle
+// multiplies by: A (smoother steps and residuals), R (restriction), P (prolongation).  autotune = 0 takes the rule below; 1 times
 // every candidate on the matrix itself (one warm-up, three timed launches) and keeps the rule's
 // choice unless another is more than 5% faster.  Decisions are cached per process by matrix
 // shape (kind, rows, columns, entries, value size), so rebuilding a hierarchy of the same shape
@@ -664,11 +666,16 @@ static int tune_tpr(int kind, int rows, int cols, int64_t nnz, int tsize, int mo
   }
   // An idle GPU ramps its clocks over the first fraction of a second: warm up on the rule's width,
   // then time every width in two passes and keep each width's faster pass.
+  // Restrictions with long rows also try a block per row.
+  constexpr int NW = 7;
+  const int width[NW] = {1, 2, 4, 8, 16, 32, 256};
+  const int nw = kind == 1 && nnz >= 64LL * rows ? NW : NW - 1;
   for (int r = 0; r < 20; ++r) launch(rule);
-  float t[6];
-  for (int k = 0; k < 6; ++k) t[k] = 1e30f;
+  float t[NW];
+  for (int k = 0; k < nw; ++k) t[k] = 1e30f;
   for (int pass = 0; pass < 2; ++pass) {
-    for (int k = 0, tpr = 1; k < 6; ++k, tpr *= 2) {
+    for (int k = 0; k < nw; ++k) {
+      const int tpr = width[k];
       launch(tpr);
       cudaEventRecord(e0, st);
       for (int r = 0; r < 3; ++r) launch(tpr);
@@ -681,11 +688,11 @@ static int tune_tpr(int kind, int rows, int cols, int64_t nnz, int tsize, int mo
   }
   float best = 1e30f, t_rule = 1e30f;
   int pick = rule;
-  for (int k = 0, tpr = 1; k < 6; ++k, tpr *= 2) {
-    if (tpr == rule) t_rule = t[k];
+  for (int k = 0; k < nw; ++k) {
+    if (width[k] == rule) t_rule = t[k];
     if (t[k] < best) {
       best = t[k];
-      pick = tpr;
+      pick = width[k];
     }
   }
   cudaEventDestroy(e0);
@@ -713,7 +720,7 @@ static ch_status autotune_levels(Hierarchy* h, std::vector<LevelT<T>>& L, int mo
     if (l + 1 < h->nlev) {
       LevelT<T>& C = L[l + 1];
       W.tprR = tune_tpr(1, W.R.nrows, W.R.ncols, W.R.nnz, sizeof(T), mode,
-                        [&](int t) { launch_spmv2<T, V2, false>(t, W.R, W.r, C.b, st); }, st);
+                        [&](int t) { launch_restrict<T, V2>(t, W.R, W.r, C.b, st, false); }, st);
       W.tprP = tune_tpr(2, W.P.nrows, W.P.ncols, W.P.nnz, sizeof(T), mode,
                         [&](int t) { launch_spmv2<T, V2, true>(t, W.P, C.x, W.x, st); }, st);
     }
@@ -1130,10 +1137,14 @@ __global__ void k_cheb_first(int n, const T* dinv, const V2* b, T invtheta, V2* 
 }
 
 // Row sums of A x for both right-hand sides with TPR lanes per row: lane `sub` takes entries
-// sub, sub+TPR, ... of the row and a butterfly of shuffles adds the lanes' partial sums, so the
-// summation order is fixed for a given TPR.  Threads past the last row contribute zeros (no
-// early return before the shuffles).  The sum adds onto the caller's (s0, s1), which lane 0 of a
-// row may seed (with -b: the sum is then A x - b at no extra FP64 instruction).
+// sub, sub+TPR, ... of the row and shuffles add the lanes' partial sums in a fixed order.  The two sums
+// are separated in the first round (each half of the lanes keeps one and takes the other half's part of
+// it), so they cost log2 TPR additions and not twice as many, and what follows a row sum runs in two
+// lanes, one per right-hand side: an FP64 instruction holds the SM's pipe 16 clocks however few lanes it
+// serves (Algorithm 1 per application, us: FP64 800 x 400 1049 -> 993, 63 x 47 x 41 2105 -> 1710 with
+// k_restrict_wide; FP32 128 x 128 x 32 960 -> 882).  Threads past the last row contribute zeros (no early return before the shuffles).  The
+// sum adds onto the caller's (s0, s1), which lane 0 of a row may seed (with -b: the sum is then A x - b at
+// no extra FP64 instruction).
 //
 // The row's structure and values are set-up data, so a kernel reads them before its programmatic
 // dependency wait (row_prefetch: the lane's first CsrRow::PF entries, i.e. rowptr, then val and col)
@@ -1185,18 +1196,52 @@ __device__ __forceinline__ void row_acc(const Csr<T>& A, const CsrRow<T, TPR>& r
       s0 = fma(r.a[k], xj[k].x, s0);
       s1 = fma(r.a[k], xj[k].y, s1);
     }
+#pragma unroll 4
   for (int q = r.q; q < r.e; q += TPR) {
     const T a = A.val[q];
     const V2 v = x[A.col[q]];
     s0 = fma(a, v.x, s0);
     s1 = fma(a, v.y, s1);
   }
+}
+
+// The row sums over the TPR lanes of a row: component 0 in the row's lane 0, component 1 in its lane
+// TPR / 2 (TPR = 1: both in the one lane).
+template <typename T, int TPR>
+struct RowSum {
+  T v[TPR == 1 ? 2 : 1];
+};
+template <typename T, int TPR>
+__device__ __forceinline__ RowSum<T, TPR> row_sum(T s0, T s1, int sub) {
+  RowSum<T, TPR> r;
+  r.v[0] = s0;
+  if constexpr (TPR == 1) {
+    r.v[1] = s1;
+  } else {
+    constexpr int H = TPR / 2;
+    const bool up = sub & H;
+    const T send = up ? s0 : s1;
+    T keep = up ? s1 : s0;
+    keep += __shfl_xor_sync(0xffffffffu, send, H);
 #pragma unroll
-  for (int o = TPR / 2; o > 0; o >>= 1) {
-    s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    for (int o = H / 2; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
+    r.v[0] = keep;
+  }
+  return r;
+}
+// f(component, sum) in the lanes that hold a row's sums
+template <typename T, int TPR, typename F>
+__device__ __forceinline__ void row_finish(const RowSum<T, TPR>& r, int sub, F f) {
+  if constexpr (TPR == 1) {
+    f(0, r.v[0]);
+    f(1, r.v[1]);
+  } else {
+    constexpr int H = TPR / 2;
+    if ((sub & (H - 1)) == 0) f(sub != 0, r.v[0]);  // (TPR = 2: H - 1 = 0, both lanes)
   }
 }
+template <typename V2> __device__ __forceinline__ auto* comps(V2* p) { return &p->x; }
+template <typename V2> __device__ __forceinline__ const auto* comps(const V2* p) { return &p->x; }
 
 // One Chebyshev step of the two-term form, x' = x + alpha (x - xp) + beta D^-1 (b - A x), with the
 // iterate before x in the output's own place: xo holds xp on entry and x' on exit, so a step moves
@@ -1212,7 +1257,7 @@ __global__ void __launch_bounds__(TPB) k_cheb_step(Csr<T> A, const T* __restrict
   const int i = t / TPR, sub = t % TPR;
   CsrRow<T, TPR> row;
   row_prefetch<T, TPR>(A, i, sub, row);
-  const T di = (sub == 0 && i < A.nrows) ? dinv[i] * nbeta : T(0);
+  const T di = i < A.nrows ? dinv[i] * nbeta : T(0);
   pdl_wait();
   pdl_trigger_t<T>();
   T s0 = 0, s1 = 0;
@@ -1222,19 +1267,14 @@ __global__ void __launch_bounds__(TPB) k_cheb_step(Csr<T> A, const T* __restrict
     s1 = -bi.y;
   }
   row_acc<T, V2, TPR>(A, row, x, s0, s1);
-  if (i >= A.nrows || sub != 0) return;
-  V2 y = x[i];
-  if (mode != XP_NONE) {
-    V2 d = y;
-    if (mode == XP_READ) {
-      const V2 xp = xo[i];
-      d.x -= xp.x;
-      d.y -= xp.y;
-    }
-    y.x = fma(alpha, d.x, y.x);
-    y.y = fma(alpha, d.y, y.y);
-  }
-  xo[i] = mk2<T, V2>(fma(di, s0, y.x), fma(di, s1, y.y));
+  const RowSum<T, TPR> r = row_sum<T, TPR>(s0, s1, sub);
+  if (i >= A.nrows) return;
+  row_finish<T, TPR>(r, sub, [&](int c, T s) {
+    T y = comps(x + i)[c];
+    T* o = comps(xo + i) + c;
+    if (mode != XP_NONE) y = fma(alpha, mode == XP_READ ? y - *o : y, y);
+    *o = fma(di, s, y);
+  });
 }
 
 template <typename T, typename V2, int TPR>
@@ -1248,9 +1288,9 @@ __global__ void __launch_bounds__(TPB) k_residual(Csr<T> A, const V2* __restrict
   pdl_trigger_t<T>();
   T s0 = 0, s1 = 0;
   row_acc<T, V2, TPR>(A, row, x, s0, s1);
-  if (i >= A.nrows || sub != 0) return;
-  const V2 bi = b[i];
-  r[i] = mk2<T, V2>(bi.x - s0, bi.y - s1);
+  const RowSum<T, TPR> rs = row_sum<T, TPR>(s0, s1, sub);
+  if (i >= A.nrows) return;
+  row_finish<T, TPR>(rs, sub, [&](int c, T s) { comps(r + i)[c] = comps(b + i)[c] - s; });
 }
 
 // y = A x (ACC = false) or y += A x (ACC = true)
@@ -1264,13 +1304,12 @@ __global__ void __launch_bounds__(TPB) k_spmv2(Csr<T> A, const V2* __restrict__ 
   pdl_trigger_t<T>();
   T s0 = 0, s1 = 0;
   row_acc<T, V2, TPR>(A, row, x, s0, s1);
-  if (i >= A.nrows || sub != 0) return;
-  if (ACC) {
-    const V2 yi = y[i];
-    y[i] = mk2<T, V2>(yi.x + s0, yi.y + s1);
-  } else {
-    y[i] = mk2<T, V2>(s0, s1);
-  }
+  const RowSum<T, TPR> rs = row_sum<T, TPR>(s0, s1, sub);
+  if (i >= A.nrows) return;
+  row_finish<T, TPR>(rs, sub, [&](int c, T s) {
+    T* o = comps(y + i) + c;
+    *o = ACC ? *o + s : s;
+  });
 }
 
 // ---------------------------------------------------------------- structured (lattice) fine level
@@ -1586,14 +1625,46 @@ __global__ void __launch_bounds__(TPB) k_restrict_first(Csr<T> R, const V2* __re
   const int i = t / TPR, sub = t % TPR;
   CsrRow<T, TPR> row;
   row_prefetch<T, TPR>(R, i, sub, row);
-  const T s = (sub == 0 && i < R.nrows) ? invtheta * dinv_c[i] : T(0);
+  const T f = i < R.nrows ? invtheta * dinv_c[i] : T(0);
   pdl_wait();
   pdl_trigger_t<T>();
   T s0 = 0, s1 = 0;
   row_acc<T, V2, TPR>(R, row, r, s0, s1);
-  if (i >= R.nrows || sub != 0) return;
-  bc[i] = mk2<T, V2>(s0, s1);
-  xc[i] = mk2<T, V2>(s * s0, s * s1);
+  const RowSum<T, TPR> rs = row_sum<T, TPR>(s0, s1, sub);
+  if (i >= R.nrows) return;
+  row_finish<T, TPR>(rs, sub, [&](int c, T s) {
+    comps(bc + i)[c] = s;
+    comps(xc + i)[c] = f * s;
+  });
+}
+
+// A restriction whose rows are long and few (the coarsest levels of a 3D hierarchy: 443 rows of 700
+// entries gave 443 warps, 17.8 us in FP32 and 32.6 in FP64, now 8.2 in FP64): one block per row.  FIRST: fused with the coarse
+// level's first Chebyshev step as k_restrict_first.  Chosen by the set-up's timing (WIDE lanes per row).
+constexpr int WIDE = TPB;
+template <typename T, typename V2, bool FIRST>
+__global__ void __launch_bounds__(TPB) k_restrict_wide(Csr<T> R, const V2* __restrict__ r, V2* __restrict__ bc,
+                                                       const T* __restrict__ dinv_c, T invtheta,
+                                                       V2* __restrict__ xc) {
+  __shared__ T part[2][TPB / 32];
+  const int i = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  CsrRow<T, WIDE> row;
+  row_prefetch<T, WIDE>(R, i, threadIdx.x, row);
+  const T f = FIRST ? invtheta * dinv_c[i] : T(0);
+  pdl_wait();
+  pdl_trigger_t<T>();
+  T s0 = 0, s1 = 0;
+  row_acc<T, V2, WIDE>(R, row, r, s0, s1);
+  const RowSum<T, 32> rs = row_sum<T, 32>(s0, s1, lane);
+  if ((lane & 15) == 0) part[lane >> 4][w] = rs.v[0];
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    T s = part[threadIdx.x][0];
+#pragma unroll
+    for (int q = 1; q < TPB / 32; ++q) s += part[threadIdx.x][q];
+    comps(bc + i)[threadIdx.x] = s;
+    if (FIRST) comps(xc + i)[threadIdx.x] = f * s;
+  }
 }
 
 #define CH_TPR_DISPATCH(tpr, KCALL)                      \
@@ -1642,9 +1713,18 @@ static void launch_spmv2(int tpr, const Csr<T>& A, const V2* x, V2* y, cudaStrea
   CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_spmv2<T, V2, TPRC, ACC>, g, TPB, 0, st, A, x, y)));
 }
 
+// y = R x
+template <typename T, typename V2>
+static void launch_restrict(int tpr, const Csr<T>& R, const V2* x, V2* y, cudaStream_t st, bool pdl) {
+  if (tpr == WIDE)
+    launch_k(pdl, k_restrict_wide<T, V2, false>, R.nrows, TPB, 0, st, R, x, y, (const T*)nullptr, T(0), (V2*)nullptr);
+  else
+    launch_spmv2<T, V2, false>(tpr, R, x, y, st, pdl);
+}
+
 // x = Ainv b, dense nc x nc.  WPR warps per row: lane l of the row's warp `sub` takes columns
 // sub * 32 + l + k * 32 WPR, with its first U entries of Ainv read before the dependency wait and
-// 8 loads in flight after it; the lanes' sums are added by a butterfly and the warps' in warp order.
+// 8 loads in flight after it; the lanes' sums are added as in row_sum and the warps' in warp order.
 template <typename T, typename V2, int WPR>
 __global__ void __launch_bounds__(TPB) k_dense_solve(int n, const T* __restrict__ inv, const V2* __restrict__ b,
                                                      V2* __restrict__ x) {
@@ -1688,28 +1768,13 @@ __global__ void __launch_bounds__(TPB) k_dense_solve(int n, const T* __restrict_
       s1 = fma(aj, v.y, s1);
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-  }
-  if (WPR == 1) {
-    if (on && lane == 0) x[row] = mk2<T, V2>(s0, s1);
-    return;
-  }
-  if (lane == 0) {
-    part[w][0] = s0;
-    part[w][1] = s1;
-  }
+  T t = row_sum<T, 32>(s0, s1, lane).v[0];  // component 0 in lane 0, 1 in lane 16
+  if ((lane & 15) == 0) part[w][lane >> 4] = t;
   __syncthreads();
-  if (on && sub == 0 && lane == 0) {
-    T t0 = s0, t1 = s1;
+  if (on && sub == 0 && (lane & 15) == 0) {
 #pragma unroll
-    for (int q = 1; q < WPR; ++q) {
-      t0 += part[w + q][0];
-      t1 += part[w + q][1];
-    }
-    x[row] = mk2<T, V2>(t0, t1);
+    for (int q = 1; q < WPR; ++q) t += part[w + q][lane >> 4];
+    comps(x + row)[lane >> 4] = t;
   }
 }
 
@@ -1927,10 +1992,14 @@ static ch_status vcycle(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l,
       const int degc = h->cheb_degree_coarse;
       const ChebCoef cc = cheb_coef(h->rho[l + 1], degc, h->cheb_lower);
       const int g = blocks_for((int64_t)L.R.nrows * L.tprR);
-      CH_TPR_DISPATCH(L.tprR, (launch_k(L.pdl, k_restrict_first<T, V2, TPRC>, g, TPB, 0, st, L.R, L.r, C.b,
-                                        C.dinv, (T)cc.invtheta, C.x)));
+      if (L.tprR == WIDE)
+        launch_k(L.pdl, k_restrict_wide<T, V2, true>, L.R.nrows, TPB, 0, st, L.R, L.r, C.b, C.dinv,
+                 (T)cc.invtheta, C.x);
+      else
+        CH_TPR_DISPATCH(L.tprR, (launch_k(L.pdl, k_restrict_first<T, V2, TPRC>, g, TPB, 0, st, L.R, L.r, C.b,
+                                          C.dinv, (T)cc.invtheta, C.x)));
     } else {
-      launch_spmv2<T, V2, false>(L.tprR, L.R, L.r, C.b, st, L.pdl);
+      launch_restrict<T, V2>(L.tprR, L.R, L.r, C.b, st, L.pdl);
     }
   }
   CH_LAUNCHED();
