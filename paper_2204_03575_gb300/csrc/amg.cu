@@ -52,16 +52,21 @@ struct LatOp {
 struct LatTile {
   int off, W, H, x0, y0, id0;
 };
-template <typename T> struct TileShape;  // columns of a region, nodes per thread, most groups
-template <> struct TileShape<float> { static constexpr int RW = 64, ROWS = 4, GMAX = 16; };
-template <> struct TileShape<double> { static constexpr int RW = 16, ROWS = 1, GMAX = 16; };
+// columns of a region, nodes per thread, groups (thread rows) of a block at most, and of a block that
+// shares its SM with another
+template <typename T> struct TileShape;
+template <> struct TileShape<float> { static constexpr int RW = 64, ROWS = 4, GMAX = 12, GPAIR = 8; };
+template <> struct TileShape<double> { static constexpr int RW = 16, ROWS = 1, GMAX = 16, GPAIR = 16; };
 // FP64 passes are bound by the FP64 pipe, where recomputed halo nodes cost as much as any: tiles only
-// while the mesh is too small to fill the chip and a step is a launch's latency
-constexpr int TILE_MAX_F64 = 152;
+// while the mesh gives the chip at most two per SM and a step is a launch's latency (us per application
+// of Algorithm 1 with tiles / a launch per step: 32 x 32 88 / 131, 64 x 64 175 / 189, 96 x 96 with four
+// tiles per SM 256 / 192)
+constexpr int TILE_MAX_F64 = 304;
 struct TilePlan {
-  int ntiles = 0;  // 0: the pass runs as one launch per step
-  int groups = 0;  // thread rows of a block
-  int halo = 0;    // operator applications of the pass
+  int ntiles = 0;     // 0: the pass runs as one launch per step
+  int groups = 0;     // thread rows of a block
+  int halo = 0;       // operator applications of the pass
+  bool pair = false;  // two blocks share an SM
   const LatTile* tiles = nullptr;
 };
 
@@ -837,12 +842,18 @@ static void lat_step_tables(const double* tab64, const LatOp<double>& op, const 
   k_lat_steps<<<dim3(blocks_for(op.L.nids, 64), deg), 64, 0, st>>>(tab64, op.L.nids, op.nd, op.ts, sc, out);
 }
 
-// Tiles of a pass of `halo` operator applications over every run of a 2D mesh: the block height whose
-// tiles leave the busiest SM the fewest region nodes (tall blocks recompute less halo, short ones
-// spread a small mesh over more SMs).
+// Tiles of a pass of `halo` operator applications over every run of a 2D mesh.  FP32 block heights by the
+// time they take in units of region rows, measured over 64 x 64 .. 1024 x 1024 and the 64-run batch (Algorithm
+// 1, us per application): a block alone on its SM costs its rows and 24 for its latencies, and as many waves as
+// there are, so a mesh that fits one wave takes the shortest block that does (512 x 512: 12 groups 186, 10
+// groups in two waves 215, pairs 206); larger meshes take two blocks of 8 groups per SM, which overlap
+// (a wave costs 80, and the last one only its share: 1024 x 1024 510, single blocks 518 to 595; batch 939,
+// 966 to 1100).  Fewer than 4 groups are too few warps to hide anything (256 x 256: 142, 4 groups 113).
+// FP64: the fewest region rows on the busiest SM.
 template <typename T>
 static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* out, cudaStream_t st) {
   using S = TileShape<T>;
+  constexpr bool F32 = sizeof(T) == 4;
   *out = TilePlan();
   const int tw = S::RW - 2 * halo;
   if (tw < S::RW / 4) return CH_OK;
@@ -851,22 +862,26 @@ static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* o
     for (const ch_params& p : m->runs) n += (int64_t)((p.nx + tw) / tw) * ((p.ny + th) / th);
     return n;
   };
-  int64_t best = 0;
+  double best = 0.0;
   int G = 0;
-  for (int g = 2; g <= S::GMAX; ++g) {
+  bool pair = false;
+  const auto consider = [&](int g, bool two) {
     const int rh = S::ROWS * g, th = rh - 2 * halo;
-    if (th < 1 || S::RW * g % 32 != 0) continue;
-    // region rows on the busiest SM, in tenths; two blocks of up to 8 groups share an SM and overlap,
-    // taller ones run alone and wait out their loads once there is more than one per SM
-    const int64_t n = count(th), cost = (n + 151) / 152 * rh * (g > 8 && n > 152 ? 11 : 10);
+    if (th < 1 || S::RW * g % 32 != 0) return;
+    const int64_t n = count(th);
+    const double waves = (double)((n + 151) / 152);
+    const double cost = two ? 80.0 * std::max(1.0, n / 304.0) : waves * (rh + (F32 ? 24 : 0));
     if (G == 0 || cost < best) {
       best = cost;
       G = g;
+      pair = two;
     }
-  }
+  };
+  for (int g = F32 ? 4 : 2; g <= S::GMAX; ++g) consider(g, false);
+  if (F32) consider(S::GPAIR, true);
   if (G == 0) return CH_OK;
   const int th = S::ROWS * G - 2 * halo;
-  if (sizeof(T) == 8 && count(th) > TILE_MAX_F64) return CH_OK;
+  if (!F32 && count(th) > TILE_MAX_F64) return CH_OK;
   std::vector<LatTile> tiles;
   for (size_t r = 0; r < m->runs.size(); ++r) {
     const ch_params& p = m->runs[r];
@@ -881,6 +896,7 @@ static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* o
   out->ntiles = (int)tiles.size();
   out->groups = G;
   out->halo = halo;
+  out->pair = pair;
   out->tiles = d;
   return CH_OK;
 }
@@ -1436,10 +1452,9 @@ __global__ void __launch_bounds__(TPB) k_spmv2_lat(LatOp<T> D, int n, const V2* 
 // the pass starts from zero) is read, once per pass instead of four vectors per step.
 //   ZERO: the pass starts from a zero guess (its first step is pointwise);  RES: r = b - A x' as well.
 // Nodes outside the mesh stay zero (their coefficients are zero).
-// Bound by instruction issue and the waves' load latency, not memory.  Algorithm 1 per application, us, one
-// launch per step -> per pass: FP32 64 x 64 77.8 -> 51.6, 256 x 256 143 -> 124, 512 x 512 247 -> 202, 1024 x
-// 1024 655 -> 523, 64 runs 1071 -> 960; FP64 32 x 32 131 -> 117 (larger FP64 meshes keep the steps: 96 x 96
-// 202 either way).
+// Bound by the latencies of a block's loads and steps, not memory.  Algorithm 1 per application, us, one
+// launch per step -> per pass: FP32 64 x 64 77.8 -> 49, 256 x 256 143 -> 113, 512 x 512 247 -> 186, 1024 x
+// 1024 655 -> 510, 64 runs 1071 -> 939; FP64 32 x 32 131 -> 88, 64 x 64 189 -> 175.
 template <typename T, typename V2>
 struct TileArgs {
   const LatTile* tiles;
@@ -1478,8 +1493,9 @@ __device__ __forceinline__ double2 fma2(double c, double2 x, double2 a) {
 __device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 
 // One block's tile.  EDGE: the region reaches the mesh's boundary (or past it), so nodes carry their own
-// class row and those outside the mesh stay zero; the other tiles (all but the rim) keep one row in
-// registers and test nothing.
+// class row (a thread's one node in FP64 for good; in FP32 a column's, and nodes of the first and last mesh
+// row load theirs) and those outside the mesh stay zero; the other tiles (all but the rim) keep one
+// row in registers and test nothing.
 template <typename T, typename V2, bool ZERO, bool RES, bool EDGE>
 __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatTile& tl, V2* buf) {
   constexpr int RW = TileShape<T>::RW, ROWS = TileShape<T>::ROWS, ST = RW + 2;
@@ -1488,7 +1504,7 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   const int h = a.halo, x = tl.x0 - h + c, y0 = tl.y0 - h + g * ROWS;
   const bool col_in = !EDGE || (x >= 0 && x < tl.W);
   const int cx = !EDGE ? 1 : (x <= 0 ? 0 : (x >= tl.W - 1 ? 2 : 1));
-  const auto in = [&](int t) { return !EDGE || (col_in && y0 + t >= 0 && y0 + t < tl.H); };
+  const auto in = [&](int t) { return !EDGE || (col_in && (unsigned)(y0 + t) < (unsigned)tl.H); };
   const auto load_row = [&](const T* tab, int cy, T (&o)[8]) {
     constexpr int NQ = 8 * (int)sizeof(T) / 16;
     const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)(tl.id0 + cx + 3 * cy) * 8);
@@ -1497,16 +1513,18 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   };
   const auto edge = [&](int t) { return y0 + t == 0 ? 0 : (y0 + t == tl.H - 1 ? 2 : 1); };
   T row[8];
-  load_row(a.tab, 1, row);
+  constexpr bool OWN = EDGE && ROWS == 1;  // the node's class row is the thread's
+  load_row(a.tab, OWN ? edge(0) : 1, row);
   pdl_wait();
   pdl_trigger_t<T>();
   const size_t node0 = (size_t)tl.off + (size_t)((long long)y0 * tl.W) + x;  // (used only inside the mesh)
-  V2 b[ROWS], cur[ROWS], prev[ROWS];
+  V2 nb[ROWS], cur[ROWS], prev[ROWS];  // -b, the iterate and the one before it
 #pragma unroll
   for (int t = 0; t < ROWS; ++t) {
-    b[t] = cur[t] = prev[t] = mk2<T, V2>(T(0), T(0));
+    nb[t] = cur[t] = prev[t] = mk2<T, V2>(T(0), T(0));
     if (in(t)) {
-      b[t] = a.b[node0 + (size_t)t * tl.W];
+      const V2 bt = a.b[node0 + (size_t)t * tl.W];
+      nb[t] = mk2<T, V2>(-bt.x, -bt.y);
       if (!ZERO) cur[t] = a.x[node0 + (size_t)t * tl.W];
     }
   }
@@ -1514,22 +1532,22 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
 #pragma unroll
     for (int t = 0; t < ROWS; ++t) {
       T di = row[7];
-      if (EDGE && edge(t) != 1) {
+      if (EDGE && !OWN && edge(t) != 1) {
         T e[8];
         load_row(a.tab, edge(t), e);
         di = e[7];
       }
-      const T s = a.invtheta * di;
-      cur[t] = mk2<T, V2>(s * b[t].x, s * b[t].y);
+      const T s = -(a.invtheta * di);
+      cur[t] = mk2<T, V2>(s * nb[t].x, s * nb[t].y);
     }
   }
   V2* mine = buf + (g * ROWS + 1) * ST + c + 1;  // this thread's first node in buffer 0
 #pragma unroll
   for (int t = 0; t < ROWS; ++t) mine[t * ST] = cur[t];
   __syncthreads();
-  int p = 0, margin = 0;  // rings of the region that are spoiled
-  // one application of the rows `tab` (the interior one in `row`) to the iterate, seeded with -b or 0:
-  // f(t, row, sum) for the thread's nodes that a later application or the output needs
+  int p = 0, margin = 0;
+  // f(t, row's last entry, sum) for the thread's nodes, sum = one application of the rows `tab` (the
+  // interior one is in `row`) to the iterate, seeded with -b or 0
   const auto apply = [&](const T* tab, bool seed_b, auto f) {
     const V2* q = mine + p * plane;
     V2 south = q[-ST], wprev = q[-ST - 1], wcur = q[-1], ecur = q[1], enext = q[ST + 1];
@@ -1539,17 +1557,17 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
       const V2 center = cur[t];
       const int r = g * ROWS + t;
       if (r > margin && r < RH - 1 - margin && in(t)) {
-        V2 s = seed_b ? mk2<T, V2>(-b[t].x, -b[t].y) : mk2<T, V2>(T(0), T(0));
-        const V2 nb[7] = {wprev, south, wcur, center, ecur, north, enext};
-        if (EDGE && edge(t) != 1) {
+        V2 s = seed_b ? nb[t] : mk2<T, V2>(T(0), T(0));
+        const V2 nbr[7] = {wprev, south, wcur, center, ecur, north, enext};
+        if (EDGE && !OWN && edge(t) != 1) {
           T e[8];
           load_row(tab, edge(t), e);
 #pragma unroll
-          for (int d = 0; d < 7; ++d) s = fma2(e[d], nb[d], s);
+          for (int d = 0; d < 7; ++d) s = fma2(e[d], nbr[d], s);
           f(t, e[7], s);
         } else {
 #pragma unroll
-          for (int d = 0; d < 7; ++d) s = fma2(row[d], nb[d], s);
+          for (int d = 0; d < 7; ++d) s = fma2(row[d], nbr[d], s);
           f(t, row[7], s);
         }
       }
@@ -1562,20 +1580,20 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
     ++margin;
   };
   for (int s = ZERO ? 1 : 0; s < a.deg; ++s) {
-    const int mode = s == 0 ? XP_NONE : (ZERO && s == 1 ? XP_ZERO : XP_READ);
     const T alpha = a.alpha[s], nbeta = a.nbeta[s];
     const T* tab = sizeof(T) == 8 ? a.steps + (size_t)s * a.nids * 8 : a.tab;
-    if (sizeof(T) == 8) load_row(tab, 1, row);
-    apply(tab, true, [&](int t, T g7, V2 sum) {
+    if (sizeof(T) == 8) load_row(tab, OWN ? edge(0) : 1, row);
+    const bool has_prev = s > 0;
+    // (before the first step of a pass from zero the iterate was zero, as prev starts out)
+    apply(tab, true, [&](int t, T last, V2 sum) {
       V2 v;
       if (sizeof(T) == 8) {
-        v = mode == XP_READ ? fma2(g7, sum, mk2<T, V2>(-alpha * prev[t].x, -alpha * prev[t].y))
-                            : mk2<T, V2>(g7 * sum.x, g7 * sum.y);
+        v = has_prev ? fma2(last, sum, mk2<T, V2>(-alpha * prev[t].x, -alpha * prev[t].y))
+                     : mk2<T, V2>(last * sum.x, last * sum.y);
       } else {
         v = cur[t];
-        if (mode == XP_READ) v = fma2(alpha, sub2(v, prev[t]), v);
-        else if (mode == XP_ZERO) v = fma2(alpha, v, v);
-        v = fma2(g7 * nbeta, sum, v);
+        if (has_prev) v = fma2(alpha, sub2(v, prev[t]), v);
+        v = fma2(last * nbeta, sum, v);
       }
       prev[t] = cur[t];
       cur[t] = v;
@@ -1591,15 +1609,17 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   for (int t = 0; t < ROWS; ++t)
     if (out(t)) a.xo[node0 + (size_t)t * tl.W] = cur[t];
   if (RES) {
-    if (sizeof(T) == 8) load_row(a.tab, 1, row);
+    if (sizeof(T) == 8) load_row(a.tab, OWN ? edge(0) : 1, row);
     apply(a.tab, false, [&](int t, T, V2 sum) {
-      if (out(t)) a.r[node0 + (size_t)t * tl.W] = sub2(b[t], sum);
+      if (out(t)) a.r[node0 + (size_t)t * tl.W] = mk2<T, V2>(-nb[t].x - sum.x, -nb[t].y - sum.y);
     });
   }
 }
 
-template <typename T, typename V2, bool ZERO, bool RES>
-__global__ void __launch_bounds__(TileShape<T>::RW* TileShape<T>::GMAX) k_smooth_tile(TileArgs<T, V2> a) {
+// PAIR: two blocks per SM (64 registers a thread in FP32; the single blocks take up to 80 and spill nothing)
+template <typename T, typename V2, bool ZERO, bool RES, bool PAIR>
+__global__ void __launch_bounds__(TileShape<T>::RW*(PAIR ? TileShape<T>::GPAIR : TileShape<T>::GMAX), PAIR ? 2 : 1)
+    k_smooth_tile(TileArgs<T, V2> a) {
   extern __shared__ __align__(16) unsigned char tile_raw[];
   V2* buf = reinterpret_cast<V2*>(tile_raw);
   const LatTile tl = a.tiles[blockIdx.x];
@@ -1854,9 +1874,14 @@ static ch_status tile_setup() {
   const auto set = [](auto kern) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem<T>(TileShape<T>::GMAX));
   };
-  CH_CUDA(set(k_smooth_tile<T, V2, true, true>));
-  CH_CUDA(set(k_smooth_tile<T, V2, false, true>));
-  CH_CUDA(set(k_smooth_tile<T, V2, false, false>));
+  CH_CUDA(set(k_smooth_tile<T, V2, true, true, false>));
+  CH_CUDA(set(k_smooth_tile<T, V2, false, true, false>));
+  CH_CUDA(set(k_smooth_tile<T, V2, false, false, false>));
+  if constexpr (sizeof(T) == 4) {
+    CH_CUDA(set(k_smooth_tile<T, V2, true, true, true>));
+    CH_CUDA(set(k_smooth_tile<T, V2, false, true, true>));
+    CH_CUDA(set(k_smooth_tile<T, V2, false, false, true>));
+  }
   return CH_OK;
 }
 
@@ -1886,8 +1911,14 @@ static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename 
   const double n = L.A.nrows, apps = pl.halo;
   ProfScope ps(st, K_CHEB_STEP, sizeof(T) == 4, n * 2.0 * sizeof(T) * ((ZERO ? 1 : 2) + (RES ? 2 : 1)),
                apps * (2.0 * L.A.nnz + 4.0 * n));
-  launch_k(L.pdl, k_smooth_tile<T, V2, ZERO, RES>, pl.ntiles, TileShape<T>::RW * pl.groups, tile_smem<T>(pl.groups),
-           st, a);
+  const int threads = TileShape<T>::RW * pl.groups, smem = tile_smem<T>(pl.groups);
+  if constexpr (sizeof(T) == 4) {
+    if (pl.pair) {
+      launch_k(L.pdl, k_smooth_tile<T, V2, ZERO, RES, true>, pl.ntiles, threads, smem, st, a);
+      return;
+    }
+  }
+  launch_k(L.pdl, k_smooth_tile<T, V2, ZERO, RES, false>, pl.ntiles, threads, smem, st, a);
 }
 
 // bytes per row of the fine level's lattice form beyond its vectors: the class id

@@ -1,7 +1,8 @@
 """The tile form of the finest level's smoothing passes (2D, one launch per pass) against the oracle's
 V-cycle, at sizes around the tiles' edges: 64-column regions in FP32 (52 to 62 output columns at halos 6 to
 1), 16-column ones in FP64, meshes of one row of cells, meshes smaller than a tile, several runs of unlike
-size in one batch, and FP64 meshes on both sides of the line where the single steps take over.
+size in one batch, a mesh large enough for two blocks per SM, and FP64 meshes on both sides of the line where
+the single steps take over.
 
 The hierarchy is the device's (coarsest level capped at 32 rows, or one level's direct solve would answer);
 bounds as in the other V-cycle tests: FP64 1e-12 relative (sums of at most 9 terms over a handful of
@@ -17,7 +18,7 @@ pytestmark = pytest.mark.gpu
 
 SIZES = [dict(nx=53, ny=3), dict(nx=54, ny=58), dict(nx=57, ny=1), dict(nx=1, ny=130), dict(nx=109, ny=53),
          dict(nx=12, ny=11), dict(nx=66, ny=127), dict(nx=54, ny=54, cheb_degree=1), dict(nx=107, ny=9, cheb_degree=5),
-         "batch"]
+         dict(nx=64, ny=64), dict(nx=640, ny=640), "batch"]
 
 
 @pytest.mark.parametrize("precision", [0, 1])
