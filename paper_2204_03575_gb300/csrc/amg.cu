@@ -73,6 +73,7 @@ struct TilePlan {
 template <typename T>
 struct LevelT {
   Csr<T> A, P, R;
+  Csr<T> RB;  // [R, -R A] over the stacked (b, x): the coarse right-hand side without the residual
   LatOp<T> lat;                        // level 0 of a structured mesh
   TilePlan plan, plan_r;               // ... its smoothing passes as single launches, and those from a
                                        // given iterate that also form the residual
@@ -86,6 +87,7 @@ struct Hierarchy {
   int precision = 0;
   int nlev = 0;
   std::vector<Csr<double>> A, P, R;  // FP64 set-up results
+  std::vector<Csr<double>> RA;       // R A where the cycle restricts with it (set-up only)
   std::vector<double*> dinv;
   std::vector<double> rho;            // per level: min(Gershgorin bound, 1.05 x power estimate) of
                                       // lambda_max(D^-1 A); Chebyshev interval [lower, 1] x 1.1 rho
@@ -393,6 +395,25 @@ __global__ void k_copy_cast(const double* a, T* b, int64_t n) {
   if (i < n) b[i] = (T)a[i];
 }
 
+// B = [R, -RA], a warp per row
+template <typename T>
+__global__ void k_stack(Csr<double> R, Csr<double> RA, Csr<T> B) {
+  const int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
+  if (i >= R.nrows) return;
+  const int r0 = R.rowptr[i], r1 = R.rowptr[i + 1], q0 = RA.rowptr[i], q1 = RA.rowptr[i + 1];
+  if (lane == 0) B.rowptr[i] = r0 + q0;
+  if (lane == 1 && i == R.nrows - 1) B.rowptr[i + 1] = r1 + q1;
+  const int o = r0 + q0, o2 = r1 + q0;
+  for (int k = r0 + lane; k < r1; k += 32) {
+    B.col[o + k - r0] = R.col[k];
+    B.val[o + k - r0] = (T)R.val[k];
+  }
+  for (int k = q0 + lane; k < q1; k += 32) {
+    B.col[o2 + k - q0] = R.ncols + RA.col[k];
+    B.val[o2 + k - q0] = (T)-RA.val[k];
+  }
+}
+
 // ---------------------------------------------------------------- spectral radius of D^-1 A
 // Power iteration with the D-weighted Rayleigh quotient lambda = (x, A x) / (x, D x), which for
 // symmetric A converges twice as fast as the norm ratio.  One launch per iteration: y = D^-1 A x with x
@@ -484,7 +505,7 @@ static ch_status power_estimate(const Csr<double>& A, const double* dinv, cudaSt
 }
 
 // ---------------------------------------------------------------- set-up driver
-static ch_status level_setup(Hierarchy* h, int l, const ch_params& p, cudaStream_t st,
+static ch_status level_setup(Hierarchy* h, int l, const ch_params& p, cudaStream_t st, Alloc& ra,
                              bool* last) {
   const Csr<double>& A = h->A[l];
   const int n = A.nrows;
@@ -615,11 +636,24 @@ static ch_status level_setup(Hierarchy* h, int l, const ch_params& p, cudaStream
   Csr<double> R, AP, Ac;
   CH_TRY(transpose(P, &R, st, h->mem));
   Alloc aptmp;
-  CH_TRY(spgemm(A, P, &AP, st, aptmp));
-  CH_TRY(spgemm(R, AP, &Ac, st, h->mem));
+  Csr<double> RA;
+  if (h->precision == 1 && l > 0 && n <= 65536 && n >= 4 * nc && A.nnz <= 32LL * n) {
+    // R A first: where it has no more entries than A, the cycle restricts by R b - (R A) x, one launch less and
+    // no residual vector.  FP32 cycles below the finest level are bound by their launches (Algorithm 1, us per
+    // application: 256 x 256 115.7 -> 108.5, 512 x 512 195.5 -> 183.6, 800 x 400 235 -> 220); FP64 ones by the
+    // FP64 pipe (512 x 512 780 and 778), and larger levels by their entries (64 runs, 200000 rows: 942 -> 950).
+    // Long rows of A (3D) or coarsening by less than 4 would give R A rows of thousands of entries.
+    CH_TRY(spgemm(R, A, &RA, st, ra));
+    CH_TRY(spgemm(RA, P, &Ac, st, h->mem));
+    if (RA.nnz > A.nnz) RA = Csr<double>();
+  } else {
+    CH_TRY(spgemm(A, P, &AP, st, aptmp));
+    CH_TRY(spgemm(R, AP, &Ac, st, h->mem));
+  }
   h->P.push_back(P);
   h->R.push_back(R);
   h->A.push_back(Ac);
+  h->RA.push_back(RA);
   CH_CUDA(cudaStreamSynchronize(st));
   return CH_OK;
 }
@@ -632,7 +666,8 @@ static void launch_residual(int tpr, const Csr<T>& A, const V2* b, const V2* x, 
 template <typename T, typename V2, bool ACC>
 static void launch_spmv2(int tpr, const Csr<T>& A, const V2* x, V2* y, cudaStream_t st, bool pdl = false);
 template <typename T, typename V2>
-static void launch_restrict(int tpr, const Csr<T>& R, const V2* x, V2* y, cudaStream_t st, bool pdl);
+static void launch_restrict(const LevelT<T>& L, int tpr, const V2* x, V2* bc, const T* dinv, T invtheta, V2* xc,
+                            cudaStream_t st, bool pdl);
 
 // ---------------------------------------------------------------- SpMV tile autotuner
 // Lanes per row (1..32, or a whole block for restrictions of long rows) for each matrix the V-cycle
@@ -724,8 +759,11 @@ static ch_status autotune_levels(Hierarchy* h, std::vector<LevelT<T>>& L, int mo
                                  [&](int t) { launch_residual<T, V2>(t, W.A, W.b, W.x, W.r, st); }, st);
     if (l + 1 < h->nlev) {
       LevelT<T>& C = L[l + 1];
-      W.tprR = tune_tpr(1, W.R.nrows, W.R.ncols, W.R.nnz, sizeof(T), mode,
-                        [&](int t) { launch_restrict<T, V2>(t, W.R, W.r, C.b, st, false); }, st);
+      const Csr<T>& R = W.RB.nnz > 0 ? W.RB : W.R;
+      W.tprR = tune_tpr(1, R.nrows, R.ncols, R.nnz, sizeof(T), mode,
+                        [&](int t) {
+                          launch_restrict<T, V2>(W, t, W.x, C.b, (const T*)nullptr, T(0), (V2*)nullptr, st, false);
+                        }, st);
       W.tprP = tune_tpr(2, W.P.nrows, W.P.ncols, W.P.nnz, sizeof(T), mode,
                         [&](int t) { launch_spmv2<T, V2, true>(t, W.P, C.x, W.x, st); }, st);
     }
@@ -931,6 +969,17 @@ static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, const ch_para
     if (l + 1 < h->nlev) {
       CH_TRY(cast_csr(h->P[l], w.P));
       CH_TRY(cast_csr(h->R[l], w.R));
+      if (h->RA[l].nnz > 0) {
+        const Csr<double>&R = h->R[l], &RA = h->RA[l];
+        w.RB.nrows = R.nrows;
+        w.RB.ncols = R.ncols + RA.ncols;
+        w.RB.nnz = R.nnz + RA.nnz;
+        CH_TRY(h->mem.get(&w.RB.rowptr, (size_t)R.nrows + 1));
+        CH_TRY(h->mem.get(&w.RB.col, (size_t)w.RB.nnz));
+        CH_TRY(h->mem.get(&w.RB.val, (size_t)w.RB.nnz));
+        k_stack<T><<<blocks_for(R.nrows, TPB / 32), TPB, 0, st>>>(R, RA, w.RB);
+        CH_LAUNCHED();
+      }
     }
     const int n = h->A[l].nrows;
     if (std::is_same<T, double>::value) {
@@ -995,6 +1044,7 @@ ch_status hierarchy_build(const Csr<double>& A0, const ch_mesh_s* mesh, const ch
   h->pdl = p.pdl != 0;
   h->cheb_lower = p.cheb_lower;
   h->A.push_back(A0);
+  Alloc ra;  // the R A products, until the working copies hold them
   ch_status s = CH_OK;
   for (int l = 0;; ++l) {
     if (l >= 25) {
@@ -1003,7 +1053,7 @@ ch_status hierarchy_build(const Csr<double>& A0, const ch_mesh_s* mesh, const ch
       break;
     }
     bool last = false;
-    s = level_setup(h, l, p, st, &last);
+    s = level_setup(h, l, p, st, ra, &last);
     if (s != CH_OK || last) break;
   }
   if (s == CH_OK) {
@@ -1060,6 +1110,7 @@ ch_status hierarchy_build(const Csr<double>& A0, const ch_mesh_s* mesh, const ch
       set_error("AMG: building working copies failed");
       s = CH_ERR_CUDA;
     }
+    h->RA.clear();
   }
   if (s != CH_OK) {
     delete h;
@@ -1198,9 +1249,22 @@ __device__ __forceinline__ void row_prefetch(const Csr<T>& A, int row, int sub, 
   }
 }
 
-template <typename T, typename V2, int TPR>
-__device__ __forceinline__ void row_acc(const Csr<T>& A, const CsrRow<T, TPR>& r, const V2* __restrict__ x,
-                                        T& s0, T& s1) {
+// What a matrix multiplies: a vector, or two stacked ones (n entries of b, then x).
+template <typename V2>
+struct OneVec {
+  const V2* __restrict__ x;
+  __device__ __forceinline__ V2 operator[](int c) const { return x[c]; }
+};
+template <typename V2>
+struct TwoVecs {
+  const V2* __restrict__ b;
+  const V2* __restrict__ x;
+  int n;
+  __device__ __forceinline__ V2 operator[](int c) const { return c < n ? b[c] : x[c - n]; }
+};
+
+template <typename T, typename V2, int TPR, typename X>
+__device__ __forceinline__ void row_acc(const Csr<T>& A, const CsrRow<T, TPR>& r, const X& x, T& s0, T& s1) {
   constexpr int PF = CsrRow<T, TPR>::PF;
   V2 xj[PF];
 #pragma unroll
@@ -1282,7 +1346,7 @@ __global__ void __launch_bounds__(TPB) k_cheb_step(Csr<T> A, const T* __restrict
     s0 = -bi.x;
     s1 = -bi.y;
   }
-  row_acc<T, V2, TPR>(A, row, x, s0, s1);
+  row_acc<T, V2, TPR>(A, row, OneVec<V2>{x}, s0, s1);
   const RowSum<T, TPR> r = row_sum<T, TPR>(s0, s1, sub);
   if (i >= A.nrows) return;
   row_finish<T, TPR>(r, sub, [&](int c, T s) {
@@ -1303,15 +1367,15 @@ __global__ void __launch_bounds__(TPB) k_residual(Csr<T> A, const V2* __restrict
   pdl_wait();
   pdl_trigger_t<T>();
   T s0 = 0, s1 = 0;
-  row_acc<T, V2, TPR>(A, row, x, s0, s1);
+  row_acc<T, V2, TPR>(A, row, OneVec<V2>{x}, s0, s1);
   const RowSum<T, TPR> rs = row_sum<T, TPR>(s0, s1, sub);
   if (i >= A.nrows) return;
   row_finish<T, TPR>(rs, sub, [&](int c, T s) { comps(r + i)[c] = comps(b + i)[c] - s; });
 }
 
 // y = A x (ACC = false) or y += A x (ACC = true)
-template <typename T, typename V2, int TPR, bool ACC>
-__global__ void __launch_bounds__(TPB) k_spmv2(Csr<T> A, const V2* __restrict__ x, V2* __restrict__ y) {
+template <typename T, typename V2, int TPR, bool ACC, typename X>
+__global__ void __launch_bounds__(TPB) k_spmv2(Csr<T> A, X x, V2* __restrict__ y) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = t / TPR, sub = t % TPR;
   CsrRow<T, TPR> row;
@@ -1635,10 +1699,10 @@ __global__ void __launch_bounds__(TileShape<T>::RW*(PAIR ? TileShape<T>::GPAIR :
     default: { constexpr int NDC = 15; KCALL; } break; \
   }
 
-// b_c = R r, fused with the coarse level's first Chebyshev step from a zero guess (pointwise:
-// x_c = invtheta D_c^-1 b_c, the arithmetic of k_cheb_first): one launch instead of two.
-template <typename T, typename V2, int TPR>
-__global__ void __launch_bounds__(TPB) k_restrict_first(Csr<T> R, const V2* __restrict__ r, V2* __restrict__ bc,
+// b_c = R r (or R b - R A x), fused with the coarse level's first Chebyshev step from a zero guess
+// (pointwise: x_c = invtheta D_c^-1 b_c, the arithmetic of k_cheb_first): one launch instead of two.
+template <typename T, typename V2, int TPR, typename X>
+__global__ void __launch_bounds__(TPB) k_restrict_first(Csr<T> R, X r, V2* __restrict__ bc,
                                                         const T* __restrict__ dinv_c, T invtheta,
                                                         V2* __restrict__ xc) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1659,11 +1723,12 @@ __global__ void __launch_bounds__(TPB) k_restrict_first(Csr<T> R, const V2* __re
 }
 
 // A restriction whose rows are long and few (the coarsest levels of a 3D hierarchy: 443 rows of 700
-// entries gave 443 warps, 17.8 us in FP32 and 32.6 in FP64, now 8.2 in FP64): one block per row.  FIRST: fused with the coarse
-// level's first Chebyshev step as k_restrict_first.  Chosen by the set-up's timing (WIDE lanes per row).
+// entries gave 443 warps, 17.8 us in FP32 and 32.6 in FP64, now 8.2 in FP64): one block per row.  FIRST:
+// fused with the coarse level's first Chebyshev step as k_restrict_first.  Chosen by the set-up's timing
+// (WIDE lanes per row).
 constexpr int WIDE = TPB;
-template <typename T, typename V2, bool FIRST>
-__global__ void __launch_bounds__(TPB) k_restrict_wide(Csr<T> R, const V2* __restrict__ r, V2* __restrict__ bc,
+template <typename T, typename V2, bool FIRST, typename X>
+__global__ void __launch_bounds__(TPB) k_restrict_wide(Csr<T> R, X r, V2* __restrict__ bc,
                                                        const T* __restrict__ dinv_c, T invtheta,
                                                        V2* __restrict__ xc) {
   __shared__ T part[2][TPB / 32];
@@ -1730,16 +1795,32 @@ static void launch_apply_level(const LevelT<T>& L, const V2* x, V2* y, cudaStrea
 template <typename T, typename V2, bool ACC>
 static void launch_spmv2(int tpr, const Csr<T>& A, const V2* x, V2* y, cudaStream_t st, bool pdl) {
   const int g = blocks_for((int64_t)A.nrows * tpr);
-  CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_spmv2<T, V2, TPRC, ACC>, g, TPB, 0, st, A, x, y)));
+  CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_spmv2<T, V2, TPRC, ACC, OneVec<V2>>, g, TPB, 0, st, A, OneVec<V2>{x}, y)));
 }
 
-// y = R x
+// bc = R x, and with dinv the coarse level's first step from zero, xc = invtheta D^-1 bc
+template <typename T, typename V2, typename X>
+static void launch_restrict_x(int tpr, const Csr<T>& R, const X& x, V2* bc, const T* dinv, T invtheta, V2* xc,
+                              cudaStream_t st, bool pdl) {
+  const int g = blocks_for((int64_t)R.nrows * tpr);
+  if (tpr == WIDE) {
+    if (dinv) launch_k(pdl, k_restrict_wide<T, V2, true, X>, R.nrows, TPB, 0, st, R, x, bc, dinv, invtheta, xc);
+    else launch_k(pdl, k_restrict_wide<T, V2, false, X>, R.nrows, TPB, 0, st, R, x, bc, dinv, invtheta, xc);
+  } else if (dinv) {
+    CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_restrict_first<T, V2, TPRC, X>, g, TPB, 0, st, R, x, bc, dinv, invtheta,
+                                   xc)));
+  } else {
+    CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_spmv2<T, V2, TPRC, false, X>, g, TPB, 0, st, R, x, bc)));
+  }
+}
+// a level's restriction: R r, or [R, -R A] (b, x) where it has the product
 template <typename T, typename V2>
-static void launch_restrict(int tpr, const Csr<T>& R, const V2* x, V2* y, cudaStream_t st, bool pdl) {
-  if (tpr == WIDE)
-    launch_k(pdl, k_restrict_wide<T, V2, false>, R.nrows, TPB, 0, st, R, x, y, (const T*)nullptr, T(0), (V2*)nullptr);
+static void launch_restrict(const LevelT<T>& L, int tpr, const V2* x, V2* bc, const T* dinv, T invtheta, V2* xc,
+                            cudaStream_t st, bool pdl) {
+  if (L.RB.nnz > 0)
+    launch_restrict_x<T, V2>(tpr, L.RB, TwoVecs<V2>{L.b, x, L.A.nrows}, bc, dinv, invtheta, xc, st, pdl);
   else
-    launch_spmv2<T, V2, false>(tpr, R, x, y, st, pdl);
+    launch_restrict_x<T, V2>(tpr, L.R, OneVec<V2>{L.r}, bc, dinv, invtheta, xc, st, pdl);
 }
 
 // x = Ainv b, dense nc x nc.  WPR warps per row: lane l of the row's warp `sub` takes columns
@@ -2010,28 +2091,20 @@ static ch_status vcycle(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l,
     x = to;
   } else {
     CH_TRY(smooth<T>(h, L, l, zero_guess, &x, st));
-    const double opb = L.lat.nd ? lat_bytes(L.lat.L, n) : L.A.nnz * (4 + Tb) + 4.0 * (n + 1);
-    ProfScope ps(st, l == 0 ? K_VRESIDUAL : K_VRESIDUAL_C, sizeof(T) == 4, opb + 6.0 * Tb * n, 2.0 * L.A.nnz);
-    launch_residual<T, V2>(L.tprA, L.A, L.b, x, L.r, st, &L.lat, L.pdl);
+    if (L.RB.nnz == 0) {
+      const double opb = L.lat.nd ? lat_bytes(L.lat.L, n) : L.A.nnz * (4 + Tb) + 4.0 * (n + 1);
+      ProfScope ps(st, l == 0 ? K_VRESIDUAL : K_VRESIDUAL_C, sizeof(T) == 4, opb + 6.0 * Tb * n, 2.0 * L.A.nnz);
+      launch_residual<T, V2>(L.tprA, L.A, L.b, x, L.r, st, &L.lat, L.pdl);
+    }
   }
   const bool fuse = l + 1 < h->nlev - 1;  // the coarse level smooths: fuse its first step
   {
+    const Csr<T>& R = L.RB.nnz > 0 ? L.RB : L.R;
     ProfScope ps(st, l == 0 ? K_RESTRICT : K_RESTRICT_C, sizeof(T) == 4,
-                 L.R.nnz * (4 + Tb) + 4.0 * (nc + 1) + 2.0 * Tb * (n + nc) + (fuse ? 3.0 * Tb * nc : 0.0),
-                 2.0 * L.R.nnz + (fuse ? 2.0 * nc : 0.0));
-    if (fuse) {
-      const int degc = h->cheb_degree_coarse;
-      const ChebCoef cc = cheb_coef(h->rho[l + 1], degc, h->cheb_lower);
-      const int g = blocks_for((int64_t)L.R.nrows * L.tprR);
-      if (L.tprR == WIDE)
-        launch_k(L.pdl, k_restrict_wide<T, V2, true>, L.R.nrows, TPB, 0, st, L.R, L.r, C.b, C.dinv,
-                 (T)cc.invtheta, C.x);
-      else
-        CH_TPR_DISPATCH(L.tprR, (launch_k(L.pdl, k_restrict_first<T, V2, TPRC>, g, TPB, 0, st, L.R, L.r, C.b,
-                                          C.dinv, (T)cc.invtheta, C.x)));
-    } else {
-      launch_restrict<T, V2>(L.tprR, L.R, L.r, C.b, st, L.pdl);
-    }
+                 R.nnz * (4 + Tb) + 4.0 * (nc + 1) + 2.0 * Tb * (R.ncols + nc) + (fuse ? 3.0 * Tb * nc : 0.0),
+                 2.0 * R.nnz + (fuse ? 2.0 * nc : 0.0));
+    const T invtheta = (T)cheb_coef(h->rho[l + 1], h->cheb_degree_coarse, h->cheb_lower).invtheta;
+    launch_restrict<T, V2>(L, L.tprR, x, C.b, fuse ? C.dinv : nullptr, invtheta, C.x, st, L.pdl);
   }
   CH_LAUNCHED();
   V2* xc = C.x;
