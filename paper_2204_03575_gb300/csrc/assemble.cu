@@ -816,54 +816,87 @@ __device__ __forceinline__ constexpr double gl_w(int i) { return i == 1 ? 4.0 / 
 
 // Natural logarithm of a positive value by tables over the mantissa and the exponent (Tang 1990,
 // "Table-driven implementation of the logarithm function in IEEE floating-point arithmetic"): x = 2^k m,
-// with f the reciprocal of the middle of m's interval (1024 of them) rounded to FP32, r = m f - 1 (one
-// FMA; |r| <= 2^-11 and a little), log x = k log 2 - log f + log1p(r) and log1p by its Taylor series
-// through r^4 (the next term is below 2^-57).  Seven FP64 instructions where the general function
-// takes several times as many, and the kernel is bound by that pipe; the absolute error stays within
-// 2^-53 (1 + |log x|) and a rounding, which is what the sums it enters can resolve.  Other values (zero,
-// negative, denormal, infinite, NaN) take CUDA's log.
+// with f the reciprocal of the middle of m's interval (4096 of them) cut to 21 bits, r = m f - 1 (one
+// FMA; |r| <= a = 2^-13 and a little), log x = k log 2 - log f + log1p(r), and log1p by its Taylor series
+// through r^3 with r^4 replaced by a^2 r^2, its part in the Chebyshev polynomials below the fourth (the
+// rest is below 2^-56).  Six FP64 instructions where the general function takes several times as many, and
+// the kernel is bound by that pipe (1024 intervals and one more term took seven); the absolute error
+// stays within 2^-53 (1 + |log x|) and a rounding, which is what the sums it enters can resolve.  Other
+// values (zero, negative, denormal, above 2^65, infinite, NaN) take CUDA's log.
+constexpr int LOG_M = 4096, LOG_K = 1088;
 struct LogTables {
-  double2 m[1024];  // f, -log f
-  double k[2048];   // (biased exponent - 1023) log 2
+  double y[LOG_M];  // -log f
+  int f[LOG_M];     // upper word of f, the lower one is zero
+  double k[LOG_K];  // (biased exponent - 1023) log 2
 };
+static_assert(sizeof(LogTables) % 16 == 0, "copied in 16-byte pieces");
 __global__ void k_log_tables(LogTables* t) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < 1024) {
-    const double f = (double)(float)(1.0 / (1.0 + (i + 0.5) / 1024.0));
-    t->m[i] = make_double2(f, -log(f));
+  if (i < LOG_M) {
+    const int hi = __double2hiint(1.0 / (1.0 + (i + 0.5) / LOG_M));
+    t->f[i] = hi;
+    t->y[i] = -log(__hiloint2double(hi, 0));
   }
-  if (i < 2048) t->k[i] = (i - 1023) * 0.69314718055994530942;
+  if (i < LOG_K) t->k[i] = (i - 1023) * 0.69314718055994530942;
 }
 // log of max(x, delta), delta > 0; a NaN stays a NaN.  Positive doubles compare like their bits (an FP64
 // comparison would take the pipe).
 __device__ __forceinline__ double guarded_log(double x, double delta, const LogTables* tab) {
+  constexpr unsigned LO = 0x00100000u, SPAN = ((unsigned)LOG_K << 20) - LO;  // upper words within the tables
   long long bits = __double_as_longlong(x);
   const long long lo = __double_as_longlong(delta);
-  if ((unsigned)(bits >> 32) - 0x00100000u >= 0x7fe00000u) {
+  if ((unsigned)(bits >> 32) - LO >= SPAN) {
     x = x < delta ? delta : x;
     bits = __double_as_longlong(x);
-    if ((unsigned)(bits >> 32) - 0x00100000u >= 0x7fe00000u) return log(x);
+    if ((unsigned)(bits >> 32) - LO >= SPAN) return log(x);
   }
   bits = bits < lo ? lo : bits;
   const unsigned hi = (unsigned)(bits >> 32);
-  if (hi < 0x00100000u) return log(__longlong_as_double(bits));  // a denormal delta
+  if (hi - LO >= SPAN) return log(__longlong_as_double(bits));  // a denormal or enormous delta
   const double m = __longlong_as_double((bits & 0x000fffffffffffffLL) | 0x3ff0000000000000LL);
-  const double2 e = tab->m[(hi >> 10) & 1023u];
-  const double r = fma(m, e.x, -1.0), r2 = r * r;
-  const double p = fma(r, fma(r, -0.25, 1.0 / 3.0), -0.5);
-  return (tab->k[hi >> 20] + e.y) + fma(r2, p, r);
+  const int j = (hi >> 8) & (LOG_M - 1);
+  const double r = fma(m, __hiloint2double(tab->f[j], 0), -1.0), r2 = r * r;
+  const double p = fma(r, 1.0 / 3.0, -0.5 - 0x1p-28);
+  return (tab->k[hi >> 20] + tab->y[j]) + fma(r2, p, r);
 }
+
+// A line of the product rule: its place (u, v (1 - u)) in the simplex, its length w2, and the weights of its
+// sums A and B (see k_cell_loads_fh) against 1, lambda_1, lambda_2 and lambda_D.
+struct FhLine {
+  double u, vv, w2, c, cu, cv, ca, cb;
+};
+template <int D>
+__device__ __forceinline__ constexpr FhLine fh_line(int ij) {
+  constexpr double h = 0.38729833462074168852;  // sqrt(15) / 10
+  const int i = D == 2 ? ij : ij / 3, j = ij % 3;
+  const double u = gl_x(i), w1 = 1.0 - u, v = D == 2 ? 0.0 : gl_x(j);
+  const double vv = v * w1, w2 = w1 * (1.0 - v);
+  const double c = (D == 2 ? 2.0 * gl_w(i) * w1 : 6.0 * gl_w(i) * gl_w(j) * w1 * w2) * gl_w(0);
+  return {u, vv, w2, c, c * u, c * vv, 0.5 * c * w2, c * w2 * h};
+}
+struct FhLines {
+  FhLine line[9];
+};
+template <int D>
+constexpr FhLines fh_lines() {
+  FhLines t{};
+  for (int q = 0; q < (D == 2 ? 3 : 9); ++q) t.line[q] = fh_line<D>(q);
+  return t;
+}
+__constant__ FhLines c_fh_lines[2] = {fh_lines<2>(), fh_lines<3>()};
 
 // eload as k_cell_loads, f' of the Flory-Huggins energy by the product rule.  The terms of f' that are
 // linear in the concentrations are integrated exactly (the rule is exact for them); the rule takes the
 // logarithms' part
 //   g_p = ln phi_p / N_p - ln phi_s / N_s,  g_n = ln phi_n / N_n - ln phi_s / N_s,
-// along the innermost direction the concentrations are a + t b and the hat functions 1 and t, so a
-// point costs three FMAs for the concentrations, three logarithms, three for g and four to
-// accumulate (about 38 FP64 instructions against 144 with the hat functions tabulated per point and
-// CUDA's log: 19.5 ms on 128 x 128 x 32 cells, 7.1 ms now).  A thread takes a simplex, a block 32 cells at a time;
-// the simplices' corner values are added in shared memory in simplex order.  Three blocks per SM
-// with the tables in shared memory.
+// along the innermost direction the concentrations are a + t b and the hat functions 1 and t.  With the
+// logarithms L_0, L_1, L_2 of one concentration at a line's points, E = L_0 + L_2, A = E + 8/5 L_1 (5/18 A is
+// the line's integral) and B = L_2 - L_0 (its moment is 5/18 (A / 2 + h B), h = sqrt(15) / 10): 105 FP64
+// instructions for a line's nine logarithms against 121 with the weights applied point by point (144 a point
+// with the hat functions tabulated and CUDA's log).  128 x 128 x 32 cells: 19.5 ms at first, 7.1 ms point by point
+// and with seven-instruction logarithms, 5.9 ms now.  The three concentrations are summed apart and
+// combined at the end.  A thread takes a simplex, a block 32 cells at a time; the simplices' corner values
+// are added in shared memory in simplex order.  Three blocks per SM with the tables in shared memory.
 template <int D>
 constexpr int fh_smem() {
   return (int)(sizeof(LogTables) + sizeof(double2) * CellSimplices<D>::NT * (D + 1) * 32);
@@ -891,56 +924,39 @@ __global__ void __launch_bounds__(32 * CellSimplices<D>::NT) k_cell_loads_fh(con
         P[a] = pp[(size_t)ld * ev[a]];
         Q[a] = pn[(size_t)ld * ev[a]];
       }
-      double Gp[D + 1], Gn[D + 1];  // [0]: against 1, [a]: against lambda_a
+      double Lp[D + 1], Ln[D + 1], Ls[D + 1];  // the logarithms' integrals, [0]: against 1, [a]: against lambda_a
 #pragma unroll
-      for (int a = 0; a <= D; ++a) Gp[a] = Gn[a] = 0.0;
-      const auto line = [&](double p0, double dp, double n0, double dn, double (&s)[4]) {
-        // s = sums over the innermost points of w g_p, w x g_p, w g_n, w x g_n
+      for (int a = 0; a <= D; ++a) Lp[a] = Ln[a] = Ls[a] = 0.0;
+#pragma unroll 1
+      for (int ij = 0; ij < (D == 2 ? 3 : 9); ++ij) {
+        const FhLine& q = c_fh_lines[D - 2].line[ij];
+        double p0 = fma(q.u, P[1] - P[0], P[0]), n0 = fma(q.u, Q[1] - Q[0], Q[0]);
+        if (D == 3) {
+          p0 = fma(q.vv, P[2] - P[0], p0);
+          n0 = fma(q.vv, Q[2] - Q[0], n0);
+        }
+        const double dp = q.w2 * (P[D] - P[0]), dn = q.w2 * (Q[D] - Q[0]);
         const double s0 = 1.0 - p0 - n0, ds = -(dp + dn);
-        s[0] = s[1] = s[2] = s[3] = 0.0;
+        const auto sums = [&](double v0, double dv, double (&G)[D + 1]) {
+          const double l0 = guarded_log(fma(gl_x(0), dv, v0), F.delta, tab);
+          const double l1 = guarded_log(fma(gl_x(1), dv, v0), F.delta, tab);
+          const double l2 = guarded_log(fma(gl_x(2), dv, v0), F.delta, tab);
+          const double A = fma(1.6, l1, l0 + l2), B = l2 - l0;
+          G[0] = fma(q.c, A, G[0]);
+          G[1] = fma(q.cu, A, G[1]);
+          if (D == 3) G[2] = fma(q.cv, A, G[2]);
+          G[D] = fma(q.ca, A, fma(q.cb, B, G[D]));
+        };
+        sums(p0, dp, Lp);
+        sums(n0, dn, Ln);
+        sums(s0, ds, Ls);
+      }
+      double Gp[D + 1], Gn[D + 1];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const double x = gl_x(k), w = gl_w(k);
-          const double p = fma(x, dp, p0), n = fma(x, dn, n0), ps = fma(x, ds, s0);
-          const double ls = guarded_log(ps, F.delta, tab) * F.inv_ns;
-          const double gp = fma(guarded_log(p, F.delta, tab), F.inv_np, -ls);
-          const double gn = fma(guarded_log(n, F.delta, tab), F.inv_nn, -ls);
-          s[0] = fma(w, gp, s[0]);
-          s[1] = fma(w * x, gp, s[1]);
-          s[2] = fma(w, gn, s[2]);
-          s[3] = fma(w * x, gn, s[3]);
-        }
-      };
-      if (D == 2) {
-#pragma unroll 1
-        for (int i = 0; i < 3; ++i) {
-          const double u = gl_x(i), w1 = 1.0 - u, c = 2.0 * gl_w(i) * w1;
-          double s[4];
-          line(fma(u, P[1] - P[0], P[0]), w1 * (P[2] - P[0]), fma(u, Q[1] - Q[0], Q[0]), w1 * (Q[2] - Q[0]), s);
-          Gp[0] = fma(c, s[0], Gp[0]);
-          Gp[1] = fma(c * u, s[0], Gp[1]);
-          Gp[2] = fma(c * w1, s[1], Gp[2]);
-          Gn[0] = fma(c, s[2], Gn[0]);
-          Gn[1] = fma(c * u, s[2], Gn[1]);
-          Gn[2] = fma(c * w1, s[3], Gn[2]);
-        }
-      } else {
-#pragma unroll 1
-        for (int ij = 0; ij < 9; ++ij) {
-          const double u = gl_x(ij / 3), v = gl_x(ij % 3), w1 = 1.0 - u, w2 = w1 * (1.0 - v), vv = v * w1;
-          const double c = 6.0 * gl_w(ij / 3) * gl_w(ij % 3) * w1 * w2;
-          double s[4];
-          line(fma(u, P[1] - P[0], fma(vv, P[2] - P[0], P[0])), w2 * (P[D] - P[0]),
-               fma(u, Q[1] - Q[0], fma(vv, Q[2] - Q[0], Q[0])), w2 * (Q[D] - Q[0]), s);
-          Gp[0] = fma(c, s[0], Gp[0]);
-          Gp[1] = fma(c * u, s[0], Gp[1]);
-          Gp[2] = fma(c * vv, s[0], Gp[2]);
-          Gp[D] = fma(c * w2, s[1], Gp[D]);
-          Gn[0] = fma(c, s[2], Gn[0]);
-          Gn[1] = fma(c * u, s[2], Gn[1]);
-          Gn[2] = fma(c * vv, s[2], Gn[2]);
-          Gn[D] = fma(c * w2, s[3], Gn[D]);
-        }
+      for (int a = 0; a <= D; ++a) {
+        const double ls = Ls[a] * F.inv_ns;
+        Gp[a] = fma(Lp[a], F.inv_np, -ls);
+        Gn[a] = fma(Ln[a], F.inv_nn, -ls);
       }
 #pragma unroll
       for (int a = 1; a <= D; ++a) {  // lambda_0 = 1 - the others
@@ -991,7 +1007,7 @@ static ch_status log_tables(ch_system_s* s, cudaStream_t st) {
   LogTables* t = nullptr;
   CH_TRY(s->mem.get(&t, 1));
   s->log_tables = t;
-  k_log_tables<<<blocks_for(2048), TPB, 0, st>>>(t);
+  k_log_tables<<<blocks_for(std::max(LOG_M, LOG_K)), TPB, 0, st>>>(t);
   CH_LAUNCHED();
   CH_CUDA(cudaFuncSetAttribute(k_cell_loads_fh<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, fh_smem<2>()));
   CH_CUDA(cudaFuncSetAttribute(k_cell_loads_fh<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, fh_smem<3>()));
