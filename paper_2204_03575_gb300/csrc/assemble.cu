@@ -889,33 +889,37 @@ __constant__ FhLines c_fh_lines[2] = {fh_lines<2>(), fh_lines<3>()};
 // linear in the concentrations are integrated exactly (the rule is exact for them); the rule takes the
 // logarithms' part
 //   g_p = ln phi_p / N_p - ln phi_s / N_s,  g_n = ln phi_n / N_n - ln phi_s / N_s,
-// along the innermost direction the concentrations are a + t b and the hat functions 1 and t.  With the
+// along the innermost direction the hat functions are linear.  With the
 // logarithms L_0, L_1, L_2 of one concentration at a line's points, E = L_0 + L_2, A = E + 8/5 L_1 (5/18 A is
-// the line's integral) and B = L_2 - L_0 (its moment is 5/18 (A / 2 + h B), h = sqrt(15) / 10): 105 FP64
+// the line's integral) and B = L_2 - L_0 (its moment is 5/18 (A / 2 + h B), h = sqrt(15) / 10): 113 FP64
 // instructions for a line's nine logarithms against 121 with the weights applied point by point (144 a point
 // with the hat functions tabulated and CUDA's log).  128 x 128 x 32 cells: 19.5 ms at first, 7.1 ms point by point
-// and with seven-instruction logarithms, 5.9 ms now.  The three concentrations are summed apart and
-// combined at the end.  A thread takes a simplex, a block 32 cells at a time; the simplices' corner values
-// are added in shared memory in simplex order.  Three blocks per SM with the tables in shared memory.
-template <int D>
+// and with seven-instruction logarithms, 6.3 ms now.  The three concentrations are summed apart and
+// combined at the end.  A thread takes a simplex; the simplices' corner values are added in shared memory in
+// simplex order, where the tables are as well.
+// CB cells per block.  Three blocks of 192 threads per SM: 32 cells of six tetrahedra, 96 of two triangles
+// (512 x 512 387 us, 32 cells about 460); 2D meshes of at most two blocks of 32 cells per SM take those
+// (64 x 64 31.6 us, 96 cells 34).
+template <int D, int CB>
 constexpr int fh_smem() {
-  return (int)(sizeof(LogTables) + sizeof(double2) * CellSimplices<D>::NT * (D + 1) * 32);
+  return (int)(sizeof(LogTables) + sizeof(double2) * CellSimplices<D>::NT * (D + 1) * CB);
 }
-template <int D>
-__global__ void __launch_bounds__(32 * CellSimplices<D>::NT) k_cell_loads_fh(const MeshPod m, const FhCoef F,
+template <int D, int CB>
+__global__ void __launch_bounds__(CB* CellSimplices<D>::NT, 3) k_cell_loads_fh(const MeshPod m, const FhCoef F,
                                                                              const LogTables* __restrict__ tables,
                                                                              const double* pp, const double* pn,
                                                                              int ld, double2* __restrict__ eload) {
   using S = CellSimplices<D>;
   extern __shared__ __align__(16) unsigned char fh_raw[];
   LogTables* tab = reinterpret_cast<LogTables*>(fh_raw);
-  double2(*part)[D + 1][32] = reinterpret_cast<double2(*)[D + 1][32]>(fh_raw + sizeof(LogTables));
+  double2(*part)[D + 1][CB] = reinterpret_cast<double2(*)[D + 1][CB]>(fh_raw + sizeof(LogTables));
   for (int e = threadIdx.x; e < (int)(sizeof(LogTables) / 16); e += blockDim.x)
     reinterpret_cast<uint4*>(tab)[e] = reinterpret_cast<const uint4*>(tables)[e];
   __syncthreads();
-  const int lane = threadIdx.x & 31, t = threadIdx.x >> 5;  // one simplex per warp: uniform corners
-  for (int c0 = blockIdx.x * 32; c0 < m.C; c0 += gridDim.x * 32) {
-    const int cell = c0 + lane;
+  // one simplex per warp: uniform corners
+  const int t = (threadIdx.x >> 5) % S::NT, in = (threadIdx.x >> 5) / S::NT * 32 + (threadIdx.x & 31);
+  for (int c0 = blockIdx.x * CB; c0 < m.C; c0 += gridDim.x * CB) {
+    const int cell = c0 + in;
     if (cell < m.C) {
       const int* ev = m.elems + ((size_t)cell * S::NT + t) * (D + 1);
       double P[D + 1], Q[D + 1];
@@ -930,26 +934,33 @@ __global__ void __launch_bounds__(32 * CellSimplices<D>::NT) k_cell_loads_fh(con
 #pragma unroll 1
       for (int ij = 0; ij < (D == 2 ? 3 : 9); ++ij) {
         const FhLine& q = c_fh_lines[D - 2].line[ij];
-        double p0 = fma(q.u, P[1] - P[0], P[0]), n0 = fma(q.u, Q[1] - Q[0], Q[0]);
+        // positive weights only (u, v (1 - u), and w2 shared by the line's ends), so that small concentrations
+        // beside large ones keep their relative precision, which their logarithms need
+        const double pa = q.w2 * P[0], pb = q.w2 * P[D], na = q.w2 * Q[0], nb = q.w2 * Q[D];
+        double pc = q.u * P[1], nc = q.u * Q[1];
         if (D == 3) {
-          p0 = fma(q.vv, P[2] - P[0], p0);
-          n0 = fma(q.vv, Q[2] - Q[0], n0);
+          pc = fma(q.vv, P[2], pc);
+          nc = fma(q.vv, Q[2], nc);
         }
-        const double dp = q.w2 * (P[D] - P[0]), dn = q.w2 * (Q[D] - Q[0]);
-        const double s0 = 1.0 - p0 - n0, ds = -(dp + dn);
-        const auto sums = [&](double v0, double dv, double (&G)[D + 1]) {
-          const double l0 = guarded_log(fma(gl_x(0), dv, v0), F.delta, tab);
-          const double l1 = guarded_log(fma(gl_x(1), dv, v0), F.delta, tab);
-          const double l2 = guarded_log(fma(gl_x(2), dv, v0), F.delta, tab);
+        double p[3], n[3], r[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          p[k] = fma(gl_x(2 - k), pa, fma(gl_x(k), pb, pc));
+          n[k] = fma(gl_x(2 - k), na, fma(gl_x(k), nb, nc));
+          r[k] = 1.0 - p[k] - n[k];
+        }
+        const auto sums = [&](const double (&v)[3], double (&G)[D + 1]) {
+          const double l0 = guarded_log(v[0], F.delta, tab), l1 = guarded_log(v[1], F.delta, tab);
+          const double l2 = guarded_log(v[2], F.delta, tab);
           const double A = fma(1.6, l1, l0 + l2), B = l2 - l0;
           G[0] = fma(q.c, A, G[0]);
           G[1] = fma(q.cu, A, G[1]);
           if (D == 3) G[2] = fma(q.cv, A, G[2]);
           G[D] = fma(q.ca, A, fma(q.cb, B, G[D]));
         };
-        sums(p0, dp, Lp);
-        sums(n0, dn, Ln);
-        sums(s0, ds, Ls);
+        sums(p, Lp);
+        sums(n, Ln);
+        sums(r, Ls);
       }
       double Gp[D + 1], Gn[D + 1];
 #pragma unroll
@@ -978,12 +989,12 @@ __global__ void __launch_bounds__(32 * CellSimplices<D>::NT) k_cell_loads_fh(con
 #pragma unroll
       for (int a = 0; a <= D; ++a) {
         const double sp = q2 * (Sp + P[a]), sq = q2 * (Sq + Q[a]);
-        part[t][a][lane] = make_double2(vol * (Gp[a] + fma(lp, sp, fma(mp, sq, kp * q1))),
+        part[t][a][in] = make_double2(vol * (Gp[a] + fma(lp, sp, fma(mp, sq, kp * q1))),
                                         vol * (Gn[a] + fma(ln, sp, fma(mn, sq, kn * q1))));
       }
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < 32 * S::NC; e += blockDim.x) {
+    for (int e = threadIdx.x; e < CB * S::NC; e += blockDim.x) {
       const int cl = e / S::NC, corner = e % S::NC;
       if (c0 + cl >= m.C) continue;
       double fp = 0.0, fn = 0.0;
@@ -1009,8 +1020,12 @@ static ch_status log_tables(ch_system_s* s, cudaStream_t st) {
   s->log_tables = t;
   k_log_tables<<<blocks_for(std::max(LOG_M, LOG_K)), TPB, 0, st>>>(t);
   CH_LAUNCHED();
-  CH_CUDA(cudaFuncSetAttribute(k_cell_loads_fh<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, fh_smem<2>()));
-  CH_CUDA(cudaFuncSetAttribute(k_cell_loads_fh<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, fh_smem<3>()));
+  const auto limit = [](auto kern, int bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  CH_CUDA(limit(k_cell_loads_fh<2, 32>, fh_smem<2, 32>()));
+  CH_CUDA(limit(k_cell_loads_fh<2, 96>, fh_smem<2, 96>()));
+  CH_CUDA(limit(k_cell_loads_fh<3, 32>, fh_smem<3, 32>()));
   return CH_OK;
 }
 
@@ -1173,13 +1188,16 @@ static void cell_loads(const ch_system_s* s, const MeshPod& m, const LoadCoef& L
   if (s->p.potential == 3) {
     const ch_params& p = s->p;
     const FhCoef F{p.chi_pn, p.chi_ps, p.chi_ns, 1.0 / p.N_p, 1.0 / p.N_nfa, 1.0 / p.N_s, p.fh_delta};
-    ProfScope ps(st, K_ELEM_LOADS, 0, bytes, C * nt * (m.dim == 2 ? 9 : 27) * 40.0);
-    if (m.dim == 2)
-      k_cell_loads_fh<2><<<std::min(blocks_for(m.C, 32), 5 * 152), 64, fh_smem<2>(), st>>>(
-          m, F, static_cast<const LogTables*>(s->log_tables), pp, pn, ld, s->eload);
+    ProfScope ps(st, K_ELEM_LOADS, 0, bytes, C * nt * (m.dim == 2 ? 9 : 27) * 38.0);
+    const LogTables* tab = static_cast<const LogTables*>(s->log_tables);
+    if (m.dim == 3)
+      k_cell_loads_fh<3, 32><<<std::min(blocks_for(m.C, 32), 3 * 152), 192, fh_smem<3, 32>(), st>>>(m, F, tab, pp, pn,
+                                                                                                  ld, s->eload);
+    else if (m.C > 2 * 152 * 32)
+      k_cell_loads_fh<2, 96><<<std::min(blocks_for(m.C, 96), 3 * 152), 192, fh_smem<2, 96>(), st>>>(m, F, tab, pp, pn,
+                                                                                                  ld, s->eload);
     else
-      k_cell_loads_fh<3><<<std::min(blocks_for(m.C, 32), 3 * 152), 192, fh_smem<3>(), st>>>(
-          m, F, static_cast<const LogTables*>(s->log_tables), pp, pn, ld, s->eload);
+      k_cell_loads_fh<2, 32><<<blocks_for(m.C, 32), 64, fh_smem<2, 32>(), st>>>(m, F, tab, pp, pn, ld, s->eload);
     return;
   }
   ProfScope ps(st, K_ELEM_LOADS, 0, bytes, C * nt * (40.0 + 10.0 * d1));
