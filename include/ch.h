@@ -204,7 +204,7 @@ ch_status ch_apply_A(const ch_system_t* s, const double* x, double* y, void* str
  * connection, MIS(2) aggregation, Jacobi-smoothed prolongator, Galerkin coarse operators,
  * dense inverse of the coarsest level), Chebyshev smoother bounds per level and, when
  * precision = 1, FP32 copies of every level.  On a uniform mesh (one run or a batch of them) the
- * finest level is also stored by lattice diagonals.  The preconditioner owns a non-blocking
+ * finest level is also stored as one row per class of nodes.  The preconditioner owns a non-blocking
  * CUDA stream and two events on the current device: ch_precond_apply runs step 1 of Algorithm 1
  * on that stream, forked from and joined back into the caller's stream. */
 ch_status ch_precond_setup(const ch_system_t* s, void* stream, ch_precond_t** out);

@@ -102,7 +102,7 @@ inline int red_blocks(int64_t n) {
 // still running (its blocks wait in pdl_wait() until that kernel has finished and its writes are
 // visible).  The rules every such kernel keeps:
 //   - before pdl_wait() it reads only data that no kernel of the current solve writes (operator
-//     values, diagonals: set-up results) and writes no global memory;
+//     values, class rows: set-up results) and writes no global memory;
 //   - it calls pdl_trigger(), which lets its own successor be scheduled, only after pdl_wait(), so
 //     that when the successor's blocks start every kernel but this one has finished.  Without the
 //     call the successor is scheduled when this kernel's blocks have all exited (still before
