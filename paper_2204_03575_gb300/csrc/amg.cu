@@ -1525,7 +1525,8 @@ struct TileArgs {
   const T *tab, *steps;  // the operator's table; FP64: the steps' tables
   const V2 *b, *x;
   V2 *xo, *r;
-  int nids, deg, halo;
+  double* wo;  // the last pass of an application: the result goes here in FP64, ldw values per node, not to xo
+  int ldw, nids, deg, halo;
   T invtheta, alpha[16], nbeta[16];
 };
 template <typename T>
@@ -1671,7 +1672,13 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   const auto out = [&](int t) { return col_out && in(t) && g * ROWS + t >= h && g * ROWS + t < RH - h; };
 #pragma unroll
   for (int t = 0; t < ROWS; ++t)
-    if (out(t)) a.xo[node0 + (size_t)t * tl.W] = cur[t];
+    if (out(t)) {
+      const size_t i = node0 + (size_t)t * tl.W;
+      if (!ZERO && !RES && a.wo)
+        *reinterpret_cast<double2*>(a.wo + i * a.ldw) = make_double2((double)cur[t].x, (double)cur[t].y);
+      else
+        a.xo[i] = cur[t];
+    }
   if (RES) {
     if (sizeof(T) == 8) load_row(a.tab, OWN ? edge(0) : 1, row);
     apply(a.tab, false, [&](int t, T, V2 sum) {
@@ -1969,7 +1976,7 @@ static ch_status tile_setup() {
 // the V-cycle smoother's pass on the finest level in one launch (see k_smooth_tile)
 template <typename T, bool ZERO, bool RES>
 static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename V2T<T>::t* x,
-                               typename V2T<T>::t* xo, cudaStream_t st) {
+                               typename V2T<T>::t* xo, cudaStream_t st, double* wo = nullptr, int ldw = 0) {
   using V2 = typename V2T<T>::t;
   const TilePlan& pl = RES && !ZERO ? L.plan_r : L.plan;
   const ChebCoef c = cheb_coef(h->rho[0], h->cheb_degree, h->cheb_lower);
@@ -1981,6 +1988,8 @@ static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename 
   a.x = x;
   a.xo = xo;
   a.r = L.r;
+  a.wo = wo;
+  a.ldw = ldw;
   a.nids = L.lat.L.nids;
   a.deg = h->cheb_degree;
   a.halo = pl.halo;
@@ -1990,7 +1999,8 @@ static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename 
     a.nbeta[s] = (T)-c.beta[s];
   }
   const double n = L.A.nrows, apps = pl.halo;
-  ProfScope ps(st, K_CHEB_STEP, sizeof(T) == 4, n * 2.0 * sizeof(T) * ((ZERO ? 1 : 2) + (RES ? 2 : 1)),
+  ProfScope ps(st, K_CHEB_STEP, sizeof(T) == 4,
+               n * (2.0 * sizeof(T) * ((ZERO ? 1 : 2) + (RES ? 2 : (wo ? 0 : 1))) + (wo ? 16.0 : 0.0)),
                apps * (2.0 * L.A.nnz + 4.0 * n));
   const int threads = TileShape<T>::RW * pl.groups, smem = tile_smem<T>(pl.groups);
   if constexpr (sizeof(T) == 4) {
@@ -2065,9 +2075,18 @@ static ch_status semi_iteration(LevelT<T_>& L, int dim, int steps, typename V2T<
 }
 
 // one V-cycle at level l on L[l].b; result in *xres (L[l].x or L[l].x2).  zero_guess: as smooth_coef
+// the level's smoothing passes run as tiles
+template <typename T>
+static bool tiled(const LevelT<T>& L) {
+  return L.plan.ntiles > 0 && L.plan_r.ntiles > 0;
+}
+
+// (wo, ldw): where the finest level is tiled, the last pass stores the result there in FP64 (see TileArgs) and
+// no conversion follows: Algorithm 1, us per application, 512 x 512 182.4 -> 180.0, 64 runs 940 -> 921
 template <typename T>
 static ch_status vcycle(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l,
-                        int zero_guess, typename V2T<T>::t** xres, cudaStream_t st) {
+                        int zero_guess, typename V2T<T>::t** xres, cudaStream_t st, double* wo = nullptr,
+                        int ldw = 0) {
   using V2 = typename V2T<T>::t;
   LevelT<T>& L = Ls[l];
   const int n = L.A.nrows;
@@ -2082,7 +2101,7 @@ static ch_status vcycle(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l,
   V2* x = *xres;
   LevelT<T>& C = Ls[l + 1];
   const int nc = C.A.nrows;
-  const bool tiles = l == 0 && L.plan.ntiles > 0 && L.plan_r.ntiles > 0;
+  const bool tiles = l == 0 && tiled(L);
   if (tiles) {
     V2* to = x == L.x ? L.x2 : L.x;
     if (zero_guess) launch_smooth_tile<T, true, true>(h, L, nullptr, to, st);
@@ -2117,7 +2136,7 @@ static ch_status vcycle(Hierarchy* h, LevelT<T>* Ls, const T* cinv, int l,
   CH_LAUNCHED();
   if (tiles) {
     V2* to = x == L.x ? L.x2 : L.x;
-    launch_smooth_tile<T, false, false>(h, L, x, to, st);
+    launch_smooth_tile<T, false, false>(h, L, x, to, st, wo, ldw);
     CH_LAUNCHED();
     x = to;
   } else {
@@ -2240,9 +2259,10 @@ static ch_status precond_t(ch_precond_s* pc, std::vector<LevelT<T>>& LM, std::ve
     if (p.precond_M == 1) {
       CH_TRY(semi_iteration<T>(L, pc->sys->mesh->dim, semi_steps(p), &xr, sm));
     } else {
-      for (int c = 0; c < p.vcycles_M; ++c) CH_TRY(vcycle<T>(pc->hM, LM.data(), cinvM, 0, c == 0 ? zg : 0, &xr, sm));
+      for (int c = 0; c < p.vcycles_M; ++c)
+        CH_TRY(vcycle<T>(pc->hM, LM.data(), cinvM, 0, c == 0 ? zg : 0, &xr, sm, c + 1 == p.vcycles_M ? w : nullptr, 4));
     }
-    {
+    if (p.precond_M == 1 || !tiled(L)) {
       ProfScope ps(sm, K_VSTORE, sizeof(T) == 4, n * (16.0 + 2.0 * sizeof(T)), 0.0);
       launch_k(L.pdl, k_store2<T, V2>, blocks_for(n), TPB, 0, sm, n, xr, w, 4);
     }
@@ -2264,8 +2284,9 @@ static ch_status precond_t(ch_precond_s* pc, std::vector<LevelT<T>>& LM, std::ve
     }
     CH_LAUNCHED();
     xr = L.x;  // the first solve's result now lives in L.b as M x; start afresh
-    for (int c = 0; c < p.vcycles_H; ++c) CH_TRY(vcycle<T>(pc->hH, LH.data(), cinvH, 0, c == 0, &xr, st));
-    {
+    for (int c = 0; c < p.vcycles_H; ++c)
+      CH_TRY(vcycle<T>(pc->hH, LH.data(), cinvH, 0, c == 0, &xr, st, c + 1 == p.vcycles_H ? w + 2 : nullptr, 4));
+    if (!tiled(L)) {
       ProfScope ps(st, K_VSTORE, sizeof(T) == 4, n * (16.0 + 2.0 * sizeof(T)), 0.0);
       launch_k(L.pdl, k_store2<T, V2>, blocks_for(n), TPB, 0, st, n, xr, w + 2, 4);
     }

@@ -43,3 +43,17 @@ def test_tiled_passes_equal_the_oracle_vcycle(lib, kw, which, precision):
                 want = o.vcycle(levels, b[:, k]) if want is None else o.vcycle(levels, b[:, k], x0=want.copy())
             err = np.abs(got[:, k] - want).max() / np.abs(want).max()
             assert err <= TOL[precision], (kw, which, k, cycles, err)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("kw", [dict(nx=57, ny=1), dict(nx=66, ny=53), dict(nx=20, ny=20, vcycles_M=2)], ids=str)
+def test_last_pass_stores_the_application(lib, kw, precision):
+    """Algorithm 1's first half is M's V-cycles alone: the tile pass that stores its result in FP64 and the cycle
+    that a conversion follows are the same arithmetic, bit for bit."""
+    p = lib.Params(precision=precision, coarse_max=32, **kw)
+    system = lib.System(lib.Mesh(p), p)
+    pc = lib.Precond(system)
+    v = torch.from_numpy(np.random.default_rng(8).standard_normal((system.n, 4))).cuda()
+    w = pc.apply(v)
+    assert torch.equal(w[:, :2], pc.vcycle(0, v[:, :2].contiguous(), kw.get("vcycles_M", 1)))
+    assert torch.isfinite(w).all()
