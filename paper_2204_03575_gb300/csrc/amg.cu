@@ -32,9 +32,10 @@ template <> struct V2T<float> { using t = float2; };
 // Fine-level operator of a uniform mesh in lattice form: node i's neighbours sit at i + lat_off(d)
 // and its row is the table row of its class id (Lattice): nd values in ascending direction, i.e. in
 // CSR column order (zero where the class has no such neighbour: the clamped index is then read but
-// multiplied by zero), padded to `ts` with the class's factor in slot nd (LatTab).  The assembled
-// rows of a class agree to the rounding of the node coordinates (checked at set-up, below 2^-36 of
-// the diagonal), and the table holds those of the class's representative node.
+// multiplied by zero), padded to `ts` with the class's factor in slot nd.  FP64 V-cycles take the classes
+// by cell widths, whose rows are the assembled ones bit for bit; FP32 V-cycles the few classes by position
+// where the rows of a class agree to 2^-36 of the diagonal, far below FP32's rounding (checked at set-up),
+// or else those by widths.
 template <typename T>
 struct LatOp {
   int nd = 0;                      // 7 (2D) or 15 (3D); 0: not structured, use the CSR form
@@ -74,7 +75,7 @@ template <typename T>
 struct LevelT {
   Csr<T> A, P, R;
   Csr<T> RB;  // [R, -R A] over the stacked (b, x): the coarse right-hand side without the residual
-  LatOp<T> lat;                        // level 0 of a structured mesh
+  LatOp<T> lat;                        // level 0 of a box mesh
   TilePlan plan, plan_r;               // ... its smoothing passes as single launches, and those from a
                                        // given iterate that also form the residual
   int tprA = 1, tprP = 1, tprR = 1;  // lanes per row of the SpMV-type kernels (autotuned)
@@ -787,25 +788,26 @@ __global__ void k_lat_table(Csr<double> A, Lattice L, int nd, int ts, double* ta
   row[nd] = 1.0 / row[nd / 2];
 }
 
-// bad = 1 if a stored entry lies off its run's lattice stencil or away from its class's table value
-__global__ void k_lat_check(Csr<double> A, Lattice L, int nd, int ts, const double* tab, int* bad) {
+// bad = 1 if a stored entry lies off its run's lattice stencil or further than `rel` of the diagonal from its
+// class's table value
+__global__ void k_lat_check(Csr<double> A, Lattice L, int nd, int ts, const double* tab, double rel, int* bad) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.nrows) return;
   const int id = lat_id(L, i);
   const int2 w = L.wh[id];
   const double* row = tab + (size_t)id * ts;
-  const double tol = 0x1p-36 * fabs(row[nd / 2]);
+  const double tol = rel * fabs(row[nd / 2]);
   bool ok = true;
-  double seen = 0.0, sum = 0.0;
+  unsigned seen = 0;
   for (int q = A.rowptr[i]; q < A.rowptr[i + 1]; ++q) {
     int at = -1;
     for (int d = 0; d < nd; ++d)
       if (lat_off(nd, d, w.x, w.y) == A.col[q] - i) at = d;
     if (at < 0 || !(fabs(A.val[q] - row[at]) <= tol)) ok = false;
-    if (at >= 0) seen += fabs(row[at]);
+    if (at >= 0) seen |= 1u << at;
   }
-  for (int d = 0; d < nd; ++d) sum += fabs(row[d]);
-  if (!(fabs(sum - seen) <= tol)) ok = false;  // the class has an entry that the row lacks
+  for (int d = 0; d < nd; ++d)
+    if (!(seen >> d & 1) && row[d] != 0.0) ok = false;  // the class has an entry that the row lacks
   if (!ok) *bad = 1;
 }
 
@@ -841,9 +843,9 @@ __global__ void k_lat_steps(const double* tab, int nids, int nd, int ts, StepCoe
 
 // The lattice form's FP64 table of A where every row fits it (tab stays null where not: the level
 // then keeps the CSR form).
-static ch_status lat_build(const Csr<double>& A, const Lattice* L, Alloc& mem, double** tab, cudaStream_t st) {
+static ch_status lat_build(const Csr<double>& A, const Lattice* L, double rel, Alloc& mem, double** tab,
+                           cudaStream_t st) {
   *tab = nullptr;
-  if (!L || (L->dim != 2 && L->dim != 3)) return CH_OK;
   const int nd = L->dim == 2 ? 7 : 15, ts = nd + 1;
   Alloc tmp;
   int* bad = nullptr;
@@ -852,7 +854,7 @@ static ch_status lat_build(const Csr<double>& A, const Lattice* L, Alloc& mem, d
   CH_TRY(mem.get(&t, (size_t)L->nids * ts));
   CH_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), st));
   k_lat_table<<<blocks_for(L->nids), TPB, 0, st>>>(A, *L, nd, ts, t);
-  k_lat_check<<<blocks_for(A.nrows), TPB, 0, st>>>(A, *L, nd, ts, t, bad);
+  k_lat_check<<<blocks_for(A.nrows), TPB, 0, st>>>(A, *L, nd, ts, t, rel, bad);
   CH_LAUNCHED();
   int hb = 0;
   CH_CUDA(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -925,7 +927,7 @@ static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* o
     const ch_params& p = m->runs[r];
     for (int y = 0; y <= p.ny; y += th)
       for (int x = 0; x <= p.nx; x += tw)
-        tiles.push_back({m->run_off[r], p.nx + 1, p.ny + 1, x, y, (int)r * m->lat.ncls});
+        tiles.push_back({m->run_off[r], p.nx + 1, p.ny + 1, x, y, (int)r * m->pos.ncls});
   }
   LatTile* d = nullptr;
   CH_TRY(mem.get(&d, tiles.size()));
@@ -996,9 +998,15 @@ static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, const ch_para
     w.pdl = h->pdl;
   }
 
-  // the fine level of a uniform mesh in lattice form
-  const Lattice* lat = &mesh->lat;
-  CH_TRY(lat_build(h->A[0], lat, h->mem, &h->lat_tab, st));
+  // the fine level in lattice form (LatOp)
+  constexpr bool F32 = sizeof(T) == 4;
+  const Lattice* lat = F32 ? &mesh->pos : &mesh->lat;
+  CH_TRY(lat_build(h->A[0], lat, F32 ? 0x1p-36 : 0.0, h->mem, &h->lat_tab, st));
+  const bool by_position = F32 && h->lat_tab;
+  if (F32 && !h->lat_tab) {
+    lat = &mesh->lat;
+    CH_TRY(lat_build(h->A[0], lat, 0.0, h->mem, &h->lat_tab, st));
+  }
   if (h->lat_tab) {
     LatOp<T>& op = L[0].lat;
     op.nd = lat->dim == 2 ? 7 : 15;
@@ -1021,7 +1029,7 @@ static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, const ch_para
       }
     }
     CH_LAUNCHED();
-    if (lat->dim == 2 && h->nlev > 1) {
+    if (lat->dim == 2 && h->nlev > 1 && (by_position || !F32)) {
       CH_TRY(tile_setup<T>());
       CH_TRY(tile_plan<T>(mesh, h->cheb_degree, h->mem, &L[0].plan, st));
       CH_TRY(tile_plan<T>(mesh, h->cheb_degree + 1, h->mem, &L[0].plan_r, st));
@@ -1407,7 +1415,7 @@ __device__ __forceinline__ LatRow<T, ND> lat_row(const LatOp<T>& D, const T* __r
   const int id = lat_id(D.L, i);
   r.W = D.L.W;
   r.WH = D.L.WH;
-  if (D.L.nids > D.L.ncls) {
+  if (D.L.multi) {
     const int2 w = D.L.wh[id];
     r.W = w.x;
     r.WH = w.y;
@@ -1526,6 +1534,7 @@ struct TileArgs {
   const V2 *b, *x;
   V2 *xo, *r;
   double* wo;  // the last pass of an application: the result goes here in FP64, ldw values per node, not to xo
+  Lattice L;   // FP64: the nodes' class ids
   int ldw, nids, deg, halo;
   T invtheta, alpha[16], nbeta[16];
 };
@@ -1557,10 +1566,10 @@ __device__ __forceinline__ double2 fma2(double c, double2 x, double2 a) {
 }
 __device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 
-// One block's tile.  EDGE: the region reaches the mesh's boundary (or past it), so nodes carry their own
-// class row (a thread's one node in FP64 for good; in FP32 a column's, and nodes of the first and last mesh
-// row load theirs) and those outside the mesh stay zero; the other tiles (all but the rim) keep one
-// row in registers and test nothing.
+// One block's tile.  FP64: a thread's one node has its class's row (by cell widths).  FP32 (classes by
+// position): a thread's nodes share the column's row, and those of the first and last mesh row load theirs.
+// EDGE: the region reaches the mesh's boundary (or past it), and nodes outside the mesh stay zero; the other
+// tiles (all but the rim) test nothing.
 template <typename T, typename V2, bool ZERO, bool RES, bool EDGE>
 __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatTile& tl, V2* buf) {
   constexpr int RW = TileShape<T>::RW, ROWS = TileShape<T>::ROWS, ST = RW + 2;
@@ -1570,19 +1579,20 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   const bool col_in = !EDGE || (x >= 0 && x < tl.W);
   const int cx = !EDGE ? 1 : (x <= 0 ? 0 : (x >= tl.W - 1 ? 2 : 1));
   const auto in = [&](int t) { return !EDGE || (col_in && (unsigned)(y0 + t) < (unsigned)tl.H); };
+  const size_t node0 = (size_t)tl.off + (size_t)((long long)y0 * tl.W) + x;  // (used only inside the mesh)
+  constexpr bool OWN = ROWS == 1;  // the thread has one node, with its own row
+  const int own = OWN && in(0) ? lat_id(a.L, (int)node0) : 0;
   const auto load_row = [&](const T* tab, int cy, T (&o)[8]) {
     constexpr int NQ = 8 * (int)sizeof(T) / 16;
-    const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)(tl.id0 + cx + 3 * cy) * 8);
+    const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)(OWN ? own : tl.id0 + cx + 3 * cy) * 8);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) reinterpret_cast<uint4*>(o)[q] = src[q];
   };
   const auto edge = [&](int t) { return y0 + t == 0 ? 0 : (y0 + t == tl.H - 1 ? 2 : 1); };
   T row[8];
-  constexpr bool OWN = EDGE && ROWS == 1;  // the node's class row is the thread's
-  load_row(a.tab, OWN ? edge(0) : 1, row);
+  load_row(a.tab, 1, row);
   pdl_wait();
   pdl_trigger_t<T>();
-  const size_t node0 = (size_t)tl.off + (size_t)((long long)y0 * tl.W) + x;  // (used only inside the mesh)
   V2 nb[ROWS], cur[ROWS], prev[ROWS];  // -b, the iterate and the one before it
 #pragma unroll
   for (int t = 0; t < ROWS; ++t) {
@@ -1647,7 +1657,7 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   for (int s = ZERO ? 1 : 0; s < a.deg; ++s) {
     const T alpha = a.alpha[s], nbeta = a.nbeta[s];
     const T* tab = sizeof(T) == 8 ? a.steps + (size_t)s * a.nids * 8 : a.tab;
-    if (sizeof(T) == 8) load_row(tab, OWN ? edge(0) : 1, row);
+    if (sizeof(T) == 8) load_row(tab, 1, row);
     const bool has_prev = s > 0;
     // (before the first step of a pass from zero the iterate was zero, as prev starts out)
     apply(tab, true, [&](int t, T last, V2 sum) {
@@ -1680,7 +1690,7 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
         a.xo[i] = cur[t];
     }
   if (RES) {
-    if (sizeof(T) == 8) load_row(a.tab, OWN ? edge(0) : 1, row);
+    if (sizeof(T) == 8) load_row(a.tab, 1, row);
     apply(a.tab, false, [&](int t, T, V2 sum) {
       if (out(t)) a.r[node0 + (size_t)t * tl.W] = mk2<T, V2>(-nb[t].x - sum.x, -nb[t].y - sum.y);
     });
@@ -1990,6 +2000,7 @@ static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename 
   a.r = L.r;
   a.wo = wo;
   a.ldw = ldw;
+  a.L = L.lat.L;
   a.nids = L.lat.L.nids;
   a.deg = h->cheb_degree;
   a.halo = pl.halo;

@@ -155,18 +155,104 @@ __global__ void k_facet_vol(const double* X, const int* f, int F, double* vol) {
   }
 }
 
-// class id of every node of one run (Lattice)
-__global__ void k_lat_ids(ch_params p, int N, int node_off, int base, int id32, void* out) {
+// class id of every node of one run (Lattice) from the classes along its axes (nx + 1, ny + 1 and in 3D
+// nz + 1 of them), ncx and ncy of which are distinct on the first two
+__global__ void k_lat_ids(ch_params p, int N, int node_off, const int* axes, int ncx, int ncy, int base, int id32,
+                          void* out) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
   const int i = n % (p.nx + 1), j = (n / (p.nx + 1)) % (p.ny + 1);
-  int c = (i == 0 ? 0 : (i == p.nx ? 2 : 1)) + 3 * (j == 0 ? 0 : (j == p.ny ? 2 : 1));
-  if (p.dim == 3) {
-    const int k = n / ((p.nx + 1) * (p.ny + 1));
-    c += 9 * (k == 0 ? 0 : (k == p.nz ? 2 : 1));
-  }
+  int c = axes[i] + ncx * axes[p.nx + 1 + j];
+  if (p.dim == 3) c += ncx * ncy * axes[p.nx + p.ny + 2 + n / ((p.nx + 1) * (p.ny + 1))];
   if (id32) static_cast<int*>(out)[node_off + n] = base + c;
   else static_cast<uint16_t*>(out)[node_off + n] = (uint16_t)(base + c);
+}
+
+// The classes of one axis (appended to cls, one per node) and a node of each: by position, or by the widths
+// of the cells on either side, computed as k_mesh_nodes and the element matrices do (volatile: no fused
+// multiply-add, the coordinates are rounded; the set-up checks find a difference).
+static std::vector<int> axis_classes(int cells, double length, bool widths, std::vector<int>& cls) {
+  if (!widths) {
+    for (int i = 0; i <= cells; ++i) cls.push_back(i == 0 ? 0 : (i == cells ? 2 : 1));
+    return {0, cells / 2, cells};
+  }
+  std::vector<int> rep;
+  std::vector<double> left, right;
+  const double h = length / cells;
+  double before = 0.0;
+  size_t at = 0;
+  for (int i = 0; i <= cells; ++i) {
+    volatile double x0 = i * h, x1 = (i + 1) * h;
+    const double after = i < cells ? x1 - x0 : 0.0;
+    const auto is = [&](size_t q) { return left[q] == before && right[q] == after; };
+    if (at >= rep.size() || !is(at)) {  // (mostly the class of the node before)
+      for (at = 0; at < rep.size() && !is(at); ++at) {}
+      if (at == rep.size()) {
+        rep.push_back(i);
+        left.push_back(before);
+        right.push_back(after);
+      }
+    }
+    cls.push_back((int)at);
+    before = after;
+  }
+  return rep;
+}
+
+static ch_status lattice_build(ch_mesh_s* m, bool widths, Lattice* L, cudaStream_t st) {
+  const int R = (int)m->runs.size(), d = m->dim;
+  struct Run {
+    size_t axes;
+    int ncx, ncy, base;
+  };
+  std::vector<Run> runs(R);
+  std::vector<int> cls, rep;
+  std::vector<int2> wh;
+  int64_t nids = 0;
+  for (int r = 0; r < R; ++r) {
+    const ch_params& p = m->runs[r];
+    const size_t axes = cls.size();
+    const std::vector<int> rx = axis_classes(p.nx, p.Lx, widths, cls), ry = axis_classes(p.ny, p.Ly, widths, cls);
+    const std::vector<int> rz = d == 3 ? axis_classes(p.nz, p.Lz, widths, cls) : std::vector<int>{0};
+    runs[r] = {axes, (int)rx.size(), (int)ry.size(), (int)nids};
+    nids += (int64_t)rx.size() * ry.size() * rz.size();
+    if (nids > 2000000000LL) {
+      set_error("batched mesh too large for int32 indexing");
+      return CH_ERR_ARG;
+    }
+    const int W = p.nx + 1, WH = W * (p.ny + 1);
+    for (int z : rz)
+      for (int y : ry)
+        for (int x : rx) {
+          wh.push_back(make_int2(W, WH));
+          rep.push_back(m->run_off[r] + x + W * y + WH * z);
+        }
+  }
+  L->dim = d;
+  L->ncls = widths ? 0 : (d == 2 ? 9 : 27);
+  L->nids = (int)nids;
+  L->multi = R > 1;
+  L->W = m->runs[0].nx + 1;
+  L->WH = L->W * (m->runs[0].ny + 1);
+  L->id32 = L->nids > 65536;
+  uint8_t* ids = nullptr;
+  int* axes = nullptr;
+  CH_TRY(m->mem.get(&ids, (size_t)m->N * (L->id32 ? 4 : 2)));
+  CH_TRY(m->mem.get(&axes, cls.size()));
+  CH_TRY(m->mem.get(&L->wh, wh.size()));
+  CH_TRY(m->mem.get(&L->rep, rep.size()));
+  L->id = ids;
+  CH_CUDA(cudaMemcpyAsync(axes, cls.data(), sizeof(int) * cls.size(), cudaMemcpyHostToDevice, st));
+  CH_CUDA(cudaMemcpyAsync(L->wh, wh.data(), sizeof(int2) * wh.size(), cudaMemcpyHostToDevice, st));
+  CH_CUDA(cudaMemcpyAsync(L->rep, rep.data(), sizeof(int) * rep.size(), cudaMemcpyHostToDevice, st));
+  for (int r = 0; r < R; ++r) {
+    const int n = m->run_off[r + 1] - m->run_off[r];
+    k_lat_ids<<<blocks_for(n), TPB, 0, st>>>(m->runs[r], n, m->run_off[r], axes + runs[r].axes, runs[r].ncx,
+                                             runs[r].ncy, runs[r].base, L->id32, L->id);
+  }
+  CH_LAUNCHED();
+  CH_CUDA(cudaStreamSynchronize(st));  // the host arrays end here
+  return CH_OK;
 }
 
 // counts of one box mesh
@@ -215,35 +301,8 @@ ch_status mesh_build(ch_mesh_s* m, cudaStream_t st) {
   CH_TRY(m->mem.get(&m->tvol, (size_t)m->Ft));
   CH_TRY(m->mem.get(&m->node_run, (size_t)m->N));
   CH_TRY(m->mem.get(&m->run_off_d, (size_t)R + 1));
-  Lattice& L = m->lat;
-  L.dim = d;
-  L.ncls = d == 2 ? 9 : 27;
-  if ((int64_t)R * L.ncls > 2000000000LL) {
-    set_error("batched mesh too large for int32 indexing");
-    return CH_ERR_ARG;
-  }
-  L.nids = R * L.ncls;
-  L.id32 = L.nids > 65536;
-  L.W = m->runs[0].nx + 1;
-  L.WH = L.W * (m->runs[0].ny + 1);
-  uint8_t* ids = nullptr;
-  CH_TRY(m->mem.get(&ids, (size_t)m->N * (L.id32 ? 4 : 2)));
-  L.id = ids;
-  CH_TRY(m->mem.get(&L.wh, (size_t)L.nids));
-  CH_TRY(m->mem.get(&L.rep, (size_t)L.nids));
-  std::vector<int2> wh(L.nids);
-  std::vector<int> rep(L.nids);
-  for (int r = 0; r < R; ++r) {
-    const ch_params& p = m->runs[r];
-    const int W = p.nx + 1, WH = W * (p.ny + 1), nz = d == 3 ? p.nz : 0;
-    for (int c = 0; c < L.ncls; ++c) {
-      const auto pick = [](int cls, int cells) { return cls == 0 ? 0 : (cls == 1 ? cells / 2 : cells); };
-      const int x = pick(c % 3, p.nx), y = pick(c / 3 % 3, p.ny), z = d == 3 ? pick(c / 9, nz) : 0;
-      wh[(size_t)r * L.ncls + c] = make_int2(W, WH);
-      rep[(size_t)r * L.ncls + c] = m->run_off[r] + x + W * y + WH * z;
-    }
-  }
-  CH_CUDA(cudaMemcpyAsync(L.wh, wh.data(), sizeof(int2) * L.nids, cudaMemcpyHostToDevice, st));
+  CH_TRY(lattice_build(m, true, &m->lat, st));
+  CH_TRY(lattice_build(m, false, &m->pos, st));
   std::vector<CellGrid> grid(R);
   for (int r = 0; r < R; ++r) {
     const ch_params& p = m->runs[r];
@@ -251,7 +310,6 @@ ch_status mesh_build(ch_mesh_s* m, cudaStream_t st) {
   }
   CH_TRY(m->mem.get(&m->cell_grid, (size_t)R));
   CH_CUDA(cudaMemcpyAsync(m->cell_grid, grid.data(), sizeof(CellGrid) * R, cudaMemcpyHostToDevice, st));
-  CH_CUDA(cudaMemcpyAsync(L.rep, rep.data(), sizeof(int) * L.nids, cudaMemcpyHostToDevice, st));
   for (int r = 0; r < R; ++r) {
     const ch_params& p = m->runs[r];
     const int n = m->run_off[r + 1] - m->run_off[r], e = eoff[r + 1] - eoff[r], f = foff[r + 1] - foff[r];
@@ -260,7 +318,6 @@ ch_status mesh_build(ch_mesh_s* m, cudaStream_t st) {
     k_mesh_facets<<<blocks_for(f), TPB, 0, st>>>(p, f, m->run_off[r], m->bot + (size_t)foff[r] * d,
                                                   m->top + (size_t)foff[r] * d);
     k_fill_int<<<blocks_for(n), TPB, 0, st>>>(m->node_run + m->run_off[r], n, r);
-    k_lat_ids<<<blocks_for(n), TPB, 0, st>>>(p, n, m->run_off[r], r * L.ncls, L.id32, L.id);
   }
   CH_LAUNCHED();
   CH_CUDA(cudaMemcpyAsync(m->run_off_d, m->run_off.data(), sizeof(int) * (R + 1), cudaMemcpyHostToDevice, st));
@@ -519,7 +576,7 @@ static ch_status substrate_weights(const ch_mesh_s* m, ch_system_s* s, cudaStrea
 // ---------------------------------------------------------------- the operator's lattice table
 template <int ND>
 __global__ void k_lat_operator(int nids, const int* rep, const int2* wh, const int* rowptr, const int* col,
-                               const double* valM, const double* valK, double a, double c, double* tab) {
+                               const double* valM, const double* valK, double* tab) {
   using X = LatAxes<ND>;
   const int id = blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= nids) return;
@@ -531,25 +588,24 @@ __global__ void k_lat_operator(int nids, const int* rep, const int2* wh, const i
     for (int d = 0; d < ND; ++d)
       if (lat_off(ND, d, w.x, w.y) == col[q] - i) {
         t[d] = valM[q];
-        t[ND + d] = -c * valM[q];
-        if (X::index(d) >= 0) t[2 * ND + X::index(d)] = a * valK[q];
+        if (X::index(d) >= 0) t[ND + X::index(d)] = valK[q];
       }
 }
 
-// bad = 1 where a row's entries differ from its class's table by more than 2^-36 of its diagonal, or K
-// has an entry off the axes
+// bad = 1 where a row is not its class's table row bit for bit, apart from K's entries off the axes: zero but
+// for the rounding of the products in the tetrahedra's gradients (2^-50 of the diagonal at most)
 template <int ND>
 __global__ void k_lat_operator_check(Lattice L, int N, const int* rowptr, const int* col, const double* valM,
-                                     const double* valK, double a, const double* tab, int* bad) {
+                                     const double* valK, const double* tab, int* bad) {
   using X = LatAxes<ND>;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   const int id = lat_id(L, i);
   const int2 w = L.wh[id];
   const double* t = tab + (size_t)id * X::TS;
-  const double tm = 0x1p-36 * fabs(t[ND / 2]), tk = 0x1p-36 * fabs(t[2 * ND + X::index(ND / 2)]);
+  const double tk = 0x1p-50 * fabs(t[ND + X::index(ND / 2)]);
   bool ok = true;
-  double seen = 0.0, sum = 0.0;
+  unsigned seen = 0;
   for (int q = rowptr[i]; q < rowptr[i + 1]; ++q) {
     int at = -1;
     for (int d = 0; d < ND; ++d)
@@ -561,12 +617,13 @@ __global__ void k_lat_operator_check(Lattice L, int N, const int* rowptr, const 
     int e = -1;
     for (int d = 0; d < ND; ++d)
       if (d == at) e = X::index(d);
-    const double k = e >= 0 ? t[2 * ND + e] : 0.0;
-    if (!(fabs(valM[q] - t[at]) <= tm) || !(fabs(a * valK[q] - k) <= tk)) ok = false;
-    seen += fabs(t[at]);
+    // (an entry whose upper word is zero would pass for an absent neighbour)
+    if (!(valM[q] == t[at]) || __double2hiint(t[at]) == 0) ok = false;
+    if (e >= 0 ? !(valK[q] == t[ND + e]) : !(fabs(valK[q]) <= tk)) ok = false;
+    seen |= 1u << at;
   }
-  for (int d = 0; d < ND; ++d) sum += fabs(t[d]);
-  if (!(fabs(sum - seen) <= tm)) ok = false;  // the class has an entry that the row lacks
+  for (int d = 0; d < ND; ++d)
+    if (!(seen >> d & 1) && t[d] != 0.0) ok = false;  // the class has an entry that the row lacks
   if (!ok) *bad = 1;
 }
 
@@ -576,17 +633,17 @@ static ch_status lattice_operator(const ch_mesh_s* m, ch_system_s* s, int* bad, 
   double* tab = nullptr;
   CH_TRY(s->mem.get(&tab, (size_t)L.nids * ts));
   s->lat.L = L;
+  s->lat.a = s->a;
+  s->lat.c = s->c;
   s->lat.tab = tab;
   if (m->dim == 2) {
     k_lat_operator<7><<<blocks_for(L.nids, 64), 64, 0, st>>>(L.nids, L.rep, L.wh, s->rowptr, s->col, s->valM, s->valK,
-                                                             s->a, s->c, tab);
-    k_lat_operator_check<7><<<blocks_for(s->N), TPB, 0, st>>>(L, s->N, s->rowptr, s->col, s->valM, s->valK, s->a, tab,
-                                                              bad);
+                                                             tab);
+    k_lat_operator_check<7><<<blocks_for(s->N), TPB, 0, st>>>(L, s->N, s->rowptr, s->col, s->valM, s->valK, tab, bad);
   } else {
     k_lat_operator<15><<<blocks_for(L.nids, 64), 64, 0, st>>>(L.nids, L.rep, L.wh, s->rowptr, s->col, s->valM,
-                                                              s->valK, s->a, s->c, tab);
-    k_lat_operator_check<15><<<blocks_for(s->N), TPB, 0, st>>>(L, s->N, s->rowptr, s->col, s->valM, s->valK, s->a,
-                                                               tab, bad);
+                                                              s->valK, tab);
+    k_lat_operator_check<15><<<blocks_for(s->N), TPB, 0, st>>>(L, s->N, s->rowptr, s->col, s->valM, s->valK, tab, bad);
   }
   CH_LAUNCHED();
   return CH_OK;
@@ -632,7 +689,7 @@ ch_status assemble_system(const ch_mesh_s* m, ch_system_s* s, cudaStream_t st) {
   int ovf[2] = {0, 0};
   CH_CUDA(cudaMemcpyAsync(ovf, overflow, sizeof(ovf), cudaMemcpyDeviceToHost, st));
   CH_CUDA(cudaStreamSynchronize(st));
-  if (ovf[1]) s->lat.tab = nullptr;  // (a very long, thin grid's coordinates round too unevenly)
+  if (ovf[1]) s->lat.tab = nullptr;
   if (ovf[0]) {
     set_error("a node has more than %d incident simplex vertices", MAXADJ);
     return CH_ERR_INTERNAL;
@@ -1159,7 +1216,8 @@ __global__ void k_rhs(const MeshPod m, LoadCoef L, const double2* eload, const L
     const double* t = A.tab + (size_t)id * LatAxes<ND>::TS;
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
-      const int j = __double2hiint(t[d]) != 0 ? v + lat_off(ND, d, w.x, w.y) : v;  // (as lat_apply_A)
+      if (__double2hiint(t[d]) == 0) continue;  // (as lat_apply_A)
+      const int j = v + lat_off(ND, d, w.x, w.y);
       mp = fma(t[d], pp[(size_t)ld * j], mp);
       mn = fma(t[d], pn[(size_t)ld * j], mn);
     }
@@ -1271,9 +1329,9 @@ __global__ void k_apply_A(int N, const int* rowptr, const int* col, const double
   y[v] = out;
 }
 
-// The lattice form: no indices or values but the class id, so the FP64 pipe alone bounds it (54
-// instructions per node at most).  512 x 512: 23.9 us, 33.6 in CSR form; 3D 128 x 128 x 32: 83, 127 in
-// CSR form.
+// The lattice form: no indices or values but the class id, so the FP64 pipe alone bounds it (54 or 94
+// instructions per node).  512 x 512: 29.3 us, 33.6 in CSR form; 3D 128 x 128 x 32: 93, 127 in
+// CSR form.  Several classes along an axis cost little: 511 x 509 29.3, 127 x 129 x 33 95.
 template <int ND>
 __global__ void __launch_bounds__(128) k_apply_A_lat(LatOperator A, int N, const double4_32a* __restrict__ x,
                                                      double4_32a* __restrict__ y) {
@@ -1285,7 +1343,7 @@ ch_status apply_A(const ch_system_s* s, const double* x, double* y, cudaStream_t
   const double4_32a* x4 = reinterpret_cast<const double4_32a*>(x);
   double4_32a* y4 = reinterpret_cast<double4_32a*>(y);
   if (s->lat.tab) {
-    const double f = s->mesh->dim == 2 ? 48.0 : 88.0;
+    const double f = s->mesh->dim == 2 ? 54.0 : 94.0;
     ProfScope ps(st, K_APPLY_A, 0, 66.0 * s->N, f * s->N);
     if (s->mesh->dim == 2) k_apply_A_lat<7><<<blocks_for(s->N, 128), 128, 0, st>>>(s->lat, s->N, x4, y4);
     else k_apply_A_lat<15><<<blocks_for(s->N, 128), 128, 0, st>>>(s->lat, s->N, x4, y4);

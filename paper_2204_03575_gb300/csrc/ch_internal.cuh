@@ -190,18 +190,25 @@ void prof_add_slot(int kid, int f32, int64_t launches, double bytes, double fmas
 
 // ---------------------------------------------------------------- lattice classes of a uniform mesh
 namespace ch {
-// On a uniform box mesh an assembled row depends only on the run's cell size and on whether the node
-// is the first, an inner or the last one along each axis: 9 classes in 2D, 27 in 3D.  Every node
-// carries its class id, run * classes + class, and a fine-level operator is one table row per id
-// instead of one value per stored entry.
+// On a box mesh an assembled row depends only on the widths of the cells on either side of the node along
+// each axis (none beyond a rim).  Every node carries a class id and a fine-level operator is one table row
+// per id instead of one value per stored entry.  Two partitions of a run's nodes:
+//   ch_mesh_s::lat  by the pairs of widths as the node coordinates have them.  Coordinates are rounded, so
+//                   the widths of a uniform axis take two values per binade: 3 pairs for 512 cells of 1 / 512,
+//                   24 for 799 cells on [0, 10].  The rows of a class are equal bit for bit.
+//   ch_mesh_s::pos  by position alone: the first, an inner or the last node along each axis, 9 classes in 2D
+//                   and 27 in 3D.  The rows of a class agree to the rounding of the coordinates (1e-13 of an
+//                   entry for those 799 cells): below FP32's rounding, and used by FP32 V-cycles only.
 struct Lattice {
-  int dim = 0, ncls = 0;        // 9 (2D) or 27 (3D) classes per run
-  int nids = 0;                 // runs x ncls
+  int dim = 0;
+  int ncls = 0;                 // pos: 9 (2D) or 27 (3D) classes per run
+  int nids = 0;                 // classes of all runs
+  int multi = 0;                // several runs: the strides are the id's
   int W = 0, WH = 0;            // strides nx + 1 and (nx + 1)(ny + 1) of a single run
   int id32 = 0;                 // ids are 32-bit (more than 65536 of them), else 16-bit
   void* id = nullptr;           // N class ids
   int2* wh = nullptr;           // nids: strides of the id's run
-  int* rep = nullptr;           // nids: a node of the class (the middle one along its inner axes)
+  int* rep = nullptr;           // nids: a node of the class
 };
 // The grid of one run: first node, first cell, cells per axis.
 struct CellGrid {
@@ -220,35 +227,38 @@ __device__ __forceinline__ int lat_id(const Lattice& L, int i) {
   return L.id32 ? static_cast<const int*>(L.id)[i] : static_cast<const uint16_t*>(L.id)[i];
 }
 
-// The block operator of Eq. (14) on the lattice: per class id a table row of the mass entries m_d, of
-// -c m_d and of a k_e over the axis directions e -- the only ones where the stiffness matrix of a box
-// mesh is not zero (5 of 7 in 2D, 7 of 15 in 3D).  tab is null where the mesh does not fit its
-// classes (set-up check): the CSR form then.
+// The block operator of Eq. (14) on the lattice: per class id a table row of the mass entries m_d and of
+// the stiffness entries k_e over the axis directions e -- the only ones where the stiffness matrix of a box
+// mesh is not zero (5 of 7 in 2D, 7 of 15 in 3D).  The entries are the assembled ones (set-up check, bit
+// for bit); tab is null where they are not, and the CSR form is taken: entries below FP64's normal range.
 struct LatOperator {
   Lattice L;
+  double a = 0, c = 0;
   const double* tab = nullptr;
 };
 template <int ND> struct LatAxes;
 template <> struct LatAxes<7> {
-  static constexpr int NK = 5, TS = 20;  // axis directions; doubles per table row (2 ND + NK, even)
+  static constexpr int NK = 5, TS = 12;  // axis directions; doubles per table row (ND + NK, even)
   __host__ __device__ static constexpr int index(int d) { return d >= 1 && d <= 5 ? d - 1 : -1; }
 };
 template <> struct LatAxes<15> {
-  static constexpr int NK = 7, TS = 38;
+  static constexpr int NK = 7, TS = 22;
   __host__ __device__ static constexpr int index(int d) {
     constexpr int k[15] = {-1, -1, -1, 0, -1, 1, 2, 3, 4, 5, -1, 6, -1, -1, -1};
     return k[d];
   }
 };
 
-// (A x)_i for both species: y1 = M x1 + a K x2, y2 = a K x1 - c M x2.  4 FMAs per direction and 4 more
-// per axis direction (48 in 2D, 88 in 3D, against 8 per stored entry, 56 and 120, in CSR form).
+// (A x)_i for both species: y1 = M x1 + a K x2, y2 = a K x1 - c M x2, in the order and with the roundings of
+// the CSR form (products m c and k a formed beforehand, six instructions fewer, rounded 1.2 to 1.5 times as
+// far from the exact sum).  4 FMAs per direction, 4 more per axis direction and 6 at the end (54 in 2D, 94 in
+// 3D, against 8 per stored entry, 62 and 126, in CSR form).
 template <int ND>
 __device__ __forceinline__ double4_32a lat_apply_A(const LatOperator& A, int i, const double4_32a* __restrict__ x) {
   using X = LatAxes<ND>;
   const int id = lat_id(A.L, i);
   int W = A.L.W, WH = A.L.WH;
-  if (A.L.nids > A.L.ncls) {
+  if (A.L.multi) {
     const int2 w = A.L.wh[id];
     W = w.x;
     WH = w.y;
@@ -261,25 +271,26 @@ __device__ __forceinline__ double4_32a lat_apply_A(const LatOperator& A, int i, 
     t[2 * q] = v.x;
     t[2 * q + 1] = v.y;
   }
-  double4_32a y = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+  double4_32a m = make_double4_32a(0.0, 0.0, 0.0, 0.0), k = m;
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
-    // a neighbour the class lacks (mass entry zero) reads the node itself, not another row's or run's value
-    const int j = __double2hiint(t[d]) != 0 ? i + lat_off(ND, d, W, WH) : i;
-    const double4_32a z = x[j];
-    y.x = fma(t[d], z.x, y.x);
-    y.y = fma(t[d], z.y, y.y);
-    y.z = fma(t[ND + d], z.z, y.z);
-    y.w = fma(t[ND + d], z.w, y.w);
+    // a neighbour the class lacks (mass entry zero) is not read: it would be another row's or run's value
+    double4_32a z = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+    if (__double2hiint(t[d]) != 0) z = x[i + lat_off(ND, d, W, WH)];
+    m.x = fma(t[d], z.x, m.x);
+    m.y = fma(t[d], z.y, m.y);
+    m.z = fma(t[d], z.z, m.z);
+    m.w = fma(t[d], z.w, m.w);
     if (X::index(d) >= 0) {
-      const double k = t[2 * ND + (X::index(d) >= 0 ? X::index(d) : 0)];
-      y.x = fma(k, z.z, y.x);
-      y.y = fma(k, z.w, y.y);
-      y.z = fma(k, z.x, y.z);
-      y.w = fma(k, z.y, y.w);
+      const double s = t[ND + (X::index(d) >= 0 ? X::index(d) : 0)];
+      k.x = fma(s, z.x, k.x);
+      k.y = fma(s, z.y, k.y);
+      k.z = fma(s, z.z, k.z);
+      k.w = fma(s, z.w, k.w);
     }
   }
-  return y;
+  return make_double4_32a(fma(A.a, k.z, m.x), fma(A.a, k.w, m.y), fma(A.a, k.x, -A.c * m.z),
+                          fma(A.a, k.y, -A.c * m.w));
 }
 }  // namespace ch
 
@@ -302,7 +313,7 @@ struct ch_mesh_s {
   int *n2e_ptr = nullptr, *n2e = nullptr;  // node -> incident elements (sorted)
   int *n2b_ptr = nullptr, *n2b = nullptr;  // node -> incident bottom facets
   int *n2t_ptr = nullptr, *n2t = nullptr;  // node -> incident top facets
-  ch::Lattice lat;
+  ch::Lattice lat, pos;  // classes by cell widths, by position
   ch::CellGrid* cell_grid = nullptr;  // device, per run
   ch::Alloc mem;
 };

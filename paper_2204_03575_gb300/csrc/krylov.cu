@@ -1371,7 +1371,7 @@ static ch_status residual_launch(ch_state_s* S, int init, cudaStream_t st, const
   const double4_32a* b4 = reinterpret_cast<const double4_32a*>(S->b);
   double4_32a* W4 = reinterpret_cast<double4_32a*>(S->W);
   if (s->lat.tab) {
-    const double f = s->mesh->dim == 2 ? 48.0 : 88.0;
+    const double f = s->mesh->dim == 2 ? 54.0 : 94.0;
     ProfScope ps(st, K_RESIDUAL4, 0, 98.0 * S->N, (f + 12.0) * S->N);
     if (s->mesh->dim == 2)
       k_residual4_lat<7><<<S->nblocks, TPB, 0, st>>>(S->seg, s->lat, x4, b4, W4, S->partials, S->kd, init,
