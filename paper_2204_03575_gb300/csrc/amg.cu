@@ -42,10 +42,6 @@ struct LatOp {
   int ts = 0;                      // values per table row: 8 or 16
   Lattice L;
   const T* tab = nullptr;          // nids x ts: the operator's rows (slot nd: 1 / diagonal)
-  // FP64: the Chebyshev steps' tables (deg x nids x ts each, see lat_step_tables); FP32 steps use tab
-  T* steps = nullptr;              // of the V-cycle's smoother
-  T* semi = nullptr;               // of the semi-iteration (precond_M = 1)
-  T* scratch = nullptr;            // of ch_smooth's own degree, rebuilt by each call
 };
 
 // One tile of the 2D lattice form for k_smooth_tile: the run's first node, strides and ids, and the
@@ -817,30 +813,6 @@ __global__ void k_lat_cast(const double* a, T* b, int n) {
   if (i < n) b[i] = (T)a[i];
 }
 
-// The Chebyshev step x' = x + alpha (x - xp) + beta D^-1 (b - A x) with everything that depends on the
-// class folded into one table row: x' = g (A' x - b) - alpha xp with g = -beta / a_ii (slot nd) and
-// A' = A but for the diagonal, a_ii' = a_ii + (1 + alpha) / g = a_ii (1 - (1 + alpha) / beta).  Nine
-// FP64 instructions per right-hand side in 2D (seven for the row, two for g and xp) instead of ten
-// and a scaling per row: FP64 V-cycles are bound by that pipe.  FP32 steps are bound by their vectors
-// and keep the operator's own rounded values (k_cheb_step_lat).
-struct StepCoefs {
-  int n;
-  double alpha[16], beta[16];
-};
-__global__ void k_lat_steps(const double* tab, int nids, int nd, int ts, StepCoefs c, double* out) {
-  const int id = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
-  if (id >= nids) return;
-  const double* row = tab + (size_t)id * ts;
-  double* o = out + ((size_t)s * nids + id) * ts;
-  const double diag = row[nd / 2];
-  for (int d = 0; d < ts; ++d) {
-    double v = d < nd ? row[d] : 0.0;
-    if (d == nd / 2) v = diag * (1.0 - (1.0 + c.alpha[s]) / c.beta[s]);
-    if (d == nd) v = -c.beta[s] / diag;
-    o[d] = v;
-  }
-}
-
 // The lattice form's FP64 table of A where every row fits it (tab stays null where not: the level
 // then keeps the CSR form).
 static ch_status lat_build(const Csr<double>& A, const Lattice* L, double rel, Alloc& mem, double** tab,
@@ -863,24 +835,18 @@ static ch_status lat_build(const Csr<double>& A, const Lattice* L, double rel, A
   return CH_OK;
 }
 
+// Coefficients of the Chebyshev smoother.  Step s from x with the carried direction e and r = A x - b:
+//   e' = carry_s e + D^-1 r,  x' = x - beta_s e'
+// (e is the usual direction d = x' - x over -beta: no factor per row is left).  The direction is kept rather
+// than x - x_prev, which would feed x's rounding into the next steps (FP32 errors 3 to 24 % larger, FP64 ones
+// 1.3 to 3.3 times with the diagonal folded as well).  A pass from zero starts with x = invtheta D^-1 b and
+// its first step carries from_x x.
 struct ChebCoef {
-  double invtheta;
-  double alpha[16], beta[16];
+  double invtheta, from_x;
+  double carry[16], beta[16];
 };
 static ChebCoef cheb_coef(double rho, int deg, double lower);
 static ChebCoef cheb_coef_interval(double lo, double hi, int deg);
-
-// the tables of `deg` steps with coefficients c
-static void lat_step_tables(const double* tab64, const LatOp<double>& op, const ChebCoef& c, int deg, double* out,
-                            cudaStream_t st) {
-  StepCoefs sc;
-  sc.n = deg;
-  for (int s = 0; s < 16; ++s) {
-    sc.alpha[s] = c.alpha[s];
-    sc.beta[s] = c.beta[s];
-  }
-  k_lat_steps<<<dim3(blocks_for(op.L.nids, 64), deg), 64, 0, st>>>(tab64, op.L.nids, op.nd, op.ts, sc, out);
-}
 
 // Tiles of a pass of `halo` operator applications over every run of a 2D mesh.  FP32 block heights by the
 // time they take in units of region rows, measured over 64 x 64 .. 1024 x 1024 and the 64-run batch (Algorithm
@@ -1017,17 +983,6 @@ static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, const ch_para
     CH_TRY(h->mem.get(&tab, (size_t)cnt));
     k_lat_cast<T><<<blocks_for(cnt), TPB, 0, st>>>(h->lat_tab, tab, cnt);
     op.tab = tab;
-    if constexpr (std::is_same<T, double>::value) {
-      CH_TRY(h->mem.get(&op.steps, (size_t)h->cheb_degree * cnt));
-      CH_TRY(h->mem.get(&op.scratch, (size_t)16 * cnt));
-      lat_step_tables(h->lat_tab, op, cheb_coef(h->rho[0], h->cheb_degree, h->cheb_lower), h->cheb_degree, op.steps,
-                      st);
-      if (p.precond_M == 1) {
-        const int ns = semi_steps(p);
-        CH_TRY(h->mem.get(&op.semi, (size_t)ns * cnt));
-        lat_step_tables(h->lat_tab, op, semi_coef(lat->dim, ns), ns, op.semi, st);
-      }
-    }
     CH_LAUNCHED();
     if (lat->dim == 2 && h->nlev > 1 && (by_position || !F32)) {
       CH_TRY(tile_setup<T>());
@@ -1331,21 +1286,19 @@ __device__ __forceinline__ void row_finish(const RowSum<T, TPR>& r, int sub, F f
 template <typename V2> __device__ __forceinline__ auto* comps(V2* p) { return &p->x; }
 template <typename V2> __device__ __forceinline__ const auto* comps(const V2* p) { return &p->x; }
 
-// One Chebyshev step of the two-term form, x' = x + alpha (x - xp) + beta D^-1 (b - A x), with the
-// iterate before x in the output's own place: xo holds xp on entry and x' on exit, so a step moves
-// four vectors (x, xp, b, x') and keeps no direction.
-enum XPrev { XP_NONE = 0, XP_READ = 1, XP_ZERO = 2 };  // alpha = 0; xp in xo; xp = 0 (x is the first iterate)
-
-// The row sum starts from -b, so it is -r, and nbeta = -beta turns it back.
+// One Chebyshev step (ChebCoef); the row sum starts from -b.  `from`: what the direction carries on from;
+// keep: the next step of the pass reads it.
+enum Carry { CARRY_NONE = 0, CARRY_E = 1, CARRY_X = 2 };  // nothing; e; x (the pass's first iterate, from zero)
 template <typename T, typename V2, int TPR>
 __global__ void __launch_bounds__(TPB) k_cheb_step(Csr<T> A, const T* __restrict__ dinv,
                                                    const V2* __restrict__ b, const V2* __restrict__ x,
-                                                   V2* __restrict__ xo, T alpha, T nbeta, int mode) {
+                                                   V2* __restrict__ xo, V2* __restrict__ e, T carry, T nbeta,
+                                                   int from, bool keep) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = t / TPR, sub = t % TPR;
   CsrRow<T, TPR> row;
   row_prefetch<T, TPR>(A, i, sub, row);
-  const T di = i < A.nrows ? dinv[i] * nbeta : T(0);
+  const T di = i < A.nrows ? dinv[i] : T(0);
   pdl_wait();
   pdl_trigger_t<T>();
   T s0 = 0, s1 = 0;
@@ -1358,10 +1311,11 @@ __global__ void __launch_bounds__(TPB) k_cheb_step(Csr<T> A, const T* __restrict
   const RowSum<T, TPR> r = row_sum<T, TPR>(s0, s1, sub);
   if (i >= A.nrows) return;
   row_finish<T, TPR>(r, sub, [&](int c, T s) {
-    T y = comps(x + i)[c];
-    T* o = comps(xo + i) + c;
-    if (mode != XP_NONE) y = fma(alpha, mode == XP_READ ? y - *o : y, y);
-    *o = fma(di, s, y);
+    const T y = comps(x + i)[c];
+    T v = di * s;
+    if (from != CARRY_NONE) v = fma(carry, from == CARRY_E ? comps(e + i)[c] : y, v);
+    if (keep) comps(e + i)[c] = v;
+    comps(xo + i)[c] = fma(nbeta, v, y);
   });
 }
 
@@ -1442,49 +1396,30 @@ __device__ __forceinline__ void lat_row_acc(const LatRow<T, ND>& r, int n, int i
   }
 }
 
-// One Chebyshev step on the lattice form.  FP32 is bound by its vectors (34 bytes per row: x, xp, b, x'
-// and the class id; one value per stored entry and a kept direction made it 72 in 2D, 104 in 3D), FP64
-// by its pipe.  Measured, us per step in a run of launches: FP32 4.01 -> 3.26 (512 x 512), 9.88 -> 8.21
-// (3D 128 x 128 x 32), 16.8 -> 10.2 (64 runs, 1.46 M rows); 512 x 512 FP64 steps 20.8 -> 18.9 ms.
-// xp is read from and x' written to xo.  FP64: the step's table
-// (lat_step_tables), x' = g (A' x - b) - alpha xp.  FP32: the operator's table, x' = x + alpha (x - xp)
-// + (nbeta D^-1) (A x - b).
+// One Chebyshev step on the lattice form: k_cheb_step's arithmetic.  FP32 is bound by its vectors (42 bytes
+// per row: x, b, e read and written, x' and the class id; one value per stored entry as well made it 72 in 2D,
+// 104 in 3D), FP64 by its pipe (ten instructions per right-hand side in 2D).
 template <typename T, typename V2, int ND>
-__global__ void __launch_bounds__(TPB) k_cheb_step_lat(LatOp<T> D, int n, const T* __restrict__ tab,
-                                                       const V2* __restrict__ b, const V2* __restrict__ x,
-                                                       V2* __restrict__ xo, T alpha, T nbeta, int mode) {
+__global__ void __launch_bounds__(TPB) k_cheb_step_lat(LatOp<T> D, int n, const V2* __restrict__ b,
+                                                       const V2* __restrict__ x, V2* __restrict__ xo,
+                                                       V2* __restrict__ e, T carry, T nbeta, int from, bool keep) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   LatRow<T, ND> row;
-  if (i < n) row = lat_row<T, ND>(D, tab, i);
+  if (i < n) row = lat_row<T, ND>(D, D.tab, i);
   pdl_wait();
   pdl_trigger_t<T>();
   if (i >= n) return;
   const V2 bi = b[i];
   T s0 = -bi.x, s1 = -bi.y;
   lat_row_acc<T, V2, ND>(row, n, i, x, s0, s1);
-  const T g = row.a[ND];
-  if (sizeof(T) == 8) {
-    if (mode == XP_READ) {
-      const V2 xp = xo[i];
-      xo[i] = mk2<T, V2>(fma(g, s0, -alpha * xp.x), fma(g, s1, -alpha * xp.y));
-    } else {
-      xo[i] = mk2<T, V2>(g * s0, g * s1);
-    }
-  } else {
-    V2 y = x[i];
-    if (mode != XP_NONE) {
-      V2 d = y;
-      if (mode == XP_READ) {
-        const V2 xp = xo[i];
-        d.x -= xp.x;
-        d.y -= xp.y;
-      }
-      y.x = fma(alpha, d.x, y.x);
-      y.y = fma(alpha, d.y, y.y);
-    }
-    const T di = g * nbeta;
-    xo[i] = mk2<T, V2>(fma(di, s0, y.x), fma(di, s1, y.y));
+  const V2 y = x[i];
+  V2 v = mk2<T, V2>(row.a[ND] * s0, row.a[ND] * s1);
+  if (from != CARRY_NONE) {
+    const V2 d = from == CARRY_E ? e[i] : y;
+    v = mk2<T, V2>(fma(carry, d.x, v.x), fma(carry, d.y, v.y));
   }
+  if (keep) e[i] = v;
+  xo[i] = mk2<T, V2>(fma(nbeta, v.x, y.x), fma(nbeta, v.y, y.y));
 }
 
 template <typename T, typename V2, int ND>
@@ -1518,7 +1453,7 @@ __global__ void __launch_bounds__(TPB) k_spmv2_lat(LatOp<T> D, int n, const V2* 
 // A whole smoothing pass of the 2D lattice form in one launch.  A block holds a region of RW columns x
 // (ROWS x groups) rows: a tile of outputs and a halo as deep as the pass applies the operator
 // (deg times), in shared memory (two buffers of the iterate); a thread owns ROWS nodes of one column
-// with their iterate, the one before it and b in registers.  Every application spoils one ring of the
+// with their iterate, the direction and b in registers.  Every application spoils one ring of the
 // region, so the tile's own nodes end exact: the same operations in the same order as k_cheb_step_lat
 // and k_residual_lat, bitwise.  Operators being one table row per class, nothing but b (and x, unless
 // the pass starts from zero) is read, once per pass instead of four vectors per step.
@@ -1530,13 +1465,13 @@ __global__ void __launch_bounds__(TPB) k_spmv2_lat(LatOp<T> D, int n, const V2* 
 template <typename T, typename V2>
 struct TileArgs {
   const LatTile* tiles;
-  const T *tab, *steps;  // the operator's table; FP64: the steps' tables
+  const T* tab;  // the operator's table
   const V2 *b, *x;
   V2 *xo, *r;
   double* wo;  // the last pass of an application: the result goes here in FP64, ldw values per node, not to xo
   Lattice L;   // FP64: the nodes' class ids
-  int ldw, nids, deg, halo;
-  T invtheta, alpha[16], nbeta[16];
+  int ldw, deg, halo;
+  T invtheta, carry[16], nbeta[16];
 };
 template <typename T>
 constexpr int tile_smem(int groups) {
@@ -1560,11 +1495,15 @@ __device__ __forceinline__ float2 fma2(float c, float2 x, float2 a) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pk2(c, c)), "l"(pk2(x.x, x.y)), "l"(pk2(a.x, a.y)));
   return up2(r);
 }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(-1.f, b, a); }  // exact product
+__device__ __forceinline__ float2 mul2(float c, float2 x) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pk2(c, c)), "l"(pk2(x.x, x.y)));
+  return up2(r);
+}
 __device__ __forceinline__ double2 fma2(double c, double2 x, double2 a) {
   return make_double2(fma(c, x.x, a.x), fma(c, x.y, a.y));
 }
-__device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 mul2(double c, double2 x) { return make_double2(c * x.x, c * x.y); }
 
 // One block's tile.  FP64: a thread's one node has its class's row (by cell widths).  FP32 (classes by
 // position): a thread's nodes share the column's row, and those of the first and last mesh row load theirs.
@@ -1593,10 +1532,10 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   load_row(a.tab, 1, row);
   pdl_wait();
   pdl_trigger_t<T>();
-  V2 nb[ROWS], cur[ROWS], prev[ROWS];  // -b, the iterate and the one before it
+  V2 nb[ROWS], cur[ROWS], dir[ROWS];  // -b, the iterate and the direction (ChebCoef's e)
 #pragma unroll
   for (int t = 0; t < ROWS; ++t) {
-    nb[t] = cur[t] = prev[t] = mk2<T, V2>(T(0), T(0));
+    nb[t] = cur[t] = dir[t] = mk2<T, V2>(T(0), T(0));
     if (in(t)) {
       const V2 bt = a.b[node0 + (size_t)t * tl.W];
       nb[t] = mk2<T, V2>(-bt.x, -bt.y);
@@ -1613,7 +1552,7 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
         di = e[7];
       }
       const T s = -(a.invtheta * di);
-      cur[t] = mk2<T, V2>(s * nb[t].x, s * nb[t].y);
+      dir[t] = cur[t] = mk2<T, V2>(s * nb[t].x, s * nb[t].y);  // (carry[1] is ChebCoef's from_x)
     }
   }
   V2* mine = buf + (g * ROWS + 1) * ST + c + 1;  // this thread's first node in buffer 0
@@ -1621,9 +1560,9 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   for (int t = 0; t < ROWS; ++t) mine[t * ST] = cur[t];
   __syncthreads();
   int p = 0, margin = 0;
-  // f(t, row's last entry, sum) for the thread's nodes, sum = one application of the rows `tab` (the
-  // interior one is in `row`) to the iterate, seeded with -b or 0
-  const auto apply = [&](const T* tab, bool seed_b, auto f) {
+  // f(t, 1 / diagonal, sum) for the thread's nodes, sum = the operator applied to the iterate, seeded with -b
+  // or 0 (the thread's row, or the interior one of its column, is in `row`)
+  const auto apply = [&](bool seed_b, auto f) {
     const V2* q = mine + p * plane;
     V2 south = q[-ST], wprev = q[-ST - 1], wcur = q[-1], ecur = q[1], enext = q[ST + 1];
 #pragma unroll
@@ -1636,7 +1575,7 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
         const V2 nbr[7] = {wprev, south, wcur, center, ecur, north, enext};
         if (EDGE && !OWN && edge(t) != 1) {
           T e[8];
-          load_row(tab, edge(t), e);
+          load_row(a.tab, edge(t), e);
 #pragma unroll
           for (int d = 0; d < 7; ++d) s = fma2(e[d], nbr[d], s);
           f(t, e[7], s);
@@ -1655,23 +1594,10 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
     ++margin;
   };
   for (int s = ZERO ? 1 : 0; s < a.deg; ++s) {
-    const T alpha = a.alpha[s], nbeta = a.nbeta[s];
-    const T* tab = sizeof(T) == 8 ? a.steps + (size_t)s * a.nids * 8 : a.tab;
-    if (sizeof(T) == 8) load_row(tab, 1, row);
-    const bool has_prev = s > 0;
-    // (before the first step of a pass from zero the iterate was zero, as prev starts out)
-    apply(tab, true, [&](int t, T last, V2 sum) {
-      V2 v;
-      if (sizeof(T) == 8) {
-        v = has_prev ? fma2(last, sum, mk2<T, V2>(-alpha * prev[t].x, -alpha * prev[t].y))
-                     : mk2<T, V2>(last * sum.x, last * sum.y);
-      } else {
-        v = cur[t];
-        if (has_prev) v = fma2(alpha, sub2(v, prev[t]), v);
-        v = fma2(last * nbeta, sum, v);
-      }
-      prev[t] = cur[t];
-      cur[t] = v;
+    const T carry = a.carry[s], nbeta = a.nbeta[s];
+    apply(true, [&](int t, T dinv, V2 sum) {
+      dir[t] = fma2(carry, dir[t], mul2(dinv, sum));
+      cur[t] = fma2(nbeta, dir[t], cur[t]);
     });
     p ^= 1;
 #pragma unroll
@@ -1690,8 +1616,7 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
         a.xo[i] = cur[t];
     }
   if (RES) {
-    if (sizeof(T) == 8) load_row(a.tab, 1, row);
-    apply(a.tab, false, [&](int t, T, V2 sum) {
+    apply(false, [&](int t, T, V2 sum) {
       if (out(t)) a.r[node0 + (size_t)t * tl.W] = mk2<T, V2>(-nb[t].x - sum.x, -nb[t].y - sum.y);
     });
   }
@@ -1779,14 +1704,13 @@ __global__ void __launch_bounds__(TPB) k_restrict_wide(Csr<T> R, X r, V2* __rest
     default: { constexpr int TPRC = 32; KCALL; } break;  \
   }
 
-// one Chebyshev step on a CSR level (the kernel takes -beta)
+// one Chebyshev step on a CSR level
 template <typename T, typename V2>
-static void launch_cheb_step(int tpr, const Csr<T>& A, const T* dinv, const V2* b, const V2* x, V2* xo, T alpha,
-                             T beta, int mode, cudaStream_t st, bool pdl) {
-  const T nbeta = -beta;
+static void launch_cheb_step(int tpr, const Csr<T>& A, const T* dinv, const V2* b, const V2* x, V2* xo,
+                             V2* e, T carry, T nbeta, int from, bool keep, cudaStream_t st, bool pdl) {
   const int g = blocks_for((int64_t)A.nrows * tpr);
-  CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_cheb_step<T, V2, TPRC>, g, TPB, 0, st, A, dinv, b, x, xo, alpha, nbeta,
-                                 mode)));
+  CH_TPR_DISPATCH(tpr, (launch_k(pdl, k_cheb_step<T, V2, TPRC>, g, TPB, 0, st, A, dinv, b, x, xo, e, carry,
+                                 nbeta, from, keep)));
 }
 template <typename T, typename V2>
 static void launch_residual(int tpr, const Csr<T>& A, const V2* b, const V2* x, V2* r, cudaStream_t st,
@@ -1942,18 +1866,20 @@ __global__ void k_store2(int n, const V2* src, double* dst, int ld) {
 
 // ---------------------------------------------------------------- V-cycle driver
 // Coefficients of `deg` Chebyshev semi-iteration steps for eigenvalues in [lo, hi]: the first
-// step from zero is x = D^-1 b / theta, then d = alpha_s d + beta_s D^-1 (b - A x), x += d.
+// step from zero is x = D^-1 b / theta, then d = alpha_s d + beta_s D^-1 (b - A x), x += d, kept as ChebCoef
+// says.
 static ChebCoef cheb_coef_interval(double lo, double hi, int deg) {
   ChebCoef c{};
   const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
   c.invtheta = 1.0 / theta;
-  c.alpha[0] = 0.0;
   c.beta[0] = 1.0 / theta;
   double rho_prev = 1.0 / sigma;
   for (int s = 1; s < deg && s < 16; ++s) {
     const double r = 1.0 / (2.0 * sigma - rho_prev);
-    c.alpha[s] = r * rho_prev;
+    const double alpha = r * rho_prev;
     c.beta[s] = 2.0 * r / delta;
+    c.carry[s] = alpha * c.beta[s - 1] / c.beta[s];
+    if (s == 1) c.from_x = -alpha / c.beta[1];
     rho_prev = r;
   }
   return c;
@@ -1993,7 +1919,6 @@ static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename 
   TileArgs<T, V2> a;
   a.tiles = pl.tiles;
   a.tab = L.lat.tab;
-  a.steps = L.lat.steps;
   a.b = L.b;
   a.x = x;
   a.xo = xo;
@@ -2001,18 +1926,17 @@ static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename 
   a.wo = wo;
   a.ldw = ldw;
   a.L = L.lat.L;
-  a.nids = L.lat.L.nids;
   a.deg = h->cheb_degree;
   a.halo = pl.halo;
   a.invtheta = (T)c.invtheta;
   for (int s = 0; s < 16; ++s) {
-    a.alpha[s] = (T)c.alpha[s];
+    a.carry[s] = (T)(ZERO && s == 1 ? c.from_x : c.carry[s]);
     a.nbeta[s] = (T)-c.beta[s];
   }
   const double n = L.A.nrows, apps = pl.halo;
   ProfScope ps(st, K_CHEB_STEP, sizeof(T) == 4,
                n * (2.0 * sizeof(T) * ((ZERO ? 1 : 2) + (RES ? 2 : (wo ? 0 : 1))) + (wo ? 16.0 : 0.0)),
-               apps * (2.0 * L.A.nnz + 4.0 * n));
+               apps * (2.0 * L.A.nnz + 6.0 * n));
   const int threads = TileShape<T>::RW * pl.groups, smem = tile_smem<T>(pl.groups);
   if constexpr (sizeof(T) == 4) {
     if (pl.pair) {
@@ -2026,12 +1950,12 @@ static void launch_smooth_tile(const Hierarchy* h, LevelT<T>& L, const typename 
 // bytes per row of the fine level's lattice form beyond its vectors: the class id
 static double lat_bytes(const Lattice& L, double n) { return (L.id32 ? 4.0 : 2.0) * n; }
 
-// `deg` Chebyshev steps with coefficients c on level L (accounted as kernels kfirst / kstep); tabs: the
-// steps' tables where the level has the lattice form in FP64.  zero_guess: 0 continue from *xcur; 1 start from
+// `deg` Chebyshev steps with coefficients c on level L (accounted as kernels kfirst / kstep), the direction in
+// L.r (the residual's place, free while a level smooths).  zero_guess: 0 continue from *xcur; 1 start from
 // zero (the first step is pointwise); 2 start from zero with that first step already taken by the
 // caller (fused into the restriction or the input conversion)
 template <typename T_>
-static ch_status smooth_coef(LevelT<T_>& L, const ChebCoef& c, const T_* tabs, int deg, int zero_guess, int kfirst,
+static ch_status smooth_coef(LevelT<T_>& L, const ChebCoef& c, int deg, int zero_guess, int kfirst,
                              int kstep, typename V2T<T_>::t** xcur, cudaStream_t st) {
   using V2 = typename V2T<T_>::t;
   const int n = L.A.nrows;
@@ -2049,14 +1973,16 @@ static ch_status smooth_coef(LevelT<T_>& L, const ChebCoef& c, const T_* tabs, i
   // operator bytes: CSR values + column indices + row pointers and D^-1, or the class ids
   const double opb = L.lat.nd ? lat_bytes(L.lat.L, n) : nnz * (4 + T) + 4.0 * (n + 1) + T * n;
   for (int s = s0; s < deg; ++s) {
-    const int mode = s == 0 ? XP_NONE : (s == 1 && s0 == 1 ? XP_ZERO : XP_READ);
-    ProfScope ps(st, kstep, sizeof(T_) == 4, opb + T * n * (mode == XP_READ ? 8 : 6), 2.0 * nnz + 4.0 * n);
+    const int from = s == 0 ? CARRY_NONE : (s == 1 && s0 == 1 ? CARRY_X : CARRY_E);
+    const bool keep = s + 1 < deg;
+    const T_ carry = (T_)(from == CARRY_X ? c.from_x : c.carry[s]), nbeta = (T_)-c.beta[s];
+    ProfScope ps(st, kstep, sizeof(T_) == 4, opb + T * n * (6 + (from == CARRY_E ? 2 : 0) + (keep ? 2 : 0)),
+                 2.0 * nnz + 6.0 * n);
     if (L.lat.nd) {
-      const T_* tab = sizeof(T_) == 8 ? tabs + (size_t)s * L.lat.L.nids * L.lat.ts : L.lat.tab;
       CH_LAT_DISPATCH(L.lat.nd, (launch_k(L.pdl, k_cheb_step_lat<T_, V2, NDC>, blocks_for(n), TPB, 0, st, L.lat, n,
-                                          tab, L.b, x, other, (T_)c.alpha[s], (T_)-c.beta[s], mode)));
+                                          L.b, x, other, L.r, carry, nbeta, from, keep)));
     } else {
-      launch_cheb_step<T_, V2>(L.tprA, L.A, L.dinv, L.b, x, other, (T_)c.alpha[s], (T_)c.beta[s], mode, st, L.pdl);
+      launch_cheb_step<T_, V2>(L.tprA, L.A, L.dinv, L.b, x, other, L.r, carry, nbeta, from, keep, st, L.pdl);
     }
     std::swap(x, other);
   }
@@ -2071,7 +1997,7 @@ static ch_status smooth(Hierarchy* h, LevelT<T_>& L, int l, int zero_guess,
                         typename V2T<T_>::t** xcur, cudaStream_t st) {
   const int deg = l == 0 ? h->cheb_degree : h->cheb_degree_coarse;
   const ChebCoef c = cheb_coef(h->rho[l], deg, h->cheb_lower);
-  return smooth_coef<T_>(L, c, L.lat.steps, deg, zero_guess, l == 0 ? K_CHEB_FIRST : K_CHEB_FIRST_C,
+  return smooth_coef<T_>(L, c, deg, zero_guess, l == 0 ? K_CHEB_FIRST : K_CHEB_FIRST_C,
                          l == 0 ? K_CHEB_STEP : K_CHEB_STEP_C, xcur, st);
 }
 
@@ -2082,7 +2008,7 @@ static ch_status smooth(Hierarchy* h, LevelT<T_>& L, int l, int zero_guess,
 template <typename T_>
 static ch_status semi_iteration(LevelT<T_>& L, int dim, int steps, typename V2T<T_>::t** xres, cudaStream_t st) {
   *xres = L.x;
-  return smooth_coef<T_>(L, semi_coef(dim, steps), L.lat.semi, steps, 1, K_CHEB_SEMI, K_CHEB_SEMI, xres, st);
+  return smooth_coef<T_>(L, semi_coef(dim, steps), steps, 1, K_CHEB_SEMI, K_CHEB_SEMI, xres, st);
 }
 
 // one V-cycle at level l on L[l].b; result in *xres (L[l].x or L[l].x2).  zero_guess: as smooth_coef
@@ -2182,15 +2108,6 @@ static ch_status smooth_t(Hierarchy* h, std::vector<LevelT<T>>& Ls, const double
   const int n = L.A.nrows;
   const double io = n * (16.0 + 2.0 * sizeof(T));
   const ChebCoef c = cheb_coef(h->rho[0], degree, h->cheb_lower);
-  const T* tabs = L.lat.steps;
-  if constexpr (std::is_same<T, double>::value) {
-    if (L.lat.nd && degree != h->cheb_degree) {
-      // this degree's tables; the two loads below lie between them and the steps, which read the
-      // tables before their dependency wait
-      lat_step_tables(h->lat_tab, L.lat, c, degree, L.lat.scratch, st);
-      tabs = L.lat.scratch;
-    }
-  }
   {
     ProfScope ps(st, K_VLOAD, sizeof(T) == 4, 2.0 * io, 0.0);
     launch_k(L.pdl, k_load2<T, V2>, blocks_for(n), TPB, 0, st, n, b, 2, L.b);
@@ -2202,7 +2119,7 @@ static ch_status smooth_t(Hierarchy* h, std::vector<LevelT<T>>& Ls, const double
   CH_LAUNCHED();
   V2* xr = L.x;
   for (int k = 0; k < passes; ++k)
-    CH_TRY(smooth_coef<T>(L, c, tabs, degree, 0, K_CHEB_FIRST, K_CHEB_STEP, &xr, st));
+    CH_TRY(smooth_coef<T>(L, c, degree, 0, K_CHEB_FIRST, K_CHEB_STEP, &xr, st));
   {
     ProfScope ps(st, K_VSTORE, sizeof(T) == 4, io, 0.0);
     launch_k(L.pdl, k_store2<T, V2>, blocks_for(n), TPB, 0, st, n, xr, x, 2);
