@@ -858,78 +858,172 @@ __global__ void __launch_bounds__(128) k_cell_loads(const MeshPod m, LoadCoef L,
 // with each logarithm taken at max(phi, delta) (a NaN stays a NaN).  The integrand is not a
 // polynomial, so a fixed rule defines the load: on every simplex the product of 3-point
 // Gauss-Legendre rules collapsed onto it (Duffy), 9 points on a triangle, 27 on a tetrahedron.
+// f_p' = ln+ phi_p / N_p - ln+ phi_s / N_s + chi_ps + mix phi_n - 2 chi_ps phi_p and f_n' alike, ln+ x =
+// 1 + ln x, mix = chi_pn - chi_ps - chi_ns (mix_lo: what its rounding left out)
 struct FhCoef {
-  double chi_pn, chi_ps, chi_ns, inv_np, inv_nn, inv_ns, delta;
+  double chi_ps, chi_ns, mix, mix_lo, inv_np, inv_nn, inv_ns, delta;
 };
+static FhCoef fh_coef(const ch_params& p) {
+  const auto rest = [](double a, double b, double d) {  // a - b - d for d = fl(a - b)
+    const double t = a - d;
+    return (a - (d + t)) + (t - b);
+  };
+  const double d = p.chi_pn - p.chi_ps, mix = d - p.chi_ns;
+  return {p.chi_ps, p.chi_ns, mix, rest(p.chi_pn, p.chi_ps, d) + rest(d, p.chi_ns, mix), 1.0 / p.N_p, 1.0 / p.N_nfa,
+          1.0 / p.N_s, p.fh_delta};
+}
+
+// Constants and tables are formed in double-double arithmetic (Dekker 1971) and rounded once.
+struct DD {
+  double h, l;
+};
+constexpr DD dd_sum(double a, double b) {
+  const double s = a + b, t = s - a;
+  return {s, (a - (s - t)) + (b - t)};
+}
+constexpr DD dd_prod(double a, double b) {  // exact: products of halves
+  const double ca = 134217729.0 * a, ah = ca - (ca - a), al = a - ah;
+  const double cb = 134217729.0 * b, bh = cb - (cb - b), bl = b - bh, p = a * b;
+  return {p, ((ah * bh - p) + ah * bl + al * bh) + al * bl};
+}
+constexpr DD operator+(DD a, DD b) {
+  const DD s = dd_sum(a.h, b.h);
+  return dd_sum(s.h, s.l + a.l + b.l);
+}
+constexpr DD operator*(DD a, DD b) {
+  const DD p = dd_prod(a.h, b.h);
+  return dd_sum(p.h, p.l + (a.h * b.l + a.l * b.h));
+}
+constexpr DD dd_div(DD a, DD b) {
+  const double q = a.h / b.h;
+  const DD p = b * DD{q, 0.0};
+  return dd_sum(q, ((a.h - p.h) + (a.l - p.l)) / b.h);
+}
 
 // Gauss-Legendre on [0, 1] with 3 points: 1/2 -+ sqrt(15)/10 and 1/2, weights 5/18, 4/9, 5/18.
 // Square (u, v) -> triangle (u, v (1 - u)), Jacobian 1 - u; cube (u, v, t) -> tetrahedron
 // (u, v (1 - u), t (1 - u)(1 - v)), Jacobian (1 - u)^2 (1 - v); normalised by the reference
-// simplex's measure (1/2, 1/6).
-__device__ __forceinline__ constexpr double gl_x(int i) {
-  return i == 0 ? 0.11270166537925831148 : (i == 1 ? 0.5 : 0.88729833462074168852);
-}
-__device__ __forceinline__ constexpr double gl_w(int i) { return i == 1 ? 4.0 / 9.0 : 5.0 / 18.0; }
+// simplex's measure (1/2, 1/6).  The vertices' weights are multiples of 2^-53, so that a point's sum to one
+// exactly: a sum off by one rounding is common to all points, and 1 - phi_p - phi_n moves by as much.
+constexpr double gl_grid(double x) { return (x + 1.0) - 1.0; }
+constexpr DD gl_w(int i) { return dd_div({i == 1 ? 4.0 : 2.5, 0.0}, {9.0, 0.0}); }
 
-// Natural logarithm of a positive value by tables over the mantissa and the exponent (Tang 1990,
-// "Table-driven implementation of the logarithm function in IEEE floating-point arithmetic"): x = 2^k m,
-// with f the reciprocal of the middle of m's interval (4096 of them) cut to 21 bits, r = m f - 1 (one
-// FMA; |r| <= a = 2^-13 and a little), log x = k log 2 - log f + log1p(r), and log1p by its Taylor series
-// through r^3 with r^4 replaced by a^2 r^2, its part in the Chebyshev polynomials below the fourth (the
-// rest is below 2^-56).  Six FP64 instructions where the general function takes several times as many, and
-// the kernel is bound by that pipe (1024 intervals and one more term took seven); the absolute error
-// stays within 2^-53 (1 + |log x|) and a rounding, which is what the sums it enters can resolve.  Other
-// values (zero, negative, denormal, above 2^65, infinite, NaN) take CUDA's log.
-constexpr int LOG_M = 4096, LOG_K = 1088;
+// 1 + ln x of a positive value by tables over the mantissa and the exponent (Tang 1990, "Table-driven
+// implementation of the logarithm function in IEEE floating-point arithmetic", with his leading and trailing
+// parts): x = 2^k m, f the reciprocal of the middle of m's interval (2048 of them) cut to 21 bits, r = m f - 1
+// (one FMA, |r| <= 2^-11), 1 + ln x = (k ln 2)_lead + (1 - ln f)_lead + r - r^2 / 2 + t, t = r^3 / 3 - r^4 / 4 +
+// r^5 / 5 + (k ln 2)_trail - (ln f)_trail.  The leading parts are multiples of 2^-42, so their sum is exact;
+// t, below 2^-34, takes FP32.  Five FP64 instructions (the pipe that bounds the kernel), the rest integer and
+// FP32 ones.  Error against extended precision 0.29 ulp of ln x rms and 0.502 at most over [1e-10, 1/2], as a
+// correctly rounded logarithm; around x = 1, where f is 1 and 1/2, below 2^-60.  Other values (zero, negative,
+// denormal, above 2^65, infinite, NaN) take CUDA's log.
+constexpr int LOG_M = 2048, LOG_K = 1088;
 struct LogTables {
-  double y[LOG_M];  // -log f
+  double y[LOG_M];  // 1 - ln f, leading part
+  double k[LOG_K];  // (biased exponent - 1023) ln 2, leading part
   int f[LOG_M];     // upper word of f, the lower one is zero
-  double k[LOG_K];  // (biased exponent - 1023) log 2
+  float yt[LOG_M];  // trailing parts
+  float kt[LOG_K];
 };
 static_assert(sizeof(LogTables) % 16 == 0, "copied in 16-byte pieces");
+// the same on the device (no contraction into other fused multiply-adds)
+__device__ DD dv_sum(double a, double b) {
+  const double s = __dadd_rn(a, b), t = __dadd_rn(s, -a);
+  return {s, __dadd_rn(__dadd_rn(a, -__dadd_rn(s, -t)), __dadd_rn(b, -t))};
+}
+__device__ DD dv_add(DD a, DD b) {
+  const DD s = dv_sum(a.h, b.h);
+  return dv_sum(s.h, __dadd_rn(s.l, __dadd_rn(a.l, b.l)));
+}
+__device__ DD dv_mul(DD a, DD b) {
+  const double p = __dmul_rn(a.h, b.h);
+  return dv_sum(p, __fma_rn(a.h, b.l, __fma_rn(a.l, b.h, __fma_rn(a.h, b.h, -p))));
+}
+__device__ DD dv_div(double a, double b) {
+  const double q = __ddiv_rn(a, b);
+  return dv_sum(q, __ddiv_rn(__fma_rn(-q, b, a), b));
+}
+// ln f = 2 (z + z^3 / 3 + ...), z = (f - 1) / (f + 1), for f in [1/2, 1] of few bits: z^2 <= 1/9, 32 terms to
+// 2^-100
+__device__ DD dv_log(double f) {
+  const DD z = dv_div(f - 1.0, f + 1.0), z2 = dv_mul(z, z);
+  DD s = {0.0, 0.0};
+  for (int n = 63; n >= 1; n -= 2) s = dv_add(dv_mul(s, z2), dv_div(2.0, n));
+  return dv_mul(s, z);
+}
 __global__ void k_log_tables(LogTables* t) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const auto lead = [](DD v) { return rint(v.h * 0x1p42) * 0x1p-42; };
   if (i < LOG_M) {
-    const int hi = __double2hiint(1.0 / (1.0 + (i + 0.5) / LOG_M));
+    // (the first and the last interval have f = 1 and 1/2, where the sums for x around 1 vanish)
+    const int hi = __double2hiint(i == 0 ? 1.0 : (i == LOG_M - 1 ? 0.5 : 1.0 / (1.0 + (i + 0.5) / LOG_M)));
+    const DD v = dv_log(__hiloint2double(hi, 0));
+    const double a = lead(v);
     t->f[i] = hi;
-    t->y[i] = -log(__hiloint2double(hi, 0));
+    t->y[i] = 1.0 - a;
+    t->yt[i] = -(float)((v.h - a) + v.l);
   }
-  if (i < LOG_K) t->k[i] = (i - 1023) * 0.69314718055994530942;
+  if (i < LOG_K) {
+    const DD v = dv_mul(dv_log(0.5), {1023.0 - i, 0.0});
+    const double a = lead(v);
+    t->k[i] = a;
+    t->kt[i] = (float)((v.h - a) + v.l);
+  }
 }
-// log of max(x, delta), delta > 0; a NaN stays a NaN.  Positive doubles compare like their bits (an FP64
+// FP64 <-> FP32 by integer operations (the conversion instructions run at the FP64 pipe's rate): to the
+// nearest, for values in FP32's normal range or zero; exact (zero becomes 2^-127)
+__device__ __forceinline__ float to_f32(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) + 0x10000000ull;
+  const int hi = (int)(b >> 32);
+  const unsigned e = (unsigned)max((hi & 0x7fffffff) - 0x38000000, 0);
+  return __int_as_float((int)__funnelshift_l((unsigned)b, e, 3) | (hi & 0x80000000));
+}
+__device__ __forceinline__ double to_f64(float v) {
+  const int b = __float_as_int(v);
+  return __hiloint2double((int)(((unsigned)(b & 0x7fffffff) >> 3) + 0x38000000u) | (b & 0x80000000), b << 29);
+}
+// 1 + ln max(x, delta), delta > 0; a NaN stays a NaN.  Positive doubles compare like their bits (an FP64
 // comparison would take the pipe).
-__device__ __forceinline__ double guarded_log(double x, double delta, const LogTables* tab) {
+__device__ __forceinline__ double guarded_log1(double x, double delta, const LogTables* tab) {
   constexpr unsigned LO = 0x00100000u, SPAN = ((unsigned)LOG_K << 20) - LO;  // upper words within the tables
   long long bits = __double_as_longlong(x);
   const long long lo = __double_as_longlong(delta);
   if ((unsigned)(bits >> 32) - LO >= SPAN) {
     x = x < delta ? delta : x;
     bits = __double_as_longlong(x);
-    if ((unsigned)(bits >> 32) - LO >= SPAN) return log(x);
+    if ((unsigned)(bits >> 32) - LO >= SPAN) return log(x) + 1.0;
   }
   bits = bits < lo ? lo : bits;
   const unsigned hi = (unsigned)(bits >> 32);
-  if (hi - LO >= SPAN) return log(__longlong_as_double(bits));  // a denormal or enormous delta
+  if (hi - LO >= SPAN) return log(__longlong_as_double(bits)) + 1.0;  // a denormal or enormous delta
   const double m = __longlong_as_double((bits & 0x000fffffffffffffLL) | 0x3ff0000000000000LL);
-  const int j = (hi >> 8) & (LOG_M - 1);
-  const double r = fma(m, __hiloint2double(tab->f[j], 0), -1.0), r2 = r * r;
-  const double p = fma(r, 1.0 / 3.0, -0.5 - 0x1p-28);
-  return (tab->k[hi >> 20] + tab->y[j]) + fma(r2, p, r);
+  const int j = (hi >> 9) & (LOG_M - 1);
+  const double r = fma(m, __hiloint2double(tab->f[j], 0), -1.0);
+  const int rh = __double2hiint(r);
+  const double half = __hiloint2double(rh == 0 ? 0 : (rh - 0x00100000) ^ 0x80000000, __double2loint(r));  // -r / 2
+  const float s = to_f32(r);
+  const float t = fmaf(s * s * s, fmaf(s, fmaf(s, 0.2f, -0.25f), 1.f / 3.f), tab->kt[hi >> 20] + tab->yt[j]);
+  return (tab->k[hi >> 20] + tab->y[j]) + (fma(half, r, r) + to_f64(t));
 }
 
-// A line of the product rule: its place (u, v (1 - u)) in the simplex, its length w2, and the weights of its
-// sums A and B (see k_cell_loads_fh) against 1, lambda_1, lambda_2 and lambda_D.
+// A line of the product rule: the weights of the simplex's vertices in its points -- u and vv of vertices 1 and 2,
+// end[k] of vertex 0 and end[2 - k] of vertex D in point k -- and those of its sums A and B (see k_cell_loads_fh)
+// against lambda_1, lambda_2 and lambda_0 or lambda_D.
 struct FhLine {
-  double u, vv, w2, c, cu, cv, ca, cb;
+  double u, vv, end[3], cu, cv, ca, cb;
 };
 template <int D>
-__device__ __forceinline__ constexpr FhLine fh_line(int ij) {
-  constexpr double h = 0.38729833462074168852;  // sqrt(15) / 10
+constexpr FhLine fh_line(int ij) {
   const int i = D == 2 ? ij : ij / 3, j = ij % 3;
-  const double u = gl_x(i), w1 = 1.0 - u, v = D == 2 ? 0.0 : gl_x(j);
-  const double vv = v * w1, w2 = w1 * (1.0 - v);
-  const double c = (D == 2 ? 2.0 * gl_w(i) * w1 : 6.0 * gl_w(i) * gl_w(j) * w1 * w2) * gl_w(0);
-  return {u, vv, w2, c, c * u, c * vv, 0.5 * c * w2, c * w2 * h};
+  const double root = 3.8729833462074168852;  // sqrt(15), then its rest
+  const DD sq = dd_prod(root, root), h = dd_div({root, ((15.0 - sq.h) - sq.l) / (2.0 * root)}, {10.0, 0.0});
+  const DD one = {1.0, 0.0}, x[3] = {DD{0.5, 0.0} + DD{-h.h, -h.l}, {0.5, 0.0}, DD{0.5, 0.0} + h};
+  const DD u = x[i], w1 = one + DD{-u.h, -u.l}, v = D == 2 ? DD{0.0, 0.0} : x[j], vv = v * w1;
+  const DD w2 = w1 + DD{-vv.h, -vv.l};
+  DD c = DD{D == 2 ? 2.0 : 6.0, 0.0} * gl_w(i) * w1 * gl_w(0);
+  if (D == 3) c = c * gl_w(j) * w2;
+  const double gu = gl_grid(u.h), gv = gl_grid(vv.h), gw = (1.0 - gu) - gv, far = gl_grid((w2 * x[0]).h);
+  return {gu, gv, {gw - far, 0.5 * gw, far}, (c * u).h, (c * vv).h, 0.5 * (c * w2).h, (c * w2 * h).h};
 }
 struct FhLines {
   FhLine line[9];
@@ -942,21 +1036,17 @@ constexpr FhLines fh_lines() {
 }
 __constant__ FhLines c_fh_lines[2] = {fh_lines<2>(), fh_lines<3>()};
 
-// eload as k_cell_loads, f' of the Flory-Huggins energy by the product rule.  The terms of f' that are
-// linear in the concentrations are integrated exactly (the rule is exact for them); the rule takes the
-// logarithms' part
-//   g_p = ln phi_p / N_p - ln phi_s / N_s,  g_n = ln phi_n / N_n - ln phi_s / N_s,
-// along the innermost direction the hat functions are linear.  With the
-// logarithms L_0, L_1, L_2 of one concentration at a line's points, E = L_0 + L_2, A = E + 8/5 L_1 (5/18 A is
-// the line's integral) and B = L_2 - L_0 (its moment is 5/18 (A / 2 + h B), h = sqrt(15) / 10): 113 FP64
-// instructions for a line's nine logarithms against 121 with the weights applied point by point (144 a point
-// with the hat functions tabulated and CUDA's log).  128 x 128 x 32 cells: 19.5 ms at first, 7.1 ms point by point
-// and with seven-instruction logarithms, 6.3 ms now.  The three concentrations are summed apart and
-// combined at the end.  A thread takes a simplex; the simplices' corner values are added in shared memory in
-// simplex order, where the tables are as well.
+// eload as k_cell_loads, f' of the Flory-Huggins energy by the product rule: along the innermost direction the
+// hat functions are linear.  With f' at a line's points f_0, f_1, f_2, E = f_0 + f_2, A = E + 8/5 f_1 (5/18 A is
+// the line's integral) and B = f_2 - f_0 (its moment is 5/18 (A / 2 + h B), h = sqrt(15) / 10).  109 FP64
+// instructions for a line's nine logarithms and six values of f' (144 a point with the hat functions tabulated and
+// CUDA's log).  f' is summed up at each point, where its large terms cancel: the three logarithms' integrals, summed
+// apart and combined at the end, saved nine instructions a line and left three to six times the error.  128 x 128 x
+// 32 cells: 19.5 ms at first, 6.1 ms now.  A thread takes a simplex; the simplices' corner values are added in
+// shared memory in simplex order, where the tables are as well.
 // CB cells per block.  Three blocks of 192 threads per SM: 32 cells of six tetrahedra, 96 of two triangles
-// (512 x 512 387 us, 32 cells about 460); 2D meshes of at most two blocks of 32 cells per SM take those
-// (64 x 64 31.6 us, 96 cells 34).
+// (512 x 512 369 us, a fifth more with 32 cells); 2D meshes of at most two blocks of 32 cells per SM take those
+// (64 x 64 29 us, a tenth more with 96 cells).
 template <int D, int CB>
 constexpr int fh_smem() {
   return (int)(sizeof(LogTables) + sizeof(double2) * CellSimplices<D>::NT * (D + 1) * CB);
@@ -985,70 +1075,52 @@ __global__ void __launch_bounds__(CB* CellSimplices<D>::NT, 3) k_cell_loads_fh(c
         P[a] = pp[(size_t)ld * ev[a]];
         Q[a] = pn[(size_t)ld * ev[a]];
       }
-      double Lp[D + 1], Ln[D + 1], Ls[D + 1];  // the logarithms' integrals, [0]: against 1, [a]: against lambda_a
+      double Gp[D + 1], Gn[D + 1];
 #pragma unroll
-      for (int a = 0; a <= D; ++a) Lp[a] = Ln[a] = Ls[a] = 0.0;
+      for (int a = 0; a <= D; ++a) Gp[a] = Gn[a] = 0.0;
 #pragma unroll 1
       for (int ij = 0; ij < (D == 2 ? 3 : 9); ++ij) {
         const FhLine& q = c_fh_lines[D - 2].line[ij];
-        // positive weights only (u, v (1 - u), and w2 shared by the line's ends), so that small concentrations
-        // beside large ones keep their relative precision, which their logarithms need
-        const double pa = q.w2 * P[0], pb = q.w2 * P[D], na = q.w2 * Q[0], nb = q.w2 * Q[D];
+        // positive weights only, so that small concentrations beside large ones keep their relative precision,
+        // which their logarithms need
         double pc = q.u * P[1], nc = q.u * Q[1];
         if (D == 3) {
           pc = fma(q.vv, P[2], pc);
           nc = fma(q.vv, Q[2], nc);
         }
-        double p[3], n[3], r[3];
+        double fp[3], fn[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          p[k] = fma(gl_x(2 - k), pa, fma(gl_x(k), pb, pc));
-          n[k] = fma(gl_x(2 - k), na, fma(gl_x(k), nb, nc));
-          r[k] = 1.0 - p[k] - n[k];
+          const double p = fma(q.end[k], P[0], fma(q.end[2 - k], P[D], pc));
+          const double n = fma(q.end[k], Q[0], fma(q.end[2 - k], Q[D], nc));
+          const double ls = guarded_log1(1.0 - p - n, F.delta, tab);
+          fp[k] = fma(F.inv_np, guarded_log1(p, F.delta, tab),
+                      fma(-F.inv_ns, ls, fma(-2.0 * F.chi_ps, p, fma(F.mix, n, F.chi_ps))));
+          fn[k] = fma(F.inv_nn, guarded_log1(n, F.delta, tab),
+                      fma(-F.inv_ns, ls, fma(-2.0 * F.chi_ns, n, fma(F.mix, p, F.chi_ns))));
         }
-        const auto sums = [&](const double (&v)[3], double (&G)[D + 1]) {
-          const double l0 = guarded_log(v[0], F.delta, tab), l1 = guarded_log(v[1], F.delta, tab);
-          const double l2 = guarded_log(v[2], F.delta, tab);
-          const double A = fma(1.6, l1, l0 + l2), B = l2 - l0;
-          G[0] = fma(q.c, A, G[0]);
+        const auto sums = [&](const double (&f)[3], double (&G)[D + 1]) {
+          const double A = fma(1.6, f[1], f[0] + f[2]), B = f[2] - f[0];
+          G[0] = fma(q.ca, A, fma(-q.cb, B, G[0]));
           G[1] = fma(q.cu, A, G[1]);
           if (D == 3) G[2] = fma(q.cv, A, G[2]);
           G[D] = fma(q.ca, A, fma(q.cb, B, G[D]));
         };
-        sums(p, Lp);
-        sums(n, Ln);
-        sums(r, Ls);
+        sums(fp, Gp);
+        sums(fn, Gn);
       }
-      double Gp[D + 1], Gn[D + 1];
-#pragma unroll
-      for (int a = 0; a <= D; ++a) {
-        const double ls = Ls[a] * F.inv_ns;
-        Gp[a] = fma(Lp[a], F.inv_np, -ls);
-        Gn[a] = fma(Ln[a], F.inv_nn, -ls);
-      }
-#pragma unroll
-      for (int a = 1; a <= D; ++a) {  // lambda_0 = 1 - the others
-        Gp[0] -= Gp[a];
-        Gn[0] -= Gn[a];
-      }
-      // the linear part, f_p' = kp + lp phi_p + mp phi_n and f_n' alike: int lambda_i = 1 / (d+1),
-      // int phi lambda_i = (<phi> + phi_i) / ((d+1)(d+2)), in units of |T|
-      const double kp = F.inv_np - F.inv_ns + F.chi_ps, lp = -2.0 * F.chi_ps, mp = F.chi_pn - F.chi_ps - F.chi_ns;
-      const double kn = F.inv_nn - F.inv_ns + F.chi_ns, ln = F.chi_pn - F.chi_ps - F.chi_ns, mn = -2.0 * F.chi_ns;
-      constexpr double q1 = 1.0 / (D + 1), q2 = 1.0 / ((D + 1) * (D + 2));
+      // mix_lo int phi lambda_i = mix_lo (<phi> + phi_i) / ((d+1)(d+2)), in units of |T|
+      constexpr double q2 = 1.0 / ((D + 1) * (D + 2));
       double Sp = 0.0, Sq = 0.0;
 #pragma unroll
       for (int a = 0; a <= D; ++a) {
         Sp += P[a];
         Sq += Q[a];
       }
-      const double vol = m.vol[(size_t)cell * S::NT + t];
+      const double vol = m.vol[(size_t)cell * S::NT + t], lo = F.mix_lo * q2;
 #pragma unroll
-      for (int a = 0; a <= D; ++a) {
-        const double sp = q2 * (Sp + P[a]), sq = q2 * (Sq + Q[a]);
-        part[t][a][in] = make_double2(vol * (Gp[a] + fma(lp, sp, fma(mp, sq, kp * q1))),
-                                        vol * (Gn[a] + fma(ln, sp, fma(mn, sq, kn * q1))));
-      }
+      for (int a = 0; a <= D; ++a)
+        part[t][a][in] = make_double2(vol * fma(lo, Sq + Q[a], Gp[a]), vol * fma(lo, Sp + P[a], Gn[a]));
     }
     __syncthreads();
     for (int e = threadIdx.x; e < CB * S::NC; e += blockDim.x) {
@@ -1245,7 +1317,7 @@ static void cell_loads(const ch_system_s* s, const MeshPod& m, const LoadCoef& L
   const double bytes = C * (nc * (4.0 + 16.0 + 16.0) + 8.0);
   if (s->p.potential == 3) {
     const ch_params& p = s->p;
-    const FhCoef F{p.chi_pn, p.chi_ps, p.chi_ns, 1.0 / p.N_p, 1.0 / p.N_nfa, 1.0 / p.N_s, p.fh_delta};
+    const FhCoef F = fh_coef(p);
     ProfScope ps(st, K_ELEM_LOADS, 0, bytes, C * nt * (m.dim == 2 ? 9 : 27) * 38.0);
     const LogTables* tab = static_cast<const LogTables*>(s->log_tables);
     if (m.dim == 3)
