@@ -47,7 +47,6 @@ struct KrylovDev {
   int reorth[2];          // ... this Arnoldi step needs the second Gram-Schmidt pass
   int reorth_count[2];    // Arnoldi steps of this time step that took the second pass
   double hsq[2];          // ||w||^2 after both Gram-Schmidt passes (CGS2)
-  int corr32;             // the second pass's update may be formed in FP32 (k_orth_close)
 };
 
 // Preconditioned MINRES scalars of one run, per species (the Lanczos process on P^-1 A in the
@@ -337,7 +336,6 @@ __global__ void k_scale4(Seg sg, const double4_32a* src, double4_32a* dst, const
 // MODE 5: W -= sum_k h2[s][k] V_k;  ||W||_s^2, the column of the flagged species
 // Blocks of a run with no flagged species leave MODE 4 and 5 at entry.
 // <a, b>_s sums components (x, z) for species 0 and (y, w) for species 1 over the run's nodes.
-constexpr double ORTH_CORR32 = 0x1p-30;  // largest |h2_k| / ||W|| whose correction may be formed in FP32
 constexpr int KC = 16;                // basis vectors per chunk: 2 KC = 32 values, one per lane
 constexpr int ORTH_BLOCKS = 152 * 2;  // target grid of the segmented kernels (2 blocks per SM)
 // threads per block of the Gram-Schmidt passes; measured (ms per step, 512 x 512 FP64 / mixed /
@@ -613,17 +611,13 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
     if (MODE == 0 && norm && threadIdx.x < 2) kd->w2[threadIdx.x] = tot[2 * nv + threadIdx.x];
     if (MODE == 1 && threadIdx.x < 64) {  // warp s: ||W - V h2||_s^2 and 1 / h_{j+1,j} of species s
       const int sp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-      double q = 0.0, mx = 0.0;
+      double q = 0.0;
       for (int k = lane; k < nv; k += 32) {
         const double h = tot[2 * k + sp];
         q = fma(h, h, q);
-        mx = fmax(mx, fabs(h));
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        q += __shfl_xor_sync(0xffffffffu, q, o);
-        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      }
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
       if (lane == 0) {
         const double w2 = tot[2 * nv + sp];
         double hsq = w2 - q;
@@ -631,12 +625,7 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
         const double hn = sqrt(hsq);
         kd->hsq[sp] = hsq;
         kd->hinv[sp] = (kd->cycle_active[sp] && hn > 1e-300) ? 1.0 / hn : 0.0;
-        sm[sp] = (isfinite(w2) && isfinite(q) && mx <= ORTH_CORR32 * sqrt(w2)) ? 1.0 : 0.0;
       }
-    }
-    if (MODE == 1) {
-      __syncthreads();
-      if (threadIdx.x == 0) kd->corr32 = sm[0] != 0.0 && sm[1] != 0.0;
     }
     if (threadIdx.x == 0) kd->ticket = 0;
   } else {
@@ -680,25 +669,12 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
   }
 }
 
-// v rounded towards zero to FP32 by integer operations (the conversion instruction runs at the FP64
-// pipe's rate).  For |v| < 2^128; values below FP32's normal range come out as zero or denormal.
-__device__ __forceinline__ float trunc_f32(double v) {
-  const int hi = __double2hiint(v), lo = __double2loint(v);
-  const int e = max((hi & 0x7fffffff) - 0x38000000, 0);  // exponent bias 1023 -> 127
-  return __int_as_float((int)__funnelshift_l((unsigned)lo, (unsigned)e, 3) | (hi & 0x80000000));
-}
-
 // The end of CGS2: V_{j+1} = (W - sum_k h2[s][k] V_k) / h_{j+1,j} (0 for a species that sits out).  W
 // itself is not written: the next Arnoldi step overwrites it.  The blocks past the segments, one per
 // run, apply the column's Givens rotations meanwhile.
 //
-// h2 is the rounding error that the first projection left (1e-16 to 1e-14 of ||W||), so where every
-// |h2_k| <= 2^-30 ||W|| (kd->corr32) the correction V h2 is formed in FP32: its error, nv 2^-23 2^-30
-// ||W|| |V_k[v]|, is below the FP64 rounding of W, and the FP64 pipe (2 FMA per clock and SM, what
-// bounds these passes) is left with three instructions per component instead of nv + 2.  A larger h2
-// (a vector that lies almost in the span of the basis) or a non-finite value takes the FP64 sum.
-// Measured (512 x 512, 10 basis vectors on average): 20.6 us, where the FP64 update with its own norm
-// reduction and the scaling kernel after it took 43.6.
+// Bound by the FP64 pipe, which forming the correction in FP32 would leave idle (512 x 512 mixed 6.80 ms per
+// step, 7.19 in FP64); the basis is FP64's, so its correction is.
 __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth_close(Seg sg, int N, int nv, const double4_32a* __restrict__ V,
                                                             const double4_32a* __restrict__ W,
                                                             double4_32a* __restrict__ vnext, KrylovDev* kds) {
@@ -716,39 +692,17 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth_close(Seg sg, int N, int n
     return;
   }
   __shared__ double coef[2][MAXM + 1];
-  __shared__ float coef32[2][MAXM + 1];
   const KrylovDev* kd = kds + sg.run[blockIdx.x];
   for (int k = threadIdx.x; k < nv; k += blockDim.x) {
-    const double h0 = kd->h2[0][k], h1 = kd->h2[1][k];
-    coef[0][k] = h0;
-    coef[1][k] = h1;
-    coef32[0][k] = (float)h0;
-    coef32[1][k] = (float)h1;
+    coef[0][k] = kd->h2[0][k];
+    coef[1][k] = kd->h2[1][k];
   }
   const double s0 = kd->hinv[0], s1 = kd->hinv[1];
-  const bool c32 = kd->corr32 != 0;
   __syncthreads();
   const int v1 = sg.hi[blockIdx.x];
   for (int v = sg.lo[blockIdx.x] + threadIdx.x; v < v1; v += blockDim.x) {
     double4_32a w = W[v];
-    if (c32) {
-      float ax = 0.f, ay = 0.f, az = 0.f, aw = 0.f;
-#pragma unroll 4
-      for (int k = 0; k < nv; ++k) {
-        const double4_32a q = V[(size_t)k * N + v];
-        const float c0 = coef32[0][k], c1 = coef32[1][k];
-        ax = fmaf(c0, trunc_f32(q.x), ax);
-        ay = fmaf(c1, trunc_f32(q.y), ay);
-        az = fmaf(c0, trunc_f32(q.z), az);
-        aw = fmaf(c1, trunc_f32(q.w), aw);
-      }
-      w.x -= (double)ax;
-      w.y -= (double)ay;
-      w.z -= (double)az;
-      w.w -= (double)aw;
-    } else {
-      orth_update_value(V, w, (size_t)N, nv, coef, v);
-    }
+    orth_update_value(V, w, (size_t)N, nv, coef, v);
     vnext[v] = make_double4_32a(w.x * s0, w.y * s1, w.z * s0, w.w * s1);
   }
 }
@@ -1350,7 +1304,7 @@ static ch_status arnoldi_step(ch_state_s* S, int j, cudaStream_t st) {
       k_orth<1><<<nb, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, S->partials, S->kd);
     }
     {
-      ProfScope ps(st, K_ORTH2, 0, (nv + 2) * n32, 12.0 * N);
+      ProfScope ps(st, K_ORTH2, 0, (nv + 2) * n32, 4.0 * nv * N + 8.0 * N);
       k_orth_close<<<nb + S->R, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, V4 + (size_t)(j + 1) * N, S->kd);
     }
   }
