@@ -47,6 +47,7 @@ struct KrylovDev {
   int reorth[2];          // ... this Arnoldi step needs the second Gram-Schmidt pass
   int reorth_count[2];    // Arnoldi steps of this time step that took the second pass
   double hsq[2];          // ||w||^2 after both Gram-Schmidt passes (CGS2)
+  int renorm;             // that norm has to be summed (k_orth_close)
 };
 
 // Preconditioned MINRES scalars of one run, per species (the Lanczos process on P^-1 A in the
@@ -324,7 +325,8 @@ __global__ void k_scale4(Seg sg, const double4_32a* src, double4_32a* dst, const
 // Classical Gram-Schmidt twice (CGS2, gs_reorth = 0):
 // MODE 0: h1[s][k] = <V_k, W>_s                       k = 0..nv-1
 // MODE 1: W -= sum_k h1[s][k] V_k;  h2[s][k] = <V_k, W>_s and ||W||_s^2, hence the norm after the
-//         second projection, ||W - V h2||^2 = ||W||^2 - ||h2||^2 (V orthonormal)
+//         second projection, ||W - V h2||^2 = ||W||^2 - ||h2||^2 (V orthonormal) where ||h2||^2 is at
+//         most ORTH_SMALL ||W||^2: the difference then has the rounding of ||W||^2
 // then k_orth_close: V_{j+1} = (W - sum_k h2[s][k] V_k) / h_{j+1,j} and, beside it, the column's Givens
 // update.
 // Selective reorthogonalisation (gs_reorth = 1; Daniel, Gragg, Kaufman and Stewart 1976): MODE 0
@@ -336,6 +338,9 @@ __global__ void k_scale4(Seg sg, const double4_32a* src, double4_32a* dst, const
 // MODE 5: W -= sum_k h2[s][k] V_k;  ||W||_s^2, the column of the flagged species
 // Blocks of a run with no flagged species leave MODE 4 and 5 at entry.
 // <a, b>_s sums components (x, z) for species 0 and (y, w) for species 1 over the run's nodes.
+// (h2 is the first projection's rounding error, 1e-16 to 1e-12 of ||W||, unless W lies almost in the basis's
+// span, where the difference would cancel: k_orth_close then sums the norm)
+constexpr double ORTH_SMALL = 0x1p-20;
 constexpr int KC = 16;                // basis vectors per chunk: 2 KC = 32 values, one per lane
 constexpr int ORTH_BLOCKS = 152 * 2;  // target grid of the segmented kernels (2 blocks per SM)
 // threads per block of the Gram-Schmidt passes; measured (ms per step, 512 x 512 FP64 / mixed /
@@ -625,7 +630,12 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
         const double hn = sqrt(hsq);
         kd->hsq[sp] = hsq;
         kd->hinv[sp] = (kd->cycle_active[sp] && hn > 1e-300) ? 1.0 / hn : 0.0;
+        sm[sp] = q > ORTH_SMALL * w2 ? 1.0 : 0.0;
       }
+    }
+    if (MODE == 1) {
+      __syncthreads();
+      if (threadIdx.x == 0) kd->renorm = sm[0] + sm[1] > 0.0;
     }
     if (threadIdx.x == 0) kd->ticket = 0;
   } else {
@@ -671,16 +681,19 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
 
 // The end of CGS2: V_{j+1} = (W - sum_k h2[s][k] V_k) / h_{j+1,j} (0 for a species that sits out).  W
 // itself is not written: the next Arnoldi step overwrites it.  The blocks past the segments, one per
-// run, apply the column's Givens rotations meanwhile.
+// run, apply the column's Givens rotations meanwhile.  With kd->renorm the norm is summed here instead: V_{j+1}
+// is stored unscaled, and the run's last block has the norm, applies the rotations and scales the run's nodes
+// (alone: about a millisecond for a million nodes, where a basis is all but exhausted).
 //
 // Bound by the FP64 pipe, which forming the correction in FP32 would leave idle (512 x 512 mixed 6.80 ms per
 // step, 7.19 in FP64); the basis is FP64's, so its correction is.
 __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth_close(Seg sg, int N, int nv, const double4_32a* __restrict__ V,
                                                             const double4_32a* __restrict__ W,
-                                                            double4_32a* __restrict__ vnext, KrylovDev* kds) {
+                                                            double4_32a* vnext, double* partials, KrylovDev* kds) {
+  __shared__ ColumnStage cst;
   if ((int)blockIdx.x >= sg.nblocks) {
     KrylovDev* kd = kds + ((int)blockIdx.x - sg.nblocks);
-    __shared__ ColumnStage cst;
+    if (kd->renorm) return;
     stage_columns(kd, nv - 1, false, &cst);
     if (threadIdx.x < 2) {
       const int sp = threadIdx.x;
@@ -692,18 +705,52 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth_close(Seg sg, int N, int n
     return;
   }
   __shared__ double coef[2][MAXM + 1];
-  const KrylovDev* kd = kds + sg.run[blockIdx.x];
+  const int run = sg.run[blockIdx.x];
+  KrylovDev* kd = kds + run;
+  const bool renorm = kd->renorm != 0;
   for (int k = threadIdx.x; k < nv; k += blockDim.x) {
     coef[0][k] = kd->h2[0][k];
     coef[1][k] = kd->h2[1][k];
   }
-  const double s0 = kd->hinv[0], s1 = kd->hinv[1];
+  const double s0 = renorm ? 1.0 : kd->hinv[0], s1 = renorm ? 1.0 : kd->hinv[1];
   __syncthreads();
   const int v1 = sg.hi[blockIdx.x];
   for (int v = sg.lo[blockIdx.x] + threadIdx.x; v < v1; v += blockDim.x) {
     double4_32a w = W[v];
     orth_update_value(V, w, (size_t)N, nv, coef, v);
     vnext[v] = make_double4_32a(w.x * s0, w.y * s1, w.z * s0, w.w * s1);
+  }
+  if (!renorm) return;
+  __shared__ double sm[(ORTH_TPB / 32) * 32], tot[2], scale[2];
+  double acc[32];
+  acc[0] = acc[1] = 0.0;
+  for (int v = sg.lo[blockIdx.x] + threadIdx.x; v < v1; v += blockDim.x) {  // (the thread's own nodes)
+    const double4_32a w = vnext[v];
+    acc[0] = fma(w.x, w.x, fma(w.z, w.z, acc[0]));
+    acc[1] = fma(w.y, w.y, fma(w.w, w.w, acc[1]));
+  }
+  const double bt = block_sum_v<ORTH_TPB, 2>(acc, sm);
+  if (threadIdx.x < 2) partials[(size_t)blockIdx.x * MAXV + threadIdx.x] = bt;
+  const int b0 = sg.first[run], b1 = sg.first[run + 1];
+  if (!reduce_run(sg, partials, &kd->ticket, b0, b1, 2, tot)) return;
+  stage_columns(kd, nv - 1, false, &cst);
+  if (threadIdx.x < 2) {
+    const int sp = threadIdx.x;
+    if (cst.active[sp]) {
+      arnoldi_column(kd, sp, nv - 1, tot[sp], &cst, true);
+      kd->reorth_count[sp] = cst.rcount[sp] + 1;
+    } else {
+      kd->hinv[sp] = 0.0;
+    }
+    scale[sp] = kd->hinv[sp];
+  }
+  if (threadIdx.x == 0) kd->ticket = 0;
+  __syncthreads();
+  double2* o = reinterpret_cast<double2*>(vnext);
+  for (int v = sg.lo[b0] + threadIdx.x; v < sg.hi[b1 - 1]; v += blockDim.x) {
+    const double2 a = __ldcg(o + 2 * v), b = __ldcg(o + 2 * v + 1);  // past L1: other blocks wrote them
+    o[2 * v] = make_double2(a.x * scale[0], a.y * scale[1]);
+    o[2 * v + 1] = make_double2(b.x * scale[0], b.y * scale[1]);
   }
 }
 
@@ -1305,7 +1352,8 @@ static ch_status arnoldi_step(ch_state_s* S, int j, cudaStream_t st) {
     }
     {
       ProfScope ps(st, K_ORTH2, 0, (nv + 2) * n32, 4.0 * nv * N + 8.0 * N);
-      k_orth_close<<<nb + S->R, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, V4 + (size_t)(j + 1) * N, S->kd);
+      k_orth_close<<<nb + S->R, ORTH_TPB, 0, st>>>(S->seg, N, j + 1, V4, W4, V4 + (size_t)(j + 1) * N, S->partials,
+                                                       S->kd);
     }
   }
   CH_LAUNCHED();

@@ -42,7 +42,8 @@ extern "C" int orth_probe(int N, int nv, int blocks, const double* V, double* W,
   double4_32a* W4 = reinterpret_cast<double4_32a*>(W);
   k_orth<0><<<blocks, ORTH_TPB>>>(sg, N, nv, V4, W4, partials, kd);
   k_orth<1><<<blocks, ORTH_TPB>>>(sg, N, nv, V4, W4, partials, kd);
-  k_orth_close<<<blocks + 1, ORTH_TPB>>>(sg, N, nv, V4, W4, reinterpret_cast<double4_32a*>(vnext), kd);
+  k_orth_close<<<blocks + 1, ORTH_TPB>>>(sg, N, nv, V4, W4, reinterpret_cast<double4_32a*>(vnext), partials,
+                                         kd);
   CH_LAUNCHED();
   CH_CUDA(cudaDeviceSynchronize());
   CH_CUDA(cudaMemcpy(k.data(), kd, sizeof(KrylovDev), cudaMemcpyDeviceToHost));

@@ -73,3 +73,17 @@ def test_correction_is_fp64(probe, n, nv, blocks, kind):
         corr, size = h2[s] @ v, abs(h2[s]) @ abs(v)
         bound = U * ((nv / 2 + 4) * size + 3 * abs(w - corr)) * hinv[s]
         assert (abs(_species(got, s) - (w - corr) * np.longdouble(hinv[s])) <= bound).all()
+
+
+@pytest.mark.parametrize("n,nv,blocks,kind", [(4, 8, 1, "random"), (4, 7, 1, "random"), (40, 64, 3, "lean 1e-15"), (32, 64, 20, "random"),
+                                              (3000, 30, 20, "lean 0"), (3000, 30, 20, "lean 1e-12"), (3000, 30, 20, "random")])
+def test_the_next_vector_has_unit_length(probe, n, nv, blocks, kind):
+    """Also where the basis spans the space, or W to rounding, and the second projection takes most of what the
+    first left.  The norm is a sum of 2 n squares, its rounding below 1e-13.  h_{j+1,j} belongs to the column: with
+    earlier rotations that are identities the new entry of R is the hypotenuse of h_{j,j} and h_{j+1,j}."""
+    V, W = _vectors(n, nv, kind, seed=nv)
+    _, got, h1, h2, hinv, R = _run(probe, n, nv, blocks, V, W)
+    for s in (0, 1):
+        assert hinv[s] > 0.0
+        assert abs(np.linalg.norm(_species(got, s)) - 1.0) <= 1e-13
+        assert abs(R[s, nv - 1] / np.hypot(h1[s, nv - 1] + h2[s, nv - 1], 1.0 / hinv[s]) - 1.0) <= 1e-13
