@@ -848,13 +848,19 @@ struct ChebCoef {
 static ChebCoef cheb_coef(double rho, int deg, double lower);
 static ChebCoef cheb_coef_interval(double lo, double hi, int deg);
 
-// Tiles of a pass of `halo` operator applications over every run of a 2D mesh.  FP32 block heights by the
-// time they take in units of region rows, measured over 64 x 64 .. 1024 x 1024 and the 64-run batch (Algorithm
-// 1, us per application): a block alone on its SM costs its rows and 24 for its latencies, and as many waves as
-// there are, so a mesh that fits one wave takes the shortest block that does (512 x 512: 12 groups 186, 10
-// groups in two waves 215, pairs 206); larger meshes take two blocks of 8 groups per SM, which overlap
-// (a wave costs 80, and the last one only its share: 1024 x 1024 510, single blocks 518 to 595; batch 939,
-// 966 to 1100).  Fewer than 4 groups are too few warps to hide anything (256 x 256: 142, 4 groups 113).
+// Tiles of a pass of `halo` operator applications over every run of a 2D mesh, none where a launch per step is
+// faster.  FP32 block heights by the time they take in units of region rows, measured at degrees 1 to 16 over 256 x
+// 256 .. 2048 x 2048, 800 x 400, 4000 x 60, 33 x 2000 and 16- and 64-run batches: a block alone on its SM costs its
+// rows and 24 for its latencies, and as many waves as there are, so a mesh that fits one wave takes the shortest
+// block that does; small halos on larger meshes take two blocks of 8 groups per SM, which overlap (a wave costs
+// 62 and 10 per application -- a smaller region recomputes more -- and the last one only its share; vectors
+// beyond L2 wait longer for their loads, and the overlap is worth more: 80).  Algorithm 1, us per application, two
+// blocks / one: 1024 x 1024 degree 3 486 / 489, degree 8 726 / 685; 64 runs 909 / 926 and 1411 / 1308; 2048 x 2048
+// 1655 / 1730 and 2496 / 2420.  Fewer than 4 groups are too few warps to hide anything.
+// Tiles or steps: an application recomputes a tile's halo, so a step by tiles costs 1.3e-6 us per region node and a
+// launch over the mesh 1.1 us and 5.9e-6 per node (1e-5 beyond L2), 2 us at least.  Times by tiles / by steps:
+// 1024 x 1024 degree 5 546 / 714, 12 976 / 1159, 14 1255 / 1288, 15 1472 / 1357, 16 1754 / 1420; 64 runs degree 13
+// 1911 / 1923, 16 3226 / 2214; 256 x 256 degree 16 266 / 381.
 // FP64: the fewest region rows on the busiest SM.
 template <typename T>
 static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* out, cudaStream_t st) {
@@ -868,6 +874,7 @@ static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* o
     for (const ch_params& p : m->runs) n += (int64_t)((p.nx + tw) / tw) * ((p.ny + th) / th);
     return n;
   };
+  const bool far = m->N > 3000000;  // four vectors and more of FP32 pairs do not fit L2
   double best = 0.0;
   int G = 0;
   bool pair = false;
@@ -876,7 +883,8 @@ static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* o
     if (th < 1 || S::RW * g % 32 != 0) return;
     const int64_t n = count(th);
     const double waves = (double)((n + 151) / 152);
-    const double cost = two ? 80.0 * std::max(1.0, n / 304.0) : waves * (rh + (F32 ? 24 : 0));
+    const double cost =
+        two ? (far ? 80.0 : 62.0 + 10.0 * halo) * std::max(1.0, n / 304.0) : waves * (rh + (F32 ? 24 : 0));
     if (G == 0 || cost < best) {
       best = cost;
       G = g;
@@ -888,6 +896,8 @@ static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* o
   if (G == 0) return CH_OK;
   const int th = S::ROWS * G - 2 * halo;
   if (!F32 && count(th) > TILE_MAX_F64) return CH_OK;
+  const double step = far ? 1e-5 * m->N : std::max(2.0, 1.1 + 5.9e-6 * m->N);
+  if (F32 && 1.3e-6 * S::RW * S::ROWS * G * count(th) > step) return CH_OK;
   std::vector<LatTile> tiles;
   for (size_t r = 0; r < m->runs.size(); ++r) {
     const ch_params& p = m->runs[r];
