@@ -382,6 +382,7 @@ __global__ void __launch_bounds__(TC_M) k_conv3x3_tc(const __nv_bfloat16* __rest
 // pixels [b chunk, (b + 1) chunk) in FP64, thread-strided and then by a tree over its threads, into
 // part[smp][b][8]; k_ws_rms_fin adds a sample's block partials in block order.
 constexpr int WS_RMS_BLOCKS = 256;  // most blocks per sample of the first pass
+constexpr int RN_BLOCKS = 152;      // most blocks of a residual norm (k_ws_resnorm)
 
 // The four channels of pixel i (N x 4 node-major arrays): one vector load where the caller's array is
 // aligned for it (al: 32 bytes for fp64, 16 for fp32), four scalar loads otherwise.
@@ -1025,6 +1026,8 @@ ch_status ws_create(int H, int W, int Bmax, ch_ws_s** out) {
   if (r == CH_OK) r = w->mem.get(&w->part, nparts * (9 * WS_C * WS_C + WS_C));
   if (r == CH_OK) r = w->mem.get(&w->loss_part, 1024);
   if (r == CH_OK) r = w->mem.get(&w->rms_part, (size_t)Bmax * WS_RMS_BLOCKS * 8);
+  if (r == CH_OK) r = w->mem.get(&w->rn_part, (size_t)RN_BLOCKS * 8);
+  if (r == CH_OK) r = w->mem.get(&w->rn_ticket, 1);
   if (r == CH_OK) {
     if (cudaHostAlloc(&w->err_host, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer(&w->err_dev, w->err_host, 0) != cudaSuccess) {
@@ -1041,6 +1044,7 @@ ch_status ws_create(int H, int W, int Bmax, ch_ws_s** out) {
     cudaMemset(w->params, 0, sizeof(float) * WS_NPARAM);
     cudaMemset(w->adam_m, 0, sizeof(float) * WS_NPARAM);
     cudaMemset(w->adam_v, 0, sizeof(float) * WS_NPARAM);
+    cudaMemset(w->rn_ticket, 0, sizeof(unsigned int));
     const float nrm[20] = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1};
     if (cudaMemcpy(w->norm, nrm, sizeof(nrm), cudaMemcpyHostToDevice) != cudaSuccess) {
       set_error("warm-start initialisation failed");
@@ -1206,7 +1210,6 @@ __global__ void k_ws_sub(int P, const double4_32a* __restrict__ a, const double4
 // (or z = r for the plain norm), in a fixed order: block b adds its chunk of pixels into part[b][8]
 // and the last block to finish adds the blocks' sums in block order.  (One block over the whole
 // image took 222 us at 257 x 257, latency alone.)
-constexpr int RN_BLOCKS = 152;
 __global__ void __launch_bounds__(256) k_ws_resnorm(int P, const double4_32a* __restrict__ rex,
                                                     const double4_32a* __restrict__ zex,
                                                     const double4_32a* __restrict__ r,
@@ -1300,20 +1303,17 @@ ch_status ws_train_residual(ch_ws_s* w, const ch_system_s* sys, ch_precond_s* pc
     return CH_ERR_ARG;
   }
   const int P = w->P;
-  if (pc != nullptr && !w->zex) {
-    CH_TRY(w->mem.get(&w->zex, (size_t)P * 4));
-    CH_TRY(w->mem.get(&w->zr, (size_t)w->Bmax * P * 4));
+  // each buffer by itself: a call after one that ran out of memory allocates what is missing
+  const auto once = [&](double** buf, size_t n) { return *buf ? CH_OK : w->mem.get(buf, n); };
+  if (pc != nullptr) {
+    CH_TRY(once(&w->zex, (size_t)P * 4));
+    CH_TRY(once(&w->zr, (size_t)w->Bmax * P * 4));
   }
-  if (!w->rex) {
-    CH_TRY(w->mem.get(&w->rex, (size_t)w->Bmax * P * 4));
-    CH_TRY(w->mem.get(&w->rres, (size_t)w->Bmax * P * 4));
-    CH_TRY(w->mem.get(&w->tmp1, (size_t)P * 4));
-    CH_TRY(w->mem.get(&w->tmp2, (size_t)P * 4));
-    CH_TRY(w->mem.get(&w->nrm, (size_t)w->Bmax * 8));
-    CH_TRY(w->mem.get(&w->rn_part, (size_t)RN_BLOCKS * 8));
-    CH_TRY(w->mem.get(&w->rn_ticket, 1));
-    CH_CUDA(cudaMemsetAsync(w->rn_ticket, 0, sizeof(unsigned int), st));
-  }
+  CH_TRY(once(&w->rex, (size_t)w->Bmax * P * 4));
+  CH_TRY(once(&w->rres, (size_t)w->Bmax * P * 4));
+  CH_TRY(once(&w->tmp1, (size_t)P * 4));
+  CH_TRY(once(&w->tmp2, (size_t)P * 4));
+  CH_TRY(once(&w->nrm, (size_t)w->Bmax * 8));
   ws_rms<double>(w, x, q, q2, B, st);
   const bool al = aligned4(8, {x, q, q2});  // (a sample is a multiple of 32 bytes)
   k_ws_pack<double><<<dim3(blocks_for(P), B), TPB, 0, st>>>(x, q, q2, P, al, w->norm, w->norm + 8, w->dinv, w->x0);
