@@ -2261,11 +2261,8 @@ ch_status state_step_learned(ch_state_s* S, ch_ws_s* w, cudaStream_t st, ch_step
               H, W, H, W);
     return CH_ERR_ARG;
   }
-  if (!S->x_prev) {
-    CH_TRY(S->mem.get(&S->x_prev, (size_t)S->N * 4));
-    CH_TRY(S->mem.get(&S->x_prev2, (size_t)S->N * 4));
-    CH_TRY(S->mem.get(&S->guess, (size_t)S->N * 4));
-  }
+  for (double** buf : {&S->x_prev, &S->x_prev2, &S->guess})  // (a call after one that ran out of memory: the rest)
+    if (!*buf) CH_TRY(S->mem.get(buf, (size_t)S->N * 4));
   const bool use_net = S->learn_k >= 2 && S->since_set >= 3;
   CH_CUDA(cudaEventRecord(S->ev0, st));
   if (use_net) CH_TRY(ws_predict(w, S->x, S->x_prev, S->x_prev2, S->guess, st));
