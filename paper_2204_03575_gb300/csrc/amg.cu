@@ -1373,6 +1373,27 @@ struct LatRow {
   T a[ND + 1];
   int W, WH;
 };
+// a table row in 16-byte loads (rows are 32 to 128 bytes, aligned to their size), value by value into o
+template <int N>
+__device__ __forceinline__ void load_table_row(const float* __restrict__ src, float (&o)[N]) {
+#pragma unroll
+  for (int q = 0; q < N / 4; ++q) {
+    const float4 v = reinterpret_cast<const float4*>(src)[q];
+    o[4 * q] = v.x;
+    o[4 * q + 1] = v.y;
+    o[4 * q + 2] = v.z;
+    o[4 * q + 3] = v.w;
+  }
+}
+template <int N>
+__device__ __forceinline__ void load_table_row(const double* __restrict__ src, double (&o)[N]) {
+#pragma unroll
+  for (int q = 0; q < N / 2; ++q) {
+    const double2 v = reinterpret_cast<const double2*>(src)[q];
+    o[2 * q] = v.x;
+    o[2 * q + 1] = v.y;
+  }
+}
 template <typename T, int ND>
 __device__ __forceinline__ LatRow<T, ND> lat_row(const LatOp<T>& D, const T* __restrict__ tab, int i) {
   LatRow<T, ND> r;
@@ -1384,11 +1405,7 @@ __device__ __forceinline__ LatRow<T, ND> lat_row(const LatOp<T>& D, const T* __r
     r.W = w.x;
     r.WH = w.y;
   }
-  constexpr int NQ = (ND + 1) * (int)sizeof(T) / 16;  // 16-byte loads (rows are 32 to 128 bytes, aligned)
-  const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)id * (ND + 1));
-  uint4* dst = reinterpret_cast<uint4*>(r.a);
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) dst[q] = src[q];
+  load_table_row(tab + (size_t)id * (ND + 1), r.a);
   return r;
 }
 
@@ -1532,10 +1549,7 @@ __device__ __forceinline__ void smooth_tile(const TileArgs<T, V2>& a, const LatT
   constexpr bool OWN = ROWS == 1;  // the thread has one node, with its own row
   const int own = OWN && in(0) ? lat_id(a.L, (int)node0) : 0;
   const auto load_row = [&](const T* tab, int cy, T (&o)[8]) {
-    constexpr int NQ = 8 * (int)sizeof(T) / 16;
-    const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)(OWN ? own : tl.id0 + cx + 3 * cy) * 8);
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) reinterpret_cast<uint4*>(o)[q] = src[q];
+    load_table_row(tab + (size_t)(OWN ? own : tl.id0 + cx + 3 * cy) * 8, o);
   };
   const auto edge = [&](int t) { return y0 + t == 0 ? 0 : (y0 + t == tl.H - 1 ? 2 : 1); };
   T row[8];
