@@ -776,6 +776,27 @@ __device__ __forceinline__ void cell_nodes(const int* elems, int cell, int (&v)[
     }
 }
 
+// eload of the CB cells from c0 on: per corner the simplices' values (part[simplex][vertex][cell]) in simplex order
+template <int D, int CB>
+__device__ __forceinline__ void cell_sums(const double2 (*part)[D + 1][CB], int c0, int C, double2* __restrict__ eload) {
+  using S = CellSimplices<D>;
+  for (int e = threadIdx.x; e < CB * S::NC; e += blockDim.x) {
+    const int cl = e / S::NC, corner = e % S::NC;
+    if (c0 + cl >= C) continue;
+    double fp = 0.0, fn = 0.0;
+#pragma unroll
+    for (int q = 0; q < S::NT; ++q)
+#pragma unroll
+      for (int a = 0; a <= D; ++a)
+        if (S::corner(q, a) == corner) {
+          const double2 v = part[q][a][cl];
+          fp += v.x;
+          fn += v.y;
+        }
+    eload[((size_t)c0 + cl) * S::NC + corner] = make_double2(fp, fn);
+  }
+}
+
 struct LoadCoef {
   double cs;      // coefficient of phi_s in f' (0.2 for Eq. (15), 0 otherwise)
   double cubic;   // 7 for Eq. (15), 0 for f' = 0
@@ -796,13 +817,46 @@ struct LoadCoef {
 // thread takes a cell, so the products of the nodal values are formed once for its simplices and
 // there is one entry per corner instead of one per simplex and vertex (a third of the stores in 3D).
 template <int D>
+struct LoadScale {
+  static constexpr double c4 = (D == 2) ? 1.0 / 360.0 : 1.0 / 840.0;  // d!/(d+4)!
+  static constexpr double c2 = 1.0 / ((D + 1) * (D + 2));             // int lambda_a lambda_i / |T|, a != i
+};
+template <int D, typename F>
+__device__ __forceinline__ void simplex_loads(const double (&P)[D + 1], const double (&Q)[D + 1],
+                                              const double (&PQ)[D + 1], double c, double b, F add) {
+  const double c_2 = 2.0 * c, c_4 = 4.0 * c, c_6 = 6.0 * c;
+  double Sp = 0, Sq = 0, Spq = 0, Spp = 0, Sqq = 0, Spqq = 0, Sppq = 0;
+#pragma unroll
+  for (int a = 0; a <= D; ++a) {
+    Sp += P[a];
+    Sq += Q[a];
+    Spq += PQ[a];
+    Spp = fma(P[a], P[a], Spp);
+    Sqq = fma(Q[a], Q[a], Sqq);
+    Spqq = fma(PQ[a], Q[a], Spqq);
+    Sppq = fma(PQ[a], P[a], Sppq);
+  }
+  const double bs = b * ((D + 2) - Sp - Sq);  // b (<phi_s> + 1)
+  const double cSp = c * Sp, cSq = c * Sq, cpq = c_2 * Spq;
+  const double Ap = fma(c_2, Spqq, fma(cSp, fma(Sq, Sq, Sqq), cpq * Sq)) - bs;
+  const double An = fma(c_2, Sppq, fma(cSq, fma(Sp, Sp, Spp), cpq * Sp)) - bs;
+  const double Bp = fma(c, fma(Sq, Sq, Sqq), b), Bn = fma(c, fma(Sp, Sp, Spp), b);
+  const double C = fma(2.0 * cSp, Sq, cpq) + b;
+  const double Sp2 = 2.0 * cSp, Sq2 = 2.0 * cSq, Sp4 = c_4 * Sp, Sq4 = c_4 * Sq;
+#pragma unroll
+  for (int a = 0; a <= D; ++a) {
+    const double p = P[a], q = Q[a];
+    add(a, fma(p, fma(q, fma(c_6, q, Sq4), Bp), fma(q, fma(Sp2, q, C), Ap)),
+        fma(q, fma(p, fma(c_6, p, Sp4), Bn), fma(p, fma(Sq2, p, C), An)));
+  }
+}
+
+template <int D>
 __global__ void __launch_bounds__(128) k_cell_loads(const MeshPod m, LoadCoef L, const double* pp, const double* pn,
                                                     int ld, double2* __restrict__ eload) {
   using S = CellSimplices<D>;
   const int cell = blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= m.C) return;
-  constexpr double c4 = (D == 2) ? 1.0 / 360.0 : 1.0 / 840.0;  // d!/(d+4)!
-  constexpr double c2 = 1.0 / ((D + 1) * (D + 2));             // int lambda_a lambda_i / |T|, a != i
   int v[S::NC];
   cell_nodes<D>(m.elems, cell, v);
   double P[S::NC], Q[S::NC], PQ[S::NC], Fp[S::NC], Fn[S::NC];
@@ -814,39 +868,51 @@ __global__ void __launch_bounds__(128) k_cell_loads(const MeshPod m, LoadCoef L,
     Fp[a] = Fn[a] = 0.0;
   }
   const double vol = m.vol[(size_t)cell * S::NT];  // the cell's simplices are congruent
-  const double c = vol * L.cubic * c4, b = vol * L.cs * c2;
-  const double c_2 = 2.0 * c, c_4 = 4.0 * c, c_6 = 6.0 * c;
+  const double c = vol * L.cubic * LoadScale<D>::c4, b = vol * L.cs * LoadScale<D>::c2;
 #pragma unroll
   for (int t = 0; t < S::NT; ++t) {
-    double Sp = 0, Sq = 0, Spq = 0, Spp = 0, Sqq = 0, Spqq = 0, Sppq = 0;
+    double p[D + 1], q[D + 1], pq[D + 1];
 #pragma unroll
     for (int a = 0; a <= D; ++a) {
-      const int k = S::corner(t, a);
-      Sp += P[k];
-      Sq += Q[k];
-      Spq += PQ[k];
-      Spp = fma(P[k], P[k], Spp);
-      Sqq = fma(Q[k], Q[k], Sqq);
-      Spqq = fma(PQ[k], Q[k], Spqq);
-      Sppq = fma(PQ[k], P[k], Sppq);
+      p[a] = P[S::corner(t, a)];
+      q[a] = Q[S::corner(t, a)];
+      pq[a] = PQ[S::corner(t, a)];
     }
-    const double bs = b * ((D + 2) - Sp - Sq);  // b (<phi_s> + 1)
-    const double cSp = c * Sp, cSq = c * Sq, cpq = c_2 * Spq;
-    const double Ap = fma(c_2, Spqq, fma(cSp, fma(Sq, Sq, Sqq), cpq * Sq)) - bs;
-    const double An = fma(c_2, Sppq, fma(cSq, fma(Sp, Sp, Spp), cpq * Sp)) - bs;
-    const double Bp = fma(c, fma(Sq, Sq, Sqq), b), Bn = fma(c, fma(Sp, Sp, Spp), b);
-    const double C = fma(2.0 * cSp, Sq, cpq) + b;
-    const double Sp2 = 2.0 * cSp, Sq2 = 2.0 * cSq, Sp4 = c_4 * Sp, Sq4 = c_4 * Sq;
-#pragma unroll
-    for (int a = 0; a <= D; ++a) {
-      const int k = S::corner(t, a);
-      const double p = P[k], q = Q[k];
-      Fp[k] += fma(p, fma(q, fma(c_6, q, Sq4), Bp), fma(q, fma(Sp2, q, C), Ap));
-      Fn[k] += fma(q, fma(p, fma(c_6, p, Sp4), Bn), fma(p, fma(Sq2, p, C), An));
-    }
+    simplex_loads<D>(p, q, pq, c, b, [&](int a, double fp, double fn) {
+      Fp[S::corner(t, a)] += fp;
+      Fn[S::corner(t, a)] += fn;
+    });
   }
 #pragma unroll
   for (int a = 0; a < S::NC; ++a) eload[(size_t)cell * S::NC + a] = make_double2(Fp[a], Fn[a]);
+}
+
+// The same for meshes of few cells, a thread per simplex (32 cells and a warp per simplex of theirs in a block), whose
+// corner values are added in shared memory in simplex order: k_cell_loads' sums, bit for bit.  A warp's FP64
+// instructions hold its quarter of the SM 64 clocks each, so six tetrahedra one after another take 20 us however few
+// the cells: right-hand sides of 16 x 16 x 16 cells 33 us, 43 by cells.
+template <int D>
+__global__ void __launch_bounds__(32 * CellSimplices<D>::NT) k_cell_loads_split(const MeshPod m, LoadCoef L,
+                                                                                const double* pp, const double* pn,
+                                                                                int ld, double2* __restrict__ eload) {
+  using S = CellSimplices<D>;
+  __shared__ double2 part[S::NT][D + 1][32];
+  const int t = threadIdx.x >> 5, in = threadIdx.x & 31, cell0 = blockIdx.x * 32;
+  if (cell0 + in < m.C) {
+    const int* ev = m.elems + ((size_t)(cell0 + in) * S::NT + t) * (D + 1);
+    double P[D + 1], Q[D + 1], PQ[D + 1];
+#pragma unroll
+    for (int a = 0; a <= D; ++a) {
+      P[a] = pp[(size_t)ld * ev[a]];
+      Q[a] = pn[(size_t)ld * ev[a]];
+      PQ[a] = P[a] * Q[a];
+    }
+    const double vol = m.vol[(size_t)(cell0 + in) * S::NT];
+    simplex_loads<D>(P, Q, PQ, vol * L.cubic * LoadScale<D>::c4, vol * L.cs * LoadScale<D>::c2,
+                     [&](int a, double fp, double fn) { part[t][a][in] = make_double2(fp, fn); });
+  }
+  __syncthreads();
+  cell_sums<D, 32>(part, cell0, m.C, eload);
 }
 
 // ---- The Flory-Huggins load (potential = 3).  Section 2's bulk energy
@@ -1123,21 +1189,7 @@ __global__ void __launch_bounds__(CB* CellSimplices<D>::NT, 3) k_cell_loads_fh(c
         part[t][a][in] = make_double2(vol * fma(lo, Sq + Q[a], Gp[a]), vol * fma(lo, Sp + P[a], Gn[a]));
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < CB * S::NC; e += blockDim.x) {
-      const int cl = e / S::NC, corner = e % S::NC;
-      if (c0 + cl >= m.C) continue;
-      double fp = 0.0, fn = 0.0;
-#pragma unroll
-      for (int q = 0; q < S::NT; ++q)
-#pragma unroll
-        for (int a = 0; a <= D; ++a)
-          if (S::corner(q, a) == corner) {
-            const double2 v = part[q][a][cl];
-            fp += v.x;
-            fn += v.y;
-          }
-      eload[((size_t)c0 + cl) * S::NC + corner] = make_double2(fp, fn);
-    }
+    cell_sums<D, CB>(part, c0, m.C, eload);
     __syncthreads();  // before the next cells' values
   }
 }
@@ -1333,6 +1385,8 @@ static void cell_loads(const ch_system_s* s, const MeshPod& m, const LoadCoef& L
   ProfScope ps(st, K_ELEM_LOADS, 0, bytes, C * nt * (40.0 + 10.0 * d1));
   if (m.dim == 2)
     k_cell_loads<2><<<blocks_for(m.C, 128), 128, 0, st>>>(m, L, pp, pn, ld, s->eload);
+  else if (m.C <= 152 * 64)  // two warps of cells per SM, twelve of simplices
+    k_cell_loads_split<3><<<blocks_for(m.C, 32), 192, 0, st>>>(m, L, pp, pn, ld, s->eload);
   else
     k_cell_loads<3><<<blocks_for(m.C, 128), 128, 0, st>>>(m, L, pp, pn, ld, s->eload);
 }
