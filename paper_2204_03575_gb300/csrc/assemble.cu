@@ -798,8 +798,8 @@ __device__ __forceinline__ void cell_sums(const double2 (*part)[D + 1][CB], int 
 }
 
 struct LoadCoef {
-  double cs;      // coefficient of phi_s in f' (0.2 for Eq. (15), 0 otherwise)
-  double cubic;   // 7 for Eq. (15), 0 for f' = 0
+  double cs;      // coefficient of phi_s in f' (0.2 for Eq. (15), 0 otherwise) / ((d+1)(d+2))
+  double cubic;   // 7 for Eq. (15), 0 for f' = 0, times d!/(d+4)!
   int bc;         // boundary loads on/off
   double gp, gn, hp, hn, kev;
   const double* bw;  // patterned substrate weights (Fb x 2 x (D + D^2)), or null for p = 1
@@ -816,11 +816,6 @@ struct LoadCoef {
 // took 875 and 122 us.  A
 // thread takes a cell, so the products of the nodal values are formed once for its simplices and
 // there is one entry per corner instead of one per simplex and vertex (a third of the stores in 3D).
-template <int D>
-struct LoadScale {
-  static constexpr double c4 = (D == 2) ? 1.0 / 360.0 : 1.0 / 840.0;  // d!/(d+4)!
-  static constexpr double c2 = 1.0 / ((D + 1) * (D + 2));             // int lambda_a lambda_i / |T|, a != i
-};
 template <int D, typename F>
 __device__ __forceinline__ void simplex_loads(const double (&P)[D + 1], const double (&Q)[D + 1],
                                               const double (&PQ)[D + 1], double c, double b, F add) {
@@ -868,7 +863,7 @@ __global__ void __launch_bounds__(128) k_cell_loads(const MeshPod m, LoadCoef L,
     Fp[a] = Fn[a] = 0.0;
   }
   const double vol = m.vol[(size_t)cell * S::NT];  // the cell's simplices are congruent
-  const double c = vol * L.cubic * LoadScale<D>::c4, b = vol * L.cs * LoadScale<D>::c2;
+  const double c = vol * L.cubic, b = vol * L.cs;  // (common to the cell's nodes, as their roundings are)
 #pragma unroll
   for (int t = 0; t < S::NT; ++t) {
     double p[D + 1], q[D + 1], pq[D + 1];
@@ -908,7 +903,7 @@ __global__ void __launch_bounds__(32 * CellSimplices<D>::NT) k_cell_loads_split(
       PQ[a] = P[a] * Q[a];
     }
     const double vol = m.vol[(size_t)(cell0 + in) * S::NT];
-    simplex_loads<D>(P, Q, PQ, vol * L.cubic * LoadScale<D>::c4, vol * L.cs * LoadScale<D>::c2,
+    simplex_loads<D>(P, Q, PQ, vol * L.cubic, vol * L.cs,
                      [&](int a, double fp, double fn) { part[t][a][in] = make_double2(fp, fn); });
   }
   __syncthreads();
@@ -1296,10 +1291,10 @@ __device__ void node_loads(const MeshPod& m, const LoadCoef& L, const double2* _
   *Gn = gn;
 }
 
-static LoadCoef load_coef(const ch_params& p) {
+static LoadCoef load_coef(const ch_params& p, int dim) {
   LoadCoef L;
-  L.cubic = p.potential == 2 ? 0.0 : 7.0;
-  L.cs = p.potential == 0 ? 0.2 : 0.0;
+  L.cubic = p.potential == 2 ? 0.0 : 7.0 / (dim == 2 ? 360.0 : 840.0);
+  L.cs = p.potential == 0 ? 0.2 / (dim == 2 ? 12.0 : 20.0) : 0.0;
   L.bc = p.bc_mode;
   L.gp = p.g_p;
   L.gn = p.g_nfa;
@@ -1394,7 +1389,7 @@ static void cell_loads(const ch_system_s* s, const MeshPod& m, const LoadCoef& L
 ch_status loads(const ch_system_s* s, const double* pp, const double* pn, double* Fp, double* Fn,
                 double* gp, double* gn, cudaStream_t st) {
   const MeshPod m = mesh_pod(s->mesh);
-  LoadCoef L = load_coef(s->p);
+  LoadCoef L = load_coef(s->p, s->mesh->dim);
   L.bw = s->bw;
   cell_loads(s, m, L, pp, pn, 1, st);
   ProfScope ps(st, K_LOADS, 0, 16.0 * m.N + 32.0 * m.N, 0.0);
@@ -1409,7 +1404,7 @@ ch_status loads(const ch_system_s* s, const double* pp, const double* pn, double
 ch_status rhs_strided(const ch_system_s* s, const double* pp, const double* pn, int ld, double* b,
                       cudaStream_t st) {
   const MeshPod m = mesh_pod(s->mesh);
-  LoadCoef L = load_coef(s->p);
+  LoadCoef L = load_coef(s->p, s->mesh->dim);
   L.bw = s->bw;
   cell_loads(s, m, L, pp, pn, ld, st);
   // phi read + b written + M (values, columns, row pointers) + the cells' contributions gathered
