@@ -4,11 +4,11 @@ kernels): V_{j+1} = (W - V h2) / h_{j+1,j} in FP64, node by node, however small 
 Tolerance: the sum over nv terms runs in two halves of fused multiply-adds, then one addition, one subtraction
 and the scaling: (nv / 2 + 4) u sum |h2_k V_k| + 3 u |W - V h2| per entry, u = 2^-53, all divided by h_{j+1,j}."""
 import ctypes
-import os
-import subprocess
 
 import numpy as np
 import pytest
+
+import probes
 
 pytestmark = pytest.mark.gpu
 
@@ -18,14 +18,7 @@ MAXM = 64
 
 @pytest.fixture(scope="module")
 def probe(lib, tmp_path_factory):
-    from paper_2204_03575_gb300 import build
-    here, out = os.path.dirname(os.path.abspath(__file__)), str(tmp_path_factory.mktemp("probe") / "probe.so")
-    cmd = [build.nvcc(), *build.ARCH, *build.FLAGS, "-shared", "-o", out, os.path.join(here, "krylov_probe.cu"),
-           lib.LIB_PATH, "-Xlinker", "-rpath", "-Xlinker", os.path.dirname(lib.LIB_PATH)]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    assert r.returncode == 0, r.stderr
-    lib.lib()
-    f = ctypes.CDLL(out).orth_probe
+    f = probes.load(lib, "krylov_probe.cu", tmp_path_factory.mktemp("probe")).orth_probe
     f.argtypes = [ctypes.c_int] * 3 + [ctypes.c_void_p] * 4
     return f
 

@@ -2,25 +2,19 @@
 it are those of a state that never failed, bit for bit.  The failure is made on the host (learned_probe.cu compiles the
 library's own source with a counted allocator), one allocation after another."""
 import ctypes
-import os
-import subprocess
 
 import numpy as np
 import pytest
+
+import probes
 
 pytestmark = pytest.mark.gpu
 
 
 def test_the_next_call_after_a_failed_allocation(lib, tmp_path):
     import torch
-    from paper_2204_03575_gb300 import build, warmstart
-    here, out = os.path.dirname(os.path.abspath(__file__)), str(tmp_path / "probe.so")
-    cmd = [build.nvcc(), *build.ARCH, *build.FLAGS, "-shared", "-o", out, os.path.join(here, "learned_probe.cu"),
-           lib.LIB_PATH, "-Xlinker", "-rpath", "-Xlinker", os.path.dirname(lib.LIB_PATH)]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    assert r.returncode == 0, r.stderr
-    lib.lib()
-    probe = ctypes.CDLL(out).learned_probe
+    from paper_2204_03575_gb300 import warmstart
+    probe = probes.load(lib, "learned_probe.cu", tmp_path).learned_probe
     probe.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int] * 2 + [ctypes.c_void_p]
     nx, ny = 20, 17
     system = warmstart.make_system(nx, ny)

@@ -2,25 +2,18 @@
 allocates what is missing and returns the same loss and gradients as a network that never failed.  The failure is made on
 the host (warmstart_probe.cu compiles the library's own source with a counted allocator), one allocation after another."""
 import ctypes
-import os
-import subprocess
 
 import numpy as np
 import pytest
+
+import probes
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.fixture(scope="module")
 def probe(lib, tmp_path_factory):
-    from paper_2204_03575_gb300 import build
-    here, out = os.path.dirname(os.path.abspath(__file__)), str(tmp_path_factory.mktemp("probe") / "probe.so")
-    cmd = [build.nvcc(), *build.ARCH, *build.FLAGS, "-shared", "-o", out, os.path.join(here, "warmstart_probe.cu"),
-           lib.LIB_PATH, "-Xlinker", "-rpath", "-Xlinker", os.path.dirname(lib.LIB_PATH)]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    assert r.returncode == 0, r.stderr
-    lib.lib()
-    f = ctypes.CDLL(out).train_probe
+    f = probes.load(lib, "warmstart_probe.cu", tmp_path_factory.mktemp("probe")).train_probe
     f.argtypes = [ctypes.c_void_p] * 2 + [ctypes.c_int] * 3 + [ctypes.c_void_p] * 5 + [ctypes.c_int] + [ctypes.c_void_p] * 2
     return f
 
