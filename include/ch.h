@@ -203,8 +203,10 @@ ch_status ch_apply_A(const ch_system_t* s, const double* x, double* y, void* str
  * Builds, on the device, smoothed-aggregation AMG hierarchies for M and H (strength of
  * connection, MIS(2) aggregation, Jacobi-smoothed prolongator, Galerkin coarse operators,
  * dense inverse of the coarsest level), Chebyshev smoother bounds per level and, when
- * precision = 1, FP32 copies of every level.  On a uniform mesh (one run or a batch of them) the
- * finest level is also stored as one row per class of nodes.  The preconditioner owns a non-blocking
+ * precision = 1, FP32 copies of every level.  The finest level is also stored as one row per class of
+ * nodes with equal cell widths around them: the assembled rows bit for bit, in FP64 V-cycles as in the
+ * system's operator; FP32 V-cycles take the widths to be equal along each axis where the rows differ by
+ * less than 2^-36 of the diagonal, far below FP32's rounding.  The preconditioner owns a non-blocking
  * CUDA stream and two events on the current device: ch_precond_apply runs step 1 of Algorithm 1
  * on that stream, forked from and joined back into the caller's stream. */
 ch_status ch_precond_setup(const ch_system_t* s, void* stream, ch_precond_t** out);

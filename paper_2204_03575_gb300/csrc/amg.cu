@@ -56,8 +56,8 @@ template <> struct TileShape<float> { static constexpr int RW = 64, ROWS = 4, GM
 template <> struct TileShape<double> { static constexpr int RW = 16, ROWS = 1, GMAX = 16, GPAIR = 16; };
 // FP64 passes are bound by the FP64 pipe, where recomputed halo nodes cost as much as any: tiles only
 // while the mesh gives the chip at most two per SM and a step is a launch's latency (us per application
-// of Algorithm 1 with tiles / a launch per step: 32 x 32 88 / 131, 64 x 64 175 / 189, 96 x 96 with four
-// tiles per SM 256 / 192)
+// of Algorithm 1 with tiles / a launch per step: 32 x 32 90 / 146, 64 x 64 164 / 214; 96 x 96 with four
+// tiles per SM took a third more than by steps)
 constexpr int TILE_MAX_F64 = 304;
 struct TilePlan {
   int ntiles = 0;     // 0: the pass runs as one launch per step
@@ -1425,7 +1425,8 @@ __device__ __forceinline__ void lat_row_acc(const LatRow<T, ND>& r, int n, int i
 
 // One Chebyshev step on the lattice form: k_cheb_step's arithmetic.  FP32 is bound by its vectors (42 bytes
 // per row: x, b, e read and written, x' and the class id; one value per stored entry as well made it 72 in 2D,
-// 104 in 3D), FP64 by its pipe (ten instructions per right-hand side in 2D).
+// 104 in 3D), FP64 by its pipe (ten instructions per right-hand side in 2D).  A step with its launch, event-timed:
+// FP32 512 x 512 7.4 us, 3D 128 x 128 x 32 11.7, 64 runs 14.7; FP64 512 x 512 15.9.
 template <typename T, typename V2, int ND>
 __global__ void __launch_bounds__(TPB) k_cheb_step_lat(LatOp<T> D, int n, const V2* __restrict__ b,
                                                        const V2* __restrict__ x, V2* __restrict__ xo,
@@ -1487,8 +1488,8 @@ __global__ void __launch_bounds__(TPB) k_spmv2_lat(LatOp<T> D, int n, const V2* 
 //   ZERO: the pass starts from a zero guess (its first step is pointwise);  RES: r = b - A x' as well.
 // Nodes outside the mesh stay zero (their coefficients are zero).
 // Bound by the latencies of a block's loads and steps, not memory.  Algorithm 1 per application, us, one
-// launch per step -> per pass: FP32 64 x 64 77.8 -> 49, 256 x 256 143 -> 113, 512 x 512 247 -> 186, 1024 x
-// 1024 655 -> 510, 64 runs 1071 -> 939; FP64 32 x 32 131 -> 88, 64 x 64 189 -> 175.
+// launch per step -> per pass: FP32 64 x 64 141 -> 67, 256 x 256 183 -> 118, 512 x 512 268 -> 197, 1024 x
+// 1024 695 -> 532, 64 runs 1138 -> 969; FP64 32 x 32 146 -> 90, 64 x 64 214 -> 164.
 template <typename T, typename V2>
 struct TileArgs {
   const LatTile* tiles;

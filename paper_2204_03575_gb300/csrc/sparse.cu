@@ -20,8 +20,8 @@ void set_error(const char* fmt, ...) {
 const char* last_error() { return g_err.c_str(); }
 
 // ---------------------------------------------------------------- exclusive scan
-// Row pointers from counts: tile sums, their scan (int64, recursive for more than one tile of tiles),
-// then the tiles' own scans on top.
+// Row pointers from counts: tile sums, their scan (int64, one block, tile after tile), then the tiles' own
+// scans on top.
 constexpr int SCAN_IT = 4;
 constexpr int SCAN_TILE = TPB * SCAN_IT;
 

@@ -130,3 +130,26 @@ def test_fp64_smoothing_has_the_assembled_rows(lib, kw, which):
     want = _vcycle(levels, bl, np.zeros(b.shape, np.longdouble))
     got = pc.vcycle(which, bd).cpu().numpy()
     assert float(abs(got - want).max()) <= 16 * U * float(abs(want).max())
+
+
+def test_fp32_cycles_of_a_long_thin_grid(lib):
+    """400000 x 1 cells: the rows of one position differ by more than 2^-36 of the diagonal, and FP32 V-cycles take the
+    classes by cell widths, a launch per step (the lattice form counts 2 bytes of class id per node and its vectors).  Against
+    the oracle to the bound of the other FP32 V-cycle tests."""
+    import torch
+    from oracle import ch_oracle as o
+    from test_zy_vcycle_oracle import TOL, _exported, _oracle_levels
+    system, _ = _system(lib, dict(nx=400000, ny=1), precision=1)
+    pc = lib.Precond(system)
+    levels = _oracle_levels(_exported(pc, 0))
+    degree, n = levels[0]["degree"], system.n
+    b = np.random.default_rng(4).standard_normal((n, 2))
+    bd = torch.from_numpy(b).cuda()
+    lib.profile_read(reset=True)
+    got = pc.vcycle(0, bd).cpu().numpy()
+    step = lib.profile_read(reset=True)["cheb_step_f32"]
+    assert step["launches"] == 2 * degree - 1
+    assert step["bytes"] <= (2.0 + 4.0 * 10) * n * step["launches"]
+    for k in range(2):
+        want = o.vcycle(levels, b[:, k])
+        assert np.abs(got[:, k] - want).max() / np.abs(want).max() <= TOL[1]
