@@ -689,6 +689,30 @@ def top_kernels(prof, n=8):
     return out
 
 
+# what the printed line keeps of the sections whose full form goes to stderr
+SECTION_KEYS = {
+    "roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac", "peak_source", "share_of_kernel_time",
+                 "avg_launch_us", "traffic"),
+    "mixed": ("value", "ms_per_step", "iters_per_step_mean", "max_rel_diff_phi_vs_fp64_form_after_run"),
+    "batch": ("runs", "nodes", "run_steps_per_s", "ms_per_step", "launches_per_step", "max_relres_last_step"),
+    "cpu_baseline": ("value", "unit", "cores", "host_cores", "kind", "sample"),
+    "learned": ("selected", "fp64", "mixed", "mixed_learned_over_fp64_previous_state"),
+    "fine_smoother_hbm_bound": ("avg_launch_us", "achieved_GBps", "frac_hbm"),
+}
+DETAIL_ONLY = ("top_kernels", "configs", "variants", "eoc_tau", "morphology_projection")
+
+
+def stdout_line(line):
+    """The JSON line for stdout: the measurement and its context, 3 to 4 kB.  Readers that keep the tail of a run's
+    output cut a line of 20 kB; the sections in full are on stderr ("bench detail: ")."""
+    out = {k: v for k, v in line.items() if k not in DETAIL_ONLY}
+    for name, keys in SECTION_KEYS.items():
+        if isinstance(out.get(name), dict):
+            out[name] = {k: out[name][k] for k in keys if k in out[name]}
+    out["detail"] = "stderr"
+    return out
+
+
 def main():
     args = parse()
     rank = int(os.environ.get("RANK", "0"))
@@ -912,7 +936,8 @@ def main():
         "cpu_baseline": cpu,
     }
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print("bench detail: " + json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(stdout_line(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
