@@ -1425,8 +1425,8 @@ __device__ __forceinline__ void lat_row_acc(const LatRow<T, ND>& r, int n, int i
 
 // One Chebyshev step on the lattice form: k_cheb_step's arithmetic.  FP32 is bound by its vectors (42 bytes
 // per row: x, b, e read and written, x' and the class id; one value per stored entry as well made it 72 in 2D,
-// 104 in 3D), FP64 by its pipe (ten instructions per right-hand side in 2D).  A step with its launch, event-timed:
-// FP32 512 x 512 7.4 us, 3D 128 x 128 x 32 11.7, 64 runs 14.7; FP64 512 x 512 15.9.
+// 104 in 3D), FP64 by its pipe (ten instructions per right-hand side in 2D).  FP32 128 x
+// 128 x 32 8.7 us, FP64 512 x 512 11.8.
 template <typename T, typename V2, int ND>
 __global__ void __launch_bounds__(TPB) k_cheb_step_lat(LatOp<T> D, int n, const V2* __restrict__ b,
                                                        const V2* __restrict__ x, V2* __restrict__ xo,

@@ -1451,8 +1451,9 @@ __global__ void k_apply_A(int N, const int* rowptr, const int* col, const double
 }
 
 // The lattice form: no indices or values but the class id, so the FP64 pipe alone bounds it (54 or 94
-// instructions per node).  512 x 512: 29.3 us, 33.6 in CSR form; 3D 128 x 128 x 32: 93, 127 in
-// CSR form.  Several classes along an axis cost little: 511 x 509 29.3, 127 x 129 x 33 95.
+// instructions per node).  512 x 512: 27.3 us, 33.6 in CSR form; 3D 128 x 128 x 32: 91, 127 in
+// CSR form.  Several classes along an axis cost little (in a run of launches: 512 x 512 and 511 x 509 29.3 us, 128 x
+// 128 x 32 93 and 127 x 129 x 33 95).
 template <int ND>
 __global__ void __launch_bounds__(128) k_apply_A_lat(LatOperator A, int N, const double4_32a* __restrict__ x,
                                                      double4_32a* __restrict__ y) {

@@ -291,7 +291,7 @@ __global__ void k_residual4(Seg sg, const int* rowptr, const int* col, const dou
 }
 
 // k_residual4 with the operator in lattice form (lat_apply_A), two nodes per iteration so that both rows'
-// gathers are in flight.  512 x 512: 49 us, 53 in CSR form; 3D 128 x 128 x 32: 120, 161 in CSR form.
+// gathers are in flight.  512 x 512: 47 us, 53 in CSR form; 3D 128 x 128 x 32: 118, 161 in CSR form.
 template <int ND>
 __global__ void __launch_bounds__(TPB, 2) k_residual4_lat(Seg sg, LatOperator A, const double4_32a* __restrict__ x,
                                                           const double4_32a* __restrict__ b, double4_32a* __restrict__ W,
@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth(Seg sg, int N, int nv, con
 // (alone: about a millisecond for a million nodes, where a basis is all but exhausted).
 //
 // Bound by the FP64 pipe, which forming the correction in FP32 would leave idle (512 x 512 mixed 6.80 ms per
-// step, 7.05 in FP64); the basis is FP64's, so its correction is.  36 us at 512 x 512, 10 vectors on average.
+// step, 7.05 in FP64); the basis is FP64's, so its correction is.  32 us at 512 x 512 with 10 vectors on average.
 __global__ void __launch_bounds__(ORTH_TPB, 2) k_orth_close(Seg sg, int N, int nv, const double4_32a* __restrict__ V,
                                                             const double4_32a* __restrict__ W,
                                                             double4_32a* vnext, double* partials, KrylovDev* kds) {
