@@ -98,7 +98,6 @@ struct Hierarchy {
   double cheb_lower = 0.3;
   int autotune = 1;
   bool pdl = true;
-  double* lat_tab = nullptr;          // FP64 table of the finest level's lattice form (null: CSR form)
   Alloc mem;
 };
 
@@ -845,8 +844,6 @@ struct ChebCoef {
   double invtheta, from_x;
   double carry[16], beta[16];
 };
-static ChebCoef cheb_coef(double rho, int deg, double lower);
-static ChebCoef cheb_coef_interval(double lo, double hi, int deg);
 
 // Tiles of a pass of `halo` operator applications over every run of a 2D mesh, none where a launch per step is
 // faster.  FP32 block heights by the time they take in units of region rows, measured at degrees 1 to 16 over 256 x
@@ -917,12 +914,8 @@ static ch_status tile_plan(const ch_mesh_s* m, int halo, Alloc& mem, TilePlan* o
   return CH_OK;
 }
 
-static int semi_steps(const ch_params& p) { return p.cheb_M_steps > 0 ? p.cheb_M_steps : 5; }
-// Wathen's bounds of the eigenvalues of D^-1 M: [1/2, 2] (triangles), [1/2, 5/2] (tetrahedra)
-static ChebCoef semi_coef(int dim, int steps) { return cheb_coef_interval(0.5, dim == 2 ? 2.0 : 2.5, steps); }
-
 template <typename T>
-static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, const ch_params& p, std::vector<LevelT<T>>& L,
+static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, std::vector<LevelT<T>>& L,
                               cudaStream_t st) {
   using V2 = typename V2T<T>::t;
   L.resize(h->nlev);
@@ -977,13 +970,14 @@ static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, const ch_para
   // the fine level in lattice form (LatOp)
   constexpr bool F32 = sizeof(T) == 4;
   const Lattice* lat = F32 ? &mesh->pos : &mesh->lat;
-  CH_TRY(lat_build(h->A[0], lat, F32 ? 0x1p-36 : 0.0, h->mem, &h->lat_tab, st));
-  const bool by_position = F32 && h->lat_tab;
-  if (F32 && !h->lat_tab) {
+  double* tab64 = nullptr;
+  CH_TRY(lat_build(h->A[0], lat, F32 ? 0x1p-36 : 0.0, h->mem, &tab64, st));
+  const bool by_position = F32 && tab64;
+  if (F32 && !tab64) {
     lat = &mesh->lat;
-    CH_TRY(lat_build(h->A[0], lat, 0.0, h->mem, &h->lat_tab, st));
+    CH_TRY(lat_build(h->A[0], lat, 0.0, h->mem, &tab64, st));
   }
-  if (h->lat_tab) {
+  if (tab64) {
     LatOp<T>& op = L[0].lat;
     op.nd = lat->dim == 2 ? 7 : 15;
     op.ts = op.nd + 1;
@@ -991,7 +985,7 @@ static ch_status make_working(Hierarchy* h, const ch_mesh_s* mesh, const ch_para
     const int cnt = lat->nids * op.ts;
     T* tab = nullptr;
     CH_TRY(h->mem.get(&tab, (size_t)cnt));
-    k_lat_cast<T><<<blocks_for(cnt), TPB, 0, st>>>(h->lat_tab, tab, cnt);
+    k_lat_cast<T><<<blocks_for(cnt), TPB, 0, st>>>(tab64, tab, cnt);
     op.tab = tab;
     CH_LAUNCHED();
     if (lat->dim == 2 && h->nlev > 1 && (by_position || !F32)) {
@@ -1070,9 +1064,9 @@ ch_status hierarchy_build(const Csr<double>& A0, const ch_mesh_s* mesh, const ch
   }
   if (s == CH_OK) {
     if (precision == 0) {
-      s = make_working<double>(h, mesh, p, h->Ld, st);
+      s = make_working<double>(h, mesh, h->Ld, st);
     } else {
-      s = make_working<float>(h, mesh, p, h->Lf, st);
+      s = make_working<float>(h, mesh, h->Lf, st);
       if (s == CH_OK) s = h->mem.get(&h->cinvf, (size_t)h->nc * h->nc);
       if (s == CH_OK) {
         k_d2f<<<blocks_for((int64_t)h->nc * h->nc), TPB, 0, st>>>(h->cinv, h->cinvf,
@@ -1366,8 +1360,8 @@ __global__ void __launch_bounds__(TPB) k_spmv2(Csr<T> A, X x, V2* __restrict__ y
 
 // ---------------------------------------------------------------- structured (lattice) fine level
 // One row of the lattice form: the class's ND values and factor and its run's strides (set-up data, so
-// the kernels read them before their dependency wait).  Rows of a warp are almost always of one class:
-// the table reads are broadcasts from L1.
+// the kernels read them before their dependency wait).  Rows of a warp are of one class by position,
+// of two to four by inexact widths: the table reads are broadcasts from L1.
 template <typename T, int ND>
 struct LatRow {
   T a[ND + 1];
@@ -1915,6 +1909,10 @@ static ChebCoef cheb_coef(double rho, int deg, double lower) {
   const double hi = 1.1 * rho;
   return cheb_coef_interval(lower * hi, hi, deg);
 }
+
+static int semi_steps(const ch_params& p) { return p.cheb_M_steps > 0 ? p.cheb_M_steps : 5; }
+// Wathen's bounds of the eigenvalues of D^-1 M: [1/2, 2] (triangles), [1/2, 5/2] (tetrahedra)
+static ChebCoef semi_coef(int dim, int steps) { return cheb_coef_interval(0.5, dim == 2 ? 2.0 : 2.5, steps); }
 
 // the tile kernels' shared-memory limits (above the 48 KB default)
 template <typename T>
